@@ -124,6 +124,8 @@ void free_ctx(Ctx& c) {
     delete[] c.prof_sites;
     c.prof_sites = nullptr;
   }
+  cudaFree(c.pp_taps);
+  cudaFree(c.pp_ctrl);
   cudaFree(c.run_rho);
   cudaFree(c.run_T);
   void* ptrs[] = {c.fixed, c.efix, c.gfix, c.q, c.rho_phys, c.ke, c.ke0, c.ke_f, c.ke0_f, c.inv_hs, c.inv_hs_df, c.rho_phys_df, c.f_offs, c.f_w,
@@ -413,6 +415,7 @@ int mgar_create(mgar_t* out, const mgar_params* p, const uint8_t* fixed_mask, co
     MGAR_CUDA(cudaMemcpy(c->q, qh.data(), n * sizeof(double), cudaMemcpyHostToDevice));
     alloc_hierarchy(*c);
     setup_filter(*c);
+    setup_postprocess(*c);
     if (P.precision == MGAR_MIXED) {
       q_to_df(*c);
       MGAR_CUDA(cudaStreamSynchronize(c->stream));

@@ -215,6 +215,11 @@ struct Ctx {
   unsigned long long seq_sent = 0;
   int* derr = nullptr;               // device error flag
 
+  // post-processing: the projection's taps and the level search's counters
+  void* pp_taps = nullptr;
+  int pp_ntaps = 0;
+  void* pp_ctrl = nullptr;
+
   // whole-run buffers (mgar_run)
   double *run_rho = nullptr, *run_T = nullptr;
 
@@ -988,6 +993,7 @@ void set_density(Ctx& c, const double* rho, bool physical);
 // instead of FP64 (dc may then be null)
 void sensitivity(Ctx& c, const double* T, double* dc, double* dv, double* compliance,
                  const float2* T_df = nullptr, float2* dc_df = nullptr);
+void setup_postprocess(Ctx& c);
 void postprocess(Ctx& c, const double* rho, const double* T, double volfrac, double* rho_out,
                  double* level_out, double* volume_out);
 // dc_df: dc as double-float pairs (then dc is not read)

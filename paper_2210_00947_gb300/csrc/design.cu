@@ -957,29 +957,389 @@ void oc_update(Ctx& c, double* rho, const double* dc, double volfrac, double mov
 
 constexpr int kPpLattice = 4;  // S: lattice intervals per axis
 
+// One element-to-node weight of the projection: the element at offset (x, y,
+// z) from the node, w = r - |centroid offset| > 0.
+struct PpTap {
+  int x, y, z;
+  double w;
+};
+
+// ns at every node, with its FP32 copy, and a flag when a value is not in
+// [0, 1e37] (then the level search below does not apply).  The taps come as a
+// list of the positive weights in the order x, y, z: forming all 8 reach^3
+// candidate weights per node instead, a square root each, took 4.1 ms on
+// 128^3 with 8 taps of 64 in use, and 0.1 ms as a list.
 template <int DIM>
-__global__ void k_pp_nodal(const double* __restrict__ dcp, double* __restrict__ ns, Dims d,
-                           double r, int reach) {
+__global__ void k_pp_nodal(const double* __restrict__ dcp, double* __restrict__ ns,
+                           float* __restrict__ ns32, Dims d, const PpTap* __restrict__ taps,
+                           int ntaps, int* __restrict__ bad) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int)d.n) return;
   int i, j, k;
   coords(idx, d.fNX, d.fNXY, i, j, k);
   double num = 0.0, den = 0.0;
-  // element (i + ox, j + oy, k + oz) has its centroid at offset o + 1/2
-  for (int ox = -reach; ox < reach; ++ox)
-    for (int oy = -reach; oy < reach; ++oy)
-      for (int oz = (DIM == 3 ? -reach : 0); oz < (DIM == 3 ? reach : 1); ++oz) {
-        const double dz = DIM == 3 ? oz + 0.5 : 0.0;
-        const double w = r - sqrt((ox + 0.5) * (ox + 0.5) + (oy + 0.5) * (oy + 0.5) + dz * dz);
-        const int ei = i + ox, ej = j + oy, ek = k + oz;
-        if (w <= 0.0 || ei < 0 || ei >= d.ex || ej < 0 || ej >= d.ey || ek < 0 || ek >= d.ez)
-          continue;
-        const int e = ei + d.ex * (ej + d.ey * ek);
-        if (!CK(e, d.ne)) continue;
-        num += w * -dcp[e];
-        den += w;
+  for (int o = 0; o < ntaps; ++o) {
+    const PpTap t = taps[o];
+    const int ei = i + t.x, ej = j + t.y, ek = k + t.z;
+    if (ei < 0 || ei >= d.ex || ej < 0 || ej >= d.ey || ek < 0 || ek >= d.ez) continue;
+    const int e = ei + d.ex * (ej + d.ey * ek);
+    if (!CK(e, d.ne)) continue;
+    num += t.w * -dcp[e];
+    den += t.w;
+  }
+  const double v = num / den;
+  ns[idx] = v;
+  ns32[idx] = (float)v;
+  if (!(v >= 0.0 && v <= 1e37)) *bad = 1;
+}
+
+// ---- The level without a pass per bisection step ------------------------
+// The mean density at a level L is the share of all lattice points (S+1)^d
+// per element whose value exceeds L.  So the bisection's answers follow from
+// counts of points, which these kernels take from few passes:
+//   two histogram passes over the points' FP32 values (as bit patterns, which
+//   order non-negative floats) find the bracket that holds the level, 384
+//   ulps wide; one pass counts the points above it and lists the FP64 values
+//   of those inside (a few thousand); one block then runs the bisection on
+//   that list, step for step with the same midpoints.
+// An FP32 value is within 8 ulps of the FP64 one (positive weights, seven
+// roundings), so every bracket is widened by kPpGuard ulps and a point outside
+// the last one is on the same side of every level in it in either precision.
+// A volume per bisection step instead, 62 passes at 4.6 ms on 128^3 (FP64-bound:
+// up to 5000 FP64 operations per element), took 290 ms; this takes 1.4 ms with
+// the projection, bound by the shared-memory atomics of the first histogram.
+constexpr int kPpBins = 4096;
+constexpr unsigned kPpGuard = 64;
+constexpr int kPpShift1 = 19, kPpShift2 = 8;  // bits per bin: 2^31 in 4096 bins, then 2^19 in 2050
+
+struct PpCtrl {
+  unsigned long long hist[2][kPpBins];
+  unsigned long long above[3];  // points past the bracket of each histogram pass and of the listing
+  unsigned lo[3], hi[3];        // bracket (bit patterns, inclusive) of each pass
+  int nlist;
+  int bad;
+};
+
+// The FP32 values of an element's lattice points, clamped to its corners'
+// range: f(value, px, py, pz).
+template <int DIM, class F>
+__device__ __forceinline__ void pp_points32(const float (&t)[1 << DIM], float tmin, float tmax, F&& f) {
+  constexpr int P = kPpLattice + 1;
+#pragma unroll 1
+  for (int px = 0; px < P; ++px) {
+    const float u = px * (1.f / kPpLattice), u1 = 1.f - u;
+    float a[1 << (DIM - 1)];
+#pragma unroll
+    for (int q = 0; q < (1 << (DIM - 1)); ++q) a[q] = fmaf(u, t[2 * q + 1], u1 * t[2 * q]);
+#pragma unroll
+    for (int py = 0; py < P; ++py) {
+      const float v = py * (1.f / kPpLattice), v1 = 1.f - v;
+      float b[1 << (DIM - 2)];
+#pragma unroll
+      for (int q = 0; q < (1 << (DIM - 2)); ++q) b[q] = fmaf(v, a[2 * q + 1], v1 * a[2 * q]);
+#pragma unroll
+      for (int pz = 0; pz < (DIM == 3 ? P : 1); ++pz) {
+        const float w = pz * (1.f / kPpLattice), w1 = 1.f - w;
+        const float s = DIM == 3 ? fmaf(w, b[DIM == 3 ? 1 : 0], w1 * b[0]) : b[0];
+        f(fminf(fmaxf(s, tmin), tmax), px, py, pz);
       }
-  ns[idx] = num / den;
+    }
+  }
+}
+
+// The FP64 value of one lattice point, the corners in order (as k_pp_density).
+template <int DIM>
+__device__ __forceinline__ double pp_value(const double (&t)[1 << DIM], int px, int py, int pz) {
+  constexpr int nen = 1 << DIM;
+  const double xi = -1.0 + 2.0 * px / kPpLattice;
+  const double eta = -1.0 + 2.0 * py / kPpLattice;
+  const double zeta = DIM == 3 ? -1.0 + 2.0 * pz / kPpLattice : 0.0;
+  double s = 0.0;
+#pragma unroll
+  for (int a = 0; a < nen; ++a) {
+    const double lx = 2 * (a & 1) - 1, ly = 2 * ((a >> 1) & 1) - 1, lz = 2 * ((a >> 2) & 1) - 1;
+    double nval = (1.0 + xi * lx) * (1.0 + eta * ly);
+    if (DIM == 3) nval *= (1.0 + zeta * lz);
+    s += nval / nen * t[a];
+  }
+  return s;
+}
+
+template <int DIM, typename T>
+__device__ __forceinline__ void pp_corners(const T* __restrict__ ns, const Dims& d, int e,
+                                           T (&t)[1 << DIM]) {
+  int i, j, k;
+  coords(e, d.fEX, d.fEXY, i, j, k);
+#pragma unroll
+  for (int a = 0; a < (1 << DIM); ++a) {
+    const int nd = (i + (a & 1)) + d.NX * ((j + ((a >> 1) & 1)) + d.NY * (k + ((a >> 2) & 1)));
+    t[a] = CK(nd, d.n) ? ns[nd] : T(0);
+  }
+}
+
+template <int N>
+__device__ __forceinline__ void pp_range(const float (&t)[N], float& lo, float& hi) {
+  lo = hi = t[0];
+#pragma unroll
+  for (int a = 1; a < N; ++a) {
+    lo = fminf(lo, t[a]);
+    hi = fmaxf(hi, t[a]);
+  }
+}
+
+// The first pass's bracket: every finite non-negative float.
+__global__ void k_pp_first(PpCtrl* c) {
+  c->lo[0] = 0u;
+  c->hi[0] = 0x7fffffffu;
+}
+
+// Histogram of the points' values in the bracket of pass `pass` (0 or 1).
+template <int DIM>
+__global__ void __launch_bounds__(512) k_pp_hist(const float* __restrict__ ns, Dims d, PpCtrl* c,
+                                                 int pass) {
+  constexpr int nen = 1 << DIM, NP = DIM == 3 ? 125 : 25;
+  __shared__ unsigned h[kPpBins];
+  __shared__ unsigned long long above;
+  const unsigned lo = c->lo[pass], hi = c->hi[pass];
+  const int shift = pass == 0 ? kPpShift1 : kPpShift2;
+  for (int b = threadIdx.x; b < kPpBins; b += blockDim.x) h[b] = 0u;
+  if (threadIdx.x == 0) above = 0ull;
+  __syncthreads();
+  unsigned long long up = 0ull;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < (int)d.ne; e += gridDim.x * blockDim.x) {
+    float t[nen], tmin, tmax;
+    pp_corners<DIM, float>(ns, d, e, t);
+    pp_range<nen>(t, tmin, tmax);
+    const unsigned bmin = __float_as_uint(tmin), bmax = __float_as_uint(tmax);
+    if (bmax < lo) continue;
+    if (bmin > hi) {
+      up += NP;
+      continue;
+    }
+    if (bmin >= lo && bmax <= hi && (bmin - lo) >> shift == (bmax - lo) >> shift) {
+      atomicAdd(&h[min((bmin - lo) >> shift, (unsigned)kPpBins - 1)], (unsigned)NP);
+      continue;
+    }
+    pp_points32<DIM>(t, tmin, tmax, [&](float s, int, int, int) {
+      const unsigned b = __float_as_uint(s);
+      if (b > hi) ++up;
+      else if (b >= lo) atomicAdd(&h[min((b - lo) >> shift, (unsigned)kPpBins - 1)], 1u);
+    });
+  }
+  if (up) atomicAdd(&above, up);
+  __syncthreads();
+  for (int b = threadIdx.x; b < kPpBins; b += blockDim.x)
+    if (h[b]) atomicAdd(&c->hist[pass][b], (unsigned long long)h[b]);
+  if (threadIdx.x == 0 && above) atomicAdd(&c->above[pass], above);
+}
+
+// The bin in which the count from the top passes `want`, widened by the
+// guard: the next pass's bracket.  One block of 1024 threads.
+__global__ void __launch_bounds__(1024) k_pp_pick(PpCtrl* c, int pass, double want) {
+  constexpr int PER = kPpBins / 1024;
+  __shared__ unsigned long long part[1024];
+  const int tid = threadIdx.x;
+  unsigned long long h[PER], s = 0ull;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    h[q] = c->hist[pass][tid * PER + q];
+    s += h[q];
+  }
+  part[tid] = s;
+  __syncthreads();
+  // suffix sums
+  for (int o = 1; o < 1024; o <<= 1) {
+    const unsigned long long v = tid + o < 1024 ? part[tid + o] : 0ull;
+    __syncthreads();
+    part[tid] += v;
+    __syncthreads();
+  }
+  const unsigned long long above = c->above[pass];
+  // points in this thread's bins and all higher ones, and in the higher ones
+  const unsigned long long incl = above + part[tid], excl = incl - s;
+  if ((double)incl > want && !((double)excl > want)) {
+    unsigned long long run = excl;
+    int bin = tid * PER;
+#pragma unroll
+    for (int q = PER - 1; q >= 0; --q) {
+      run += h[q];
+      if ((double)run > want) {
+        bin = tid * PER + q;
+        break;
+      }
+    }
+    const int shift = pass == 0 ? kPpShift1 : kPpShift2;
+    const unsigned a = c->lo[pass] + ((unsigned)bin << shift), b = a + (1u << shift) - 1u;
+    c->lo[pass + 1] = a > kPpGuard ? a - kPpGuard : 0u;
+    c->hi[pass + 1] = min(b + kPpGuard, 0x7f7fffffu);
+  }
+}
+
+// Points above the last bracket, counted, and the values of those inside,
+// listed: the level below which the point counts, which is its FP64 value
+// kept within its element's corners (an element whose corners all exceed the
+// level is solid, one whose corners are all below it void).
+template <int DIM>
+__global__ void __launch_bounds__(512) k_pp_list(const float* __restrict__ ns32,
+                                                 const double* __restrict__ ns, Dims d, PpCtrl* c,
+                                                 double* __restrict__ list, int cap) {
+  constexpr int nen = 1 << DIM, NP = DIM == 3 ? 125 : 25;
+  __shared__ unsigned long long above;
+  const unsigned lo = c->lo[2], hi = c->hi[2];
+  if (threadIdx.x == 0) above = 0ull;
+  __syncthreads();
+  unsigned long long up = 0ull;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < (int)d.ne; e += gridDim.x * blockDim.x) {
+    float t[nen], tmin, tmax;
+    pp_corners<DIM, float>(ns32, d, e, t);
+    pp_range<nen>(t, tmin, tmax);
+    if (__float_as_uint(tmax) < lo) continue;
+    if (__float_as_uint(tmin) > hi) {
+      up += NP;
+      continue;
+    }
+    pp_points32<DIM>(t, tmin, tmax, [&](float s, int px, int py, int pz) {
+      const unsigned b = __float_as_uint(s);
+      if (b > hi) ++up;
+      else if (b >= lo) {
+        double td[nen];
+        pp_corners<DIM, double>(ns, d, e, td);
+        double mn = td[0], mx = td[0];
+#pragma unroll
+        for (int a = 1; a < nen; ++a) {
+          mn = fmin(mn, td[a]);
+          mx = fmax(mx, td[a]);
+        }
+        const double v = pp_value<DIM>(td, px, py, pz);
+        // at the level mx itself the element is not void: a value rounded
+        // above mx counts there and nowhere higher
+        const double eff = v > mx ? nextafter(mx, 1e300) : fmax(v, mn);
+        const int slot = atomicAdd(&c->nlist, 1);
+        if (slot < cap) list[slot] = eff;
+      }
+    });
+  }
+  if (up) atomicAdd(&above, up);
+  __syncthreads();
+  if (threadIdx.x == 0 && above) atomicAdd(&c->above[2], above);
+}
+
+// The bisection, one block: level L has the points above the last bracket
+// plus the listed values > L.  The densities' FP64 sum and this count give the
+// same answer unless the count is the target itself; then out[0] = 1 asks for
+// that answer (tie: -1 unknown, else whether the sum exceeds the target) at
+// the level in out[1].  out[0] = 2: not applicable; 0: done, level in out[1].
+__global__ void __launch_bounds__(1024) k_pp_bisect(const PpCtrl* c, const double* __restrict__ list,
+                                                    int cap, double top, double want, double slack,
+                                                    int tie, double* out) {
+  __shared__ int part[32];
+  __shared__ int total;
+  const int n = c->nlist, tid = threadIdx.x;
+  if (c->bad || n > cap) {
+    if (tid == 0) out[0] = 2.0;
+    return;
+  }
+  const double base = (double)c->above[2];
+  // outside [La, Lb] the answer is known (a bracket cut off at 0 knows nothing below)
+  const double La = c->lo[2] ? (double)__uint_as_float(c->lo[2] + kPpGuard / 2) : -1.0;
+  const double Lb = (double)__uint_as_float(c->hi[2] - kPpGuard / 2);
+  double lo = -1.0, hi = top;
+  for (int step = 0; step < 200; ++step) {
+    const double mid = 0.5 * (lo + hi);
+    if (!(lo < mid && mid < hi)) break;
+    bool more;
+    if (mid <= La) more = true;
+    else if (mid >= Lb) more = false;
+    else {
+      int k = 0;
+      for (int q = tid; q < n; q += 1024) k += list[q] > mid ? 1 : 0;
+      k = __reduce_add_sync(0xffffffffu, k);
+      if ((tid & 31) == 0) part[tid >> 5] = k;
+      __syncthreads();
+      if (tid < 32) {
+        const int s = __reduce_add_sync(0xffffffffu, part[tid]);
+        if (tid == 0) total = s;
+      }
+      __syncthreads();
+      const double count = base + (double)total;
+      __syncthreads();
+      if (fabs(count - want) <= slack) {
+        if (tie < 0) {
+          if (tid == 0) {
+            out[0] = 1.0;
+            out[1] = mid;
+          }
+          return;
+        }
+        more = tie != 0;
+      } else {
+        more = count > want;
+      }
+    }
+    if (more) lo = mid;
+    else hi = mid;
+  }
+  if (tid == 0) {
+    out[0] = 0.0;
+    out[1] = hi;
+  }
+}
+
+// k_pp_density for nodal values in [0, 1e37]: the same counts, the points
+// (and corners) decided by their FP32 values unless those lie within the
+// FP32 error of the level.
+template <int DIM>
+__global__ void k_pp_density32(const float* __restrict__ ns32, const double* __restrict__ ns, Dims d,
+                               double level, double* __restrict__ rho, double* partials,
+                               unsigned int* counter, double* sum) {
+  constexpr int nen = 1 << DIM, NP = DIM == 3 ? 125 : 25;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  const float l32 = (float)level;
+  // points this far (16 ulps) from the level are on the same side of it in FP64
+  const float lo = l32 * (1.f - 0x1p-19f), hi = l32 * (1.f + 0x1p-19f) + 0x1p-140f;
+  double v[1] = {0.0};
+  if (e < (int)d.ne) {
+    float t[nen], tmin, tmax;
+    pp_corners<DIM, float>(ns32, d, e, t);
+    pp_range<nen>(t, tmin, tmax);
+    int count = -1;
+    if (tmin > l32) count = NP;       // rounding keeps the order: every corner above the level
+    else if (tmax < l32) count = 0;   // ... below
+    if (count < 0) {
+      double td[nen];
+      bool have = false, above = true, below = true;
+      if (!(tmin < l32 && tmax > l32)) {  // a corner rounds to the level: decide in FP64
+        pp_corners<DIM, double>(ns, d, e, td);
+        have = true;
+#pragma unroll
+        for (int a = 0; a < nen; ++a) {
+          above = above && td[a] > level;
+          below = below && td[a] < level;
+        }
+      } else {
+        above = below = false;
+      }
+      if (above) count = NP;
+      else if (below) count = 0;
+      else {
+        count = 0;
+        pp_points32<DIM>(t, 0.f, 3e38f, [&](float s, int px, int py, int pz) {
+          if (s > hi) ++count;
+          else if (!(s < lo)) {
+            if (!have) {
+              pp_corners<DIM, double>(ns, d, e, td);
+              have = true;
+            }
+            count += pp_value<DIM>(td, px, py, pz) > level ? 1 : 0;
+          }
+        });
+      }
+    }
+    const double val = count == NP ? 1.0 : count == 0 ? 0.0 : (double)count / (double)NP;
+    if (rho) rho[e] = val;
+    v[0] = val;
+  }
+  block_sum_finish<1>(v, partials, counter, sum);
 }
 
 // Eq. 24 with ev of Eq. 25-27; the densities into rho (may be null) and their
@@ -1059,19 +1419,32 @@ void postprocess(Ctx& c, const double* rho, const double* T, double volfrac, dou
                                                               c.p.penal);
   MGAR_LAUNCH_CHECK();
   const double r = c.p.rmin;
-  const int reach = (int)std::ceil(r + 0.5);
   double* ns = c.tm;
+  float* ns32 = reinterpret_cast<float*>(c.pv);
+  PpCtrl* ctrl = reinterpret_cast<PpCtrl*>(c.pp_ctrl);
+  MGAR_CUDA(cudaMemsetAsync(ctrl, 0, sizeof(PpCtrl), c.stream));
+  const PpTap* taps = reinterpret_cast<const PpTap*>(c.pp_taps);
   if (c.dim == 2)
-    k_pp_nodal<2><<<blocks_for(c.n), kThreads, 0, c.stream>>>(c.tmp_e, ns, d, r, reach);
+    k_pp_nodal<2><<<blocks_for(c.n), kThreads, 0, c.stream>>>(c.tmp_e, ns, ns32, d, taps,
+                                                              c.pp_ntaps, &ctrl->bad);
   else
-    k_pp_nodal<3><<<blocks_for(c.n), kThreads, 0, c.stream>>>(c.tmp_e, ns, d, r, reach);
+    k_pp_nodal<3><<<blocks_for(c.n), kThreads, 0, c.stream>>>(c.tmp_e, ns, ns32, d, taps,
+                                                              c.pp_ntaps, &ctrl->bad);
   MGAR_LAUNCH_CHECK();
   k_pp_max<<<c.grid_blocks, kThreads, 0, c.stream>>>(ns, (int)c.n, c.partials, c.counter,
                                                       c.dsc + S_TMP);
   MGAR_LAUNCH_CHECK();
   fetch_scalars(c, S_TMP, 1);
-  auto volume = [&](double level, double* out) {
-    if (c.dim == 2)
+  const double top = c.hsc[S_TMP];
+  // the density at a level and its mean; fast: nodal values in [0, 1e37]
+  auto volume = [&](double level, double* out, bool fast) {
+    if (fast && c.dim == 2)
+      k_pp_density32<2><<<blocks_for(ne), kThreads, 0, c.stream>>>(ns32, ns, d, level, out, c.partials,
+                                                                   c.counter, c.dsc + S_TMP);
+    else if (fast)
+      k_pp_density32<3><<<blocks_for(ne), kThreads, 0, c.stream>>>(ns32, ns, d, level, out, c.partials,
+                                                                   c.counter, c.dsc + S_TMP);
+    else if (c.dim == 2)
       k_pp_density<2><<<blocks_for(ne), kThreads, 0, c.stream>>>(ns, d, level, out, c.partials,
                                                                  c.counter, c.dsc + S_TMP);
     else
@@ -1081,17 +1454,77 @@ void postprocess(Ctx& c, const double* rho, const double* T, double volfrac, dou
     fetch_scalars(c, S_TMP, 1);
     return c.hsc[S_TMP] / (double)ne;
   };
-  // ns >= 0: below -1 every node is above the level (volume 1), at max(ns)
-  // none is (volume 0)
-  double lo = -1.0, hi = c.hsc[S_TMP];
-  for (int step = 0; step < 200; ++step) {
-    const double mid = 0.5 * (lo + hi);
-    if (!(lo < mid && mid < hi)) break;
-    if (volume(mid, nullptr) > volfrac) lo = mid;
-    else hi = mid;
+  // the level by counts of lattice points
+  const double total = (c.dim == 3 ? 125.0 : 25.0) * (double)ne, want = volfrac * total;
+  double* list = c.tmp_e;  // the element sensitivities are no longer needed
+  const int hb = std::min(blocks_for(ne, 512), 4 * c.sms);
+  k_pp_first<<<1, 1, 0, c.stream>>>(ctrl);
+  MGAR_LAUNCH_CHECK();
+  for (int pass = 0; pass < 2; ++pass) {
+    if (c.dim == 2) k_pp_hist<2><<<hb, 512, 0, c.stream>>>(ns32, d, ctrl, pass);
+    else k_pp_hist<3><<<hb, 512, 0, c.stream>>>(ns32, d, ctrl, pass);
+    MGAR_LAUNCH_CHECK();
+    k_pp_pick<<<1, 1024, 0, c.stream>>>(ctrl, pass, want);
+    MGAR_LAUNCH_CHECK();
   }
-  const double v = volume(hi, rho_out);
+  if (c.dim == 2) k_pp_list<2><<<hb, 512, 0, c.stream>>>(ns32, ns, d, ctrl, list, ne);
+  else k_pp_list<3><<<hb, 512, 0, c.stream>>>(ns32, ns, d, ctrl, list, ne);
+  MGAR_LAUNCH_CHECK();
+  // the FP64 sum of the densities is within 1e-13 of the count's share, so
+  // only a count that equals the target leaves the comparison to it
+  const double slack = 1e-12 * total;
+  double hi = top;
+  bool found = false;
+  for (int tie = -1;;) {
+    k_pp_bisect<<<1, 1024, 0, c.stream>>>(ctrl, list, ne, top, want, slack, tie, c.dsc + S_GS);
+    MGAR_LAUNCH_CHECK();
+    fetch_scalars(c, S_GS, 2);
+    const int state = (int)c.hsc[S_GS];
+    if (state == 1 && tie < 0) {
+      tie = volume(c.hsc[S_GS + 1], nullptr, true) > volfrac ? 1 : 0;
+      continue;
+    }
+    found = state == 0;
+    if (found) hi = c.hsc[S_GS + 1];
+    break;
+  }
+  if (!found) {
+    // values outside [0, 1e37], or more equal values at the level than the
+    // list holds: a volume per step.  ns >= 0: below -1 every node is above
+    // the level (volume 1), at max(ns) none is (volume 0)
+    double lo = -1.0;
+    hi = top;
+    for (int step = 0; step < 200; ++step) {
+      const double mid = 0.5 * (lo + hi);
+      if (!(lo < mid && mid < hi)) break;
+      if (volume(mid, nullptr, false) > volfrac) lo = mid;
+      else hi = mid;
+    }
+  }
+  const double v = volume(hi, rho_out, found);
   if (level_out) *level_out = hi;
   if (volume_out) *volume_out = v;
+}
+
+// The projection's taps and the level search's counters, at creation.
+void setup_postprocess(Ctx& c) {
+  const double r = c.p.rmin;
+  const int reach = (int)std::ceil(r + 0.5);
+  std::vector<PpTap> taps;
+  // element (i + ox, j + oy, k + oz) has its centroid at offset o + 1/2
+  for (int ox = -reach; ox < reach; ++ox)
+    for (int oy = -reach; oy < reach; ++oy)
+      for (int oz = (c.dim == 3 ? -reach : 0); oz < (c.dim == 3 ? reach : 1); ++oz) {
+        const double dz = c.dim == 3 ? oz + 0.5 : 0.0;
+        const double w = r - std::sqrt((ox + 0.5) * (ox + 0.5) + (oy + 0.5) * (oy + 0.5) + dz * dz);
+        if (w > 0.0) taps.push_back(PpTap{ox, oy, oz, w});
+      }
+  c.pp_ntaps = (int)taps.size();
+  if (!taps.empty()) {
+    MGAR_CUDA(cudaMalloc(&c.pp_taps, taps.size() * sizeof(PpTap)));
+    MGAR_CUDA(cudaMemcpy(c.pp_taps, taps.data(), taps.size() * sizeof(PpTap),
+                         cudaMemcpyHostToDevice));
+  }
+  MGAR_CUDA(cudaMalloc(&c.pp_ctrl, sizeof(PpCtrl)));
 }
 }  // namespace mgar
