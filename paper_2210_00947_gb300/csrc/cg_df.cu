@@ -22,32 +22,53 @@ namespace mgar {
 namespace {
 
 // y = A x; with DOT, x.y into out (warp sums in df64, FP64 across warps and
-// blocks).  NPT nodes per thread: base, base + blockDim.x, ...
-template <int DIM, bool DOT, int NPT = 1>
+// blocks).
+template <int DIM, bool DOT>
 __global__ void k_df_apply(DfOp op, const float2* __restrict__ x, float2* __restrict__ y,
                            double* partials, unsigned int* counter, double* out) {
-  const int base = blockIdx.x * blockDim.x * NPT + threadIdx.x;
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   df v{0.f, 0.f};
-#pragma unroll
-  for (int u = 0; u < NPT; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < op.n) {
-      const df yv = df_row<DIM>(op, x, idx);
-      y[idx] = pack(yv);
-      if (DOT) v = df_add(v, df_mul(unpack(x[idx]), yv));
-    }
+  if (idx < op.n) {
+    const df yv = df_row<DIM>(op, x, idx);
+    y[idx] = pack(yv);
+    if (DOT) v = df_mul(unpack(x[idx]), yv);
   }
   if (DOT) block_sum_finish_df(v, partials, counter, out);
 }
 
-// The 2D product with p . Ap, two nodes per thread.
-constexpr int kNptApply2 = 2;
+// 2D: p = z + (*rz_new / *rz_old) p_old (p = z when first), y = A p, p . y
+// into *out; odd *parity (may be null) swaps p_old and p.
+__global__ void __launch_bounds__(l2d::kThreads2) k_df_dir2(DfOp op, const float* __restrict__ z,
+                                                            const float2* p_old, float2* p,
+                                                            const double* rz_new,
+                                                            const double* rz_old, int first,
+                                                            const double* parity,
+                                                            float2* __restrict__ y, double* partials,
+                                                            unsigned int* counter, double* out) {
+  __shared__ DfDirSmem s;
+  pdl_wait();
+  pdl_trigger();
+  if (parity && (((int)*parity) & 1)) {
+    float2* t = const_cast<float2*>(p_old);
+    p_old = p;
+    p = t;
+  }
+  const df beta = first ? df{0.f, 0.f} : block_div_df(rz_new, rz_old);
+  const df v = df_dir_tile(s, op, blockIdx.x, blockIdx.y, z, p_old, first != 0, beta, p, y);
+  double t;
+  if (block_sum_last_df(v, partials, counter, t, threadIdx.x, l2d::kThreads2,
+                        blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y) &&
+      threadIdx.x == 0)
+    *out = t;
+}
 
-void df_apply2_dot(const DfOp& op, const float2* x, float2* y, double* partials,
-                   unsigned int* counter, double* out, cudaStream_t s) {
-  const int per = kThreads * kNptApply2;
-  k_df_apply<2, true, kNptApply2><<<(op.n + per - 1) / per, kThreads, 0, s>>>(op, x, y, partials,
-                                                                             counter, out);
+void df_dir2(Ctx& c, const DfOp& op, const float2* p_old, float2* p, const double* rz_new,
+             const double* rz_old, bool first, const double* parity) {
+  const dim3 grid(l2d::tiles(op.NX, l2d::kUX), l2d::tiles(op.NY, l2d::kUY));
+  launch_pdl(c.stream, c.use_pdl, k_df_dir2, grid, dim3(l2d::kThreads2), op, (const float*)c.x32,
+             p_old, p, rz_new, rz_old, first ? 1 : 0, parity, c.df_Ap, c.partials, c.counter,
+             c.dsc + S_PAP);
+  MGAR_LAUNCH_CHECK();
 }
 
 // r = q - A x and ||r||^2
@@ -65,16 +86,39 @@ __global__ void k_df_residual(DfOp op, const float2* __restrict__ q, const float
   block_sum_finish_df(v, partials, counter, out);
 }
 
+// The device-side loop's test, in the last block of an update of x and r:
+// count the iteration, flip the parity, and continue while ||r|| / ||q|| >
+// eps2 (the host loop's test, same arithmetic) and fewer than cg_max
+// iterations ran; a non-finite residual stops the loop and the host reports
+// it.  The iteration's r . z (RZ1) becomes the next one's old value (RZ0).
+struct CgCheck {
+  double* dsc;  // null: no device-side loop
+  double qnorm, eps2;
+  int cg_max;
+  cudaGraphConditionalHandle loop;
+};
+
+__device__ __forceinline__ void cg_check(const CgCheck& k) {
+  double* dsc = k.dsc;
+  const double rel = sqrt(dsc[S_RR]) / k.qnorm;
+  const int it = (int)dsc[S_CGIT] + 1;
+  dsc[S_CGIT] = (double)it;
+  dsc[S_CGPAR] = (double)(((int)dsc[S_CGPAR]) ^ 1);
+  dsc[S_RZ0] = dsc[S_RZ1];
+  const bool go = isfinite(rel) && rel > k.eps2 && it < k.cg_max;
+  cudaGraphSetConditional(k.loop, go ? 1u : 0u);
+}
+
 // alpha = rz / pAp; x += alpha p; r -= alpha Ap; ||r||^2; optionally the
 // FP32 copy of r for the preconditioner
 __global__ void k_df_cg_xr(float2* __restrict__ x, float2* __restrict__ r, const float2* __restrict__ p,
                            const float2* __restrict__ Ap, int n, const double* __restrict__ rz,
                            const double* __restrict__ pap, double* partials, unsigned int* counter,
                            double* out, float* __restrict__ r32,
-                           const float2* __restrict__ p_alt = nullptr,
-                           const double* parity = nullptr) {
+                           const float2* __restrict__ p_alt, const double* parity, CgCheck check) {
   pdl_wait();
   // device-side CG loop: the two direction buffers swap with the parity
+  // (every block reads it before the last one flips it)
   if (parity && (((int)*parity) & 1)) p = p_alt;
   const df alpha = block_div_df(rz, pap);
   df acc{0.f, 0.f};
@@ -105,7 +149,12 @@ __global__ void k_df_cg_xr(float2* __restrict__ x, float2* __restrict__ r, const
     if (r32) r32[i] = __fadd_rn(ri.hi, ri.lo);
     acc = df_add(acc, df_mul(ri, ri));
   }
-  block_sum_finish_df(acc, partials, counter, out);
+  double t;
+  if (block_sum_last_df(acc, partials, counter, t, threadIdx.x, blockDim.x, blockIdx.x, gridDim.x) &&
+      threadIdx.x == 0) {
+    *out = t;
+    if (check.dsc) cg_check(check);
+  }
 }
 
 // p = z + (rz_new / rz_old) p, z in FP32
@@ -195,26 +244,10 @@ static void precondition_df(Ctx& c) {
 }
 
 // Device-side CG loop (one graph per handle): iteration count and buffer
-// parity start at zero ...
+// parity start at zero.
 __global__ void k_cg_reset(double* dsc) {
   dsc[S_CGIT] = 0.0;
   dsc[S_CGPAR] = 0.0;
-}
-
-// ... and after each update of x and r: count the iteration, flip the
-// parity, and continue while ||r|| / ||q|| > eps2 (the host loop's test,
-// same arithmetic) and fewer than cg_max iterations ran; a non-finite
-// residual stops the loop and the host reports it.  shift: the iteration's
-// r . z (RZ1) becomes the next one's old value (RZ0).
-__global__ void k_cg_check(double* dsc, double qnorm, double eps2, int cg_max,
-                           cudaGraphConditionalHandle loop, int shift) {
-  const double rel = sqrt(dsc[S_RR]) / qnorm;
-  const int it = (int)dsc[S_CGIT] + 1;
-  dsc[S_CGIT] = (double)it;
-  dsc[S_CGPAR] = (double)(((int)dsc[S_CGPAR]) ^ 1);
-  if (shift) dsc[S_RZ0] = dsc[S_RZ1];
-  const bool go = isfinite(rel) && rel > eps2 && it < cg_max;
-  cudaGraphSetConditional(loop, go ? 1u : 0u);
 }
 
 // z32 = M r32 (the FP32 copy of r is written by the residual and update
@@ -230,28 +263,26 @@ static void precondition_f32(Ctx& c, int slot) {
 // (p = z + beta p_old, A p, p.Ap in one pass) and write the FP32 copy of r
 // beside r, so an iteration is: product, update of x and r, V-cycle, r.z.
 // One CG iteration of the device-side loop: V-cycle (r . z into RZ1), the
-// direction update and product (beta = RZ1 / RZ0, then RZ0 <- RZ1), the
-// update of x and r, the convergence check.
+// direction update and product (beta = RZ1 / RZ0), the update of x and r with
+// the convergence check (which moves RZ1 to RZ0).
 static void cg_iteration(Ctx& c, bool first, cudaGraphConditionalHandle loop) {
   const int n = (int)c.n;
   vcycle_dot(c, c.b32, c.x32, c.df_r, c.dsc + S_RZ1);
   df3d_dir(c, c.x32, c.df_p, c.df_p2, c.dsc + S_RZ1, c.dsc + S_RZ0, first, c.df_Ap, c.dsc + S_PAP,
-           c.dsc + S_CGPAR, c.dsc + S_RZ0);
+           c.dsc + S_CGPAR);
   // parity 0: the new p is in df_p2
   launch_pdl(c.stream, c.use_pdl, k_df_cg_xr, dim3(c.grid_blocks), dim3(kThreads), c.df_x, c.df_r,
-             (const float2*)c.df_p2, (const float2*)c.df_Ap, n, (const double*)(c.dsc + S_RZ0),
+             (const float2*)c.df_p2, (const float2*)c.df_Ap, n, (const double*)(c.dsc + S_RZ1),
              (const double*)(c.dsc + S_PAP), c.partials, c.counter, c.dsc + S_RR, c.b32,
-             (const float2*)c.df_p, (const double*)(c.dsc + S_CGPAR));
-  MGAR_LAUNCH_CHECK();
-  k_cg_check<<<1, 1, 0, c.stream>>>(c.dsc, c.qnorm, c.p.eps2, c.p.cg_max, loop, 0);
+             (const float2*)c.df_p, (const double*)(c.dsc + S_CGPAR),
+             CgCheck{c.dsc, c.qnorm, c.p.eps2, c.p.cg_max, loop});
   MGAR_LAUNCH_CHECK();
 }
 
-// 2D: one CG iteration of the device-side loop with the generic kernels,
-// the host loop's steps and arithmetic: V-cycle z = M r (r's FP32 copy is
-// written by the update of x and r), r . z into RZ1, p = z (first) or
-// p = z + (RZ1 / RZ0) p, A p with p . A p, the update of x and r with
-// alpha = RZ1 / pAp, the check (which moves RZ1 to RZ0).
+// 2D: one CG iteration of the device-side loop, the host loop's steps and
+// arithmetic: V-cycle z = M r (r's FP32 copy is written by the update of x
+// and r) with r . z into RZ1, p = z (first) or p = z + (RZ1 / RZ0) p with A p
+// and p . A p, the update of x and r with alpha = RZ1 / pAp and the check.
 static void cg_iteration_2d(Ctx& c, bool first, cudaGraphConditionalHandle loop) {
   const int n = (int)c.n;
   const int rb = c.grid_blocks;
@@ -269,18 +300,12 @@ static void cg_iteration_2d(Ctx& c, bool first, cudaGraphConditionalHandle loop)
                                               c.dsc + S_RZ1);
     MGAR_LAUNCH_CHECK();
   }
-  if (first)
-    k_f32_to_df<<<blocks_for(n), kThreads, 0, c.stream>>>(c.x32, c.df_p, n);
-  else
-    k_df_cg_p<<<rb, kThreads, 0, c.stream>>>(c.df_p, c.x32, n, c.dsc + S_RZ1, c.dsc + S_RZ0);
-  MGAR_LAUNCH_CHECK();
-  df_apply2_dot(op, c.df_p, c.df_Ap, c.partials, c.counter, c.dsc + S_PAP, c.stream);
-  MGAR_LAUNCH_CHECK();
-  k_df_cg_xr<<<rb, kThreads, 0, c.stream>>>(c.df_x, c.df_r, c.df_p, c.df_Ap, n, c.dsc + S_RZ1,
-                                            c.dsc + S_PAP, c.partials, c.counter, c.dsc + S_RR,
-                                            c.b32);
-  MGAR_LAUNCH_CHECK();
-  k_cg_check<<<1, 1, 0, c.stream>>>(c.dsc, c.qnorm, c.p.eps2, c.p.cg_max, loop, 1);
+  df_dir2(c, op, c.df_p, c.df_p2, c.dsc + S_RZ1, c.dsc + S_RZ0, first, c.dsc + S_CGPAR);
+  launch_pdl(c.stream, c.use_pdl, k_df_cg_xr, dim3(rb), dim3(kThreads), c.df_x, c.df_r,
+             (const float2*)c.df_p2, (const float2*)c.df_Ap, n, (const double*)(c.dsc + S_RZ1),
+             (const double*)(c.dsc + S_PAP), c.partials, c.counter, c.dsc + S_RR, c.b32,
+             (const float2*)c.df_p, (const double*)(c.dsc + S_CGPAR),
+             CgCheck{c.dsc, c.qnorm, c.p.eps2, c.p.cg_max, loop});
   MGAR_LAUNCH_CHECK();
 }
 
@@ -423,7 +448,7 @@ static int solve_mgcg_df3(Ctx& c, double* T, int* iters, double* relres) {
       launch_pdl(c.stream, c.use_pdl, k_df_cg_xr, dim3(rb), dim3(kThreads), c.df_x, c.df_r,
                  (const float2*)pcur, (const float2*)c.df_Ap, n, (const double*)(c.dsc + a),
                  (const double*)(c.dsc + S_PAP), c.partials, c.counter, c.dsc + S_RR, c.b32,
-                 (const float2*)nullptr, (const double*)nullptr);
+                 (const float2*)nullptr, (const double*)nullptr, CgCheck{});
       MGAR_LAUNCH_CHECK();
       ++it;
       fetch_scalars(c, S_RR, 1);
@@ -832,38 +857,47 @@ int solve_mgcg_df(Ctx& c, double* T, int* iters, double* relres) {
       k_df_dot_f<<<rb, kThreads, 0, c.stream>>>(c.df_r, c.x32, n, c.partials, c.counter, c.dsc + a);
       MGAR_LAUNCH_CHECK();
     }
-    k_f32_to_df<<<blocks_for(n), kThreads, 0, c.stream>>>(c.x32, c.df_p, n);
-    MGAR_LAUNCH_CHECK();
+    float2 *pcur = c.df_p, *pnext = c.df_p2;
+    bool first = true;
+    if (c.dim == 3) {
+      k_f32_to_df<<<blocks_for(n), kThreads, 0, c.stream>>>(c.x32, pcur, n);
+      MGAR_LAUNCH_CHECK();
+    }
     while (it < c.p.cg_max) {
       {
         ProfScope ps(c, MGAR_KC_APPLY64);
-        if (c.dim == 2)
-          df_apply2_dot(op, c.df_p, c.df_Ap, c.partials, c.counter, c.dsc + S_PAP, c.stream);
-        else
+        if (c.dim == 2) {
+          df_dir2(c, op, pcur, pnext, c.dsc + a, c.dsc + b, first, nullptr);
+          std::swap(pcur, pnext);
+        } else {
           k_df_apply<3, true><<<blocks_for(n), kThreads, 0, c.stream>>>(
-              op, c.df_p, c.df_Ap, c.partials, c.counter, c.dsc + S_PAP);
-        MGAR_LAUNCH_CHECK();
+              op, pcur, c.df_Ap, c.partials, c.counter, c.dsc + S_PAP);
+          MGAR_LAUNCH_CHECK();
+        }
       }
-      k_df_cg_xr<<<rb, kThreads, 0, c.stream>>>(c.df_x, c.df_r, c.df_p, c.df_Ap, n, c.dsc + a,
+      first = false;
+      k_df_cg_xr<<<rb, kThreads, 0, c.stream>>>(c.df_x, c.df_r, pcur, c.df_Ap, n, c.dsc + a,
                                                 c.dsc + S_PAP, c.partials, c.counter, c.dsc + S_RR,
-                                                fused ? c.b32 : nullptr);
+                                                fused ? c.b32 : nullptr, nullptr, nullptr, CgCheck{});
       MGAR_LAUNCH_CHECK();
       ++it;
       fetch_scalars(c, S_RR, 1);
       rel = std::sqrt(c.hsc[S_RR]) / c.qnorm;
       require(std::isfinite(rel), MGAR_ERR_NONFINITE, "CG breakdown (non-finite residual)");
       if (rel <= c.p.eps2) break;
+      std::swap(a, b);
       if (fused) {
-        precondition_f32(c, b);
+        precondition_f32(c, a);
       } else {
         precondition_df(c);
         k_df_dot_f<<<rb, kThreads, 0, c.stream>>>(c.df_r, c.x32, n, c.partials, c.counter,
-                                                  c.dsc + b);
+                                                  c.dsc + a);
         MGAR_LAUNCH_CHECK();
       }
-      k_df_cg_p<<<rb, kThreads, 0, c.stream>>>(c.df_p, c.x32, n, c.dsc + b, c.dsc + a);
-      MGAR_LAUNCH_CHECK();
-      std::swap(a, b);
+      if (c.dim == 3) {
+        k_df_cg_p<<<rb, kThreads, 0, c.stream>>>(pcur, c.x32, n, c.dsc + a, c.dsc + b);
+        MGAR_LAUNCH_CHECK();
+      }
     }
   }
   k_df_to_d<<<blocks_for(n), kThreads, 0, c.stream>>>(c.df_x, T, n);

@@ -127,6 +127,7 @@ template <typename Real>
 struct LevelBuf {
   Real* st = nullptr;    // [S][n] assembled stencil, levels >= 1
   Real* dinv = nullptr;  // [n] 1/diag, levels >= 1
+  Real* dinv_s = nullptr;  // [n] 2D, level 0: 1/diag, negated on fixed nodes
   Real* elem = nullptr;  // [ne][nen*nen] Galerkin element matrices, levels >= 1
   Real* x = nullptr;     // V-cycle iterate (levels >= 1; level 0 uses caller arrays)
   Real* b = nullptr;     // right-hand side (levels >= 1)
@@ -947,6 +948,8 @@ inline bool vcycle_dot_ok(const Ctx& c) {
   return c.p.nu_pre == 1 && c.p.nu_post == 1 && c.nl >= 2 && !c.untiled;
 }
 void vcycle_dot(Ctx& c, const float* b, float* x, const float2* r, double* dout);
+// the same in FP64 with b . x in *dout, for 2D grids where vcycle_dot_ok
+void vcycle_dot64(Ctx& c, const double* b, double* x, double* dout);
 // launch shapes of the tiled kernels (occupancy query; call outside stream capture)
 void fine3d_prepare(Ctx& c);
 // vcycle.cu: can the bottom levels run as one thread-block cluster launch
@@ -1099,7 +1102,8 @@ void run_graph(Ctx& c, int kind, const void* a, const void* b, bool profiled_ins
                                       "graph:3 mgar-vcycle64-guess", "graph:4 mgar-vcycle32-zero",
                                       "graph:5 mgar-vcycle32-guess", "graph:6 precondition-df",
                                       "graph:7", "graph:8 precondition-rz", "graph:9 precondition-rz",
-                                      "graph:10 precondition-rz32"};
-  prof_mark(kGraphSites[kind >= 0 && kind < 11 ? kind : 0]);
+                                      "graph:10 precondition-rz32", "graph:11 precondition-rz64",
+                                      "graph:12 precondition-rz64"};
+  prof_mark(kGraphSites[kind >= 0 && kind < 13 ? kind : 0]);
 }
 }  // namespace mgar

@@ -293,14 +293,16 @@ __global__ void k_assemble(const Real* __restrict__ elem, Dims d, Real* __restri
   dinv[idx] = Real(1) / acc[S / 2];
 }
 
-// Inverse diagonal of the matrix-free finest operator (1 on fixed nodes).
+// Inverse diagonal of the matrix-free finest operator (1 on fixed nodes); 2D:
+// also negated on the fixed nodes, for the tiled passes.
 template <typename Real, int DIM>
 __global__ void k_fine_dinv(const Real* __restrict__ ke, const uint8_t* __restrict__ fixed, Dims d,
-                            Real* __restrict__ dinv) {
+                            Real* __restrict__ dinv, Real* __restrict__ dinv_s) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int)d.n) return;
   if (fixed[idx]) {
     dinv[idx] = Real(1);
+    if (DIM == 2) dinv_s[idx] = Real(-1);
     return;
   }
   int i, j, k;
@@ -316,7 +318,9 @@ __global__ void k_fine_dinv(const Real* __restrict__ ke, const uint8_t* __restri
     const Real kv = CK(e, d.ne) ? ke[e] : Real(0);
     if (ok) ks += kv;
   }
-  dinv[idx] = Real(1) / (ks * Real(DIM == 2 ? 4.0 / 6.0 : 4.0 / 12.0));
+  const Real dv = Real(1) / (ks * Real(DIM == 2 ? 4.0 / 6.0 : 4.0 / 12.0));
+  dinv[idx] = dv;
+  if (DIM == 2) dinv_s[idx] = dv;
 }
 
 // Lower band of the coarsest operator: band[i*(bw+1) + (j - i + bw)].
@@ -736,6 +740,7 @@ static void alloc_levels(Ctx& c, LevelBuf<Real>* h) {
   for (int l = 0; l < c.nl; ++l) {
     const Dims& d = c.L[l];
     MGAR_CUDA(cudaMalloc(&h[l].dinv, d.n * sizeof(Real)));
+    if (l == 0 && c.dim == 2) MGAR_CUDA(cudaMalloc(&h[l].dinv_s, d.n * sizeof(Real)));
     MGAR_CUDA(cudaMalloc(&h[l].t, d.n * sizeof(Real)));
     MGAR_CUDA(cudaMalloc(&h[l].r, d.n * sizeof(Real)));
     if (l >= 1) {
@@ -751,6 +756,7 @@ template <typename Real>
 static void free_levels(LevelBuf<Real>* h) {
   for (int l = 0; l < kMaxLevels; ++l) {
     cudaFree(h[l].dinv);
+    cudaFree(h[l].dinv_s);
     cudaFree(h[l].t);
     cudaFree(h[l].r);
     cudaFree(h[l].st);
@@ -923,7 +929,8 @@ static void build_levels(Ctx& c, const Real* ke0, LevelBuf<Real>* h) {
   const int nen = 1 << DIM;
   const double* k0 = c.tables;
   const Real* G = g_tables<Real>(c);
-  k_fine_dinv<Real, DIM><<<blocks_for(c.L[0].n), kThreads, 0, s>>>(ke0, c.fixed, c.L[0], h[0].dinv);
+  k_fine_dinv<Real, DIM><<<blocks_for(c.L[0].n), kThreads, 0, s>>>(ke0, c.fixed, c.L[0], h[0].dinv,
+                                                                        h[0].dinv_s);
   MGAR_LAUNCH_CHECK();
   for (int l = 0; l + 1 < c.nl; ++l) {
     const Dims& f = c.L[l];

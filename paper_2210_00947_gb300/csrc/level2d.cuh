@@ -1,0 +1,414 @@
+// Tiled V-cycle passes of the 2D levels, shared by the single-design V-cycle
+// (FP32 and FP64) and the batched one.  Each pass of Table 1 used to be a
+// kernel of its own that gathered every operand of a node from global memory
+// with bounds and Dirichlet tests per neighbour; the finest level's passes ran
+// at 4-6 times their bytes' time and the coarse ones at the latency of a
+// launch.  A block here stages a tile with its rim in shared memory (off-grid
+// and fixed neighbours as zeros, so the stencil needs no tests) and does all
+// that follows from it:
+//   down, finest:  x = w D^-1 b (or the given x), r = b - A x, b_c = P^T r,
+//                  x_c = w D_c^-1 b_c        (three or four passes before)
+//   up, finest:    v = x + P x_c, x' = v + w D^-1 (b - A v), r . x'   (two)
+//   down, coarse:  r = b - A x, b_c = P^T r, x_c = w D_c^-1 b_c       (two)
+//   up, coarse:    v = x + P x_c, x' = v + w D^-1 (b - A v)     (one or two)
+// The residual never goes to memory.  1025^2 nodes in FP32: down 7.7 us (21.5
+// as three kernels), up with r . x 14 us (26.8), a coarse level 2.6-5.3 us each
+// way (6-8).  Bound by instruction issue (100 warp instructions per node down,
+// 165 up) and the sum's cross-block stage.  Tiles are 64 columns wide with their
+// rim (two nodes per lane), so a warp's rows are coalesced and no lane divides
+// to find its node; tall enough that the rim costs 8 % (residuals) to 24 %
+// (x) more, short enough that a 1024^2 grid fills the chip in one wave.
+#pragma once
+#include "common.cuh"
+
+namespace mgar {
+namespace l2d {
+
+constexpr int kW = 64;        // columns of a finest-level tile with its rim
+constexpr int kThreads2 = 256;
+// Each of the eight warps owns kR consecutive rows (two columns per lane), so
+// the rows' stencils share their neighbours' shared-memory loads, and one
+// address per array serves all six nodes of a thread.
+constexpr int kR = 3, kRows = 8 * kR;
+// down: coarse nodes per tile; fine columns 2 kCX + 3 = 63, rows 2 kCY + 3 = 23
+constexpr int kCX = 30, kCY = 10;
+// up: own nodes per tile
+constexpr int kUX = 62, kUY = kRows - 2;
+// coarse levels: down, coarse nodes per tile (31 x 7 residuals); up, own nodes
+constexpr int kDX = 15, kDY = 3, kDownThreads = 32 * (2 * kDY + 1);
+constexpr int kPX = 30, kPY = 8, kUpThreads = 32 * (kPY + 2);
+
+__host__ __device__ __forceinline__ int tiles(int n, int per) { return (n + per - 1) / per; }
+
+// A finest level (matrix-free operator).
+// dinv: 1/diag, negated on fixed nodes (one load for both)
+template <typename Real>
+struct Fine {
+  const Real* ke;
+  const Real* dinv;
+  int ex, ey, cNX, cNY;  // elements; nodes of the next level
+  Real omega;
+};
+
+// A coarse level (assembled stencil).
+template <typename Real>
+struct Coarse {
+  StencilOp<Real> op;
+  int ex, ey, cNX, cNY;
+  Real omega;
+};
+
+// Restriction weights of coarse node I from the fine nodes 2I-1, 2I, 2I+1 (nf
+// fine elements; off-grid residuals are zero, so only the injected last node
+// of an odd axis differs from 1/2, 1, 1/2).
+template <typename Real>
+__device__ __forceinline__ void restrict_weights(int I, int nf, Real& w0, Real& w1, Real& w2) {
+  const int f = 2 * I;
+  w0 = f - 1 == nf ? Real(1) : Real(0.5);
+  w1 = Real(1);
+  w2 = f + 1 == nf ? Real(0) : Real(0.5);
+}
+
+template <typename Real, int W>
+__device__ __forceinline__ Real restrict_sum(const Real (*r)[W], int c, int y, int I, int J, int ex,
+                                             int ey) {
+  Real x0, x1, x2, y0, y1, y2;
+  restrict_weights<Real>(I, ex, x0, x1, x2);
+  restrict_weights<Real>(J, ey, y0, y1, y2);
+  const Real a = x0 * r[y][c] + x1 * r[y][c + 1] + x2 * r[y][c + 2];
+  const Real b = x0 * r[y + 1][c] + x1 * r[y + 1][c + 1] + x2 * r[y + 1][c + 2];
+  const Real d = x0 * r[y + 2][c] + x1 * r[y + 2][c + 1] + x2 * r[y + 2][c + 2];
+  return y0 * a + y1 * b + y2 * d;
+}
+
+// The Q4 rows times 6 of column c at the tile rows y0 .. y0 + kR - 1, tile row
+// y at shared-memory row y + 1: x with off-grid and fixed values zero, k the
+// element to the lower right of the node; f(q, row) with row as a function of
+// the centre value.
+template <typename Real, class F>
+__device__ __forceinline__ void q4_rows(const Real (*x)[kW], const Real (*k)[kW], int c, int y0, F&& f) {
+  Real xl = x[y0][c - 1], xc = x[y0][c], xr = x[y0][c + 1];
+  Real yl = x[y0 + 1][c - 1], yc = x[y0 + 1][c], yr = x[y0 + 1][c + 1];
+  Real k00 = k[y0][c - 1], k01 = k[y0][c];
+#pragma unroll
+  for (int q = 0; q < kR; ++q) {
+    const Real zl = x[y0 + q + 2][c - 1], zc = x[y0 + q + 2][c], zr = x[y0 + q + 2][c + 1];
+    const Real k10 = k[y0 + q + 1][c - 1], k11 = k[y0 + q + 1][c];
+    const Real s = k00 + k01, n = k10 + k11;
+    const Real dg = k00 * xl + k01 * xr + k10 * zl + k11 * zr;
+    const Real ed = (k00 + k10) * yl + (k01 + k11) * yr + s * xc + n * zc;
+    f(q, yc, [&](Real xi) { return Real(4) * (s + n) * xi - ed - Real(2) * dg; });
+    xl = yl, xc = yc, xr = yr;
+    yl = zl, yc = zc, yr = zr;
+    k00 = k10, k01 = k11;
+  }
+}
+
+// (P x_c) at a fine node whose first coarse tap sits at c[y][x]; hx, hy:
+// halfway between two coarse nodes along x, y.  Weights are powers of two, so
+// they scale the sum exactly.
+template <typename Real, int W>
+__device__ __forceinline__ Real prolong_sum(const Real (*c)[W], int x, int y, bool hx, bool hy) {
+  Real s = c[y][x];
+  if (hx) s += c[y][x + 1];
+  if (hy) {
+    s += c[y + 1][x];
+    if (hx) s += c[y + 1][x + 1];
+  }
+  const Real wx = hx ? Real(0.5) : Real(1), wxy = hy ? Real(0.5) * wx : wx;
+  return wxy * s;
+}
+
+// First coarse tap of fine node i, and whether it is halfway.
+__device__ __forceinline__ int first_tap(int i, int nf, bool& half) {
+  half = (i & 1) && i < nf;
+  return (i & 1) && i == nf ? (i + 1) >> 1 : i >> 1;
+}
+
+// A thread's six nodes in a tile whose first node is (fx0, fy0): rows y0 + q,
+// columns lane + 32 h.
+struct Place {
+  int lane, w, y0;
+  bool con[2], eon[2];  // column on the grid, its element on the grid
+  __device__ __forceinline__ Place(int fx0, int ex) {
+    lane = threadIdx.x & 31;
+    w = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
+    y0 = kR * w;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const unsigned i = (unsigned)(fx0 + lane + 32 * h);
+      con[h] = i <= (unsigned)ex;
+      eon[h] = i < (unsigned)ex;
+    }
+  }
+};
+
+// ------------------------------------------------------------- finest, down
+// tile row y at row y + 1; the rows before the first and after the last are
+// read by the rim rows' stencils, whose results are not used
+template <typename Real>
+struct DownSmem {
+  Real x[kRows + 2][kW];
+  Real k[kRows + 1][kW];
+  Real r[kRows][kW];
+};
+
+// ZERO: x = w D^-1 b, written to t; otherwise x is read from t.  bc and (not
+// null) xc of the tile's coarse nodes.
+template <typename Real, bool ZERO>
+__device__ __forceinline__ void fine_down(DownSmem<Real>& s, const Fine<Real>& f, int tx, int ty,
+                                          const Real* __restrict__ b, Real* __restrict__ t,
+                                          Real* __restrict__ bc, const Real* __restrict__ dinvc,
+                                          Real* __restrict__ xc) {
+  const int NX = f.ex + 1, NY = f.ey + 1;
+  const int I0 = tx * kCX, J0 = ty * kCY;
+  const int fx0 = 2 * I0 - 2, fy0 = 2 * J0 - 2;
+  const Place p(fx0, f.ex);
+  const int64_t at = fx0 + p.lane + (int64_t)NX * (fy0 + p.y0);
+  const int64_t eat = fx0 + p.lane + (int64_t)f.ex * (fy0 + p.y0);
+  Real dv[kR][2], bv[kR][2];
+  bool ron[kR];
+  // hierarchy data before the wait on the predecessor
+#pragma unroll
+  for (int q = 0; q < kR; ++q) {
+    const unsigned j = (unsigned)(fy0 + p.y0 + q);
+    ron[q] = j < (unsigned)NY;
+    const bool reon = j < (unsigned)f.ey;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      dv[q][h] = Real(0);
+      if (ron[q] && p.con[h]) dv[q][h] = f.dinv[at + q * NX + 32 * h];
+      Real kv = Real(0);
+      if (reon && p.eon[h]) kv = f.ke[eat + q * f.ex + 32 * h];
+      s.k[p.y0 + q + 1][p.lane + 32 * h] = kv;
+    }
+  }
+  Real dc[2] = {Real(0), Real(0)};
+  int cidx[2];
+  bool con[2];
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    const int I = I0 + p.lane, J = J0 + p.w + 8 * g;
+    con[g] = p.w + 8 * g < kCY && p.lane < kCX && I < f.cNX && J < f.cNY;
+    cidx[g] = I + f.cNX * J;
+    if (xc && con[g]) dc[g] = dinvc[cidx[g]];
+  }
+  pdl_wait();
+  pdl_trigger();
+#pragma unroll
+  for (int q = 0; q < kR; ++q)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      bv[q][h] = Real(0);
+      if (ron[q] && p.con[h]) bv[q][h] = b[at + q * NX + 32 * h];
+    }
+#pragma unroll
+  for (int q = 0; q < kR; ++q)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int y = p.y0 + q, c = p.lane + 32 * h;
+      Real x = Real(0);
+      if (ZERO) {
+        x = f.omega * fabs(dv[q][h]) * bv[q][h];
+        if (y >= 2 && y < 2 * kCY + 2 && c >= 2 && c < 2 * kCX + 2 && ron[q] && p.con[h])
+          t[at + q * NX + 32 * h] = x;
+      } else if (ron[q] && p.con[h]) {
+        x = t[at + q * NX + 32 * h];
+      }
+      s.x[y + 1][c] = dv[q][h] > Real(0) ? x : Real(0);
+    }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int c = p.lane + 32 * h;
+    if (c >= 1 && c < 2 * kCX + 2)
+      q4_rows<Real>(s.x, s.k, c, p.y0, [&](int q, Real xi, auto&& row) {
+        const Real r = bv[q][h] - row(xi) * Real(1.0 / 6.0);
+        s.r[p.y0 + q][c] = dv[q][h] > Real(0) ? r : Real(0);
+      });
+  }
+  __syncthreads();
+#pragma unroll
+  for (int g = 0; g < 2; ++g)
+    if (con[g]) {
+      const int cy = p.w + 8 * g;
+      const Real v = restrict_sum<Real, kW>(s.r, 2 * p.lane + 1, 2 * cy + 1, I0 + p.lane, J0 + cy,
+                                            f.ex, f.ey);
+      bc[cidx[g]] = v;
+      if (xc) xc[cidx[g]] = f.omega * dc[g] * v;
+    }
+}
+
+// --------------------------------------------------------------- finest, up
+template <typename Real>
+struct UpSmem {
+  Real v[kRows + 2][kW];
+  Real k[kRows + 1][kW];
+  Real c[kRows / 2 + 3][kW / 2 + 4];
+};
+
+// xout = v + w D^-1 (b - A v), v = t + P res (fixed nodes keep t); dot(at, b,
+// x', early) is called for every node of the tile, early what pre(at) gave for
+// it beside the operands' loads.
+template <typename Real, class Pre, class Dot>
+__device__ __forceinline__ void fine_up(UpSmem<Real>& s, const Fine<Real>& f, int tx, int ty,
+                                        const Real* __restrict__ b, const Real* __restrict__ t,
+                                        const Real* __restrict__ res, Real* __restrict__ xout,
+                                        Pre&& pre, Dot&& dot) {
+  constexpr int CR = kRows / 2 + 2, CC = kW / 2 + 2;
+  const int NX = f.ex + 1, NY = f.ey + 1;
+  const int fx0 = tx * kUX - 1, fy0 = ty * kUY - 1;
+  const int ci0 = max(fx0, 0) >> 1, cj0 = max(fy0, 0) >> 1;
+  const Place p(fx0, f.ex);
+  const int64_t at = fx0 + p.lane + (int64_t)NX * (fy0 + p.y0);
+  const int64_t eat = fx0 + p.lane + (int64_t)f.ex * (fy0 + p.y0);
+  Real dv[kR][2], bv[kR][2], tv[kR][2];
+  decltype(pre(int64_t(0))) early[kR][2];
+  bool ron[kR];
+#pragma unroll
+  for (int q = 0; q < kR; ++q) {
+    const unsigned j = (unsigned)(fy0 + p.y0 + q);
+    ron[q] = j < (unsigned)NY;
+    const bool reon = j < (unsigned)f.ey;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      dv[q][h] = Real(0);
+      if (ron[q] && p.con[h]) dv[q][h] = f.dinv[at + q * NX + 32 * h];
+      Real kv = Real(0);
+      if (reon && p.eon[h]) kv = f.ke[eat + q * f.ex + 32 * h];
+      s.k[p.y0 + q + 1][p.lane + 32 * h] = kv;
+    }
+  }
+  pdl_wait();
+  pdl_trigger();
+  // coarse values under the tile (clamped: values past the grid are not used)
+  for (int cy = p.w; cy < CR; cy += 8)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int cx = p.lane + 32 * h;
+      if (cx < CC)
+        s.c[cy][cx] = res[min(ci0 + cx, f.cNX - 1) + f.cNX * min(cj0 + cy, f.cNY - 1)];
+    }
+#pragma unroll
+  for (int q = 0; q < kR; ++q)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      bv[q][h] = tv[q][h] = Real(0);
+      if (ron[q] && p.con[h]) {
+        bv[q][h] = b[at + q * NX + 32 * h];
+        tv[q][h] = t[at + q * NX + 32 * h];
+        early[q][h] = pre(at + q * NX + 32 * h);
+      }
+    }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    bool hx;
+    const int cx = min(max(first_tap(fx0 + p.lane + 32 * h, f.ex, hx) - ci0, 0), CC);
+#pragma unroll
+    for (int q = 0; q < kR; ++q) {
+      bool hy;
+      const int cy = min(max(first_tap(fy0 + p.y0 + q, f.ey, hy) - cj0, 0), CR - 1);
+      const bool in = dv[q][h] > Real(0);
+      if (in) tv[q][h] += prolong_sum<Real, kW / 2 + 4>(s.c, cx, cy, hx, hy);
+      s.v[p.y0 + q + 1][p.lane + 32 * h] = in ? tv[q][h] : Real(0);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int c = p.lane + 32 * h;
+    if (c >= 1 && c <= kUX && p.con[h])
+      q4_rows<Real>(s.v, s.k, c, p.y0, [&](int q, Real, auto&& row) {
+        const int y = p.y0 + q;
+        if (!(y >= 1 && y <= kUY && ron[q])) return;
+        const Real v = tv[q][h];
+        const Real ax = dv[q][h] < Real(0) ? v : row(v) * Real(1.0 / 6.0);
+        const Real xo = v + f.omega * fabs(dv[q][h]) * (bv[q][h] - ax);
+        const int64_t o = at + q * NX + 32 * h;
+        xout[o] = xo;
+        dot(bv[q][h], xo, early[q][h]);
+      });
+  }
+}
+
+// ------------------------------------------------------------- coarse, down
+template <typename Real>
+__device__ __forceinline__ void coarse_down(Real (*s)[32], const Coarse<Real>& f, int tx, int ty,
+                                            const Real* __restrict__ b, const Real* __restrict__ x,
+                                            Real* __restrict__ bc, const Real* __restrict__ dinvc,
+                                            Real* __restrict__ xc) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int I0 = tx * kDX, J0 = ty * kDY;
+  const int i = 2 * I0 - 1 + lane, j = 2 * J0 - 1 + w;
+  const bool on = lane < 2 * kDX + 1 && i >= 0 && i < f.op.NX && j >= 0 && j < f.op.NY;
+  Real sv[9];
+  if (on) stencil_coefs<2>(f.op, i, j, 0, sv);
+  const int I = I0 + lane, J = J0 + w;
+  const bool con = lane < kDX && w < kDY && I < f.cNX && J < f.cNY;
+  const int cidx = con ? I + f.cNX * J : 0;
+  const Real dc = xc && con ? dinvc[cidx] : Real(0);
+  pdl_wait();
+  pdl_trigger();
+  Real r = Real(0);
+  if (on) r = b[i + f.op.NX * j] - stencil_apply<2, Real, false>(f.op, x, i, j, 0, sv);
+  s[w][lane] = r;
+  __syncthreads();
+  if (con) {
+    const Real v = restrict_sum<Real, 32>(s, 2 * lane, 2 * w, I, J, f.ex, f.ey);
+    bc[cidx] = v;
+    if (xc) xc[cidx] = f.omega * dc * v;
+  }
+}
+
+// --------------------------------------------------------------- coarse, up
+template <typename Real>
+struct CoarseUpSmem {
+  Real v[kPY + 2][32];
+};
+
+template <typename Real>
+__device__ __forceinline__ void coarse_up(CoarseUpSmem<Real>& s, const Coarse<Real>& f, int tx, int ty,
+                                          const Real* __restrict__ b, const Real* __restrict__ x,
+                                          const Real* __restrict__ res, Real* __restrict__ xout) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int i = tx * kPX - 1 + lane, j = ty * kPY - 1 + w;
+  const bool on = i >= 0 && i < f.op.NX && j >= 0 && j < f.op.NY;
+  const bool own = on && lane >= 1 && lane <= kPX && w >= 1 && w <= kPY;
+  const int idx = on ? i + f.op.NX * j : 0;
+  Real sv[9], dv = Real(0);
+  if (own) {
+    stencil_coefs<2>(f.op, i, j, 0, sv);
+    dv = f.op.dinv[idx];
+  }
+  bool hx = false, hy = false;
+  const int cx = on ? first_tap(i, f.ex, hx) : 0, cy = on ? first_tap(j, f.ey, hy) : 0;
+  pdl_wait();
+  pdl_trigger();
+  Real v = Real(0), bv = Real(0);
+  if (on) {
+    // four taps, an unused one repeating the first
+    const int c0 = cx + f.cNX * cy, ox = hx ? 1 : 0, oy = hy ? f.cNX : 0;
+    const Real r0 = res[c0], r1 = res[c0 + ox], r2 = res[c0 + oy], r3 = res[c0 + ox + oy];
+    v = x[idx];
+    if (own) bv = b[idx];
+    Real p = r0;
+    if (hx) p += r1;
+    if (hy) {
+      p += r2;
+      if (hx) p += r3;
+    }
+    v += (hx ? Real(0.5) : Real(1)) * (hy ? Real(0.5) : Real(1)) * p;
+  }
+  s.v[w][lane] = v;
+  __syncthreads();
+  if (own) {
+    Real acc = Real(0);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) acc += sv[q] * s.v[w - 1 + q / 3][lane - 1 + q % 3];
+    xout[idx] = v + f.omega * dv * (bv - acc);
+  }
+}
+
+}  // namespace l2d
+}  // namespace mgar

@@ -327,9 +327,18 @@ static int solve_mgcg_fp(Ctx& c, double* T, int* iters, double* relres) {
   int it = 0;
   if (!(rel <= c.p.eps2)) {
     require(std::isfinite(rel), MGAR_ERR_NONFINITE, "non-finite initial residual");
-    precondition(c, c.r, c.z);
+    // z = M r and r . z, in one with the 2D V-cycle's tiled passes
+    auto precondition_rz = [&](int slot) {
+      if (c.dim == 2 && vcycle_dot_ok(c)) {
+        run_graph(c, slot == S_RZ0 ? 11 : 12, c.r, c.z, vcycle_profiled(c),
+                  [&] { vcycle_dot64(c, c.r, c.z, c.dsc + slot); });
+      } else {
+        precondition(c, c.r, c.z);
+        dot(c, c.r, c.z, n, c.dsc + slot);
+      }
+    };
     int a = S_RZ0, b = S_RZ1;
-    dot(c, c.r, c.z, n, c.dsc + a);
+    precondition_rz(a);
     MGAR_CUDA(cudaMemcpyAsync(c.pv, c.z, n * sizeof(double), cudaMemcpyDeviceToDevice, c.stream));
     while (it < c.p.cg_max) {
       apply_fine64(c, c.ke, c.pv, c.Ap, c.dsc + S_PAP);
@@ -342,8 +351,7 @@ static int solve_mgcg_fp(Ctx& c, double* T, int* iters, double* relres) {
       rel = std::sqrt(c.hsc[S_RR]) / c.qnorm;
       require(std::isfinite(rel), MGAR_ERR_NONFINITE, "CG breakdown (non-finite residual)");
       if (rel <= c.p.eps2) break;
-      precondition(c, c.r, c.z);
-      dot(c, c.r, c.z, n, c.dsc + b);
+      precondition_rz(b);
       k_cg_p<<<red_blocks(c), kThreads, 0, c.stream>>>(c.pv, c.z, n, c.dsc + b, c.dsc + a);
       MGAR_LAUNCH_CHECK();
       std::swap(a, b);

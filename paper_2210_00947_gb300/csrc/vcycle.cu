@@ -9,6 +9,7 @@
 // coarse ones are assembled 3^d-point stencils.  Every kernel is templated on
 // the working precision (FP64, or FP32 for the mixed preconditioner).
 #include "common.cuh"
+#include "level2d.cuh"
 #include "levelops.cuh"
 
 namespace mgar {
@@ -91,85 +92,73 @@ __global__ void k_apply(Row row, const Real* __restrict__ x, Real* __restrict__ 
   if (DOT) block_sum_finish<1>(v, partials, counter, out);
 }
 
-// The 2D finest-level passes with kNptFine nodes per thread (nodes base,
-// base + blockDim.x, ...): each thread has several nodes' loads in flight and
-// the launch a quarter of the blocks; the arithmetic per node is that of the
-// one-node kernels above.
-constexpr int kNptFine = 4;
+// The 2D levels' tiled passes (level2d.cuh).
+template <typename Real, bool ZERO>
+__global__ void __launch_bounds__(l2d::kThreads2) k_down2d(l2d::Fine<Real> f, const Real* __restrict__ b,
+                                                           Real* __restrict__ t, Real* __restrict__ bc,
+                                                           const Real* __restrict__ dinvc,
+                                                           Real* __restrict__ xc) {
+  __shared__ l2d::DownSmem<Real> s;
+  l2d::fine_down<Real, ZERO>(s, f, blockIdx.x, blockIdx.y, b, t, bc, dinvc, xc);
+}
 
-inline int blocks_npt(int64_t n) {
-  const int64_t per = (int64_t)kThreads * kNptFine;
-  return (int)((n + per - 1) / per);
+// DOT: also r . xout into *dout, r given as df64 pairs (the mixed CG's) or,
+// without them, b itself.  FP32: double-float warp sums, FP64 across warps.
+template <typename Real, bool DOT>
+__global__ void __launch_bounds__(l2d::kThreads2) k_up2d(l2d::Fine<Real> f, const Real* __restrict__ b,
+                                                         const Real* __restrict__ t,
+                                                         const Real* __restrict__ res,
+                                                         Real* __restrict__ xout,
+                                                         const float2* __restrict__ rdot,
+                                                         double* partials, unsigned int* counter,
+                                                         double* dout) {
+  __shared__ l2d::UpSmem<Real> s;
+  float ah = 0.f, al = 0.f;
+  double acc64[1] = {0.0};
+  l2d::fine_up<Real>(
+      s, f, blockIdx.x, blockIdx.y, b, t, res, xout,
+      [&](int64_t at) { return DOT && sizeof(Real) == 4 && rdot ? rdot[at] : make_float2(0.f, 0.f); },
+      [&](Real bv, Real xo, float2 rv) {
+        if constexpr (DOT && sizeof(Real) == 4)
+          df_acc_mulf(ah, al, rdot ? df{rv.x, rv.y} : df{bv, 0.f}, xo);
+        else if constexpr (DOT)
+          acc64[0] += bv * xo;
+      });
+  if constexpr (DOT) {
+    const int bid = blockIdx.x + gridDim.x * blockIdx.y, nb = gridDim.x * gridDim.y;
+    if constexpr (sizeof(Real) == 4) {
+      double v;
+      if (block_sum_last_df(df_make(ah, al), partials, counter, v, threadIdx.x, l2d::kThreads2, bid, nb) &&
+          threadIdx.x == 0)
+        *dout = v;
+    } else {
+      double v[1];
+      if (block_sum_last_ids<1>(acc64, partials, counter, v, threadIdx.x, l2d::kThreads2, bid, nb) &&
+          threadIdx.x == 0)
+        *dout = v[0];
+    }
+  }
 }
 
 template <typename Real>
-__global__ void k_jacobi_zero_n(const Real* __restrict__ b, Real* __restrict__ x,
-                                const Real* __restrict__ dinv, Real omega, int n) {
-  const int base = blockIdx.x * blockDim.x * kNptFine + threadIdx.x;
-  Real bv[kNptFine], dv[kNptFine];
-#pragma unroll
-  for (int u = 0; u < kNptFine; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < n) {
-      bv[u] = b[idx];
-      dv[u] = dinv[idx];
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < kNptFine; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < n) x[idx] = omega * dv[u] * bv[u];
-  }
+__global__ void __launch_bounds__(l2d::kDownThreads) k_coarse_down2d(l2d::Coarse<Real> f,
+                                                                     const Real* __restrict__ b,
+                                                                     const Real* __restrict__ x,
+                                                                     Real* __restrict__ bc,
+                                                                     const Real* __restrict__ dinvc,
+                                                                     Real* __restrict__ xc) {
+  __shared__ Real s[2 * l2d::kDY + 1][32];
+  l2d::coarse_down<Real>(s, f, blockIdx.x, blockIdx.y, b, x, bc, dinvc, xc);
 }
 
-template <class Row, typename Real>
-__global__ void k_residual_n(Row row, const Real* __restrict__ b, const Real* __restrict__ x,
-                             Real* __restrict__ r) {
-  const int base = blockIdx.x * blockDim.x * kNptFine + threadIdx.x;
-#pragma unroll
-  for (int u = 0; u < kNptFine; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < row.size()) r[idx] = b[idx] - row(x, idx);
-  }
-}
-
-template <typename Real, int DIM>
-__global__ void k_prolong_n(const Real* __restrict__ xc, const Real* cur, Real* dst, Dims f, Dims cd,
-                            const uint8_t* __restrict__ fixed) {
-  pdl_wait();
-  pdl_trigger();
-  const int base = blockIdx.x * blockDim.x * kNptFine + threadIdx.x;
-#pragma unroll
-  for (int u = 0; u < kNptFine; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < f.n) prolong_node<Real, DIM>(xc, cur, dst, f, cd, fixed, idx);
-  }
-}
-
-// One damped-Jacobi sweep; with DOT also r . xout (r as df64 pairs: the CG's
-// r . z) into *dout, double-float warp sums, FP64 across warps and blocks.
-template <class Row, typename Real, bool DOT>
-__global__ void k_jacobi_n(Row row, const Real* __restrict__ b, const Real* __restrict__ xin,
-                           Real* __restrict__ xout, const Real* __restrict__ dinv, Real omega,
-                           const float2* __restrict__ rdot, double* partials,
-                           unsigned int* counter, double* dout) {
-  const int base = blockIdx.x * blockDim.x * kNptFine + threadIdx.x;
-  df acc{0.f, 0.f};
-#pragma unroll
-  for (int u = 0; u < kNptFine; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < row.size()) {
-      const Real ax = row(xin, idx);
-      const Real xo = xin[idx] + omega * dinv[idx] * (b[idx] - ax);
-      xout[idx] = xo;
-      if (DOT) {
-        // r . z, or b . z when no r is given
-        const float2 rv = rdot ? rdot[idx] : make_float2((float)b[idx], 0.f);
-        acc = df_add(acc, df_mulf(df{rv.x, rv.y}, (float)xo));
-      }
-    }
-  }
-  if (DOT) block_sum_finish_df(acc, partials, counter, dout);
+template <typename Real>
+__global__ void __launch_bounds__(l2d::kUpThreads) k_coarse_up2d(l2d::Coarse<Real> f,
+                                                                 const Real* __restrict__ b,
+                                                                 const Real* __restrict__ x,
+                                                                 const Real* __restrict__ res,
+                                                                 Real* __restrict__ xout) {
+  __shared__ l2d::CoarseUpSmem<Real> s;
+  l2d::coarse_up<Real>(s, f, blockIdx.x, blockIdx.y, b, x, res, xout);
 }
 
 template <typename Real, int DIM>
@@ -563,7 +552,7 @@ static bool bottom_fits(int csize) {
 void bottom_prepare(Ctx& c) {
   c.bottom_ok = false;
   for (int csize = kBottomClusterMax; csize >= 8 && !c.bottom_ok; csize /= 2) {
-    c.bottom_ok = c.dim == 2 ? bottom_fits<float, 2>(csize) : bottom_fits<float, 3>(csize);
+    c.bottom_ok = c.dim == 3 && bottom_fits<float, 3>(csize);
     if (c.bottom_ok) c.bottom_cluster = csize;
   }
 }
@@ -583,14 +572,76 @@ static void launch_prolong(Ctx& c, bool pdl, const Real* xc, const Real* cur, Re
   }
 }
 
+// The coarsest level by its explicit inverse.
+template <typename Real>
+static void coarse_solve(Ctx& c) {
+  LevelBuf<Real>* h = levels<Real>(c);
+  const int l = c.nl - 1, rows_per_block = kThreads / 32;
+  launch_pdl(c.stream, c.use_pdl, k_coarse_solve<Real, typename CoarseT<Real>::T>,
+             dim3((c.nc + rows_per_block - 1) / rows_per_block), dim3(kThreads),
+             (const typename CoarseT<Real>::T*)CoarseT<Real>::inv(c), (const Real*)h[l].b, h[l].x, c.nc);
+  MGAR_LAUNCH_CHECK_AT(level_site(5, l));
+}
+
+// The 2D V-cycle with one pre- and one post-sweep in the tiled passes: one
+// launch per level and direction and the coarsest solve, in either precision
+// (FP64 gains from the passes saved and, on small grids, from 2 instead of 5
+// launches per level; its rims cost 8 % more FP64 operations).  dout: r . x
+// (r = b, or rdot's pairs when given).
+template <typename Real>
+static void vcycle_fused2(Ctx& c, const Real* b0, Real* x0, bool zero_guess,
+                          const float2* rdot = nullptr, double* dout = nullptr) {
+  LevelBuf<Real>* h = levels<Real>(c);
+  const int nl = c.nl;
+  const Real om = (Real)c.p.omega;
+  const Dims& d0 = c.L[0];
+  auto next_x = [&](int l) { return l + 2 < nl ? h[l + 1].x : (Real*)nullptr; };
+  auto coarse = [&](int l) {
+    return l2d::Coarse<Real>{stencil_row<Real, 2>(c, l).op, c.L[l].ex, c.L[l].ey, c.L[l + 1].NX,
+                             c.L[l + 1].NY, om};
+  };
+  const l2d::Fine<Real> f{ref_ke<Real>(c), h[0].dinv_s, d0.ex, d0.ey, c.L[1].NX, c.L[1].NY, om};
+  {
+    ProfScope ps(c, MGAR_KC_SMOOTH0);
+    if (!zero_guess) sweep<Real, 2>(c, 0, b0, x0, h[0].t);
+    ProfScope pr(c, MGAR_KC_RESID0);
+    const dim3 grid(l2d::tiles(c.L[1].NX, l2d::kCX), l2d::tiles(c.L[1].NY, l2d::kCY));
+    launch_pdl(c.stream, c.use_pdl, zero_guess ? k_down2d<Real, true> : k_down2d<Real, false>, grid,
+               dim3(l2d::kThreads2), f, b0, h[0].t, h[1].b, (const Real*)h[1].dinv, next_x(0));
+    MGAR_LAUNCH_CHECK_AT(level_site(0, 0));
+  }
+  for (int l = 1; l + 1 < nl; ++l) {
+    const dim3 grid(l2d::tiles(c.L[l + 1].NX, l2d::kDX), l2d::tiles(c.L[l + 1].NY, l2d::kDY));
+    launch_pdl(c.stream, c.use_pdl, k_coarse_down2d<Real>, grid, dim3(l2d::kDownThreads), coarse(l),
+               (const Real*)h[l].b, (const Real*)h[l].x, h[l + 1].b, (const Real*)h[l + 1].dinv,
+               next_x(l));
+    MGAR_LAUNCH_CHECK_AT(level_site(3, l));
+  }
+  coarse_solve<Real>(c);
+  const Real* res = h[nl - 1].x;
+  for (int l = nl - 2; l >= 1; --l) {
+    const dim3 grid(l2d::tiles(c.L[l].NX, l2d::kPX), l2d::tiles(c.L[l].NY, l2d::kPY));
+    launch_pdl(c.stream, c.use_pdl, k_coarse_up2d<Real>, grid, dim3(l2d::kUpThreads), coarse(l),
+               (const Real*)h[l].b, (const Real*)h[l].x, res, h[l].t);
+    MGAR_LAUNCH_CHECK_AT(level_site(4, l));
+    res = h[l].t;
+  }
+  ProfScope ps(c, MGAR_KC_SMOOTH0);
+  const dim3 grid(l2d::tiles(d0.NX, l2d::kUX), l2d::tiles(d0.NY, l2d::kUY));
+  launch_pdl(c.stream, c.use_pdl, dout ? k_up2d<Real, true> : k_up2d<Real, false>, grid,
+             dim3(l2d::kThreads2), f, b0, (const Real*)h[0].t, res, x0, rdot, c.partials, c.counter,
+             dout);
+  MGAR_LAUNCH_CHECK_AT(level_site(1, 0));
+}
+
 // Table 1 with one pre- and one post-sweep and a zero guess below the finest
 // level: per level one fused pre kernel (smooth from zero + residual), the
 // restriction, and one fused post kernel (interpolation + smooth); the small
 // levels at the bottom run in one cluster launch.
-template <int DIM>
-static void vcycle_fused(Ctx& c, const float* b0, float* x0, bool zero_guess,
+static void vcycle_fused3(Ctx& c, const float* b0, float* x0, bool zero_guess,
                          const float2* rdot = nullptr, double* dout = nullptr) {
   using Real = float;
+  constexpr int DIM = 3;
   LevelBuf<Real>* h = levels<Real>(c);
   const int nl = c.nl;
   const Real om = (Real)c.p.omega;
@@ -600,34 +651,19 @@ static void vcycle_fused(Ctx& c, const float* b0, float* x0, bool zero_guess,
   Real* cur0;
   {
     ProfScope ps(c, MGAR_KC_SMOOTH0);
-    if (DIM == 3) {
-      if (zero_guess) {
-        fine3d(c, 0, ref_ke<Real>(c), b0, h[0].dinv, nullptr, nullptr, h[0].t, h[0].r);
-      } else {
-        fine3d(c, 3, ref_ke<Real>(c), b0, h[0].dinv, x0, nullptr, h[0].t, nullptr);
-        fine3d(c, 2, ref_ke<Real>(c), b0, h[0].dinv, h[0].t, nullptr, h[0].r, nullptr);
-      }
-      cur0 = h[0].t;
+    if (zero_guess) {
+      fine3d(c, 0, ref_ke<Real>(c), b0, h[0].dinv, nullptr, nullptr, h[0].t, h[0].r);
     } else {
-      if (zero_guess) {
-        k_jacobi_zero_n<<<blocks_npt(d0.n), kThreads, 0, c.stream>>>(b0, h[0].t, h[0].dinv, om,
-                                                                     (int)d0.n);
-        MGAR_LAUNCH_CHECK_AT(level_site(0, 0));
-      } else {
-        sweep<Real, DIM>(c, 0, b0, x0, h[0].t);
-      }
-      cur0 = h[0].t;
-      ProfScope pr(c, MGAR_KC_RESID0);
-      k_residual_n<<<blocks_npt(d0.n), kThreads, 0, c.stream>>>(
-          fine_row<Real, DIM>(c, ref_ke<Real>(c), nullptr), b0, (const Real*)cur0, h[0].r);
-      MGAR_LAUNCH_CHECK_AT(level_site(2, 0));
+      fine3d(c, 3, ref_ke<Real>(c), b0, h[0].dinv, x0, nullptr, h[0].t, nullptr);
+      fine3d(c, 2, ref_ke<Real>(c), b0, h[0].dinv, h[0].t, nullptr, h[0].r, nullptr);
     }
+    cur0 = h[0].t;
   }
   // the tiled 3D kernels leave r = 0 on fixed nodes, which P^T = (Z P)^T ignores
   // each restriction into a level above the coarsest also leaves that
   // level's zero-guess sweep x = w D^-1 b
   launch_pdl(c.stream, c.use_pdl, k_restrict<Real, DIM>, dim3(blocks_for(c.L[1].n)), dim3(kThreads),
-             (const Real*)h[0].r, h[1].b, d0, c.L[1], DIM == 3 ? (const uint8_t*)nullptr : c.fixed,
+             (const Real*)h[0].r, h[1].b, d0, c.L[1], (const uint8_t*)nullptr,
              (const Real*)h[1].dinv, om, nl > 2 ? h[1].x : (Real*)nullptr);
   MGAR_LAUNCH_CHECK_AT(level_site(3, 0));
   const int lb = bottom_level(c);
@@ -649,13 +685,8 @@ static void vcycle_fused(Ctx& c, const float* b0, float* x0, bool zero_guess,
     res[nl - 1] = h[nl - 1].x;
     for (int l = lb; l + 1 < nl; ++l) res[l] = h[l].t;
   } else {
-    // coarsest level
+    coarse_solve<Real>(c);
     const int l = nl - 1;
-    const int rows_per_block = kThreads / 32;
-    k_coarse_solve<Real, typename CoarseT<Real>::T>
-        <<<(c.nc + rows_per_block - 1) / rows_per_block, kThreads, 0, c.stream>>>(
-            CoarseT<Real>::inv(c), h[l].b, h[l].x, c.nc);
-    MGAR_LAUNCH_CHECK_AT(level_site(5, l));
     res[l] = h[l].x;
   }
   // coarse levels, up
@@ -676,33 +707,16 @@ static void vcycle_fused(Ctx& c, const float* b0, float* x0, bool zero_guess,
     res[l] = h[l].t;
   }
   // finest level, post (the timed class is the tiled pass alone)
-  if (DIM == 3 && !c.split_post) {
+  if (!c.split_post) {
     ProfScope ps(c, MGAR_KC_SMOOTH0);
     fine3d(c, 1, ref_ke<Real>(c), b0, h[0].dinv, cur0, res[1], x0, nullptr, rdot, dout);
-  } else if (DIM == 3) {
+  } else {
     // interpolation in place on the pre-smoothed iterate, then the tiled sweep
     launch_prolong<Real, DIM>(c, true, (const Real*)res[1], (const Real*)cur0, cur0, d0, c.L[1],
                               (const uint8_t*)c.fixed);
     MGAR_LAUNCH_CHECK_AT(level_site(4, 0));
     ProfScope ps(c, MGAR_KC_SMOOTH0);
     fine3d(c, 3, ref_ke<Real>(c), b0, h[0].dinv, cur0, nullptr, x0, nullptr, rdot, dout);
-  } else {
-    ProfScope ps(c, MGAR_KC_SMOOTH0);
-    // interpolation in place on the pre-smoothed iterate, then the sweep into
-    // x0 (with r . x0 into *dout when asked)
-    k_prolong_n<Real, DIM><<<blocks_npt(d0.n), kThreads, 0, c.stream>>>(res[1], cur0, cur0, d0,
-                                                                         c.L[1], c.fixed);
-    MGAR_LAUNCH_CHECK_AT(level_site(4, 0));
-    const FineRow<Real, DIM> row = fine_row<Real, DIM>(c, ref_ke<Real>(c), nullptr);
-    if (dout)
-      k_jacobi_n<FineRow<Real, DIM>, Real, true><<<blocks_npt(d0.n), kThreads, 0, c.stream>>>(
-          row, b0, (const Real*)cur0, x0, (const Real*)h[0].dinv, om, rdot, c.partials, c.counter,
-          dout);
-    else
-      k_jacobi_n<FineRow<Real, DIM>, Real, false><<<blocks_npt(d0.n), kThreads, 0, c.stream>>>(
-          row, b0, (const Real*)cur0, x0, (const Real*)h[0].dinv, om, nullptr, nullptr, nullptr,
-          nullptr);
-    MGAR_LAUNCH_CHECK_AT(level_site(1, 0));
   }
 }
 
@@ -713,9 +727,12 @@ static void vcycle_fused(Ctx& c, const float* b0, float* x0, bool zero_guess,
 // FP64, where the separate kernels below are faster.
 template <typename Real, int DIM>
 static void vcycle_dim(Ctx& c, const Real* b0, Real* x0, bool zero_guess) {
-  if constexpr (sizeof(Real) == 4) {
-    if (c.p.nu_pre == 1 && c.p.nu_post == 1 && c.nl >= 2 && !c.untiled) {
-      vcycle_fused<DIM>(c, b0, x0, zero_guess);
+  if (c.p.nu_pre == 1 && c.p.nu_post == 1 && c.nl >= 2 && !c.untiled) {
+    if constexpr (DIM == 2) {
+      vcycle_fused2<Real>(c, b0, x0, zero_guess);
+      return;
+    } else if constexpr (sizeof(Real) == 4) {
+      vcycle_fused3(c, b0, x0, zero_guess);
       return;
     }
   }
@@ -752,15 +769,7 @@ static void vcycle_dim(Ctx& c, const Real* b0, Real* x0, bool zero_guess) {
         h[l].r, h[l + 1].b, d, c.L[l + 1], l == 0 ? c.fixed : nullptr);
     MGAR_LAUNCH_CHECK_AT(level_site(3, l));
   }
-  // coarsest level
-  {
-    const int l = nl - 1;
-    const int rows_per_block = kThreads / 32;
-    k_coarse_solve<Real, typename CoarseT<Real>::T>
-        <<<(c.nc + rows_per_block - 1) / rows_per_block, kThreads, 0, c.stream>>>(
-            CoarseT<Real>::inv(c), h[l].b, h[l].x, c.nc);
-    MGAR_LAUNCH_CHECK_AT(level_site(5, l));
-  }
+  coarse_solve<Real>(c);
   // upward leg
   for (int l = nl - 2; l >= 0; --l) {
     const Dims& d = c.L[l];
@@ -792,8 +801,12 @@ template void vcycle<float>(Ctx&, const float*, float*, bool);
 void vcycle_dot(Ctx& c, const float* b, float* x, const float2* r, double* dout) {
   require(vcycle_dot_ok(c), MGAR_ERR_ARG,
           "fused r.z V-cycle needs one pre- and one post-sweep, two levels and the tiled 3D kernels");
-  if (c.dim == 2) vcycle_fused<2>(c, b, x, true, r, dout);
-  else vcycle_fused<3>(c, b, x, true, r, dout);
+  if (c.dim == 2) vcycle_fused2<float>(c, b, x, true, r, dout);
+  else vcycle_fused3(c, b, x, true, r, dout);
+}
+
+void vcycle_dot64(Ctx& c, const double* b, double* x, double* dout) {
+  vcycle_fused2<double>(c, b, x, true, nullptr, dout);
 }
 
 template <typename Real, int DIM>
