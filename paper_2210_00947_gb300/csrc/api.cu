@@ -519,7 +519,7 @@ int mgar_set_load(mgar_t h, const double* q) {
 int mgar_apply_K(mgar_t h, const double* x, double* y) {
   return guarded(h, [&](Ctx& c) {
     require(x && y && x != y, MGAR_ERR_ARG, "apply_K: bad pointers");
-    apply_fine64(c, c.ke, x, y, nullptr);
+    apply_fine64(c, c.ke, x, y);
     return MGAR_OK;
   });
 }

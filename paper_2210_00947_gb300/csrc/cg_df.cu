@@ -25,7 +25,7 @@ namespace {
 // blocks).
 template <int DIM, bool DOT>
 __global__ void k_df_apply(DfOp op, const float2* __restrict__ x, float2* __restrict__ y,
-                           double* partials, unsigned int* counter, double* out) {
+                           double* partials, unsigned int* counter, SumOut out) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   df v{0.f, 0.f};
   if (idx < op.n) {
@@ -36,15 +36,13 @@ __global__ void k_df_apply(DfOp op, const float2* __restrict__ x, float2* __rest
   if (DOT) block_sum_finish_df(v, partials, counter, out);
 }
 
-// 2D: p = z + (*rz_new / *rz_old) p_old (p = z when first), y = A p, p . y
-// into *out; odd *parity (may be null) swaps p_old and p.
+// 2D: p = z + beta p_old (p = z when first), y = A p; odd *parity (may be
+// null) swaps p_old and p.
 __global__ void __launch_bounds__(l2d::kThreads2) k_df_dir2(DfOp op, const float* __restrict__ z,
                                                             const float2* p_old, float2* p,
-                                                            const double* rz_new,
-                                                            const double* rz_old, int first,
+                                                            const double* beta, int first,
                                                             const double* parity,
-                                                            float2* __restrict__ y, double* partials,
-                                                            unsigned int* counter, double* out) {
+                                                            float2* __restrict__ y) {
   __shared__ DfDirSmem s;
   pdl_wait();
   pdl_trigger();
@@ -53,21 +51,53 @@ __global__ void __launch_bounds__(l2d::kThreads2) k_df_dir2(DfOp op, const float
     p_old = p;
     p = t;
   }
-  const df beta = first ? df{0.f, 0.f} : block_div_df(rz_new, rz_old);
-  const df v = df_dir_tile(s, op, blockIdx.x, blockIdx.y, z, p_old, first != 0, beta, p, y);
-  double t;
-  if (block_sum_last_df(v, partials, counter, t, threadIdx.x, l2d::kThreads2,
-                        blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y) &&
-      threadIdx.x == 0)
-    *out = t;
+  const df b = first ? df{0.f, 0.f} : load_pair(beta);
+  df_dir_tile(s, op, blockIdx.x, blockIdx.y, z, p_old, first != 0, b, p, y);
 }
 
-void df_dir2(Ctx& c, const DfOp& op, const float2* p_old, float2* p, const double* rz_new,
-             const double* rz_old, bool first, const double* parity) {
+// p . y over the nodes in memory order (as the sum of r . z, it does not
+// follow the tiles)
+__global__ void __launch_bounds__(kThreads) k_dot_py(const float2* __restrict__ p,
+                                                     const float2* __restrict__ p_alt,
+                                                     const double* parity,
+                                                     const float2* __restrict__ y, int n,
+                                                     double* partials, unsigned int* counter,
+                                                     SumOut out) {
+  pdl_wait();
+  pdl_trigger();
+  if (parity && (((int)*parity) & 1)) p = p_alt;
+  float2 pv[2 * kSumVB], yv[2 * kSumVB];
+  double t;
+  if (ordered_sum<2>(
+          n, blockIdx.x, partials, counter, t,
+          [&](int q, int idx) {
+            pv[q] = p[idx];
+            yv[q] = y[idx];
+          },
+          [&](int q) { return df_mul(unpack(pv[q]), unpack(yv[q])); }) &&
+      threadIdx.x == 0)
+    sum_out(out, t);
+}
+
+// p . A p into S_PAP and alpha = *rz / p . A p into S_ALPHA
+SumOut pap_out(Ctx& c, const double* rz) {
+  return SumOut{c.dsc + S_PAP, rz, nullptr, c.dsc + S_ALPHA, 1};
+}
+// r . z into dsc[slot] and beta = r . z / dsc[old] into S_BETA
+SumOut rz_out(Ctx& c, int slot, int old) {
+  return SumOut{c.dsc + slot, nullptr, c.dsc + old, c.dsc + S_BETA, 1};
+}
+
+void df_dir2(Ctx& c, const DfOp& op, const float2* p_old, float2* p, const double* rz, bool first,
+             const double* parity) {
   const dim3 grid(l2d::tiles(op.NX, l2d::kUX), l2d::tiles(op.NY, l2d::kUY));
   launch_pdl(c.stream, c.use_pdl, k_df_dir2, grid, dim3(l2d::kThreads2), op, (const float*)c.x32,
-             p_old, p, rz_new, rz_old, first ? 1 : 0, parity, c.df_Ap, c.partials, c.counter,
-             c.dsc + S_PAP);
+             p_old, p, (const double*)(c.dsc + S_BETA), first ? 1 : 0, parity, c.df_Ap);
+  MGAR_LAUNCH_CHECK();
+  // odd parity: the new p is in p_old's buffer
+  launch_pdl(c.stream, c.use_pdl, k_dot_py, dim3(sum_phys(op.n, 2)), dim3(kThreads),
+             (const float2*)p, p_old, parity, (const float2*)c.df_Ap, op.n, c.partials, c.counter,
+             pap_out(c, rz));
   MGAR_LAUNCH_CHECK();
 }
 
@@ -75,7 +105,7 @@ void df_dir2(Ctx& c, const DfOp& op, const float2* p_old, float2* p, const doubl
 template <int DIM>
 __global__ void k_df_residual(DfOp op, const float2* __restrict__ q, const float2* __restrict__ x,
                               float2* __restrict__ r, double* partials, unsigned int* counter,
-                              double* out) {
+                              SumOut out) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   df v{0.f, 0.f};
   if (idx < op.n) {
@@ -109,45 +139,47 @@ __device__ __forceinline__ void cg_check(const CgCheck& k) {
   cudaGraphSetConditional(k.loop, go ? 1u : 0u);
 }
 
-// alpha = rz / pAp; x += alpha p; r -= alpha Ap; ||r||^2; optionally the
-// FP32 copy of r for the preconditioner
-__global__ void k_df_cg_xr(float2* __restrict__ x, float2* __restrict__ r, const float2* __restrict__ p,
-                           const float2* __restrict__ Ap, int n, const double* __restrict__ rz,
-                           const double* __restrict__ pap, double* partials, unsigned int* counter,
-                           double* out, float* __restrict__ r32,
-                           const float2* __restrict__ p_alt, const double* parity, CgCheck check) {
+// x += alpha p; r -= alpha Ap; ||r||^2; optionally the FP32 copy of r for the
+// preconditioner
+__global__ void __launch_bounds__(kThreads) k_df_cg_xr(float2* __restrict__ x, float2* __restrict__ r,
+                                                       const float2* __restrict__ p,
+                                                       const float2* __restrict__ Ap, int n,
+                                                       const double* __restrict__ alpha_p,
+                                                       double* partials, unsigned int* counter,
+                                                       double* out, float* __restrict__ r32,
+                                                       const float2* __restrict__ p_alt,
+                                                       const double* parity, CgCheck check) {
   pdl_wait();
   // device-side CG loop: the two direction buffers swap with the parity
   // (every block reads it before the last one flips it)
   if (parity && (((int)*parity) & 1)) p = p_alt;
-  const df alpha = block_div_df(rz, pap);
+  const df alpha = load_pair(alpha_p);
   df acc{0.f, 0.f};
   const int stride = gridDim.x * blockDim.x;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  // two nodes per iteration: their eight loads are in flight together
-  for (; i + stride < n; i += 2 * stride) {
-    const int j = i + stride;
-    const float2 xa = x[i], xb = x[j], pa = p[i], pb = p[j];
-    const float2 ra = r[i], rb = r[j], qa = Ap[i], qb = Ap[j];
-    x[i] = pack(df_add(unpack(xa), df_mul(alpha, unpack(pa))));
-    x[j] = pack(df_add(unpack(xb), df_mul(alpha, unpack(pb))));
-    const df ria = df_sub(unpack(ra), df_mul(alpha, unpack(qa)));
-    const df rib = df_sub(unpack(rb), df_mul(alpha, unpack(qb)));
-    r[i] = pack(ria);
-    r[j] = pack(rib);
-    if (r32) {
-      r32[i] = __fadd_rn(ria.hi, ria.lo);
-      r32[j] = __fadd_rn(rib.hi, rib.lo);
+  // four nodes per iteration: their sixteen loads are in flight together
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += 4 * stride) {
+    float2 xv[4], pv[4], rv[4], qv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = i + u * stride;
+      if (j < n) {
+        xv[u] = x[j];
+        pv[u] = p[j];
+        rv[u] = r[j];
+        qv[u] = Ap[j];
+      }
     }
-    acc = df_add(acc, df_mul(ria, ria));
-    acc = df_add(acc, df_mul(rib, rib));
-  }
-  for (; i < n; i += stride) {
-    x[i] = pack(df_add(unpack(x[i]), df_mul(alpha, unpack(p[i]))));
-    const df ri = df_sub(unpack(r[i]), df_mul(alpha, unpack(Ap[i])));
-    r[i] = pack(ri);
-    if (r32) r32[i] = __fadd_rn(ri.hi, ri.lo);
-    acc = df_add(acc, df_mul(ri, ri));
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = i + u * stride;
+      if (j < n) {
+        x[j] = pack(df_add(unpack(xv[u]), df_mul(alpha, unpack(pv[u]))));
+        const df ri = df_sub(unpack(rv[u]), df_mul(alpha, unpack(qv[u])));
+        r[j] = pack(ri);
+        if (r32) r32[j] = __fadd_rn(ri.hi, ri.lo);
+        acc = df_add(acc, df_mul(ri, ri));
+      }
+    }
   }
   double t;
   if (block_sum_last_df(acc, partials, counter, t, threadIdx.x, blockDim.x, blockIdx.x, gridDim.x) &&
@@ -157,17 +189,22 @@ __global__ void k_df_cg_xr(float2* __restrict__ x, float2* __restrict__ r, const
   }
 }
 
-// p = z + (rz_new / rz_old) p, z in FP32
+// Blocks of the FP32 CG's update, four nodes per access: four per SM.
+int xr32_blocks(const Ctx& c) {
+  return (int)std::min<int64_t>(blocks_for((c.n + 3) / 4), (int64_t)c.sms * 4);
+}
+
+// p = z + beta p, z in FP32
 __global__ void k_df_cg_p(float2* __restrict__ p, const float* __restrict__ z, int n,
-                          const double* __restrict__ rz_new, const double* __restrict__ rz_old) {
-  const df beta = block_div_df(rz_new, rz_old);
+                          const double* __restrict__ beta_p) {
+  const df beta = load_pair(beta_p);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     p[i] = pack(df_add(df{z[i], 0.f}, df_mul(beta, unpack(p[i]))));
 }
 
 // r . z with z in FP32
 __global__ void k_df_dot_f(const float2* __restrict__ r, const float* __restrict__ z, int n,
-                           double* partials, unsigned int* counter, double* out) {
+                           double* partials, unsigned int* counter, SumOut out) {
   df acc{0.f, 0.f};
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     acc = df_add(acc, df_mulf(unpack(r[i]), z[i]));
@@ -211,10 +248,10 @@ void apply_df64(Ctx& c, const double* x, double* y) {
   {
     if (c.dim == 2)
       k_df_apply<2, false><<<blocks_for(n), kThreads, 0, c.stream>>>(op, c.df_p, c.df_Ap, nullptr,
-                                                                     nullptr, nullptr);
+                                                                     nullptr, SumOut{});
     else
       k_df_apply<3, false><<<blocks_for(n), kThreads, 0, c.stream>>>(op, c.df_p, c.df_Ap, nullptr,
-                                                                     nullptr, nullptr);
+                                                                     nullptr, SumOut{});
     MGAR_LAUNCH_CHECK();
   }
   k_df_to_d<<<blocks_for(n), kThreads, 0, c.stream>>>(c.df_Ap, y, n);
@@ -251,12 +288,13 @@ __global__ void k_cg_reset(double* dsc) {
 }
 
 // z32 = M r32 (the FP32 copy of r is written by the residual and update
-// kernels) and r . z into dsc[slot], fused into the V-cycle's last kernel
+// kernels) and r . z into dsc[slot] with beta, fused into the V-cycle's last
+// kernel
 static void precondition_f32(Ctx& c, int slot) {
   const bool prof_inside = c.prof_class == MGAR_KC_SMOOTH0 || c.prof_class == MGAR_KC_RESID0;
-  double* out = c.dsc + slot;
-  run_graph(c, slot == S_RZ0 ? 8 : 9, c.b32, c.x32, prof_inside,
-            [&] { vcycle_dot(c, c.b32, c.x32, c.df_r, out); });
+  run_graph(c, slot == S_RZ0 ? 8 : 9, c.b32, c.x32, prof_inside, [&] {
+    vcycle_dot(c, c.b32, c.x32, c.df_r, rz_out(c, slot, slot == S_RZ0 ? S_RZ1 : S_RZ0));
+  });
 }
 
 // 3D: the tiled kernels fuse the direction update into the product
@@ -267,15 +305,14 @@ static void precondition_f32(Ctx& c, int slot) {
 // the convergence check (which moves RZ1 to RZ0).
 static void cg_iteration(Ctx& c, bool first, cudaGraphConditionalHandle loop) {
   const int n = (int)c.n;
-  vcycle_dot(c, c.b32, c.x32, c.df_r, c.dsc + S_RZ1);
-  df3d_dir(c, c.x32, c.df_p, c.df_p2, c.dsc + S_RZ1, c.dsc + S_RZ0, first, c.df_Ap, c.dsc + S_PAP,
+  vcycle_dot(c, c.b32, c.x32, c.df_r, rz_out(c, S_RZ1, S_RZ0));
+  df3d_dir(c, c.x32, c.df_p, c.df_p2, c.dsc + S_BETA, first, c.df_Ap, pap_out(c, c.dsc + S_RZ1),
            c.dsc + S_CGPAR);
   // parity 0: the new p is in df_p2
   launch_pdl(c.stream, c.use_pdl, k_df_cg_xr, dim3(c.grid_blocks), dim3(kThreads), c.df_x, c.df_r,
-             (const float2*)c.df_p2, (const float2*)c.df_Ap, n, (const double*)(c.dsc + S_RZ1),
-             (const double*)(c.dsc + S_PAP), c.partials, c.counter, c.dsc + S_RR, c.b32,
-             (const float2*)c.df_p, (const double*)(c.dsc + S_CGPAR),
-             CgCheck{c.dsc, c.qnorm, c.p.eps2, c.p.cg_max, loop});
+             (const float2*)c.df_p2, (const float2*)c.df_Ap, n, (const double*)(c.dsc + S_ALPHA),
+             c.partials, c.counter, c.dsc + S_RR, c.b32, (const float2*)c.df_p,
+             (const double*)(c.dsc + S_CGPAR), CgCheck{c.dsc, c.qnorm, c.p.eps2, c.p.cg_max, loop});
   MGAR_LAUNCH_CHECK();
 }
 
@@ -285,7 +322,6 @@ static void cg_iteration(Ctx& c, bool first, cudaGraphConditionalHandle loop) {
 // and p . A p, the update of x and r with alpha = RZ1 / pAp and the check.
 static void cg_iteration_2d(Ctx& c, bool first, cudaGraphConditionalHandle loop) {
   const int n = (int)c.n;
-  const int rb = c.grid_blocks;
   const DfOp op = make_op(c);
   if (first) {
     k_df_to_f32<<<blocks_for(n), kThreads, 0, c.stream>>>(c.df_r, c.b32, n);
@@ -293,19 +329,18 @@ static void cg_iteration_2d(Ctx& c, bool first, cudaGraphConditionalHandle loop)
   }
   if (vcycle_dot_ok(c)) {
     // r . z fused into the V-cycle's last sweep
-    vcycle_dot(c, c.b32, c.x32, c.df_r, c.dsc + S_RZ1);
+    vcycle_dot(c, c.b32, c.x32, c.df_r, rz_out(c, S_RZ1, S_RZ0));
   } else {
     vcycle<float>(c, c.b32, c.x32, true);
-    k_df_dot_f<<<rb, kThreads, 0, c.stream>>>(c.df_r, c.x32, n, c.partials, c.counter,
-                                              c.dsc + S_RZ1);
+    k_df_dot_f<<<c.grid_blocks, kThreads, 0, c.stream>>>(c.df_r, c.x32, n, c.partials, c.counter,
+                                                         rz_out(c, S_RZ1, S_RZ0));
     MGAR_LAUNCH_CHECK();
   }
-  df_dir2(c, op, c.df_p, c.df_p2, c.dsc + S_RZ1, c.dsc + S_RZ0, first, c.dsc + S_CGPAR);
-  launch_pdl(c.stream, c.use_pdl, k_df_cg_xr, dim3(rb), dim3(kThreads), c.df_x, c.df_r,
-             (const float2*)c.df_p2, (const float2*)c.df_Ap, n, (const double*)(c.dsc + S_RZ1),
-             (const double*)(c.dsc + S_PAP), c.partials, c.counter, c.dsc + S_RR, c.b32,
-             (const float2*)c.df_p, (const double*)(c.dsc + S_CGPAR),
-             CgCheck{c.dsc, c.qnorm, c.p.eps2, c.p.cg_max, loop});
+  df_dir2(c, op, c.df_p, c.df_p2, c.dsc + S_RZ1, first, c.dsc + S_CGPAR);
+  launch_pdl(c.stream, c.use_pdl, k_df_cg_xr, dim3(c.grid_blocks), dim3(kThreads), c.df_x, c.df_r,
+             (const float2*)c.df_p2, (const float2*)c.df_Ap, n, (const double*)(c.dsc + S_ALPHA),
+             c.partials, c.counter, c.dsc + S_RR, c.b32, (const float2*)c.df_p,
+             (const double*)(c.dsc + S_CGPAR), CgCheck{c.dsc, c.qnorm, c.p.eps2, c.p.cg_max, loop});
   MGAR_LAUNCH_CHECK();
 }
 
@@ -406,7 +441,6 @@ static void drop_stale_cg_graph(Ctx& c) {
 
 static int solve_mgcg_df3(Ctx& c, double* T, int* iters, double* relres) {
   const int n = (int)c.n;
-  const int rb = c.grid_blocks;
   k_d_to_df<<<blocks_for(n), kThreads, 0, c.stream>>>(T, c.df_x, n);
   MGAR_LAUNCH_CHECK();
   {
@@ -441,13 +475,13 @@ static int solve_mgcg_df3(Ctx& c, double* T, int* iters, double* relres) {
     while (it < c.p.cg_max) {
       {
         ProfScope ps(c, MGAR_KC_APPLY64);
-        df3d_dir(c, c.x32, pcur, pnext, c.dsc + a, c.dsc + b, first, c.df_Ap, c.dsc + S_PAP);
+        df3d_dir(c, c.x32, pcur, pnext, c.dsc + S_BETA, first, c.df_Ap, pap_out(c, c.dsc + a));
       }
       first = false;
       std::swap(pcur, pnext);
-      launch_pdl(c.stream, c.use_pdl, k_df_cg_xr, dim3(rb), dim3(kThreads), c.df_x, c.df_r,
-                 (const float2*)pcur, (const float2*)c.df_Ap, n, (const double*)(c.dsc + a),
-                 (const double*)(c.dsc + S_PAP), c.partials, c.counter, c.dsc + S_RR, c.b32,
+      launch_pdl(c.stream, c.use_pdl, k_df_cg_xr, dim3(c.grid_blocks), dim3(kThreads), c.df_x,
+                 c.df_r, (const float2*)pcur, (const float2*)c.df_Ap, n,
+                 (const double*)(c.dsc + S_ALPHA), c.partials, c.counter, c.dsc + S_RR, c.b32,
                  (const float2*)nullptr, (const double*)nullptr, CgCheck{});
       MGAR_LAUNCH_CHECK();
       ++it;
@@ -499,18 +533,23 @@ __device__ void ru_decide(double* dsc, double qnorm, double eps2, double delta, 
   if (set) cudaGraphSetConditional(ru, upd ? 1u : 0u);
 }
 
-// alpha = rz / pAp; xc += alpha p; r -= alpha A p; ||r||^2 into dsc[S_RR],
-// then the update decision (ru_decide) in the last block
-__global__ void k_cg_xr32(float* __restrict__ xc, float* __restrict__ r, const float* __restrict__ p,
-                          const float* __restrict__ p_alt, const double* parity,
-                          const float* __restrict__ Ap, int n, const double* __restrict__ rz,
-                          const double* __restrict__ pap, double* partials, unsigned int* counter,
-                          double* dsc, double qnorm, double eps2, double delta, int cg_max,
-                          cudaGraphConditionalHandle ru, int set) {
+// xc += alpha p; r -= alpha A p; ||r||^2 into dsc[S_RR], then the update
+// decision (ru_decide) in the last block.  Two 16-byte rows of each vector in
+// flight per thread, four blocks per SM.
+__global__ void __launch_bounds__(kThreads) k_cg_xr32(float* __restrict__ xc, float* __restrict__ r,
+                                                      const float* __restrict__ p,
+                                                      const float* __restrict__ p_alt,
+                                                      const double* parity,
+                                                      const float* __restrict__ Ap, int n,
+                                                      const double* __restrict__ alpha_p,
+                                                      double* partials, unsigned int* counter,
+                                                      double* dsc, double qnorm, double eps2,
+                                                      double delta, int cg_max,
+                                                      cudaGraphConditionalHandle ru, int set) {
   pdl_wait();
   // every block reads the parity before the last one flips it
   if (parity && (((int)*parity) & 1)) p = p_alt;
-  const float alpha = block_div_f(rz, pap);
+  const float alpha = load_pair(alpha_p).hi;
   float acc = 0.f;
   const int stride = gridDim.x * blockDim.x;
   const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -520,9 +559,7 @@ __global__ void k_cg_xr32(float* __restrict__ xc, float* __restrict__ r, const f
   float4* __restrict__ r4 = reinterpret_cast<float4*>(r);
   const float4* __restrict__ p4 = reinterpret_cast<const float4*>(p);
   const float4* __restrict__ a4 = reinterpret_cast<const float4*>(Ap);
-  for (int q = t0; q < n4; q += stride) {
-    float4 xv = xc4[q], rv = r4[q];
-    const float4 pv = p4[q], av = a4[q];
+  auto step = [&](float4& xv, float4& rv, const float4& pv, const float4& av) {
     xv.x = fmaf(alpha, pv.x, xv.x);
     xv.y = fmaf(alpha, pv.y, xv.y);
     xv.z = fmaf(alpha, pv.z, xv.z);
@@ -531,12 +568,27 @@ __global__ void k_cg_xr32(float* __restrict__ xc, float* __restrict__ r, const f
     rv.y = fmaf(-alpha, av.y, rv.y);
     rv.z = fmaf(-alpha, av.z, rv.z);
     rv.w = fmaf(-alpha, av.w, rv.w);
-    xc4[q] = xv;
-    r4[q] = rv;
     acc = fmaf(rv.x, rv.x, acc);
     acc = fmaf(rv.y, rv.y, acc);
     acc = fmaf(rv.z, rv.z, acc);
     acc = fmaf(rv.w, rv.w, acc);
+  };
+  int q = t0;
+  for (; q + stride < n4; q += 2 * stride) {
+    float4 xa = xc4[q], ra = r4[q], xb = xc4[q + stride], rb = r4[q + stride];
+    const float4 pa = p4[q], aa = a4[q], pb = p4[q + stride], ab = a4[q + stride];
+    step(xa, ra, pa, aa);
+    step(xb, rb, pb, ab);
+    xc4[q] = xa;
+    r4[q] = ra;
+    xc4[q + stride] = xb;
+    r4[q + stride] = rb;
+  }
+  if (q < n4) {
+    float4 xv = xc4[q], rv = r4[q];
+    step(xv, rv, p4[q], a4[q]);
+    xc4[q] = xv;
+    r4[q] = rv;
   }
   for (int i = 4 * n4 + t0; i < n; i += stride) {
     xc[i] = fmaf(alpha, p[i], xc[i]);
@@ -606,22 +658,21 @@ __global__ void k_ru_loop(double* dsc, double qnorm, double eps2, int cg_max,
 static void ru_iteration(Ctx& c, cudaGraphConditionalHandle ru, bool set) {
   const int n = (int)c.n;
   if (set) {
-    vcycle_dot(c, c.b32, c.x32, nullptr, c.dsc + S_RZ1);
+    vcycle_dot(c, c.b32, c.x32, nullptr, rz_out(c, S_RZ1, S_RZ0));
   } else {
     const bool prof_inside = c.prof_class == MGAR_KC_SMOOTH0 || c.prof_class == MGAR_KC_RESID0;
     run_graph(c, 10, c.b32, c.x32, prof_inside,
-              [&] { vcycle_dot(c, c.b32, c.x32, nullptr, c.dsc + S_RZ1); });
+              [&] { vcycle_dot(c, c.b32, c.x32, nullptr, rz_out(c, S_RZ1, S_RZ0)); });
   }
   {
     ProfScope ps(c, MGAR_KC_APPLY32);
-    fine3d_dir(c, c.x32, c.p32, c.p32b, c.dsc + S_RZ1, c.dsc + S_RZ0, c.dsc + S_CGFIRST,
-               c.dsc + S_CGPAR, c.y32, c.dsc + S_PAP, c.dsc + S_RZ0);
+    fine3d_dir(c, c.x32, c.p32, c.p32b, c.dsc + S_BETA, c.dsc + S_CGFIRST, c.dsc + S_CGPAR, c.y32,
+               pap_out(c, c.dsc + S_RZ1), c.dsc + S_RZ1, c.dsc + S_RZ0);
   }
   // parity 0: the new p is in p32b
-  launch_pdl(c.stream, c.use_pdl, k_cg_xr32, dim3(c.grid_blocks), dim3(kThreads), c.xc32, c.b32,
-             (const float*)c.p32b, (const float*)c.p32, (const double*)(c.dsc + S_CGPAR),
-             (const float*)c.y32, n, (const double*)(c.dsc + S_RZ0),
-             (const double*)(c.dsc + S_PAP), c.partials, c.counter, c.dsc, c.qnorm, c.p.eps2,
+  launch_pdl(c.stream, c.use_pdl, k_cg_xr32, dim3(xr32_blocks(c)), dim3(kThreads), c.xc32,
+             c.b32, (const float*)c.p32b, (const float*)c.p32, (const double*)(c.dsc + S_CGPAR),
+             (const float*)c.y32, n, (const double*)(c.dsc + S_ALPHA), c.partials, c.counter, c.dsc, c.qnorm, c.p.eps2,
              c.ru_delta, c.p.cg_max, ru, set ? 1 : 0);
   MGAR_LAUNCH_CHECK();
 }
@@ -817,10 +868,10 @@ int solve_mgcg_df(Ctx& c, double* T, int* iters, double* relres) {
     ProfScope ps(c, MGAR_KC_APPLY64);
     if (c.dim == 2)
       k_df_residual<2><<<blocks_for(n), kThreads, 0, c.stream>>>(op, c.df_q, c.df_x, c.df_r,
-                                                                 c.partials, c.counter, c.dsc + S_RR);
+                                                                 c.partials, c.counter, SumOut{c.dsc + S_RR});
     else
-      k_df_residual<3><<<blocks_for(n), kThreads, 0, c.stream>>>(op, c.df_q, c.df_x, c.df_r,
-                                                                 c.partials, c.counter, c.dsc + S_RR);
+      k_df_residual<3><<<blocks_for(n), kThreads, 0, c.stream>>>(
+          op, c.df_q, c.df_x, c.df_r, c.partials, c.counter, SumOut{c.dsc + S_RR});
     MGAR_LAUNCH_CHECK();
   }
   fetch_scalars(c, S_RR, 1);
@@ -854,7 +905,8 @@ int solve_mgcg_df(Ctx& c, double* T, int* iters, double* relres) {
       precondition_f32(c, a);
     } else {
       precondition_df(c);
-      k_df_dot_f<<<rb, kThreads, 0, c.stream>>>(c.df_r, c.x32, n, c.partials, c.counter, c.dsc + a);
+      k_df_dot_f<<<rb, kThreads, 0, c.stream>>>(c.df_r, c.x32, n, c.partials, c.counter,
+                                                rz_out(c, a, b));
       MGAR_LAUNCH_CHECK();
     }
     float2 *pcur = c.df_p, *pnext = c.df_p2;
@@ -867,18 +919,18 @@ int solve_mgcg_df(Ctx& c, double* T, int* iters, double* relres) {
       {
         ProfScope ps(c, MGAR_KC_APPLY64);
         if (c.dim == 2) {
-          df_dir2(c, op, pcur, pnext, c.dsc + a, c.dsc + b, first, nullptr);
+          df_dir2(c, op, pcur, pnext, c.dsc + a, first, nullptr);
           std::swap(pcur, pnext);
         } else {
           k_df_apply<3, true><<<blocks_for(n), kThreads, 0, c.stream>>>(
-              op, pcur, c.df_Ap, c.partials, c.counter, c.dsc + S_PAP);
+              op, pcur, c.df_Ap, c.partials, c.counter, pap_out(c, c.dsc + a));
           MGAR_LAUNCH_CHECK();
         }
       }
       first = false;
-      k_df_cg_xr<<<rb, kThreads, 0, c.stream>>>(c.df_x, c.df_r, pcur, c.df_Ap, n, c.dsc + a,
-                                                c.dsc + S_PAP, c.partials, c.counter, c.dsc + S_RR,
-                                                fused ? c.b32 : nullptr, nullptr, nullptr, CgCheck{});
+      k_df_cg_xr<<<rb, kThreads, 0, c.stream>>>(
+          c.df_x, c.df_r, pcur, c.df_Ap, n, c.dsc + S_ALPHA, c.partials, c.counter, c.dsc + S_RR,
+          fused ? c.b32 : nullptr, nullptr, nullptr, CgCheck{});
       MGAR_LAUNCH_CHECK();
       ++it;
       fetch_scalars(c, S_RR, 1);
@@ -891,11 +943,11 @@ int solve_mgcg_df(Ctx& c, double* T, int* iters, double* relres) {
       } else {
         precondition_df(c);
         k_df_dot_f<<<rb, kThreads, 0, c.stream>>>(c.df_r, c.x32, n, c.partials, c.counter,
-                                                  c.dsc + a);
+                                                  rz_out(c, a, b));
         MGAR_LAUNCH_CHECK();
       }
       if (c.dim == 3) {
-        k_df_cg_p<<<rb, kThreads, 0, c.stream>>>(pcur, c.x32, n, c.dsc + a, c.dsc + b);
+        k_df_cg_p<<<rb, kThreads, 0, c.stream>>>(pcur, c.x32, n, c.dsc + S_BETA);
         MGAR_LAUNCH_CHECK();
       }
     }

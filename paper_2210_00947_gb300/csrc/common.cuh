@@ -74,7 +74,8 @@ enum Slot : int {
   S_DERR = 191,     // host mirror only: the device error flag, published with every fetch
   S_RREC = 192,     // FP32 CG: recursive ||r|| at the last update decision
   S_RUSTALL = 193,  // FP32 CG: successive updates that did not halve the true ||r||
-  S_COUNT = 194
+  S_ALPHA = 194, S_BETA = 195,  // CG: r . z / p . A p and r . z / (r . z)_old, a double or a df64 pair
+  S_COUNT = 196
 };
 
 // 1 / sqrt(a) for a > 0: an FP32 seed refined by two Newton-Raphson steps
@@ -486,6 +487,71 @@ __device__ __forceinline__ bool block_sum_last_core(const double (&w)[N], double
   return true;
 }
 
+// One sum: block_sum_last_core's order of additions, with the warps' sums (in
+// lane 0, FP64, or as a df64 pair that one warp converts) added up by the
+// first warp and one barrier less.  Every block of a wide launch pays for this
+// stage, and on the 1/58-rate FP64 pipe a conversion per warp (three FP64
+// operations each) and a division per block were 40 % of a CG update's pipe
+// time.  The total is valid in thread 0 of the last block.
+__device__ __forceinline__ bool block_sum_last_one(bool pair, double w, df wp, double* partials,
+                                                   unsigned int* counter, double& total, int tid,
+                                                   int nthr, int bid, int nblk) {
+  __shared__ double sh[32];
+  __shared__ bool last;
+  const int lane = tid & 31, warp = tid >> 5, nw = nthr >> 5;
+  float2* shp = reinterpret_cast<float2*>(sh);
+  if (lane == 0) {
+    if (pair) shp[warp] = make_float2(wp.hi, wp.lo);
+    else sh[warp] = w;
+  }
+  __syncthreads();
+  // 0 + v_0 + v_1 + ..., v_q in lane q
+  auto in_order = [&](double v) {
+    double s = 0.0;
+    for (int q = 0; q < nw; ++q) s += __shfl_sync(0xffffffffu, v, q);
+    return s;
+  };
+  if (warp == 0) {
+    double v = 0.0;
+    if (lane < nw) {
+      if (pair) {
+        const float2 f = shp[lane];
+        v = (double)f.x + (double)f.y;
+      } else {
+        v = sh[lane];
+      }
+    }
+    const double s = in_order(v);
+    if (lane == 0) {
+      if (CK(bid, g_partials_len)) partials[bid] = s;
+      __threadfence();
+      last = atomicAdd(counter, 1u) == (unsigned int)nblk - 1;
+    }
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  // L2-coherent loads, four rows of blocks in flight together
+  constexpr int U = 4;
+  double acc = 0.0;
+  for (int b = tid; b < nblk; b += U * nthr) {
+    double v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = b + u * nthr < nblk ? __ldcg(partials + b + u * nthr) : 0.0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) acc += v[u];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+  if (lane == 0) sh[warp] = acc;
+  __syncthreads();
+  if (warp == 0) {
+    total = in_order(lane < nw ? sh[lane] : 0.0);
+    if (lane == 0) *counter = 0u;
+  }
+  return true;
+}
+
 template <int N>
 __device__ __forceinline__ bool block_sum_last_ids(double (&v)[N], double* partials,
                                                    unsigned int* counter, double (&total)[N],
@@ -497,13 +563,18 @@ __device__ __forceinline__ bool block_sum_last_ids(double (&v)[N], double* parti
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     v[k] = s;
   }
-  return block_sum_last_core<N>(v, partials, counter, total, tid, nthr, bid, nblk);
+  if constexpr (N == 1)
+    return block_sum_last_one(false, v[0], df{0.f, 0.f}, partials, counter, total[0], tid, nthr, bid,
+                              nblk);
+  else
+    return block_sum_last_core<N>(v, partials, counter, total, tid, nthr, bid, nblk);
 }
 
 // One double-float value per thread: the warp sums are formed in df64 on
 // the FP32 pipe (GB300 runs FP64 at 1/58 of the FP32 rate, and an FP64
 // shuffle tree over every warp of a wide grid costs microseconds), then
-// FP64 across warps and blocks as in block_sum_last_ids.
+// FP64 across warps and blocks.  The total is valid in thread 0 of the last
+// block.
 __device__ __forceinline__ bool block_sum_last_df(df v, double* partials, unsigned int* counter,
                                                   double& total, int tid, int nthr, int bid,
                                                   int nblk) {
@@ -513,12 +584,132 @@ __device__ __forceinline__ bool block_sum_last_df(df v, double* partials, unsign
     const float l = __shfl_down_sync(0xffffffffu, v.lo, o);
     v = df_add(v, df{h, l});
   }
-  double w[1] = {0.0};
-  if ((tid & 31) == 0) w[0] = df_to_double(v);
-  double t[1];
-  const bool last = block_sum_last_core<1>(w, partials, counter, t, tid, nthr, bid, nblk);
-  total = t[0];
-  return last;
+  return block_sum_last_one(true, 0.0, v, partials, counter, total, tid, nthr, bid, nblk);
+}
+
+// Four sums at once: v[g] is thread tid's value of the virtual block vb0 + g of
+// kThreads threads, and the total over the nvb virtual blocks is the one that
+// block_sum_last_df would give over nvb blocks, bit for bit.  A block of a sum
+// over a million values otherwise spends most of its time in the barrier,
+// fence and ticket (11.8 us for 2053 blocks of two values per thread); here a
+// quarter of the blocks pay for them, and the four warp trees share their
+// steps (six additions instead of twenty).
+constexpr int kSumVB = 4;
+__device__ __forceinline__ bool block_sums_last_df(const df (&v)[kSumVB], double* partials,
+                                                   unsigned int* counter, double& total, int vb0,
+                                                   int nvb, int nphys) {
+  static_assert(kSumVB == 4 && kThreads == 256, "the lane layout below");
+  __shared__ float2 shp[kSumVB][8];
+  __shared__ double sh[8];
+  __shared__ bool last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto swap_add = [&](bool upper, df a, df b, int o) {
+    const df send = upper ? a : b, keep = upper ? b : a;
+    return df_add(keep, df{__shfl_xor_sync(0xffffffffu, send.hi, o),
+                           __shfl_xor_sync(0xffffffffu, send.lo, o)});
+  };
+  const df w01 = swap_add(lane & 16, v[0], v[1], 16), w23 = swap_add(lane & 16, v[2], v[3], 16);
+  df u = swap_add(lane & 8, w01, w23, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+    u = df_add(u, df{__shfl_down_sync(0xffffffffu, u.hi, o), __shfl_down_sync(0xffffffffu, u.lo, o)});
+  // lanes 0, 16, 8, 24 hold the warp's sums 0, 1, 2, 3
+  if ((lane & 7) == 0) shp[((lane >> 4) & 1) + ((lane >> 2) & 2)][warp] = make_float2(u.hi, u.lo);
+  __syncthreads();
+  if (warp == 0) {
+    const float2 f = shp[lane >> 3][lane & 7];
+    const double d = (double)f.x + (double)f.y;
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s += __shfl_sync(0xffffffffu, d, q, 8);
+    const int vb = vb0 + (lane >> 3);
+    if ((lane & 7) == 0 && vb < nvb && CK(vb, g_partials_len)) {
+      partials[vb] = s;
+      __threadfence();
+    }
+    __syncwarp();
+    if (lane == 0) last = atomicAdd(counter, 1u) == (unsigned int)nphys - 1;
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  constexpr int U = 4;
+  double acc = 0.0;
+  for (int b = tid; b < nvb; b += U * kThreads) {
+    double w[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) w[q] = b + q * kThreads < nvb ? __ldcg(partials + b + q * kThreads) : 0.0;
+#pragma unroll
+    for (int q = 0; q < U; ++q) acc += w[q];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+  if (lane == 0) sh[warp] = acc;
+  __syncthreads();
+  if (warp == 0) {
+    const double w = sh[lane & 7];
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s += __shfl_sync(0xffffffffu, w, q);
+    total = s;
+    if (lane == 0) *counter = 0u;
+  }
+  return true;
+}
+
+// Sum over n nodes, NPT per thread and virtual block (nodes vb * kThreads *
+// NPT + u * kThreads + tid): load(g * NPT + u, idx) fetches a node's operands,
+// term(g * NPT + u) gives its term.  The block is block bid of the sum's
+// sum_phys(n, NPT).
+template <int NPT, class Load, class Term>
+__device__ __forceinline__ bool ordered_sum(int n, int bid, double* partials, unsigned int* counter,
+                                            double& total, Load&& load, Term&& term) {
+  const int per = kThreads * NPT, nvb = (n + per - 1) / per, vb0 = bid * kSumVB;
+  const int base = vb0 * per + threadIdx.x;
+#pragma unroll
+  for (int q = 0; q < kSumVB * NPT; ++q)
+    if (base + q * kThreads < n) load(q, base + q * kThreads);
+  df v[kSumVB];
+#pragma unroll
+  for (int g = 0; g < kSumVB; ++g) {
+    v[g] = df{0.f, 0.f};
+#pragma unroll
+    for (int u = 0; u < NPT; ++u)
+      if (base + (g * NPT + u) * kThreads < n) v[g] = df_add(v[g], term(g * NPT + u));
+  }
+  return block_sums_last_df(v, partials, counter, total, vb0, nvb, (nvb + kSumVB - 1) / kSumVB);
+}
+inline int sum_phys(int64_t n, int npt) {
+  const int64_t nvb = (n + (int64_t)kThreads * npt - 1) / ((int64_t)kThreads * npt);
+  return (int)((nvb + kSumVB - 1) / kSumVB);
+}
+
+// Where a sum goes: *out, and with num or den also a quotient of the CG, *num
+// / sum or sum / *den, into *q as a double or as a df64 pair.  The block that
+// finishes the sum divides, so the next kernel's blocks read the quotient
+// instead of dividing each (an FP64 division is about 30 FP64 operations).
+struct SumOut {
+  double* out = nullptr;
+  const double* num = nullptr;
+  const double* den = nullptr;
+  double* q = nullptr;
+  int pair = 0;
+};
+__device__ __forceinline__ void sum_out(const SumOut& s, double t) {
+  *s.out = t;
+  if (s.q) {
+    const double v = s.num ? *s.num / t : t / *s.den;
+    if (s.pair) {
+      const df p = df_from_double(v);
+      *reinterpret_cast<float2*>(s.q) = make_float2(p.hi, p.lo);
+    } else {
+      *s.q = v;
+    }
+  }
+}
+__device__ __forceinline__ df load_pair(const double* q) {
+  const float2 v = *reinterpret_cast<const float2*>(q);
+  return df{v.x, v.y};
 }
 
 template <int N>
@@ -600,32 +791,23 @@ __device__ __forceinline__ void block_sum_finish(double (&v)[N], double* partial
     for (int k = 0; k < N; ++k) out[k] = t[k];
   }
 }
+__device__ __forceinline__ void block_sum_finish(double v, double* partials, unsigned int* counter,
+                                                 const SumOut& out) {
+  double a[1] = {v}, t[1];
+  if (block_sum_last<1>(a, partials, counter, t) && threadIdx.x == 0) sum_out(out, t[0]);
+}
 
 // As block_sum_last_df over a 1D grid, storing the total to *out.
 __device__ __forceinline__ void block_sum_finish_df(df v, double* partials, unsigned int* counter,
-                                                    double* out) {
+                                                    const SumOut& out) {
   double t;
   if (block_sum_last_df(v, partials, counter, t, threadIdx.x, blockDim.x, blockIdx.x, gridDim.x) &&
       threadIdx.x == 0)
-    *out = t;
+    sum_out(out, t);
 }
 
-// *a / *b for the whole block, computed once by thread 0: GB300's FP64
-// division costs tens of FP64 operations at 1/58 of the FP32 rate, so one
-// per thread of a wide grid costs microseconds.  Every thread of the block
-// must call these, once per kernel.
-__device__ __forceinline__ double block_div(const double* a, const double* b) {
-  __shared__ double s;
-  if (threadIdx.x == 0) s = *a / *b;
-  __syncthreads();
-  return s;
-}
-__device__ __forceinline__ float block_div_f(const double* a, const double* b) {
-  __shared__ float s;
-  if (threadIdx.x == 0) s = (float)(*a / *b);
-  __syncthreads();
-  return s;
-}
+// *a / *b for the whole block as a df64 pair, computed once by thread 0.
+// Every thread of the block must call it, once per kernel.
 __device__ __forceinline__ df block_div_df(const double* a, const double* b) {
   __shared__ float2 s;
   if (threadIdx.x == 0) {
@@ -933,13 +1115,13 @@ void vcycle(Ctx& c, const Real* b, Real* x, bool zero_guess);
 // fine3d.cu: tiled finest-level 3D passes (mode 0 pre, 1 post, 2 residual, 3 sweep)
 void fine3d(Ctx& c, int mode, const float* ke, const float* b, const float* dinv, const float* x,
             const float* xc, float* out0, float* out1, const float2* rdot = nullptr,
-            double* dout = nullptr);
-// FP32 CG direction update and product: p = z + beta p_old (beta = *rz_new /
-// *rz_old, 0 while *first is nonzero), y = A p with the current k_e, p . y
-// into *dot; odd *parity swaps p_old and p; rz_set receives *rz_new
-void fine3d_dir(Ctx& c, const float* z, const float* p_old, float* p, const double* rz_new,
-                const double* rz_old, const double* first, const double* parity, float* y,
-                double* dot, double* rz_set);
+            SumOut dout = {});
+// FP32 CG direction update and product: p = z + beta p_old (beta a df64 pair,
+// 0 while *first is nonzero), y = A p with the current k_e, p . y into dot;
+// odd *parity swaps p_old and p; rz_set receives *rz_new
+void fine3d_dir(Ctx& c, const float* z, const float* p_old, float* p, const double* beta,
+                const double* first, const double* parity, float* y, SumOut dot,
+                const double* rz_new, double* rz_set);
 // zero-guess FP32 V-cycle x = M b that also leaves r . x in *dout (r in
 // double-float pairs, or r = b when r is null; 3D tiled path)
 // vcycle_dot applies: one pre- and one post-sweep, two levels or more, and
@@ -947,9 +1129,9 @@ void fine3d_dir(Ctx& c, const float* z, const float* p_old, float* p, const doub
 inline bool vcycle_dot_ok(const Ctx& c) {
   return c.p.nu_pre == 1 && c.p.nu_post == 1 && c.nl >= 2 && !c.untiled;
 }
-void vcycle_dot(Ctx& c, const float* b, float* x, const float2* r, double* dout);
+void vcycle_dot(Ctx& c, const float* b, float* x, const float2* r, SumOut dout);
 // the same in FP64 with b . x in *dout, for 2D grids where vcycle_dot_ok
-void vcycle_dot64(Ctx& c, const double* b, double* x, double* dout);
+void vcycle_dot64(Ctx& c, const double* b, double* x, SumOut dout);
 // launch shapes of the tiled kernels (occupancy query; call outside stream capture)
 void fine3d_prepare(Ctx& c);
 // vcycle.cu: can the bottom levels run as one thread-block cluster launch
@@ -959,13 +1141,11 @@ void df3d_prepare(Ctx& c);
 // kd_df from ke_df (after every change of the design)
 void df3d_node_diag(Ctx& c);
 void df3d_apply(Ctx& c, const double* x, double* y, double* dot);
-// parity (device scalar, may be null): odd swaps the roles of p_old and p;
-// rz_set (may be null) receives *rz_new after the launch has used it
-void df3d_dir(Ctx& c, const float* z, const float2* p_old, float2* p, const double* rz_new,
-              const double* rz_old, bool first, float2* y, double* dot,
-              const double* parity = nullptr, double* rz_set = nullptr);
+// parity (device scalar, may be null): odd swaps the roles of p_old and p
+void df3d_dir(Ctx& c, const float* z, const float2* p_old, float2* p, const double* beta, bool first,
+              float2* y, SumOut dot, const double* parity = nullptr);
 void df3d_resid(Ctx& c, const float2* q, const float2* x, float2* r, float* r32, double* rr);
-void apply_fine64(Ctx& c, const double* ke, const double* x, double* y, double* dot_out);
+void apply_fine64(Ctx& c, const double* ke, const double* x, double* y, SumOut dot_out = {});
 void apply_fine32(Ctx& c, const float* ke, const float* x, float* y);
 void apply_dK64(Ctx& c, const double* x, double* y);
 void apply_dK32(Ctx& c, const float* x, float* y);
@@ -981,7 +1161,10 @@ int solve_mgcg(Ctx& c, double* T, int* iters, double* relres);
 void solve_mgar(Ctx& c, const double* T_prev, double* T, double* res, int* accepted);
 void precondition(Ctx& c, const double* r, double* z);
 // reductions
-void dot(Ctx& c, const double* a, const double* b, int64_t n, double* out_dev);
+void dot(Ctx& c, const double* a, const double* b, int64_t n, SumOut out);
+inline void dot(Ctx& c, const double* a, const double* b, int64_t n, double* out_dev) {
+  dot(c, a, b, n, SumOut{out_dev});
+}
 void fetch_scalars(Ctx& c, int first, int count);
 // design.cu
 void setup_filter(Ctx& c);

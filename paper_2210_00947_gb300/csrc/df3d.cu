@@ -56,22 +56,19 @@ struct DfArgs {
   double* y64;          // APPLY: A x
   const float* z;       // DIR
   const float2* q;      // RESID
-  const double* rz_new; // DIR: beta = rz_new / rz_old
-  const double* rz_old;
+  const double* beta;   // DIR: a df64 pair
   int first;            // DIR: p = z
   float2* y;            // APPLY/DIR: A x; RESID: r
   float2* p;            // DIR: new direction
   float* r32;           // RESID
   double* partials;
   unsigned int* counter;
-  double* out;          // dot product (may be null for APPLY)
+  SumOut out;           // dot product (without one for APPLY)
   // DIR inside the device-side CG loop: with parity odd, p_old is x_alt and
-  // the new p goes to p_alt (the two direction buffers swap each iteration);
-  // rz_set, when given, receives rz_new once every block has read it
+  // the new p goes to p_alt (the two direction buffers swap each iteration)
   const float2* x_alt;
   float2* p_alt;
   const double* parity;
-  double* rz_set;
 };
 
 template <int MODE>
@@ -187,8 +184,7 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 4 : 2) k_df3d(DfArgs a)
   if (kr) T::kring(tid - KRING0, kxh, kyh);
   df beta{0.f, 0.f};
   if (MODE == DIR) {
-    const df q = block_div_df(a.rz_new, a.rz_old);  // once per block
-    if (!a.first) beta = q;
+    if (!a.first) beta = load_pair(a.beta);
   }
   const bool odd = MODE == DIR && a.parity && (((int)*a.parity) & 1);
   const float2* const xsrc = odd ? a.x_alt : a.x;
@@ -363,7 +359,7 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 4 : 2) k_df3d(DfArgs a)
         dot = df_add(dot, df_mul(ri, ri));                                                 \
       } else if (MODE == APPLY) {                                                          \
         a.y64[idx] = df_to_double(yv);                                                     \
-        if (a.out) dot = df_add(dot, df_mul(dfk(xi), yv));                                 \
+        if (a.out.out) dot = df_add(dot, df_mul(dfk(xi), yv));                                 \
       } else {                                                                             \
         a.y[idx] = make_float2(yv.hi, yv.lo);                                              \
         dot = df_add(dot, df_mul(dfk(xi), yv));                                            \
@@ -381,14 +377,12 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 4 : 2) k_df3d(DfArgs a)
 #undef D3D_FINISH
 #undef D3D_FINISH_FROM
 #undef D3D_FINISH_LAYER
-  if (a.out) {
+  if (a.out.out) {
     double t;
     const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     const int nb = gridDim.x * gridDim.y * gridDim.z;
-    if (block_sum_last_df(dot, a.partials, a.counter, t, tid, T::NTB, bid, nb) && tid == 0) {
-      a.out[0] = t;
-      if (MODE == DIR && a.rz_set) *a.rz_set = *a.rz_new;  // every block has read rz_new
-    }
+    if (block_sum_last_df(dot, a.partials, a.counter, t, tid, T::NTB, bid, nb) && tid == 0)
+      sum_out(a.out, t);
   }
 }
 
@@ -495,14 +489,13 @@ void df3d_apply(Ctx& c, const double* x, double* y, double* dot) {
   DfArgs a = base_args(c);
   a.x64 = x;
   a.y64 = y;
-  a.out = dot;
+  a.out = SumOut{dot};
   launch<APPLY>(c, a);
 }
 
-// p = z + (rz_new / rz_old) p_old (p = z when first), y = A p, p . y into *dot
-void df3d_dir(Ctx& c, const float* z, const float2* p_old, float2* p, const double* rz_new,
-              const double* rz_old, bool first, float2* y, double* dot, const double* parity,
-              double* rz_set) {
+// p = z + beta p_old (p = z when first), y = A p, p . y into dot
+void df3d_dir(Ctx& c, const float* z, const float2* p_old, float2* p, const double* beta, bool first,
+              float2* y, SumOut dot, const double* parity) {
   using namespace d3d;
   DfArgs a = base_args(c);
   a.z = z;
@@ -511,9 +504,7 @@ void df3d_dir(Ctx& c, const float* z, const float2* p_old, float2* p, const doub
   a.x_alt = p;        // odd parity: the buffers swap roles
   a.p_alt = const_cast<float2*>(p_old);
   a.parity = parity;
-  a.rz_set = rz_set;
-  a.rz_new = rz_new;
-  a.rz_old = rz_old;
+  a.beta = beta;
   a.first = first ? 1 : 0;
   a.y = y;
   a.out = dot;
@@ -528,7 +519,7 @@ void df3d_resid(Ctx& c, const float2* q, const float2* x, float2* r, float* r32,
   a.x = x;
   a.y = r;
   a.r32 = r32;
-  a.out = rr;
+  a.out = SumOut{rr};
   launch<RESID>(c, a);
 }
 

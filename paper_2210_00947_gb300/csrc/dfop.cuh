@@ -147,17 +147,16 @@ __device__ __forceinline__ df unpack(float2 v) { return df{v.x, v.y}; }
 // Tiled 2D direction update and product of the df64 CG, shared by the
 // single-design and the batched solve: p = z + beta p_old on a 64 x 24 node
 // tile (62 x 22 own nodes and their rim) in shared memory, off-grid and fixed
-// neighbours as zeros, then y = A p in the difference form and this thread's
-// terms of p . y.  As separate kernels, the product gathering each operand
+// neighbours as zeros, then y = A p in the difference form.  As separate kernels, the product gathering each operand
 // with bounds and Dirichlet tests, the two took 30 us on 1025^2 nodes; this
-// takes 19, issue-bound, against 10 us of FP32 pipe (about 250 operations per
+// takes 15, issue-bound, against 10 us of FP32 pipe (about 250 operations per
 // node and the rim) and 6 us of bytes.
 struct DfDirSmem {
   float2 p[l2d::kRows + 2][l2d::kW];
   float2 k[l2d::kRows + 1][l2d::kW];
 };
 
-__device__ __forceinline__ df df_dir_tile(DfDirSmem& s, const DfOp& op, int tx, int ty,
+__device__ __forceinline__ void df_dir_tile(DfDirSmem& s, const DfOp& op, int tx, int ty,
                                           const float* __restrict__ z,
                                           const float2* __restrict__ p_old, bool first, df beta,
                                           float2* __restrict__ pn, float2* __restrict__ y) {
@@ -200,7 +199,6 @@ __device__ __forceinline__ df df_dir_tile(DfDirSmem& s, const DfOp& op, int tx, 
       s.p[p.y0 + q + 1][p.lane + 32 * h] = fx[q][h] ? make_float2(0.f, 0.f) : v;
     }
   __syncthreads();
-  float dh = 0.f, dl = 0.f;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int c = p.lane + 32 * h, y0 = p.y0;
@@ -228,21 +226,12 @@ __device__ __forceinline__ df df_dir_tile(DfDirSmem& s, const DfOp& op, int tx, 
         const int64_t o = at + q * op.NX + 32 * h;
         pn[o] = pv[q][h];
         y[o] = pack(yv);
-        // p . y, the rounding errors gathered apart
-        float m, me, t, te;
-        two_prod(xi.hi, yv.hi, m, me);
-        me = __fmaf_rn(xi.hi, yv.lo, me);
-        me = __fmaf_rn(xi.lo, yv.hi, me);
-        two_sum(dh, m, t, te);
-        dh = t;
-        dl = __fadd_rn(dl, __fadd_rn(te, me));
       }
       xl = yl, xc = yc, xr = yr;
       yl = zl, yc = zc, yr = zr;
       k00 = k10, k01 = k11;
     }
   }
-  return df_make(dh, dl);
 }
 
 // The operator of a handle's finest level at its current design.

@@ -53,13 +53,12 @@ struct FineArgs {
   const float2* rdot;
   double* partials;
   unsigned int* counter;
-  double* dout;     // POST / SWEEP: r . x'; DIR: p . A p
-  // DIR: beta = rz_new / rz_old, or 0 while *first is nonzero; with *parity
-  // odd, p_old is x_alt and p goes to out_alt (the two direction buffers swap
-  // each iteration); rz_set, when given, receives *rz_new once every block
-  // has read it
+  SumOut dout;      // POST / SWEEP: r . x'; DIR: p . A p
+  // DIR: beta (a df64 pair), or 0 while *first is nonzero; with *parity odd,
+  // p_old is x_alt and p goes to out_alt (the two direction buffers swap each
+  // iteration); rz_set receives *rz_new once p . A p is done with it
+  const double* beta;
   const double* rz_new;
-  const double* rz_old;
   const double* first;
   const double* parity;
   const void* x_alt;
@@ -258,8 +257,7 @@ __global__ void __launch_bounds__(T::NTB, f3d_minb(MODE, T::NT)) k_fine3d(FineAr
   if (MODE == DIR) {
     const bool first = *a.first != 0.0;
     const bool odd = a.parity && (((int)*a.parity) & 1);
-    const float q = block_div_f(a.rz_new, a.rz_old);  // once per block
-    om = first ? Real(0) : (Real)q;
+    om = first ? Real(0) : (Real)load_pair(a.beta).hi;
     dsrc = first ? nullptr : (const Real*)(odd ? a.x_alt : a.x);
     pdst = (Real*)(odd ? a.out_alt : a.out0);
   }
@@ -285,7 +283,7 @@ __global__ void __launch_bounds__(T::NTB, f3d_minb(MODE, T::NT)) k_fine3d(FineAr
   // for the fused r . x')
   Real cv[4], cb[4], cd[4], mv[4];
   bool cf[4];
-  const bool rdot = (MODE == POST || MODE == SWEEP || MODE == DIR) && a.dout != nullptr;
+  const bool rdot = (MODE == POST || MODE == SWEEP || MODE == DIR) && a.dout.out != nullptr;
   // the thread's terms of p . Ap, or of r . x' with r in FP32, are few (one z
   // run, about 20): summed in FP32 and combined across threads in df64; r in
   // df64 pairs keeps a df64 sum
@@ -416,8 +414,8 @@ __global__ void __launch_bounds__(T::NTB, f3d_minb(MODE, T::NT)) k_fine3d(FineAr
     const int nb = gridDim.x * gridDim.y * gridDim.z;
     const df v = df_add(dacc, df{facc, 0.f});
     if (block_sum_last_df(v, a.partials, a.counter, t, tid, T::NTB, bid, nb) && tid == 0) {
-      a.dout[0] = t;
-      if (MODE == DIR && a.rz_set) *a.rz_set = *a.rz_new;  // every block has read rz_new
+      sum_out(a.dout, t);
+      if (MODE == DIR) *a.rz_set = *a.rz_new;
     }
   }
 }
@@ -480,7 +478,7 @@ void launch(Ctx& c, FineArgs& a) {
 // Launch one tiled finest-level pass of the FP32 V-cycle (3D only).
 // mode: 0 pre, 1 post, 2 residual, 3 sweep.
 void fine3d(Ctx& c, int mode, const float* ke, const float* b, const float* dinv, const float* x,
-            const float* xc, float* out0, float* out1, const float2* rdot, double* dout) {
+            const float* xc, float* out0, float* out1, const float2* rdot, SumOut dout) {
   using namespace f3d;
   const Dims& d = c.L[0];
   FineArgs a{};
@@ -515,11 +513,11 @@ void fine3d(Ctx& c, int mode, const float* ke, const float* b, const float* dinv
   MGAR_LAUNCH_CHECK_AT(level_site(6 + (mode == PRE ? 0 : mode == POST ? 1 : mode == SWEEP ? 2 : 3), 0));
 }
 
-// p = z + (rz_new / rz_old) p_old (p = z while *first is nonzero), y = A p,
-// p . y into *dot; FP32 vectors
-void fine3d_dir(Ctx& c, const float* z, const float* p_old, float* p, const double* rz_new,
-                const double* rz_old, const double* first, const double* parity, float* y,
-                double* dot, double* rz_set) {
+// p = z + beta p_old (p = z while *first is nonzero), y = A p, p . y into dot;
+// FP32 vectors
+void fine3d_dir(Ctx& c, const float* z, const float* p_old, float* p, const double* beta,
+                const double* first, const double* parity, float* y, SumOut dot,
+                const double* rz_new, double* rz_set) {
   using namespace f3d;
   const Dims& d = c.L[0];
   FineArgs a{};
@@ -538,7 +536,7 @@ void fine3d_dir(Ctx& c, const float* z, const float* p_old, float* p, const doub
   a.out_alt = const_cast<float*>(p_old);
   a.out1 = y;
   a.rz_new = rz_new;
-  a.rz_old = rz_old;
+  a.beta = beta;
   a.first = first;
   a.parity = parity;
   a.rz_set = rz_set;

@@ -8,13 +8,14 @@
 // that follows from it:
 //   down, finest:  x = w D^-1 b (or the given x), r = b - A x, b_c = P^T r,
 //                  x_c = w D_c^-1 b_c        (three or four passes before)
-//   up, finest:    v = x + P x_c, x' = v + w D^-1 (b - A v), r . x'   (two)
+//   up, finest:    v = x + P x_c, x' = v + w D^-1 (b - A v)           (two)
 //   down, coarse:  r = b - A x, b_c = P^T r, x_c = w D_c^-1 b_c       (two)
 //   up, coarse:    v = x + P x_c, x' = v + w D^-1 (b - A v)     (one or two)
-// The residual never goes to memory.  1025^2 nodes in FP32: down 7.7 us (21.5
-// as three kernels), up with r . x 14 us (26.8), a coarse level 2.6-5.3 us each
-// way (6-8).  Bound by instruction issue (100 warp instructions per node down,
-// 165 up) and the sum's cross-block stage.  Tiles are 64 columns wide with their
+// The residual never goes to memory.  1025^2 nodes in FP32: down 6.7 us (21.5
+// as three kernels), up 8.2 us (20 as two), a coarse level 2.6-5.3 us each way
+// (6-8); bound by instruction issue (100 warp instructions per node down, 130
+// up).  FP32 results are those of the separate passes bit for bit (the order
+// of a row's additions and its contractions are theirs).  Tiles are 64 columns wide with their
 // rim (two nodes per lane), so a warp's rows are coalesced and no lane divides
 // to find its node; tall enough that the rim costs 8 % (residuals) to 24 %
 // (x) more, short enough that a 1024^2 grid fills the chip in one wave.
@@ -75,10 +76,25 @@ __device__ __forceinline__ Real restrict_sum(const Real (*r)[W], int c, int y, i
   Real x0, x1, x2, y0, y1, y2;
   restrict_weights<Real>(I, ex, x0, x1, x2);
   restrict_weights<Real>(J, ey, y0, y1, y2);
-  const Real a = x0 * r[y][c] + x1 * r[y][c + 1] + x2 * r[y][c + 2];
-  const Real b = x0 * r[y + 1][c] + x1 * r[y + 1][c + 1] + x2 * r[y + 1][c + 2];
-  const Real d = x0 * r[y + 2][c] + x1 * r[y + 2][c + 1] + x2 * r[y + 2][c + 2];
-  return y0 * a + y1 * b + y2 * d;
+  if constexpr (sizeof(Real) == 4) {
+    // the order of restrict_node
+    Real acc = (y0 * x0) * r[y][c];
+    acc += (y0 * x1) * r[y][c + 1];
+    acc += (y0 * x2) * r[y][c + 2];
+    acc += (y1 * x0) * r[y + 1][c];
+    acc += (y1 * x1) * r[y + 1][c + 1];
+    acc += (y1 * x2) * r[y + 1][c + 2];
+    acc += (y2 * x0) * r[y + 2][c];
+    acc += (y2 * x1) * r[y + 2][c + 1];
+    acc += (y2 * x2) * r[y + 2][c + 2];
+    return acc;
+  } else {
+    // 9 FP64 products fewer
+    const Real a = x0 * r[y][c] + x1 * r[y][c + 1] + x2 * r[y][c + 2];
+    const Real b = x0 * r[y + 1][c] + x1 * r[y + 1][c + 1] + x2 * r[y + 1][c + 2];
+    const Real d = x0 * r[y + 2][c] + x1 * r[y + 2][c + 1] + x2 * r[y + 2][c + 2];
+    return y0 * a + y1 * b + y2 * d;
+  }
 }
 
 // The Q4 rows times 6 of column c at the tile rows y0 .. y0 + kR - 1, tile row
@@ -95,9 +111,25 @@ __device__ __forceinline__ void q4_rows(const Real (*x)[kW], const Real (*k)[kW]
     const Real zl = x[y0 + q + 2][c - 1], zc = x[y0 + q + 2][c], zr = x[y0 + q + 2][c + 1];
     const Real k10 = k[y0 + q + 1][c - 1], k11 = k[y0 + q + 1][c];
     const Real s = k00 + k01, n = k10 + k11;
-    const Real dg = k00 * xl + k01 * xr + k10 * zl + k11 * zr;
-    const Real ed = (k00 + k10) * yl + (k01 + k11) * yr + s * xc + n * zc;
-    f(q, yc, [&](Real xi) { return Real(4) * (s + n) * xi - ed - Real(2) * dg; });
+    f(q, yc, [&](Real xi) {
+      if constexpr (sizeof(Real) == 4) {
+        // the order of fine_row2, as compiled
+        Real acc = __fmul_rn(__fmul_rn(4.f, s + n), xi);
+        acc = __fmaf_rn(-(k00 + k10), yl, acc);
+        acc = __fmaf_rn(-(k01 + k11), yr, acc);
+        acc = __fmaf_rn(-s, xc, acc);
+        acc = __fmaf_rn(-n, zc, acc);
+        acc = __fmaf_rn(-2.f * k00, xl, acc);
+        acc = __fmaf_rn(-2.f * k01, xr, acc);
+        acc = __fmaf_rn(-2.f * k10, zl, acc);
+        acc = __fmaf_rn(-2.f * k11, zr, acc);
+        return acc;
+      } else {
+        const Real dg = k00 * xl + k01 * xr + k10 * zl + k11 * zr;
+        const Real ed = (k00 + k10) * yl + (k01 + k11) * yr + s * xc + n * zc;
+        return Real(4) * (s + n) * xi - ed - Real(2) * dg;
+      }
+    });
     xl = yl, xc = yc, xr = yr;
     yl = zl, yc = zc, yr = zr;
     k00 = k10, k01 = k11;
@@ -118,6 +150,10 @@ __device__ __forceinline__ Real prolong_sum(const Real (*c)[W], int x, int y, bo
   const Real wx = hx ? Real(0.5) : Real(1), wxy = hy ? Real(0.5) * wx : wx;
   return wxy * s;
 }
+
+// a / 6; rounded by itself in FP32, as fine_row2's result
+__device__ __forceinline__ float sixth(float a) { return __fmul_rn(a, float(1.0 / 6.0)); }
+__device__ __forceinline__ double sixth(double a) { return a * (1.0 / 6.0); }
 
 // First coarse tap of fine node i, and whether it is halfway.
 __device__ __forceinline__ int first_tap(int i, int nf, bool& half) {
@@ -223,7 +259,7 @@ __device__ __forceinline__ void fine_down(DownSmem<Real>& s, const Fine<Real>& f
     const int c = p.lane + 32 * h;
     if (c >= 1 && c < 2 * kCX + 2)
       q4_rows<Real>(s.x, s.k, c, p.y0, [&](int q, Real xi, auto&& row) {
-        const Real r = bv[q][h] - row(xi) * Real(1.0 / 6.0);
+        const Real r = bv[q][h] - sixth(row(xi));
         s.r[p.y0 + q][c] = dv[q][h] > Real(0) ? r : Real(0);
       });
   }
@@ -247,14 +283,13 @@ struct UpSmem {
   Real c[kRows / 2 + 3][kW / 2 + 4];
 };
 
-// xout = v + w D^-1 (b - A v), v = t + P res (fixed nodes keep t); dot(at, b,
-// x', early) is called for every node of the tile, early what pre(at) gave for
-// it beside the operands' loads.
-template <typename Real, class Pre, class Dot>
+// xout = v + w D^-1 (b - A v), v = t + P res (fixed nodes keep t); dot(b, x')
+// is called for every node of the tile.
+template <typename Real, class Dot>
 __device__ __forceinline__ void fine_up(UpSmem<Real>& s, const Fine<Real>& f, int tx, int ty,
                                         const Real* __restrict__ b, const Real* __restrict__ t,
                                         const Real* __restrict__ res, Real* __restrict__ xout,
-                                        Pre&& pre, Dot&& dot) {
+                                        Dot&& dot) {
   constexpr int CR = kRows / 2 + 2, CC = kW / 2 + 2;
   const int NX = f.ex + 1, NY = f.ey + 1;
   const int fx0 = tx * kUX - 1, fy0 = ty * kUY - 1;
@@ -263,7 +298,6 @@ __device__ __forceinline__ void fine_up(UpSmem<Real>& s, const Fine<Real>& f, in
   const int64_t at = fx0 + p.lane + (int64_t)NX * (fy0 + p.y0);
   const int64_t eat = fx0 + p.lane + (int64_t)f.ex * (fy0 + p.y0);
   Real dv[kR][2], bv[kR][2], tv[kR][2];
-  decltype(pre(int64_t(0))) early[kR][2];
   bool ron[kR];
 #pragma unroll
   for (int q = 0; q < kR; ++q) {
@@ -297,7 +331,6 @@ __device__ __forceinline__ void fine_up(UpSmem<Real>& s, const Fine<Real>& f, in
       if (ron[q] && p.con[h]) {
         bv[q][h] = b[at + q * NX + 32 * h];
         tv[q][h] = t[at + q * NX + 32 * h];
-        early[q][h] = pre(at + q * NX + 32 * h);
       }
     }
   __syncthreads();
@@ -323,11 +356,10 @@ __device__ __forceinline__ void fine_up(UpSmem<Real>& s, const Fine<Real>& f, in
         const int y = p.y0 + q;
         if (!(y >= 1 && y <= kUY && ron[q])) return;
         const Real v = tv[q][h];
-        const Real ax = dv[q][h] < Real(0) ? v : row(v) * Real(1.0 / 6.0);
+        const Real ax = dv[q][h] < Real(0) ? v : sixth(row(v));
         const Real xo = v + f.omega * fabs(dv[q][h]) * (bv[q][h] - ax);
-        const int64_t o = at + q * NX + 32 * h;
-        xout[o] = xo;
-        dot(bv[q][h], xo, early[q][h]);
+        xout[at + q * NX + 32 * h] = xo;
+        dot(bv[q][h], xo);
       });
   }
 }
@@ -367,7 +399,9 @@ struct CoarseUpSmem {
   Real v[kPY + 2][32];
 };
 
-template <typename Real>
+// AXES: interpolate along x, then y (post_node's order of additions), else
+// all taps in one sum (prolong_node's).
+template <typename Real, bool AXES>
 __device__ __forceinline__ void coarse_up(CoarseUpSmem<Real>& s, const Coarse<Real>& f, int tx, int ty,
                                           const Real* __restrict__ b, const Real* __restrict__ x,
                                           const Real* __restrict__ res, Real* __restrict__ xout) {
@@ -392,13 +426,18 @@ __device__ __forceinline__ void coarse_up(CoarseUpSmem<Real>& s, const Coarse<Re
     const Real r0 = res[c0], r1 = res[c0 + ox], r2 = res[c0 + oy], r3 = res[c0 + ox + oy];
     v = x[idx];
     if (own) bv = b[idx];
-    Real p = r0;
-    if (hx) p += r1;
-    if (hy) {
-      p += r2;
-      if (hx) p += r3;
+    if (AXES) {
+      const Real p = hx ? Real(0.5) * (r0 + r1) : r0, u = hx ? Real(0.5) * (r2 + r3) : r2;
+      v += hy ? Real(0.5) * (p + u) : p;
+    } else {
+      Real p = r0;
+      if (hx) p += r1;
+      if (hy) {
+        p += r2;
+        if (hx) p += r3;
+      }
+      v += (hx ? Real(0.5) : Real(1)) * (hy ? Real(0.5) : Real(1)) * p;
     }
-    v += (hx ? Real(0.5) : Real(1)) * (hy ? Real(0.5) : Real(1)) * p;
   }
   s.v[w][lane] = v;
   __syncthreads();

@@ -19,7 +19,7 @@ namespace mgar {
 
 // ----------------------------------------------------------------- kernels
 __global__ void k_dot(const double* __restrict__ a, const double* __restrict__ b, int64_t n,
-                      double* partials, unsigned int* counter, double* out) {
+                      double* partials, unsigned int* counter, SumOut out) {
   // four independent partial sums per thread: four loads in flight, and no
   // chain of dependent FP64 additions (fixed order, so still reproducible)
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -32,8 +32,7 @@ __global__ void k_dot(const double* __restrict__ a, const double* __restrict__ b
     s3 += a[i + 3 * stride] * b[i + 3 * stride];
   }
   for (; i < n; i += stride) s0 += a[i] * b[i];
-  double v[1] = {(s0 + s1) + (s2 + s3)};
-  block_sum_finish<1>(v, partials, counter, out);
+  block_sum_finish((s0 + s1) + (s2 + s3), partials, counter, out);
 }
 
 // The reduced system's products in one pass over R, W and q (Eq. 19-20):
@@ -91,27 +90,48 @@ __global__ void k_residual_norm(FineOp<double> op, const double* __restrict__ q,
   block_sum_finish<1>(v, partials, counter, out);
 }
 
-// alpha = rz / pAp; x += alpha p; r -= alpha Ap; ||r||^2.
-__global__ void k_cg_xr(double* __restrict__ x, double* __restrict__ r, const double* __restrict__ p,
-                        const double* __restrict__ Ap, int64_t n, const double* __restrict__ rz,
-                        const double* __restrict__ pap, double* partials, unsigned int* counter,
-                        double* out) {
-  const double alpha = block_div(rz, pap);
+// x += alpha p; r -= alpha Ap; ||r||^2.  Two nodes per access (the solver's own
+// vectors are aligned; the caller's x need not be) and, as in dot, two blocks
+// per SM: with eight the FP64 shuffle trees took as long as the data.
+__global__ void __launch_bounds__(kThreads) k_cg_xr(double* __restrict__ x, double* __restrict__ r,
+                                                    const double* __restrict__ p,
+                                                    const double* __restrict__ Ap, int64_t n,
+                                                    const double* __restrict__ alpha_p,
+                                                    double* partials, unsigned int* counter,
+                                                    double* out) {
+  const double alpha = *alpha_p;
   double v[1] = {0.0};
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    x[i] += alpha * p[i];
-    const double ri = r[i] - alpha * Ap[i];
-    r[i] = ri;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x, n2 = n >> 1;
+  const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  double2* __restrict__ r2 = reinterpret_cast<double2*>(r);
+  const double2* __restrict__ p2 = reinterpret_cast<const double2*>(p);
+  const double2* __restrict__ q2 = reinterpret_cast<const double2*>(Ap);
+#pragma unroll 2
+  for (int64_t i = t0; i < n2; i += stride) {
+    const double xa = x[2 * i], xb = x[2 * i + 1];
+    const double2 pv = p2[i], qv = q2[i];
+    double2 rv = r2[i];
+    x[2 * i] = xa + alpha * pv.x;
+    x[2 * i + 1] = xb + alpha * pv.y;
+    rv.x -= alpha * qv.x;
+    rv.y -= alpha * qv.y;
+    r2[i] = rv;
+    v[0] += rv.x * rv.x;
+    v[0] += rv.y * rv.y;
+  }
+  if ((n & 1) && t0 == 0) {
+    x[n - 1] += alpha * p[n - 1];
+    const double ri = r[n - 1] - alpha * Ap[n - 1];
+    r[n - 1] = ri;
     v[0] += ri * ri;
   }
   block_sum_finish<1>(v, partials, counter, out);
 }
 
-// p = z + (rz_new / rz_old) p
+// p = z + beta p
 __global__ void k_cg_p(double* __restrict__ p, const double* __restrict__ z, int64_t n,
-                       const double* __restrict__ rz_new, const double* __restrict__ rz_old) {
-  const double beta = block_div(rz_new, rz_old);
+                       const double* __restrict__ beta_p) {
+  const double beta = *beta_p;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     p[i] = z[i] + beta * p[i];
@@ -201,9 +221,15 @@ __global__ void k_reduced_combine(const double* __restrict__ Q, const double* __
 
 // -------------------------------------------------------------------- host
 static int red_blocks(Ctx& c) { return c.grid_blocks; }
+// Two blocks per SM for a sum over n values, four per thread and pass.
+static int sum_blocks(const Ctx& c, int64_t n) {
+  return (int)std::min<int64_t>(blocks_for((n + 3) / 4), (int64_t)c.sms * 2);
+}
 
-void dot(Ctx& c, const double* a, const double* b, int64_t n, double* out_dev) {
-  k_dot<<<red_blocks(c), kThreads, 0, c.stream>>>(a, b, n, c.partials, c.counter, out_dev);
+// Every warp of a sum costs an FP64 shuffle tree, so no more than two blocks
+// per SM, each thread with four loads of each vector in flight.
+void dot(Ctx& c, const double* a, const double* b, int64_t n, SumOut out) {
+  k_dot<<<sum_blocks(c, n), kThreads, 0, c.stream>>>(a, b, n, c.partials, c.counter, out);
   MGAR_LAUNCH_CHECK();
 }
 
@@ -327,24 +353,27 @@ static int solve_mgcg_fp(Ctx& c, double* T, int* iters, double* relres) {
   int it = 0;
   if (!(rel <= c.p.eps2)) {
     require(std::isfinite(rel), MGAR_ERR_NONFINITE, "non-finite initial residual");
-    // z = M r and r . z, in one with the 2D V-cycle's tiled passes
+    // z = M r, r . z into dsc[slot] and beta, in one with the 2D V-cycle's
+    // tiled passes
     auto precondition_rz = [&](int slot) {
+      const SumOut out{c.dsc + slot, nullptr, c.dsc + (slot == S_RZ0 ? S_RZ1 : S_RZ0),
+                       c.dsc + S_BETA, 0};
       if (c.dim == 2 && vcycle_dot_ok(c)) {
         run_graph(c, slot == S_RZ0 ? 11 : 12, c.r, c.z, vcycle_profiled(c),
-                  [&] { vcycle_dot64(c, c.r, c.z, c.dsc + slot); });
+                  [&] { vcycle_dot64(c, c.r, c.z, out); });
       } else {
         precondition(c, c.r, c.z);
-        dot(c, c.r, c.z, n, c.dsc + slot);
+        dot(c, c.r, c.z, n, out);
       }
     };
     int a = S_RZ0, b = S_RZ1;
     precondition_rz(a);
     MGAR_CUDA(cudaMemcpyAsync(c.pv, c.z, n * sizeof(double), cudaMemcpyDeviceToDevice, c.stream));
     while (it < c.p.cg_max) {
-      apply_fine64(c, c.ke, c.pv, c.Ap, c.dsc + S_PAP);
-      k_cg_xr<<<red_blocks(c), kThreads, 0, c.stream>>>(T, c.r, c.pv, c.Ap, n, c.dsc + a,
-                                                        c.dsc + S_PAP, c.partials, c.counter,
-                                                        c.dsc + S_RR);
+      apply_fine64(c, c.ke, c.pv, c.Ap,
+                   SumOut{c.dsc + S_PAP, c.dsc + a, nullptr, c.dsc + S_ALPHA, 0});
+      k_cg_xr<<<sum_blocks(c, n), kThreads, 0, c.stream>>>(T, c.r, c.pv, c.Ap, n, c.dsc + S_ALPHA,
+                                                        c.partials, c.counter, c.dsc + S_RR);
       MGAR_LAUNCH_CHECK();
       ++it;
       fetch_scalars(c, S_RR, 1);
@@ -352,7 +381,7 @@ static int solve_mgcg_fp(Ctx& c, double* T, int* iters, double* relres) {
       require(std::isfinite(rel), MGAR_ERR_NONFINITE, "CG breakdown (non-finite residual)");
       if (rel <= c.p.eps2) break;
       precondition_rz(b);
-      k_cg_p<<<red_blocks(c), kThreads, 0, c.stream>>>(c.pv, c.z, n, c.dsc + b, c.dsc + a);
+      k_cg_p<<<red_blocks(c), kThreads, 0, c.stream>>>(c.pv, c.z, n, c.dsc + S_BETA);
       MGAR_LAUNCH_CHECK();
       std::swap(a, b);
     }
@@ -445,7 +474,7 @@ void solve_mgar(Ctx& c, const double* T_prev, double* T, double* res, int* accep
     } else if (c.p.precision == MGAR_MIXED) {
       apply_df64(c, c.R + (int64_t)j * n, c.W + (int64_t)j * n);
     } else {
-      apply_fine64(c, c.ke, c.R + (int64_t)j * n, c.W + (int64_t)j * n, nullptr);
+      apply_fine64(c, c.ke, c.R + (int64_t)j * n, c.W + (int64_t)j * n);
     }
   }
   if (kept <= 3) {

@@ -78,18 +78,18 @@ __global__ void k_residual(Row row, const Real* __restrict__ b, const Real* __re
   r[idx] = b[idx] - row(x, idx);
 }
 
-// y = A x, optionally with the deterministic sum of x.y into out[0].
+// y = A x, optionally with the deterministic sum of x.y into out.
 template <class Row, typename Real, bool DOT>
 __global__ void k_apply(Row row, const Real* __restrict__ x, Real* __restrict__ y, Real scale,
-                        double* partials, unsigned int* counter, double* out) {
+                        double* partials, unsigned int* counter, SumOut out) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  double v[1] = {0.0};
+  double v = 0.0;
   if (idx < row.size()) {
     const Real ax = scale * row(x, idx);
     y[idx] = ax;
-    if (DOT) v[0] = (double)x[idx] * (double)ax;
+    if (DOT) v = (double)x[idx] * (double)ax;
   }
-  if (DOT) block_sum_finish<1>(v, partials, counter, out);
+  if (DOT) block_sum_finish(v, partials, counter, out);
 }
 
 // The 2D levels' tiled passes (level2d.cuh).
@@ -102,42 +102,51 @@ __global__ void __launch_bounds__(l2d::kThreads2) k_down2d(l2d::Fine<Real> f, co
   l2d::fine_down<Real, ZERO>(s, f, blockIdx.x, blockIdx.y, b, t, bc, dinvc, xc);
 }
 
-// DOT: also r . xout into *dout, r given as df64 pairs (the mixed CG's) or,
-// without them, b itself.  FP32: double-float warp sums, FP64 across warps.
+// DOT (FP64): also b . xout into dout.
 template <typename Real, bool DOT>
 __global__ void __launch_bounds__(l2d::kThreads2) k_up2d(l2d::Fine<Real> f, const Real* __restrict__ b,
                                                          const Real* __restrict__ t,
                                                          const Real* __restrict__ res,
-                                                         Real* __restrict__ xout,
-                                                         const float2* __restrict__ rdot,
-                                                         double* partials, unsigned int* counter,
-                                                         double* dout) {
+                                                         Real* __restrict__ xout, double* partials,
+                                                         unsigned int* counter, SumOut dout) {
   __shared__ l2d::UpSmem<Real> s;
-  float ah = 0.f, al = 0.f;
-  double acc64[1] = {0.0};
-  l2d::fine_up<Real>(
-      s, f, blockIdx.x, blockIdx.y, b, t, res, xout,
-      [&](int64_t at) { return DOT && sizeof(Real) == 4 && rdot ? rdot[at] : make_float2(0.f, 0.f); },
-      [&](Real bv, Real xo, float2 rv) {
-        if constexpr (DOT && sizeof(Real) == 4)
-          df_acc_mulf(ah, al, rdot ? df{rv.x, rv.y} : df{bv, 0.f}, xo);
-        else if constexpr (DOT)
-          acc64[0] += bv * xo;
-      });
-  if constexpr (DOT) {
-    const int bid = blockIdx.x + gridDim.x * blockIdx.y, nb = gridDim.x * gridDim.y;
-    if constexpr (sizeof(Real) == 4) {
-      double v;
-      if (block_sum_last_df(df_make(ah, al), partials, counter, v, threadIdx.x, l2d::kThreads2, bid, nb) &&
-          threadIdx.x == 0)
-        *dout = v;
-    } else {
-      double v[1];
-      if (block_sum_last_ids<1>(acc64, partials, counter, v, threadIdx.x, l2d::kThreads2, bid, nb) &&
-          threadIdx.x == 0)
-        *dout = v[0];
-    }
+  double acc[1] = {0.0};
+  l2d::fine_up<Real>(s, f, blockIdx.x, blockIdx.y, b, t, res, xout,
+                     [&](Real bv, Real xo) { if (DOT) acc[0] += bv * xo; });
+  if (DOT) {
+    double v[1];
+    if (block_sum_last_ids<1>(acc, partials, counter, v, threadIdx.x, l2d::kThreads2,
+                              blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y) &&
+        threadIdx.x == 0)
+      sum_out(dout, v[0]);
   }
+}
+
+// r . x (r in df64 pairs, or r = b without them) over the nodes in memory
+// order.  The mixed 2D CG is sensitive to its last bits: another order of this
+// sum changes which FP32 roundings the V-cycle meets, and with them the
+// iteration count of one design in sixty.  So the sum keeps the order of the
+// nodes and does not follow the tiles, where it cost 6 us on 1025^2 nodes at
+// the end of the pass.
+__global__ void __launch_bounds__(kThreads) k_dot_rz(const float2* __restrict__ r,
+                                                     const float* __restrict__ b,
+                                                     const float* __restrict__ x, int n,
+                                                     double* partials, unsigned int* counter,
+                                                     SumOut out) {
+  pdl_wait();
+  pdl_trigger();
+  float2 rv[4 * kSumVB];
+  float xv[4 * kSumVB];
+  double t;
+  if (ordered_sum<4>(
+          n, blockIdx.x, partials, counter, t,
+          [&](int q, int idx) {
+            rv[q] = r ? r[idx] : make_float2(b[idx], 0.f);
+            xv[q] = x[idx];
+          },
+          [&](int q) { return df_mulf(df{rv[q].x, rv[q].y}, xv[q]); }) &&
+      threadIdx.x == 0)
+    sum_out(out, t);
 }
 
 template <typename Real>
@@ -151,14 +160,14 @@ __global__ void __launch_bounds__(l2d::kDownThreads) k_coarse_down2d(l2d::Coarse
   l2d::coarse_down<Real>(s, f, blockIdx.x, blockIdx.y, b, x, bc, dinvc, xc);
 }
 
-template <typename Real>
+template <typename Real, bool AXES>
 __global__ void __launch_bounds__(l2d::kUpThreads) k_coarse_up2d(l2d::Coarse<Real> f,
                                                                  const Real* __restrict__ b,
                                                                  const Real* __restrict__ x,
                                                                  const Real* __restrict__ res,
                                                                  Real* __restrict__ xout) {
   __shared__ l2d::CoarseUpSmem<Real> s;
-  l2d::coarse_up<Real>(s, f, blockIdx.x, blockIdx.y, b, x, res, xout);
+  l2d::coarse_up<Real, AXES>(s, f, blockIdx.x, blockIdx.y, b, x, res, xout);
 }
 
 template <typename Real, int DIM>
@@ -590,7 +599,7 @@ static void coarse_solve(Ctx& c) {
 // (r = b, or rdot's pairs when given).
 template <typename Real>
 static void vcycle_fused2(Ctx& c, const Real* b0, Real* x0, bool zero_guess,
-                          const float2* rdot = nullptr, double* dout = nullptr) {
+                          const float2* rdot = nullptr, SumOut dout = {}) {
   LevelBuf<Real>* h = levels<Real>(c);
   const int nl = c.nl;
   const Real om = (Real)c.p.omega;
@@ -621,17 +630,26 @@ static void vcycle_fused2(Ctx& c, const Real* b0, Real* x0, bool zero_guess,
   const Real* res = h[nl - 1].x;
   for (int l = nl - 2; l >= 1; --l) {
     const dim3 grid(l2d::tiles(c.L[l].NX, l2d::kPX), l2d::tiles(c.L[l].NY, l2d::kPY));
-    launch_pdl(c.stream, c.use_pdl, k_coarse_up2d<Real>, grid, dim3(l2d::kUpThreads), coarse(l),
-               (const Real*)h[l].b, (const Real*)h[l].x, res, h[l].t);
+    // (large levels: the additions' order of the interpolation as a pass of its own)
+    launch_pdl(c.stream, c.use_pdl,
+               c.L[l].n > c.split_coarse_nodes ? k_coarse_up2d<Real, false> : k_coarse_up2d<Real, true>,
+               grid, dim3(l2d::kUpThreads), coarse(l), (const Real*)h[l].b, (const Real*)h[l].x, res,
+               h[l].t);
     MGAR_LAUNCH_CHECK_AT(level_site(4, l));
     res = h[l].t;
   }
   ProfScope ps(c, MGAR_KC_SMOOTH0);
   const dim3 grid(l2d::tiles(d0.NX, l2d::kUX), l2d::tiles(d0.NY, l2d::kUY));
-  launch_pdl(c.stream, c.use_pdl, dout ? k_up2d<Real, true> : k_up2d<Real, false>, grid,
-             dim3(l2d::kThreads2), f, b0, (const Real*)h[0].t, res, x0, rdot, c.partials, c.counter,
-             dout);
+  const bool fused = sizeof(Real) == 8 && dout.out;
+  launch_pdl(c.stream, c.use_pdl, fused ? k_up2d<Real, true> : k_up2d<Real, false>, grid,
+             dim3(l2d::kThreads2), f, b0, (const Real*)h[0].t, res, x0, c.partials, c.counter, dout);
   MGAR_LAUNCH_CHECK_AT(level_site(1, 0));
+  if constexpr (sizeof(Real) == 4) {
+    if (dout.out) {
+      launch_pdl(c.stream, c.use_pdl, k_dot_rz, dim3(sum_phys(d0.n, 4)), dim3(kThreads), rdot, b0, (const float*)x0, (int)d0.n, c.partials, c.counter, dout);
+      MGAR_LAUNCH_CHECK();
+    }
+  }
 }
 
 // Table 1 with one pre- and one post-sweep and a zero guess below the finest
@@ -639,7 +657,7 @@ static void vcycle_fused2(Ctx& c, const Real* b0, Real* x0, bool zero_guess,
 // restriction, and one fused post kernel (interpolation + smooth); the small
 // levels at the bottom run in one cluster launch.
 static void vcycle_fused3(Ctx& c, const float* b0, float* x0, bool zero_guess,
-                         const float2* rdot = nullptr, double* dout = nullptr) {
+                         const float2* rdot = nullptr, SumOut dout = {}) {
   using Real = float;
   constexpr int DIM = 3;
   LevelBuf<Real>* h = levels<Real>(c);
@@ -798,48 +816,48 @@ void vcycle(Ctx& c, const Real* b, Real* x, bool zero_guess) {
 template void vcycle<double>(Ctx&, const double*, double*, bool);
 template void vcycle<float>(Ctx&, const float*, float*, bool);
 
-void vcycle_dot(Ctx& c, const float* b, float* x, const float2* r, double* dout) {
+void vcycle_dot(Ctx& c, const float* b, float* x, const float2* r, SumOut dout) {
   require(vcycle_dot_ok(c), MGAR_ERR_ARG,
           "fused r.z V-cycle needs one pre- and one post-sweep, two levels and the tiled 3D kernels");
   if (c.dim == 2) vcycle_fused2<float>(c, b, x, true, r, dout);
   else vcycle_fused3(c, b, x, true, r, dout);
 }
 
-void vcycle_dot64(Ctx& c, const double* b, double* x, double* dout) {
+void vcycle_dot64(Ctx& c, const double* b, double* x, SumOut dout) {
   vcycle_fused2<double>(c, b, x, true, nullptr, dout);
 }
 
 template <typename Real, int DIM>
 static void apply_dim(Ctx& c, const Real* ke, const Real* ksub, const Real* x, Real* y, Real scale,
-                      double* dot_out) {
+                      SumOut dot_out) {
   const Dims& d = c.L[0];
   auto row = fine_row<Real, DIM>(c, ke, ksub);
-  if (dot_out)
+  if (dot_out.out)
     k_apply<FineRow<Real, DIM>, Real, true><<<blocks_for(d.n), kThreads, 0, c.stream>>>(
         row, x, y, scale, c.partials, c.counter, dot_out);
   else
     k_apply<FineRow<Real, DIM>, Real, false><<<blocks_for(d.n), kThreads, 0, c.stream>>>(
-        row, x, y, scale, nullptr, nullptr, nullptr);
+        row, x, y, scale, nullptr, nullptr, SumOut{});
   MGAR_LAUNCH_CHECK();
 }
 
-void apply_fine64(Ctx& c, const double* ke, const double* x, double* y, double* dot_out) {
+void apply_fine64(Ctx& c, const double* ke, const double* x, double* y, SumOut dot_out) {
   ProfScope ps(c, MGAR_KC_APPLY64);
   if (c.dim == 2) apply_dim<double, 2>(c, ke, nullptr, x, y, 1.0, dot_out);
   else apply_dim<double, 3>(c, ke, nullptr, x, y, 1.0, dot_out);
 }
 void apply_fine32(Ctx& c, const float* ke, const float* x, float* y) {
-  if (c.dim == 2) apply_dim<float, 2>(c, ke, nullptr, x, y, 1.f, nullptr);
-  else apply_dim<float, 3>(c, ke, nullptr, x, y, 1.f, nullptr);
+  if (c.dim == 2) apply_dim<float, 2>(c, ke, nullptr, x, y, 1.f, {});
+  else apply_dim<float, 3>(c, ke, nullptr, x, y, 1.f, {});
 }
 // y = -(A - A0) x
 void apply_dK64(Ctx& c, const double* x, double* y) {
-  if (c.dim == 2) apply_dim<double, 2>(c, c.ke, c.ke0, x, y, -1.0, nullptr);
-  else apply_dim<double, 3>(c, c.ke, c.ke0, x, y, -1.0, nullptr);
+  if (c.dim == 2) apply_dim<double, 2>(c, c.ke, c.ke0, x, y, -1.0, {});
+  else apply_dim<double, 3>(c, c.ke, c.ke0, x, y, -1.0, {});
 }
 void apply_dK32(Ctx& c, const float* x, float* y) {
-  if (c.dim == 2) apply_dim<float, 2>(c, c.ke_f, c.ke0_f, x, y, -1.f, nullptr);
-  else apply_dim<float, 3>(c, c.ke_f, c.ke0_f, x, y, -1.f, nullptr);
+  if (c.dim == 2) apply_dim<float, 2>(c, c.ke_f, c.ke0_f, x, y, -1.f, {});
+  else apply_dim<float, 3>(c, c.ke_f, c.ke0_f, x, y, -1.f, {});
 }
 
 void convert_d2f(Ctx& c, const double* a, float* b, int64_t n) {
