@@ -124,6 +124,7 @@ void free_ctx(Ctx& c) {
     delete[] c.prof_sites;
     c.prof_sites = nullptr;
   }
+  cudaFree(c.f_cls);
   cudaFree(c.pp_taps);
   cudaFree(c.pp_ctrl);
   cudaFree(c.run_rho);

@@ -171,6 +171,7 @@ struct Ctx {
   float2* dv_df = nullptr;  // dv, double-float
   int n_filter = 0;
   double filter_r = 0.0;    // radius of the current tables
+  void* f_cls = nullptr;    // mixed 3D: its classes of equal weight (filter3d.cu)
   int filter_cap = 0;       // offsets the tables have room for
   int4* f_offs_h = nullptr; // pinned staging of the tables (continuous filter)
   double* f_w_h = nullptr;

@@ -5,6 +5,7 @@
 
 #include "common.cuh"
 #include "df64.cuh"
+#include "filter3d.cuh"
 
 #include <vector>
 
@@ -90,17 +91,11 @@ __device__ __forceinline__ df filter_sum_df(const float2* __restrict__ in, const
   return df_make(ah, al);
 }
 
-// Forward filter (Eq. 6) fused with the SIMP conductivities (Eq. 4):
-// rho~_e = inv_hs_e sum_o w_o rho_{e+o}, k_e = kmin + (k0 - kmin) rho~^3,
-// written as FP64 (rho~, k_e), FP32 and df64 copies of k_e.
-// The constants come as double-float pairs (kmin_df, dk_df = k0 - kmin) and
-// 1/Hs as pairs, so no thread converts from FP64 (1/58 of the FP32 rate).
-__global__ void k_filter_simp_df(const float2* __restrict__ rho, const float2* __restrict__ inv_hs,
-                                 const int4* __restrict__ offs, const double* __restrict__ w, int noff,
-                                 Dims d, int reach, int reach_z, double k0, double kmin, double penal,
-                                 float2 kmin_df, float2 dk_df, double* __restrict__ rho_phys,
-                                 float2* __restrict__ rho_df, double* __restrict__ ke,
-                                 float* __restrict__ kf, float2* __restrict__ kdf) {
+// Forward filter (Eq. 6) fused with the SIMP conductivities (Eq. 4), offset
+// by offset.
+__global__ void k_filter_simp_df(const float2* __restrict__ rho, const int4* __restrict__ offs,
+                                 const double* __restrict__ w, int noff, Dims d, int reach, int reach_z,
+                                 SimpArgs a) {
   // offsets staged as bytes: |d| <= 127 for any radius the tables allow
   __shared__ df ws[kMaxFilterOffsets];
   __shared__ char4 os[kMaxFilterOffsets];
@@ -117,20 +112,8 @@ __global__ void k_filter_simp_df(const float2* __restrict__ rho, const float2* _
   const int e = valid ? e0 : (int)d.ne - 1;
   int i, j, k;
   coords(e, d.fEX, d.fEXY, i, j, k);
-  const df r = df_mul(filter_sum_df(rho, ws, os, noff, e, i, j, k, d, reach, reach_z),
-                      dfk2(inv_hs[e]));
-  if (!valid) return;
-  rho_phys[e] = df_to_double(r);
-  rho_df[e] = make_float2(r.hi, r.lo);  // the pair k_e comes from (rho_phys: its FP64 rounding)
-  df kv;
-  if (penal == 3.0) {
-    kv = df_add(dfk2(kmin_df), df_mul(dfk2(dk_df), df_mul(df_mul(r, r), r)));
-  } else {
-    kv = df_from_double(kmin + (k0 - kmin) * pow(df_to_double(r), penal));
-  }
-  ke[e] = df_to_double(kv);
-  kf[e] = __fadd_rn(kv.hi, kv.lo);
-  kdf[e] = make_float2(kv.hi, kv.lo);
+  const df s = filter_sum_df(rho, ws, os, noff, e, i, j, k, d, reach, reach_z);
+  if (valid) simp_store(a, e, s);
 }
 
 // Element sensitivity (Eq. 10) times inv_hs, as the transpose filter's input:
@@ -747,6 +730,7 @@ __global__ void k_filter_expand(Dims d, FilterClasses f, const double* __restric
 // update fills anew (a class grid has no more cells than the grid elements).
 static void filter_derived(Ctx& c) {
   const Dims& d = c.L[0];
+  filter3d_classes(c);
   FilterClasses f;
   f.edge = 2 * filter_reach(c);
   const int n[3] = {d.ex, d.ey, c.dim == 3 ? d.ez : 1};
@@ -841,12 +825,17 @@ void set_density(Ctx& c, const double* rho, bool physical) {
     k_to_df<<<blocks_for(c.ne), kThreads, 0, c.stream>>>(rho, c.df_e, (int)c.ne);
     MGAR_LAUNCH_CHECK();
     const df kmin_df = df_from_double(c.p.kmin), dk_df = df_from_double(c.p.k0 - c.p.kmin);
-    k_filter_simp_df<<<blocks_for(c.ne), kThreads, 0, c.stream>>>(
-        c.df_e, c.inv_hs_df, c.f_offs, c.f_w, c.n_filter, c.L[0], filter_reach(c),
-        c.dim == 3 ? filter_reach(c) : 0, c.p.k0, c.p.kmin, c.p.penal,
-        make_float2(kmin_df.hi, kmin_df.lo), make_float2(dk_df.hi, dk_df.lo), c.rho_phys,
-        c.rho_phys_df, c.ke, c.ke_f, c.ke_df);
-    MGAR_LAUNCH_CHECK();
+    const SimpArgs a{c.inv_hs_df, c.p.k0, c.p.kmin, c.p.penal, make_float2(kmin_df.hi, kmin_df.lo),
+                     make_float2(dk_df.hi, dk_df.lo), c.rho_phys, c.rho_phys_df, c.ke, c.ke_f,
+                     c.ke_df};
+    if (filter3d_ok(c)) {
+      filter3d_simp(c, c.df_e, a);
+    } else {
+      k_filter_simp_df<<<blocks_for(c.ne), kThreads, 0, c.stream>>>(
+          c.df_e, c.f_offs, c.f_w, c.n_filter, c.L[0], filter_reach(c),
+          c.dim == 3 ? filter_reach(c) : 0, a);
+      MGAR_LAUNCH_CHECK();
+    }
     if (c.dim == 3) df3d_node_diag(c);
     return;
   }
@@ -890,10 +879,14 @@ void sensitivity(Ctx& c, const double* T, double* dc, double* dv, double* compli
                                                                 c.inv_hs_df, c.df_e, d, mcoef_df,
                                                                 c.p.penal);
     MGAR_LAUNCH_CHECK();
-    k_filter_t_df<<<blocks_for(c.ne), kThreads, 0, c.stream>>>(
-        c.df_e, c.f_offs, c.f_w, c.n_filter, d, filter_reach(c), c.dim == 3 ? filter_reach(c) : 0,
-        dc_df ? nullptr : dc, dc_df);
-    MGAR_LAUNCH_CHECK();
+    if (filter3d_ok(c)) {
+      filter3d_t(c, c.df_e, dc_df ? nullptr : dc, dc_df);
+    } else {
+      k_filter_t_df<<<blocks_for(c.ne), kThreads, 0, c.stream>>>(
+          c.df_e, c.f_offs, c.f_w, c.n_filter, d, filter_reach(c), c.dim == 3 ? filter_reach(c) : 0,
+          dc_df ? nullptr : dc, dc_df);
+      MGAR_LAUNCH_CHECK();
+    }
   } else if (dc) {
     ProfScope ps(c, MGAR_KC_SENS);
     if (c.dim == 2)
