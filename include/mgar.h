@@ -276,9 +276,9 @@ int64_t mgar_kernel_launches(void);
  * and operation), the outer CG runs in double-float arithmetic (FP64
  * accuracy on the FP32 pipe; FP64 scalars) around the FP32 V-cycle, and
  * the solve after the hierarchy builds is one CUDA graph that iterates while
- * any design is unconverged.  The V-cycle kernels' block sizes come from an
+ * any design is unconverged.  The coarsest solve's block size comes from an
  * autotuner at the first solve (mgar_batch_report lists its timings and
- * choices); no choice changes a result, and each design's result does not
+ * choice); no choice changes a result, and each design's result does not
  * depend on the other designs in the batch. */
 typedef struct mgar_batch_ctx* mgar_batch_t;
 

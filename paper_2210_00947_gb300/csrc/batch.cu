@@ -4,11 +4,11 @@
 // Every handle keeps its own data (conductivities, hierarchy, vectors); the
 // batch only holds device tables of their pointers and sizes.  Each step of
 // the solve is one launch over all designs: block b of a launch belongs to
-// design bdes[b], and its nodes are (b - b0[design]) * blockDim + thread of
-// that design's level.  So one launch per V-cycle level and operation serves
-// every design, and the designs' different depths only decide which of them
-// take part in a level (a design's coarsest level is solved by one launch
-// over all designs' coarsest levels).  The outer CG runs in double-float
+// design bdes[b] and takes tile (or block of nodes) b - b0[design] of that
+// design's level.  So one launch per V-cycle level and direction serves every
+// design (the tiled passes of level2d.cuh), and the designs' different depths
+// only decide which of them take part in a level (a design's coarsest level is
+// solved by one launch over all designs' coarsest levels).  The outer CG runs in double-float
 // (df64) arithmetic on the FP32 pipe around the FP32 V-cycle (FP32
 // preconditioner, FP64-accurate refinement: GB300 runs FP64 at 1/58 of the
 // FP32 rate), with FP64 scalars; its per-design scalars
@@ -20,10 +20,13 @@
 // Reductions are per design in a fixed order (each design's blocks write
 // partials, the design's last block adds them in block order), and the
 // reduction kernels use a fixed block size, so a design's result does not
-// depend on the other designs in the batch.  The node kernels of the
-// V-cycle (no reductions) take their block size per level from an
-// autotuner run at the first solve, which times the candidates on the
-// batch's own levels and keeps the fastest.
+// depend on the other designs in the batch.
+//
+// 64 uneven designs, 4.94 M nodes: an iteration was 13 + 3 launches per coarse
+// level with a gathering kernel per pass (93 us the product, 83 the finest
+// post-sweep with r . z, 59 the update, 54 the finest residual); the tiles, the
+// product fused with the direction update and programmatic dependent launches
+// halve it, with bit-identical results.
 #include "common.cuh"
 #include "dfop.cuh"
 #include "levelops.cuh"
@@ -37,24 +40,23 @@ namespace mgar {
 namespace bat {
 
 constexpr int kRedThreads = 256;  // block size of every reducing kernel
-constexpr int kBS = 16;           // device scalars per design
+constexpr int kBS = 18;           // device scalars per design
 enum : int { BS_RZ = 0, BS_PAP = 2, BS_RR = 3, BS_IT = 4, BS_ACT = 5, BS_QN = 6, BS_EPS = 7,
              BS_CGMAX = 8, BS_BAD = 9,
              // gathered from each handle after the solve / the design cycle
-             BS_COMPL = 10, BS_LAM = 11, BS_CHANGE = 12, BS_FAIL = 13, BS_DERR = 14 };
+             BS_COMPL = 10, BS_LAM = 11, BS_CHANGE = 12, BS_FAIL = 13, BS_DERR = 14,
+             // CG quotients as df64 pairs
+             BS_ALPHA = 15, BS_BETA = 16 };
 
 // One design at one level of the V-cycle.
 struct Lev {
-  FineOp<float> f0;      // level 0: FP32 reference conductivities (matrix-free)
-  StencilOp<float> op;   // levels >= 1: assembled stencil and 1/diag
-  Dims d, dn;            // this level and the next coarser one
-  const float* dinv;     // this level's 1/diag
+  l2d::Fine<float> f0;   // level 0: FP32 reference conductivities (matrix-free)
+  l2d::Coarse<float> c;  // levels >= 1: assembled stencil and 1/diag
+  int NX, NY;            // node dims of this level
   const float* dinv_n;   // the next level's 1/diag
-  float *x, *b, *t, *r;  // level 0: x = V-cycle result, b = its input
+  float *x, *b, *t;      // level 0: x = V-cycle result, b = its input
   float *bn, *xn;        // the next level's b, and its x (null when it is the coarsest)
   const float* resn;     // the next level's result (x at the coarsest, t above)
-  const uint8_t* fixed;  // level 0: Dirichlet mask
-  float omega;
 };
 
 struct Coarse {
@@ -67,7 +69,7 @@ struct Coarse {
 struct Des {
   DfOp f;              // current conductivities (df64 pairs, matrix-free difference form)
   const float2* q;     // the load as df64 pairs
-  float2 *x, *r, *p, *Ap;  // CG vectors as df64 pairs (the handle's own buffers)
+  float2 *x, *r, *p, *p2, *Ap;  // CG vectors as df64 pairs (the handle's own buffers)
   double* T;           // the caller's solution (FP64): warm start in, solution out
   float *b32, *x32;    // FP32 input and output of the V-cycle at level 0
   const double* dsc;   // the handle's device scalars (compliance, OC outcome)
@@ -84,12 +86,17 @@ struct Shape {
 
 __device__ __forceinline__ bool active(const double* bsc, int d) { return bsc[d * kBS + BS_ACT] != 0.0; }
 
-// Nodes per thread of the level-0 launches: a thread takes nodes base,
-// base + blockDim.x, ... of its design, so each block's lookups (its design,
-// the design's tables and scalars) serve several nodes and each thread has
-// several independent loads in flight.
-constexpr int kNpt0 = 4;  // V-cycle node kernels at level 0
-constexpr int kNptR = 2;  // CG kernels (double-float vectors, reductions)
+// Nodes per thread of the CG's node kernels: a thread takes nodes base, base +
+// blockDim.x, ... of its design, so each block's lookups serve several nodes
+// and each thread has several independent loads in flight.
+constexpr int kNptR = 2;
+
+// The tile of this block in its design's launch, ntx tiles per row.
+__device__ __forceinline__ void tile_of(const int* b0, int d, int ntx, int& tx, int& ty) {
+  const int l = blockIdx.x - b0[d];
+  ty = l / ntx;
+  tx = l - ty * ntx;
+}
 
 // The first node of this thread in its design, for npt nodes per thread.
 __device__ __forceinline__ int node_base(const int* b0, int d, int npt) {
@@ -204,69 +211,128 @@ __global__ void kb_start(double* bsc, int nd) {
   s[BS_ACT] = (isfinite(rel) && rel > s[BS_EPS] && s[BS_CGMAX] > 0.0) ? 1.0 : 0.0;
 }
 
-// Ap = A p and p . Ap.
-__global__ void kb_apply_dot(const Des* D, const int* bdes, const int* b0, double* bsc,
-                             double* partials, unsigned int* counters) {
+// The direction buffers: iteration it reads one and writes the other.
+__device__ __forceinline__ float2* p_new(const Des& g, int it) { return (it & 1) ? g.p : g.p2; }
+__device__ __forceinline__ float2* p_old(const Des& g, int it) { return (it & 1) ? g.p2 : g.p; }
+
+// p = z + beta p_old (p = z in the first iteration), z the FP32 V-cycle
+// output, and Ap = A p.
+__global__ void __launch_bounds__(l2d::kThreads2) kb_dir(const Des* D, const int* bdes, const int* b0,
+                                                         const double* bsc) {
+  __shared__ DfDirSmem s;
+  pdl_wait();
+  pdl_trigger();
   const int d = bdes[blockIdx.x];
   if (!active(bsc, d)) return;
   const Des& g = D[d];
-  const int base = node_base(b0, d, kNptR);
-  df v{0.f, 0.f};
-#pragma unroll
-  for (int u = 0; u < kNptR; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < g.f.n) {
-      const df ap = df_row<2>(g.f, g.p, idx);
-      g.Ap[idx] = pack(ap);
-      v = df_add(v, df_mul(unpack(g.p[idx]), ap));
-    }
-  }
-  seg_finish_df(v, partials, counters, d, b0[d], design_blocks(g.f.n, kNptR),
-                bsc + d * kBS + BS_PAP);
+  const int it = (int)bsc[d * kBS + BS_IT];
+  int tx, ty;
+  tile_of(b0, d, l2d::tiles(g.f.NX, l2d::kUX), tx, ty);
+  const df beta = it == 0 ? df{0.f, 0.f} : load_pair(bsc + d * kBS + BS_BETA);
+  df_dir_tile(s, g.f, tx, ty, g.x32, p_old(g, it), it == 0, beta, p_new(g, it), g.Ap);
 }
 
-// alpha = r.z / p.Ap; x += alpha p; r -= alpha Ap; ||r||^2; FP32 copy of r.
-__global__ void kb_cg_xr(const Des* D, const int* bdes, const int* b0, double* bsc,
-                         double* partials, unsigned int* counters) {
+// The sums of a design run over its nodes in memory order, four virtual
+// blocks of 512 nodes per block (ordered_sum); red_b0: the design's first
+// virtual block.
+// p . Ap and alpha = r . z / p . Ap
+__global__ void __launch_bounds__(kRedThreads) kb_dot_py(const Des* D, const int* bdes, const int* b0,
+                                                         const int* red_b0, double* bsc,
+                                                         double* partials, unsigned int* counters) {
+  pdl_wait();
+  pdl_trigger();
   const int d = bdes[blockIdx.x];
   if (!active(bsc, d)) return;
   const Des& g = D[d];
-  const double* s = bsc + d * kBS;
-  const int par = ((int)s[BS_IT]) & 1;
-  const df alpha = block_div_df(s + BS_RZ + par, s + BS_PAP);
-  const int base = node_base(b0, d, kNptR);
-  // every node's four loads first, then the updates
-  float2 xv[kNptR], pv[kNptR], rv[kNptR], qv[kNptR];
-#pragma unroll
-  for (int u = 0; u < kNptR; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < g.f.n) {
-      xv[u] = g.x[idx];
-      pv[u] = g.p[idx];
-      rv[u] = g.r[idx];
-      qv[u] = g.Ap[idx];
+  double* s = bsc + d * kBS;
+  const int it = (int)s[BS_IT];
+  const float2* __restrict__ p = p_new(g, it);
+  const float2* __restrict__ y = g.Ap;
+  float2 pv[kNptR * kSumVB], yv[kNptR * kSumVB];
+  double t;
+  if (ordered_sum<kNptR>(
+          g.f.n, blockIdx.x - b0[d], partials + red_b0[d], counters + d, t,
+          [&](int q, int idx) {
+            pv[q] = p[idx];
+            yv[q] = y[idx];
+          },
+          [&](int q) { return df_mul(unpack(pv[q]), unpack(yv[q])); }) &&
+      threadIdx.x == 0)
+    sum_out(SumOut{s + BS_PAP, s + BS_RZ + (it & 1), nullptr, s + BS_ALPHA, 1}, t);
+}
+
+// r . z and beta = r . z / (r . z)_old
+__global__ void __launch_bounds__(kRedThreads) kb_dot_rz(const Des* D, const int* bdes, const int* b0,
+                                                         const int* red_b0, double* bsc,
+                                                         double* partials, unsigned int* counters) {
+  pdl_wait();
+  pdl_trigger();
+  const int d = bdes[blockIdx.x];
+  if (!active(bsc, d)) return;
+  const Des& g = D[d];
+  double* s = bsc + d * kBS;
+  const int it = (int)s[BS_IT];
+  float2 rv[kNptR * kSumVB];
+  float zv[kNptR * kSumVB];
+  double t;
+  if (ordered_sum<kNptR>(
+          g.f.n, blockIdx.x - b0[d], partials + red_b0[d], counters + d, t,
+          [&](int q, int idx) {
+            rv[q] = g.r[idx];
+            zv[q] = g.x32[idx];
+          },
+          [&](int q) { return df_mulf(unpack(rv[q]), zv[q]); }) &&
+      threadIdx.x == 0) {
+    SumOut out{s + BS_RZ + (it & 1)};
+    if (it > 0) {
+      out.den = s + BS_RZ + ((it - 1) & 1);
+      out.q = s + BS_BETA;
+      out.pair = 1;
     }
+    sum_out(out, t);
   }
-  df v{0.f, 0.f};
-#pragma unroll
-  for (int u = 0; u < kNptR; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < g.f.n) {
-      g.x[idx] = pack(df_add(unpack(xv[u]), df_mul(alpha, unpack(pv[u]))));
-      const df ri = df_sub(unpack(rv[u]), df_mul(alpha, unpack(qv[u])));
-      g.r[idx] = pack(ri);
-      g.b32[idx] = __fadd_rn(ri.hi, ri.lo);
-      v = df_add(v, df_mul(ri, ri));
-    }
-  }
-  seg_finish_df(v, partials, counters, d, b0[d], design_blocks(g.f.n, kNptR),
-                bsc + d * kBS + BS_RR);
+}
+
+// x += alpha p; r -= alpha Ap; ||r||^2; FP32 copy of r.
+__global__ void __launch_bounds__(kRedThreads) kb_cg_xr(const Des* D, const int* bdes, const int* b0,
+                                                        const int* red_b0, double* bsc,
+                                                        double* partials, unsigned int* counters) {
+  pdl_wait();
+  pdl_trigger();
+  const int d = bdes[blockIdx.x];
+  if (!active(bsc, d)) return;
+  const Des& g = D[d];
+  double* s = bsc + d * kBS;
+  const float2* __restrict__ p = p_new(g, (int)s[BS_IT]);
+  const df alpha = load_pair(s + BS_ALPHA);
+  float2 xv[kNptR * kSumVB], pv[kNptR * kSumVB], rv[kNptR * kSumVB], qv[kNptR * kSumVB];
+  int at[kNptR * kSumVB];
+  double t;
+  if (ordered_sum<kNptR>(
+          g.f.n, blockIdx.x - b0[d], partials + red_b0[d], counters + d, t,
+          [&](int q, int idx) {
+            at[q] = idx;
+            xv[q] = g.x[idx];
+            pv[q] = p[idx];
+            rv[q] = g.r[idx];
+            qv[q] = g.Ap[idx];
+          },
+          [&](int q) {
+            g.x[at[q]] = pack(df_add(unpack(xv[q]), df_mul(alpha, unpack(pv[q]))));
+            const df ri = df_sub(unpack(rv[q]), df_mul(alpha, unpack(qv[q])));
+            g.r[at[q]] = pack(ri);
+            g.b32[at[q]] = __fadd_rn(ri.hi, ri.lo);
+            return df_mul(ri, ri);
+          }) &&
+      threadIdx.x == 0)
+    s[BS_RR] = t;
 }
 
 // One iteration done: count it and decide, per design, whether to go on;
 // the WHILE node repeats while any design is active.
 __global__ void kb_check(double* bsc, int nd, cudaGraphConditionalHandle loop, int* any_out) {
   __shared__ int any;
+  pdl_wait();
   if (threadIdx.x == 0) any = 0;
   __syncthreads();
   for (int d = threadIdx.x; d < nd; d += blockDim.x) {
@@ -287,107 +353,39 @@ __global__ void kb_check(double* bsc, int nd, cudaGraphConditionalHandle loop, i
   }
 }
 
-// p = z + (r.z_new / r.z_old) p (p = z in the first iteration), z the FP32
-// V-cycle output.
-__global__ void kb_cg_p(const Des* D, const int* bdes, const int* b0, const double* bsc) {
-  const int d = bdes[blockIdx.x];
-  if (!active(bsc, d)) return;
-  const Des& g = D[d];
-  const double* s = bsc + d * kBS;
-  const int it = (int)s[BS_IT];
-  const df beta = it == 0 ? df{0.f, 0.f}
-                          : block_div_df(s + BS_RZ + (it & 1), s + BS_RZ + ((it - 1) & 1));
-  const int base = node_base(b0, d, kNptR);
-  float zv[kNptR];
-  float2 pv[kNptR];
-#pragma unroll
-  for (int u = 0; u < kNptR; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < g.f.n) {
-      zv[u] = g.x32[idx];
-      pv[u] = g.p[idx];
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < kNptR; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < g.f.n) {
-      const df z{zv[u], 0.f};
-      g.p[idx] = pack(it == 0 ? z : df_add(z, df_mul(beta, unpack(pv[u]))));
-    }
-  }
-}
-
 // --------------------------------------------------------- V-cycle kernels
-// The design and node of a thread of a level launch (false: nothing to do).
-__device__ __forceinline__ bool lev_node(const int* bdes, const int* b0, const double* bsc, int& d,
-                                         int& idx) {
-  d = bdes[blockIdx.x];
-  if (!active(bsc, d)) return false;
-  idx = (blockIdx.x - b0[d]) * blockDim.x + threadIdx.x;
-  return true;
-}
-
-// level 0, zero initial guess: t = w D^-1 b
-__global__ void kb_jz0(const Lev* L, const int* bdes, const int* b0, const double* bsc) {
+// The tiled passes of level2d.cuh, each one launch over all active designs.
+// level 0, down: t = w D^-1 b, b_1 = P^T (b - A t), x_1 = w D_1^-1 b_1 (x_1
+// unless level 1 is the coarsest)
+__global__ void __launch_bounds__(l2d::kThreads2) kb_down0(const Lev* L, const int* bdes,
+                                                           const int* b0, const double* bsc) {
+  __shared__ l2d::DownSmem<float> s;
+  pdl_wait();
   const int d = bdes[blockIdx.x];
   if (!active(bsc, d)) return;
   const Lev& v = L[d];
-  const int base = node_base(b0, d, kNpt0);
-  float dv[kNpt0], bv[kNpt0];
-#pragma unroll
-  for (int u = 0; u < kNpt0; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < v.d.n) {
-      dv[u] = v.dinv[idx];
-      bv[u] = v.b[idx];
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < kNpt0; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < v.d.n) v.t[idx] = v.omega * dv[u] * bv[u];
-  }
+  int tx, ty;
+  tile_of(b0, d, l2d::tiles(v.f0.cNX, l2d::kCX), tx, ty);
+  l2d::fine_down<float, true>(s, v.f0, tx, ty, v.b, v.t, v.bn, v.dinv_n, v.xn);
 }
 
-// level 0: r = b - A t (matrix-free FP32 operator)
-__global__ void kb_resid0(const Lev* L, const int* bdes, const int* b0, const double* bsc) {
+// levels >= 1 above the coarsest, down
+__global__ void __launch_bounds__(l2d::kDownThreads) kb_down(const Lev* L, const int* bdes,
+                                                             const int* b0, const double* bsc) {
+  __shared__ float s[2 * l2d::kDY + 1][32];
+  pdl_wait();
   const int d = bdes[blockIdx.x];
   if (!active(bsc, d)) return;
   const Lev& v = L[d];
-  const int base = node_base(b0, d, kNpt0);
-#pragma unroll
-  for (int u = 0; u < kNpt0; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < v.d.n) {
-      int i, j, k;
-      coords(idx, v.f0.fNX, v.f0.fNXY, i, j, k);
-      float diag;
-      v.r[idx] = v.b[idx] - fine_row2(v.f0, v.t, i, j, diag);
-    }
-  }
-}
-
-// b_next = P^T r (fixed fine nodes excluded at level 0), and the next level's
-// zero-guess sweep x_next = w D^-1 b_next unless it is the coarsest
-__global__ void kb_restrict(const Lev* L, const int* bdes, const int* b0, const double* bsc) {
-  int d, idx;
-  if (!lev_node(bdes, b0, bsc, d, idx)) return;
-  const Lev& v = L[d];
-  if (idx < v.dn.n)
-    restrict_node<float, 2, false>(v.r, v.bn, v.d, v.dn, v.fixed, idx, v.dinv_n, v.omega, v.xn);
-}
-
-// levels >= 1 above the coarsest: r = b - A x (x left by the restriction)
-__global__ void kb_resid(const Lev* L, const int* bdes, const int* b0, const double* bsc) {
-  int d, idx;
-  if (!lev_node(bdes, b0, bsc, d, idx)) return;
-  const Lev& v = L[d];
-  if (idx < v.d.n) resid_node<float, 2, false>(v.op, v.b, v.x, v.r, idx);
+  int tx, ty;
+  tile_of(b0, d, l2d::tiles(v.c.cNX, l2d::kDX), tx, ty);
+  l2d::coarse_down<float>(s, v.c, tx, ty, v.b, v.x, v.bn, v.dinv_n, v.xn);
 }
 
 // each design's coarsest level: x = C b, one warp per row
 __global__ void kb_coarse(const Coarse* C, const int* bdes, const int* b0, const double* bsc) {
+  pdl_wait();
+  pdl_trigger();
   const int d = bdes[blockIdx.x];
   if (!active(bsc, d)) return;
   const Coarse& c = C[d];
@@ -396,54 +394,30 @@ __global__ void kb_coarse(const Coarse* C, const int* bdes, const int* b0, const
   if (row < c.nc) coarse_row<float, false, double>(c.cinv, c.b, c.x, c.nc, row, threadIdx.x & 31);
 }
 
-// levels >= 1 above the coarsest: t = post-smoothing of x + P res_next
-__global__ void kb_post(const Lev* L, const int* bdes, const int* b0, const double* bsc) {
-  int d, idx;
-  if (!lev_node(bdes, b0, bsc, d, idx)) return;
-  const Lev& v = L[d];
-  if (idx < v.d.n)
-    post_node<float, 2, false>(v.op, v.resn, v.x, v.b, v.dinv, v.omega, v.t, v.d, v.dn, idx);
-}
-
-// level 0: t += P res_1 (fixed nodes keep t)
-__global__ void kb_prolong0(const Lev* L, const int* bdes, const int* b0, const double* bsc) {
+// levels >= 1 above the coarsest, up: t = post-smoothing of x + P res_next
+__global__ void __launch_bounds__(l2d::kUpThreads) kb_up(const Lev* L, const int* bdes, const int* b0,
+                                                         const double* bsc) {
+  __shared__ l2d::CoarseUpSmem<float> s;
+  pdl_wait();
   const int d = bdes[blockIdx.x];
   if (!active(bsc, d)) return;
   const Lev& v = L[d];
-  const int base = node_base(b0, d, kNpt0);
-#pragma unroll
-  for (int u = 0; u < kNpt0; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < v.d.n) prolong_node<float, 2>(v.resn, v.t, v.t, v.d, v.dn, v.fixed, idx);
-  }
+  int tx, ty;
+  tile_of(b0, d, l2d::tiles(v.NX, l2d::kPX), tx, ty);
+  l2d::coarse_up<float, true>(s, v.c, tx, ty, v.b, v.x, v.resn, v.t);
 }
 
-// level 0: x = t + w D^-1 (b - A t), z = x in FP64 and r . z (the CG's new
-// r.z, slot by iteration parity)
-__global__ void kb_sweep0(const Lev* L, const Des* D, const int* bdes, const int* b0,
-                          double* bsc, double* partials, unsigned int* counters) {
+// level 0, up: x = v + w D^-1 (b - A v), v = t + P res_1
+__global__ void __launch_bounds__(l2d::kThreads2) kb_up0(const Lev* L, const int* bdes, const int* b0,
+                                                         const double* bsc) {
+  __shared__ l2d::UpSmem<float> s;
+  pdl_wait();
   const int d = bdes[blockIdx.x];
   if (!active(bsc, d)) return;
   const Lev& v = L[d];
-  const Des& g = D[d];
-  const int base = node_base(b0, d, kNptR);
-  df s{0.f, 0.f};
-#pragma unroll
-  for (int u = 0; u < kNptR; ++u) {
-    const int idx = base + u * blockDim.x;
-    if (idx < v.d.n) {
-      int i, j, k;
-      coords(idx, v.f0.fNX, v.f0.fNXY, i, j, k);
-      float diag;
-      const float ti = v.t[idx];
-      const float xo = ti + v.omega * v.dinv[idx] * (v.b[idx] - fine_row2(v.f0, v.t, i, j, diag));
-      v.x[idx] = xo;
-      s = df_add(s, df_mulf(unpack(g.r[idx]), xo));
-    }
-  }
-  const int par = ((int)bsc[d * kBS + BS_IT]) & 1;
-  seg_finish_df(s, partials, counters, d, b0[d], design_blocks(v.d.n, kNptR),
-                bsc + d * kBS + BS_RZ + par);
+  int tx, ty;
+  tile_of(b0, d, l2d::tiles(v.NX, l2d::kUX), tx, ty);
+  l2d::fine_up<float>(s, v.f0, tx, ty, v.b, v.t, v.resn, v.x, [](float, float) {});
 }
 
 // ------------------------------------------------------------------- host
@@ -462,11 +436,10 @@ struct Batch {
   double* hbsc = nullptr;      // pinned
   double* partials = nullptr;
   unsigned int* counters = nullptr;
-  Shape s_red;                 // level 0, reducing kernels
-  std::vector<int> tuned;      // threads per level (node kernels); [lmax] + coarse warps last
-  std::vector<Shape> shapes;   // all shapes made (freed at destroy)
-  // per level l: nodes of l (designs with a level below l), nodes of l + 1
-  std::vector<Shape> s_node, s_next;
+  Shape s_red, s_dot;          // level 0: virtual blocks of the sums, and the sums' blocks
+  // per level l (designs with a level below l): tiles of the way down (of the
+  // nodes of l + 1 at level 0) and up; s_up[0] is also the product's
+  std::vector<Shape> s_down, s_up;
   Shape s_coarse;
   cudaGraphExec_t exec = nullptr;
   int64_t prologue = 0, body = 0;
@@ -518,22 +491,20 @@ static Shape make_shape(const std::vector<int64_t>& units, int per_block, int th
   return s;
 }
 
-// Nodes of level l per design for the level's own kernels (designs for
-// which l is above the coarsest), or of level l + 1 (its restriction).
-static std::vector<int64_t> level_units(const Batch& b, int l, bool next) {
-  std::vector<int64_t> u(b.nd, 0);
+// The tiles of level l (designs for which l is above the coarsest).
+static void make_level_shapes(Batch& b, int l) {
+  std::vector<int64_t> down(b.nd, 0), up(b.nd, 0);
   for (int d = 0; d < b.nd; ++d) {
     const Ctx& c = *b.h[d];
-    if (l + 1 < c.nl) u[d] = next ? c.L[l + 1].n : c.L[l].n;
+    if (l + 1 >= c.nl) continue;
+    const Dims &f = c.L[l], &n = c.L[l + 1];
+    down[d] = l == 0 ? l2d::tiles(n.NX, l2d::kCX) * l2d::tiles(n.NY, l2d::kCY)
+                     : l2d::tiles(n.NX, l2d::kDX) * l2d::tiles(n.NY, l2d::kDY);
+    up[d] = l == 0 ? l2d::tiles(f.NX, l2d::kUX) * l2d::tiles(f.NY, l2d::kUY)
+                   : l2d::tiles(f.NX, l2d::kPX) * l2d::tiles(f.NY, l2d::kPY);
   }
-  return u;
-}
-
-static void make_level_shapes(Batch& b, int l, int threads) {
-  free_shape(b.s_node[l]);
-  free_shape(b.s_next[l]);
-  b.s_node[l] = make_shape(level_units(b, l, false), threads * (l == 0 ? kNpt0 : 1), threads);
-  b.s_next[l] = make_shape(level_units(b, l, true), threads, threads);
+  b.s_down[l] = make_shape(down, 1, l == 0 ? l2d::kThreads2 : l2d::kDownThreads);
+  b.s_up[l] = make_shape(up, 1, l == 0 ? l2d::kThreads2 : l2d::kUpThreads);
 }
 
 static void make_coarse_shape(Batch& b, int warps) {
@@ -543,35 +514,33 @@ static void make_coarse_shape(Batch& b, int warps) {
   b.s_coarse = make_shape(rows, warps, warps * 32);
 }
 
-template <typename K, typename... Args>
-static void launch_shape(Batch& b, const Shape& s, K kernel, Args... args) {
+template <typename... KArgs, typename... Args>
+static void launch_shape(Batch& b, const Shape& s, void (*kernel)(KArgs...), Args... args) {
   if (s.nblocks == 0) return;
-  kernel<<<s.nblocks, s.threads, 0, b.stream>>>(args..., s.bdes, s.b0, b.bsc);
+  launch_pdl(b.stream, true, kernel, dim3(s.nblocks), dim3(s.threads), args..., (const int*)s.bdes,
+             (const int*)s.b0, (const double*)b.bsc);
   MGAR_LAUNCH_CHECK();
 }
 
-// The FP32 V-cycle z = M r of every active design (Table 1, zero guess).
-static void vcycle(Batch& b) {
-  Lev* L0 = b.dlev;
-  // down
-  for (int l = 0; l + 1 < b.lmax; ++l) {
-    Lev* L = b.dlev + (size_t)l * b.nd;
-    if (l == 0) {
-      launch_shape(b, b.s_node[0], kb_jz0, (const Lev*)L);
-      launch_shape(b, b.s_node[0], kb_resid0, (const Lev*)L);
-    } else {
-      launch_shape(b, b.s_node[l], kb_resid, (const Lev*)L);
-    }
-    launch_shape(b, b.s_next[l], kb_restrict, (const Lev*)L);
-  }
-  launch_shape(b, b.s_coarse, kb_coarse, (const Coarse*)b.dco);
-  // up
-  for (int l = b.lmax - 2; l >= 1; --l)
-    launch_shape(b, b.s_node[l], kb_post, (const Lev*)(b.dlev + (size_t)l * b.nd));
-  launch_shape(b, b.s_node[0], kb_prolong0, (const Lev*)L0);
-  kb_sweep0<<<b.s_red.nblocks, kRedThreads, 0, b.stream>>>(L0, b.ddes, b.s_red.bdes, b.s_red.b0,
-                                                           b.bsc, b.partials, b.counters);
+// A sum over every active design's nodes.
+static void launch_sum(Batch& b, void (*kernel)(const Des*, const int*, const int*, const int*, double*,
+                                                double*, unsigned int*)) {
+  launch_pdl(b.stream, true, kernel, dim3(b.s_dot.nblocks), dim3(kRedThreads), (const Des*)b.ddes,
+             (const int*)b.s_dot.bdes, (const int*)b.s_dot.b0, (const int*)b.s_red.b0, b.bsc,
+             b.partials, b.counters);
   MGAR_LAUNCH_CHECK();
+}
+
+// The FP32 V-cycle z = M r of every active design (Table 1, zero guess) and
+// r . z.
+static void vcycle(Batch& b) {
+  auto lev = [&](int l) { return (const Lev*)(b.dlev + (size_t)l * b.nd); };
+  launch_shape(b, b.s_down[0], kb_down0, lev(0));
+  for (int l = 1; l + 1 < b.lmax; ++l) launch_shape(b, b.s_down[l], kb_down, lev(l));
+  launch_shape(b, b.s_coarse, kb_coarse, (const Coarse*)b.dco);
+  for (int l = b.lmax - 2; l >= 1; --l) launch_shape(b, b.s_up[l], kb_up, lev(l));
+  launch_shape(b, b.s_up[0], kb_up0, lev(0));
+  launch_sum(b, kb_dot_rz);
 }
 
 static void red_launch_resid(Batch& b) {
@@ -581,20 +550,15 @@ static void red_launch_resid(Batch& b) {
 }
 
 static void iteration(Batch& b, cudaGraphConditionalHandle loop, int* any_out = nullptr) {
-  kb_apply_dot<<<b.s_red.nblocks, kRedThreads, 0, b.stream>>>(b.ddes, b.s_red.bdes, b.s_red.b0,
-                                                              b.bsc, b.partials, b.counters);
-  MGAR_LAUNCH_CHECK();
-  kb_cg_xr<<<b.s_red.nblocks, kRedThreads, 0, b.stream>>>(b.ddes, b.s_red.bdes, b.s_red.b0, b.bsc,
-                                                          b.partials, b.counters);
-  MGAR_LAUNCH_CHECK();
-  kb_check<<<1, 256, 0, b.stream>>>(b.bsc, b.nd, loop, any_out);
+  launch_shape(b, b.s_up[0], kb_dir, (const Des*)b.ddes);
+  launch_sum(b, kb_dot_py);
+  launch_sum(b, kb_cg_xr);
+  launch_pdl(b.stream, true, kb_check, dim3(1), dim3(256), b.bsc, b.nd, loop, any_out);
   MGAR_LAUNCH_CHECK();
   vcycle(b);
-  kb_cg_p<<<b.s_red.nblocks, kRedThreads, 0, b.stream>>>(b.ddes, b.s_red.bdes, b.s_red.b0, b.bsc);
-  MGAR_LAUNCH_CHECK();
 }
 
-// Per-design scalars, initial residuals, first V-cycle and direction.
+// Per-design scalars, initial residuals, first V-cycle.
 static void prologue(Batch& b) {
   const int th = 128;
   kb_init<<<(b.nd + th - 1) / th, th, 0, b.stream>>>(b.bsc, b.consts, b.nd);
@@ -605,8 +569,6 @@ static void prologue(Batch& b) {
   kb_start<<<(b.nd + th - 1) / th, th, 0, b.stream>>>(b.bsc, b.nd);
   MGAR_LAUNCH_CHECK();
   vcycle(b);
-  kb_cg_p<<<b.s_red.nblocks, kRedThreads, 0, b.stream>>>(b.ddes, b.s_red.bdes, b.s_red.b0, b.bsc);
-  MGAR_LAUNCH_CHECK();
 }
 
 // After the loop: the solutions back to the callers' FP64 vectors.
@@ -630,7 +592,7 @@ static void solve_eager(Batch& b) {
 }
 
 // The solve after the hierarchy builds as one graph: scalars, initial
-// residuals, first V-cycle and direction, then WHILE(any active) iteration.
+// residuals, first V-cycle, then WHILE(any active) iteration.
 static void build_graph(Batch& b) {
   cudaGraph_t g = nullptr;
   cudaGraphConditionalHandle loop = 0;
@@ -714,46 +676,19 @@ static float time_best(Batch& b, int reps, F&& fn) {
   return best;
 }
 
-// Autotuner: per level, the block size of its node kernels from 64 / 128 /
-// 256 / 512 threads, and the warps per block of the coarsest solve from
-// 2 / 4 / 8, each timed on the batch's own levels (the kernels are
-// node-parallel without reductions, so the choice changes no result).  The
-// device scalars mark every design active while it runs.
+// Autotuner: the warps per block of the coarsest solve from 2 / 4 / 8, timed on
+// the batch's own coarsest levels (a row per warp either way, so the choice
+// changes no result); the other launches' tiles are fixed.  The device scalars
+// mark every design active while it runs.
 static void autotune(Batch& b) {
   std::vector<double> ones((size_t)b.nd * kBS, 0.0);
   for (int d = 0; d < b.nd; ++d) ones[(size_t)d * kBS + BS_ACT] = 1.0;
   MGAR_CUDA(cudaMemcpy(b.bsc, ones.data(), ones.size() * sizeof(double), cudaMemcpyHostToDevice));
-  const int cand[4] = {64, 128, 256, 512};
   char line[160];
-  b.report = "batched V-cycle autotuner (best of 5 timed runs per candidate)\n";
+  b.report = "batched V-cycle (coarsest solve: best of 5 timed runs per candidate)\n";
   for (int l = 0; l + 1 < b.lmax; ++l) {
-    Lev* L = b.dlev + (size_t)l * b.nd;
-    float best = 1e30f;
-    int pick = 256;
-    for (int th : cand) {
-      make_level_shapes(b, l, th);
-      const float ms = time_best(b, 5, [&] {
-        if (l == 0) {
-          launch_shape(b, b.s_node[0], kb_jz0, (const Lev*)L);
-          launch_shape(b, b.s_node[0], kb_resid0, (const Lev*)L);
-          launch_shape(b, b.s_next[0], kb_restrict, (const Lev*)L);
-          launch_shape(b, b.s_node[0], kb_prolong0, (const Lev*)L);
-        } else {
-          launch_shape(b, b.s_node[l], kb_resid, (const Lev*)L);
-          launch_shape(b, b.s_next[l], kb_restrict, (const Lev*)L);
-          launch_shape(b, b.s_node[l], kb_post, (const Lev*)L);
-        }
-      });
-      snprintf(line, sizeof(line), "  level %d: %3d threads %8.2f us\n", l, th, ms * 1e3f);
-      b.report += line;
-      if (ms < best) {
-        best = ms;
-        pick = th;
-      }
-    }
-    make_level_shapes(b, l, pick);
-    b.tuned[l] = pick;
-    snprintf(line, sizeof(line), "level %d: %d threads per block\n", l, pick);
+    snprintf(line, sizeof(line), "level %d: %d tiles down, %d up\n", l, b.s_down[l].nblocks,
+             b.s_up[l].nblocks);
     b.report += line;
   }
   const int wc[3] = {2, 4, 8};
@@ -770,7 +705,6 @@ static void autotune(Batch& b) {
     }
   }
   make_coarse_shape(b, pick);
-  b.tuned[b.lmax - 1] = pick;
   snprintf(line, sizeof(line), "coarsest solve: %d warps per block\n", pick);
   b.report += line;
 }
@@ -813,10 +747,11 @@ void free_batch(Batch& b) {
   for (cudaEvent_t e : b.ev_des) cudaEventDestroy(e);
   if (b.ev_solved) cudaEventDestroy(b.ev_solved);
   if (b.ev_start) cudaEventDestroy(b.ev_start);
-  for (auto& s : b.s_node) free_shape(s);
-  for (auto& s : b.s_next) free_shape(s);
+  for (auto& s : b.s_down) free_shape(s);
+  for (auto& s : b.s_up) free_shape(s);
   free_shape(b.s_coarse);
   free_shape(b.s_red);
+  free_shape(b.s_dot);
   cudaFree(b.dlev);
   cudaFree(b.dco);
   cudaFree(b.ddes);
@@ -1036,9 +971,8 @@ int mgar_batch_create(mgar_batch_t* out, const mgar_t* handles, int count, void*
       b->lmax = std::max(b->lmax, c->nl);
     }
     const int nd = b->nd, lmax = b->lmax;
-    b->s_node.resize(lmax);
-    b->s_next.resize(lmax);
-    b->tuned.assign(lmax, 256);
+    b->s_down.resize(lmax);
+    b->s_up.resize(lmax);
     MGAR_CUDA(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
     // tables
     std::vector<Lev> lev((size_t)lmax * nd);
@@ -1054,6 +988,7 @@ int mgar_batch_create(mgar_batch_t* out, const mgar_t* handles, int count, void*
       des[d].x = c.df_x;
       des[d].r = c.df_r;
       des[d].p = c.df_p;
+      des[d].p2 = c.df_p2;
       des[d].Ap = c.df_Ap;
       des[d].b32 = c.b32;
       des[d].x32 = c.x32;
@@ -1064,25 +999,21 @@ int mgar_batch_create(mgar_batch_t* out, const mgar_t* handles, int count, void*
         Lev& v = lev[(size_t)l * nd + d];
         const Dims& dl = c.L[l];
         const Dims& dn = c.L[l + 1];
-        v.d = dl;
-        v.dn = dn;
-        v.omega = (float)c.p.omega;
-        v.dinv = c.h32[l].dinv;
+        v.NX = dl.NX;
+        v.NY = dl.NY;
         v.dinv_n = c.h32[l + 1].dinv;
         v.t = c.h32[l].t;
-        v.r = c.h32[l].r;
         if (l == 0) {
-          v.f0 = FineOp<float>{c.ke0_f, nullptr, c.fixed, dl.ex, dl.ey, dl.ez, dl.NX, dl.NY, dl.NZ,
-                               (int)dl.n, dl.fNX, dl.fNXY};
+          v.f0 = l2d::Fine<float>{c.ke0_f, c.h32[0].dinv_s, dl.ex, dl.ey, dn.NX, dn.NY,
+                                  (float)c.p.omega};
           v.x = c.x32;
           v.b = c.b32;
-          v.fixed = c.fixed;
         } else {
-          v.op = StencilOp<float>{c.h32[l].st, c.h32[l].dinv, dl.NX, dl.NY, dl.NZ, (int)dl.n,
-                                  dl.fNX, dl.fNXY};
+          v.c = l2d::Coarse<float>{StencilOp<float>{c.h32[l].st, c.h32[l].dinv, dl.NX, dl.NY, dl.NZ,
+                                                    (int)dl.n, dl.fNX, dl.fNXY},
+                                   dl.ex, dl.ey, dn.NX, dn.NY, (float)c.p.omega};
           v.x = c.h32[l].x;
           v.b = c.h32[l].b;
-          v.fixed = nullptr;
         }
         const bool next_coarsest = l + 2 == c.nl;
         v.bn = c.h32[l + 1].b;
@@ -1102,7 +1033,8 @@ int mgar_batch_create(mgar_batch_t* out, const mgar_t* handles, int count, void*
     MGAR_CUDA(cudaMemcpy(b->ddes, des.data(), des.size() * sizeof(Des), cudaMemcpyHostToDevice));
     b->hdes = des;
     b->s_red = make_shape(n0, kRedThreads * kNptR, kRedThreads);
-    for (int l = 0; l + 1 < lmax; ++l) make_level_shapes(*b, l, 256);
+    b->s_dot = make_shape(n0, kRedThreads * kNptR * kSumVB, kRedThreads);
+    for (int l = 0; l + 1 < lmax; ++l) make_level_shapes(*b, l);
     make_coarse_shape(*b, 8);
     MGAR_CUDA(cudaMalloc(&b->bsc, (size_t)nd * kBS * sizeof(double)));
     MGAR_CUDA(cudaMemset(b->bsc, 0, (size_t)nd * kBS * sizeof(double)));
