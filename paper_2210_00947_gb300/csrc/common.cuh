@@ -242,6 +242,7 @@ struct Ctx {
   bool untiled = false;  // MGAR_UNTILED=1: generic finest-level kernels (debugging aid)
   int f3d_gz[5] = {};     // z runs of the tiled finest-level kernels [mode]
   int df3d_gz[3] = {};    // z runs of the tiled df64 operator kernels [mode]
+  int f64_gz[5] = {};     // z runs of the tiled FP64 kernels [mode]
   bool df3d_tile = false; // their tile: 32 x 8, or 43 x 11 when that leaves fewer lanes idle
   bool f3d_tile = false;  // FP32 finest-level tile: 32 x 8, or 43 x 5 when that leaves fewer lanes idle
   bool bottom_ok = false; // the V-cycle's bottom levels run as one cluster launch
@@ -1117,6 +1118,19 @@ void vcycle(Ctx& c, const Real* b, Real* x, bool zero_guess);
 void fine3d(Ctx& c, int mode, const float* ke, const float* b, const float* dinv, const float* x,
             const float* xc, float* out0, float* out1, const float2* rdot = nullptr,
             SumOut dout = {});
+// the same passes in FP64 (fine3d64.cu; no mode 1)
+void fine3d(Ctx& c, int mode, const double* ke, const double* b, const double* dinv, const double* x,
+            const double* xc, double* out0, double* out1, const float2* rdot = nullptr,
+            SumOut dout = {});
+void fine3d64_prepare(Ctx& c);
+// r = q - A x with the current k_e, ||r||^2
+void fine3d_residual64(Ctx& c, const double* q, const double* x, double* r, SumOut rr);
+// p = z + *beta p_old (p = z when p_old is null), y = A p, p . y
+void fine3d_dir64(Ctx& c, const double* z, const double* p_old, double* p, const double* beta,
+                  double* y, SumOut dot);
+// y = scale A x (with ksub: conductivities k_e - ksub_e, fixed rows 0), x . y
+void fine3d_apply64(Ctx& c, const double* ke, const double* ksub, const double* x, double* y,
+                    double scale, SumOut dot);
 // FP32 CG direction update and product: p = z + beta p_old (beta a df64 pair,
 // 0 while *first is nonzero), y = A p with the current k_e, p . y into dot;
 // odd *parity swaps p_old and p; rz_set receives *rz_new
@@ -1131,7 +1145,7 @@ inline bool vcycle_dot_ok(const Ctx& c) {
   return c.p.nu_pre == 1 && c.p.nu_post == 1 && c.nl >= 2 && !c.untiled;
 }
 void vcycle_dot(Ctx& c, const float* b, float* x, const float2* r, SumOut dout);
-// the same in FP64 with b . x in *dout, for 2D grids where vcycle_dot_ok
+// the same in FP64 with b . x in dout
 void vcycle_dot64(Ctx& c, const double* b, double* x, SumOut dout);
 // launch shapes of the tiled kernels (occupancy query; call outside stream capture)
 void fine3d_prepare(Ctx& c);

@@ -347,18 +347,20 @@ static int solve_mgcg_fp(Ctx& c, double* T, int* iters, double* relres) {
   if (c.p.precision == MGAR_MIXED) return solve_mgcg_df(c, T, iters, relres);
   const int64_t n = c.n;
   if (c.dim == 2) residual_norm<2>(c, T, c.r, c.dsc + S_RR);
+  else if (!c.untiled) fine3d_residual64(c, c.q, T, c.r, SumOut{c.dsc + S_RR});
   else residual_norm<3>(c, T, c.r, c.dsc + S_RR);
   fetch_scalars(c, S_RR, 1);
   double rel = std::sqrt(c.hsc[S_RR]) / c.qnorm;
   int it = 0;
   if (!(rel <= c.p.eps2)) {
     require(std::isfinite(rel), MGAR_ERR_NONFINITE, "non-finite initial residual");
-    // z = M r, r . z into dsc[slot] and beta, in one with the 2D V-cycle's
-    // tiled passes
+    // z = M r, r . z into dsc[slot] and beta, in one with the V-cycle's tiled
+    // passes; 3D: the direction update in one with the product
+    const bool tiled = vcycle_dot_ok(c);
     auto precondition_rz = [&](int slot) {
       const SumOut out{c.dsc + slot, nullptr, c.dsc + (slot == S_RZ0 ? S_RZ1 : S_RZ0),
                        c.dsc + S_BETA, 0};
-      if (c.dim == 2 && vcycle_dot_ok(c)) {
+      if (tiled) {
         run_graph(c, slot == S_RZ0 ? 11 : 12, c.r, c.z, vcycle_profiled(c),
                   [&] { vcycle_dot64(c, c.r, c.z, out); });
       } else {
@@ -368,11 +370,23 @@ static int solve_mgcg_fp(Ctx& c, double* T, int* iters, double* relres) {
     };
     int a = S_RZ0, b = S_RZ1;
     precondition_rz(a);
-    MGAR_CUDA(cudaMemcpyAsync(c.pv, c.z, n * sizeof(double), cudaMemcpyDeviceToDevice, c.stream));
+    const bool dir = c.dim == 3 && !c.untiled;
+    // tm, the reanalysis's own solution vector, is free during a solve
+    double *pcur = c.pv, *pnext = c.tm;
+    bool first = true;
+    if (!dir)
+      MGAR_CUDA(cudaMemcpyAsync(pcur, c.z, n * sizeof(double), cudaMemcpyDeviceToDevice, c.stream));
     while (it < c.p.cg_max) {
-      apply_fine64(c, c.ke, c.pv, c.Ap,
-                   SumOut{c.dsc + S_PAP, c.dsc + a, nullptr, c.dsc + S_ALPHA, 0});
-      k_cg_xr<<<sum_blocks(c, n), kThreads, 0, c.stream>>>(T, c.r, c.pv, c.Ap, n, c.dsc + S_ALPHA,
+      const SumOut pap{c.dsc + S_PAP, c.dsc + a, nullptr, c.dsc + S_ALPHA, 0};
+      if (dir) {
+        ProfScope ps(c, MGAR_KC_APPLY64);
+        fine3d_dir64(c, c.z, first ? nullptr : pcur, pnext, c.dsc + S_BETA, c.Ap, pap);
+        std::swap(pcur, pnext);
+      } else {
+        apply_fine64(c, c.ke, pcur, c.Ap, pap);
+      }
+      first = false;
+      k_cg_xr<<<sum_blocks(c, n), kThreads, 0, c.stream>>>(T, c.r, pcur, c.Ap, n, c.dsc + S_ALPHA,
                                                         c.partials, c.counter, c.dsc + S_RR);
       MGAR_LAUNCH_CHECK();
       ++it;
@@ -380,10 +394,12 @@ static int solve_mgcg_fp(Ctx& c, double* T, int* iters, double* relres) {
       rel = std::sqrt(c.hsc[S_RR]) / c.qnorm;
       require(std::isfinite(rel), MGAR_ERR_NONFINITE, "CG breakdown (non-finite residual)");
       if (rel <= c.p.eps2) break;
-      precondition_rz(b);
-      k_cg_p<<<red_blocks(c), kThreads, 0, c.stream>>>(c.pv, c.z, n, c.dsc + S_BETA);
-      MGAR_LAUNCH_CHECK();
       std::swap(a, b);
+      precondition_rz(a);
+      if (!dir) {
+        k_cg_p<<<red_blocks(c), kThreads, 0, c.stream>>>(pcur, c.z, n, c.dsc + S_BETA);
+        MGAR_LAUNCH_CHECK();
+      }
     }
   }
   if (iters) *iters = it;

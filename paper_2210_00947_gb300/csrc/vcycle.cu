@@ -212,6 +212,9 @@ __global__ void k_prolong3(const Real* __restrict__ xc, const Real* cur, Real* d
   float wx[2], wy[2];
   prolong_taps(i, f.ex, ix, wx);
   prolong_taps(j, f.ey, iy, wy);
+  Real wxy[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) wxy[q] = (Real)(wx[q & 1] * wy[q >> 1]);
   const int cNXY = cd.NX * cd.NY;
   const int k0 = blockIdx.y * KC, Kb = k0 >> 1;
   // coarse planes Kb .. Kb + NP - 1, interpolated in x and y
@@ -226,7 +229,7 @@ __global__ void k_prolong3(const Real* __restrict__ xc, const Real* cur, Real* d
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
           const int o = ix[a] + cd.NX * iy[b] + cNXY * K;
-          if (CK(o, cd.n)) P[t] += (Real)(wx[a] * wy[b]) * xc[o];
+          if (CK(o, cd.n)) P[t] += wxy[a + 2 * b] * xc[o];
         }
     }
   }
@@ -653,12 +656,13 @@ static void vcycle_fused2(Ctx& c, const Real* b0, Real* x0, bool zero_guess,
 }
 
 // Table 1 with one pre- and one post-sweep and a zero guess below the finest
-// level: per level one fused pre kernel (smooth from zero + residual), the
-// restriction, and one fused post kernel (interpolation + smooth); the small
-// levels at the bottom run in one cluster launch.
-static void vcycle_fused3(Ctx& c, const float* b0, float* x0, bool zero_guess,
-                         const float2* rdot = nullptr, SumOut dout = {}) {
-  using Real = float;
+// level, 3D: the tiled passes on the finest level, per coarse level the
+// residual, the restriction (which leaves the next level's zero-guess sweep)
+// and one fused post kernel (interpolation + smooth) or two on large levels; on
+// request the small levels at the bottom run in one cluster launch (FP32).
+template <typename Real>
+static void vcycle_fused3(Ctx& c, const Real* b0, Real* x0, bool zero_guess,
+                          const float2* rdot = nullptr, SumOut dout = {}) {
   constexpr int DIM = 3;
   LevelBuf<Real>* h = levels<Real>(c);
   const int nl = c.nl;
@@ -670,10 +674,13 @@ static void vcycle_fused3(Ctx& c, const float* b0, float* x0, bool zero_guess,
   {
     ProfScope ps(c, MGAR_KC_SMOOTH0);
     if (zero_guess) {
-      fine3d(c, 0, ref_ke<Real>(c), b0, h[0].dinv, nullptr, nullptr, h[0].t, h[0].r);
+      fine3d(c, 0, ref_ke<Real>(c), b0, h[0].dinv, (const Real*)nullptr, (const Real*)nullptr, h[0].t,
+             h[0].r);
     } else {
-      fine3d(c, 3, ref_ke<Real>(c), b0, h[0].dinv, x0, nullptr, h[0].t, nullptr);
-      fine3d(c, 2, ref_ke<Real>(c), b0, h[0].dinv, h[0].t, nullptr, h[0].r, nullptr);
+      fine3d(c, 3, ref_ke<Real>(c), b0, h[0].dinv, (const Real*)x0, (const Real*)nullptr, h[0].t,
+             (Real*)nullptr);
+      fine3d(c, 2, ref_ke<Real>(c), b0, h[0].dinv, (const Real*)h[0].t, (const Real*)nullptr, h[0].r,
+             (Real*)nullptr);
     }
     cur0 = h[0].t;
   }
@@ -684,7 +691,7 @@ static void vcycle_fused3(Ctx& c, const float* b0, float* x0, bool zero_guess,
              (const Real*)h[0].r, h[1].b, d0, c.L[1], (const uint8_t*)nullptr,
              (const Real*)h[1].dinv, om, nl > 2 ? h[1].x : (Real*)nullptr);
   MGAR_LAUNCH_CHECK_AT(level_site(3, 0));
-  const int lb = bottom_level(c);
+  const int lb = sizeof(Real) == 4 ? bottom_level(c) : nl;
   // coarse levels, down
   for (int l = 1; l + 1 < nl && l < lb; ++l) {
     const Dims& d = c.L[l];
@@ -699,7 +706,7 @@ static void vcycle_fused3(Ctx& c, const float* b0, float* x0, bool zero_guess,
   }
   if (lb < nl) {
     // levels lb .. nl-1 in one cluster launch
-    launch_bottom<Real, DIM>(c, lb);
+    if constexpr (sizeof(Real) == 4) launch_bottom<Real, DIM>(c, lb);
     res[nl - 1] = h[nl - 1].x;
     for (int l = lb; l + 1 < nl; ++l) res[l] = h[l].t;
   } else {
@@ -710,7 +717,9 @@ static void vcycle_fused3(Ctx& c, const float* b0, float* x0, bool zero_guess,
   // coarse levels, up
   for (int l = std::min(nl - 2, lb - 1); l >= 1; --l) {
     const Dims& d = c.L[l];
-    if (d.n > c.split_coarse_nodes) {
+    // FP64: interpolating at each of 27 neighbours takes longer than a launch
+    // on every level (24 us on 9^3 and on 17^3 nodes, against 11 for the two)
+    if (sizeof(Real) == 8 || d.n > c.split_coarse_nodes) {
       // large level: thin interpolation in place on x_l, then the sweep into t_l
       launch_prolong<Real, DIM>(c, true, res[l + 1], (const Real*)h[l].x, h[l].x, d, c.L[l + 1],
                                 (const uint8_t*)nullptr);
@@ -725,34 +734,28 @@ static void vcycle_fused3(Ctx& c, const float* b0, float* x0, bool zero_guess,
     res[l] = h[l].t;
   }
   // finest level, post (the timed class is the tiled pass alone)
-  if (!c.split_post) {
+  if (sizeof(Real) == 4 && !c.split_post) {
     ProfScope ps(c, MGAR_KC_SMOOTH0);
-    fine3d(c, 1, ref_ke<Real>(c), b0, h[0].dinv, cur0, res[1], x0, nullptr, rdot, dout);
+    fine3d(c, 1, ref_ke<Real>(c), b0, h[0].dinv, (const Real*)cur0, res[1], x0, (Real*)nullptr, rdot,
+           dout);
   } else {
     // interpolation in place on the pre-smoothed iterate, then the tiled sweep
     launch_prolong<Real, DIM>(c, true, (const Real*)res[1], (const Real*)cur0, cur0, d0, c.L[1],
                               (const uint8_t*)c.fixed);
     MGAR_LAUNCH_CHECK_AT(level_site(4, 0));
     ProfScope ps(c, MGAR_KC_SMOOTH0);
-    fine3d(c, 3, ref_ke<Real>(c), b0, h[0].dinv, cur0, nullptr, x0, nullptr, rdot, dout);
+    fine3d(c, 3, ref_ke<Real>(c), b0, h[0].dinv, (const Real*)cur0, (const Real*)nullptr, x0,
+           (Real*)nullptr, rdot, dout);
   }
 }
 
-// General Table 1 V-cycle (any numbers of pre- and post-sweeps).  The fused
-// form is for the FP32 V-cycle: its kernels trade memory passes and launches
-// for recomputed arithmetic (the neighbours' smoothed values and
-// interpolations), which pays on the FP32 pipe and not at GB300's 1/58-rate
-// FP64, where the separate kernels below are faster.
+// General Table 1 V-cycle (any numbers of pre- and post-sweeps).
 template <typename Real, int DIM>
 static void vcycle_dim(Ctx& c, const Real* b0, Real* x0, bool zero_guess) {
   if (c.p.nu_pre == 1 && c.p.nu_post == 1 && c.nl >= 2 && !c.untiled) {
-    if constexpr (DIM == 2) {
-      vcycle_fused2<Real>(c, b0, x0, zero_guess);
-      return;
-    } else if constexpr (sizeof(Real) == 4) {
-      vcycle_fused3(c, b0, x0, zero_guess);
-      return;
-    }
+    if constexpr (DIM == 2) vcycle_fused2<Real>(c, b0, x0, zero_guess);
+    else vcycle_fused3<Real>(c, b0, x0, zero_guess);
+    return;
   }
   LevelBuf<Real>* h = levels<Real>(c);
   const int nl = c.nl;
@@ -820,11 +823,12 @@ void vcycle_dot(Ctx& c, const float* b, float* x, const float2* r, SumOut dout) 
   require(vcycle_dot_ok(c), MGAR_ERR_ARG,
           "fused r.z V-cycle needs one pre- and one post-sweep, two levels and the tiled 3D kernels");
   if (c.dim == 2) vcycle_fused2<float>(c, b, x, true, r, dout);
-  else vcycle_fused3(c, b, x, true, r, dout);
+  else vcycle_fused3<float>(c, b, x, true, r, dout);
 }
 
 void vcycle_dot64(Ctx& c, const double* b, double* x, SumOut dout) {
-  vcycle_fused2<double>(c, b, x, true, nullptr, dout);
+  if (c.dim == 2) vcycle_fused2<double>(c, b, x, true, nullptr, dout);
+  else vcycle_fused3<double>(c, b, x, true, nullptr, dout);
 }
 
 template <typename Real, int DIM>
@@ -844,6 +848,7 @@ static void apply_dim(Ctx& c, const Real* ke, const Real* ksub, const Real* x, R
 void apply_fine64(Ctx& c, const double* ke, const double* x, double* y, SumOut dot_out) {
   ProfScope ps(c, MGAR_KC_APPLY64);
   if (c.dim == 2) apply_dim<double, 2>(c, ke, nullptr, x, y, 1.0, dot_out);
+  else if (!c.untiled) fine3d_apply64(c, ke, nullptr, x, y, 1.0, dot_out);
   else apply_dim<double, 3>(c, ke, nullptr, x, y, 1.0, dot_out);
 }
 void apply_fine32(Ctx& c, const float* ke, const float* x, float* y) {
@@ -853,6 +858,7 @@ void apply_fine32(Ctx& c, const float* ke, const float* x, float* y) {
 // y = -(A - A0) x
 void apply_dK64(Ctx& c, const double* x, double* y) {
   if (c.dim == 2) apply_dim<double, 2>(c, c.ke, c.ke0, x, y, -1.0, {});
+  else if (!c.untiled) fine3d_apply64(c, c.ke, c.ke0, x, y, -1.0, {});
   else apply_dim<double, 3>(c, c.ke, c.ke0, x, y, -1.0, {});
 }
 void apply_dK32(Ctx& c, const float* x, float* y) {
