@@ -15,6 +15,7 @@
 // coarse solve of every V-cycle is one small dense product.
 #include "common.cuh"
 
+#include <type_traits>
 #include <vector>
 
 namespace mgar {
@@ -580,157 +581,237 @@ __global__ void k_band_inverse_df(const double* __restrict__ gband_d,
   for (int i = lane; i < n; i += 32) inv[(int64_t)i * n + col] = df_to_double(df_ld(colbuf + i));
 }
 
-// Band widths below one warp (every coarsest level the V-cycles build here:
-// 5^3 nodes in 3D, up to 17^2 in 2D): the same factorisation and inverse,
-// the same df64 operations on every entry in the same order (bit-identical
-// results), with shorter dependency chains.
-constexpr int kWinBw = 32;
-
-// The pivot of column k: sqrt(A(k,k)) into the band, 1/sqrt into rdiag and
-// *rp; *bad set when A(k,k) is not positive.
-__device__ __forceinline__ void chol_pivot_df(float2* band, float2* rdiag, int k, int ld, int bw,
-                                              float2* rp, int* bad) {
-  const df a = df_ld(band + (int64_t)k * ld + bw);
-  if (!(a.hi > 0.f) || !isfinite(a.hi)) *bad = 1;
-  const df r = df_rsqrt(a);
-  *rp = make_float2(r.hi, r.lo);
-  df_st(band + (int64_t)k * ld + bw, df_mul(a, r));
-  df_st(rdiag + k, r);
-}
-
-// Right-looking band Cholesky for bw < 32, one barrier per column: warp w
-// takes row i = k+1+w of column k's rank-1 update (lane l the entry j =
-// k+1+l <= i), scaling A(i,k) and A(j,k) by the pivot as it reads them; the
-// scaled column is stored after the barrier, when no thread reads the
-// unscaled one any more.  The first lane of warp 0, which updates A(k+1,k+1),
-// computes the next pivot at once (double-buffered pivot and flag), so the
-// pivot's rsqrt chain overlaps the other rows' updates.
-__global__ void __launch_bounds__(kCholThreads) k_band_cholesky_df_win(double* __restrict__ gband,
-                                                                       double* __restrict__ grdiag,
-                                                                       int n, int bw,
-                                                                       int* __restrict__ err) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  float2* band = reinterpret_cast<float2*>(smraw);
-  float2* out = reinterpret_cast<float2*>(gband);  // same bytes, df64 pairs
-  float2* rdiag = reinterpret_cast<float2*>(grdiag);
-  __shared__ float2 rpiv[2];
-  __shared__ int bad[2];
-  const int ld = bw + 1;
-  const int64_t size = (int64_t)n * ld;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int64_t t = tid; t < size; t += blockDim.x) {
-    const df v = df_from_double(gband[t]);
-    band[t] = make_float2(v.hi, v.lo);
+// The coarsest factor and inverse for band widths below 64 in the LDL^T form,
+// in FP64 or in double-float arithmetic.
+//
+// A chain of n pivots on one SM, whose length is the latency of a step.  The
+// Cholesky kernels above take three barriers and a square root per pivot (160
+// us in FP64 for 169 nodes of band width 14); here a step is
+//   A(i, j) -= (A(i, k) / d_k) A(j, k),  k < j <= i <= k + bw,
+// the triangle's entries dealt to the threads one by one (a row per warp left
+// most lanes idle, and an FP64 instruction costs 20 clocks of the SM however
+// many lanes it serves), the thread of A(k+1, k+1) forming 1/d_{k+1} at once (a
+// reciprocal is half the dependent operations of a square root's), and one
+// barrier.  Column k is only read in its step, so L = A(., k) / d_k is formed
+// for all columns at the end.
+struct ArD {
+  using S = double;
+  __device__ static S from(double v) { return v; }
+  __device__ static double to(S v) { return v; }
+  __device__ static S zero() { return 0.0; }
+  __device__ static S mul(S a, S b) { return a * b; }
+  // c - a b
+  __device__ static S nfma(S a, S b, S c) { return fma(-a, b, c); }
+  __device__ static bool ok(S a) { return a > 0.0 && isfinite(a); }
+  // an FP32 reciprocal refined by two Newton steps (24 -> 48 -> 96 bits)
+  __device__ static S rcp(S a) {
+    const float f = (float)a;
+    if (!(f > 1e-37f && f < 1e37f)) return 1.0 / a;
+    double y = (double)(1.f / f);
+    y = fma(y, fma(-a, y, 1.0), y);
+    return fma(y, fma(-a, y, 1.0), y);
   }
+  __device__ static S shfl(S v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+};
+struct ArDf {
+  using S = float2;
+  __device__ static df u(S v) { return df{v.x, v.y}; }
+  __device__ static S p(df v) { return make_float2(v.hi, v.lo); }
+  __device__ static S from(double v) { return p(df_from_double(v)); }
+  __device__ static double to(S v) { return df_to_double(u(v)); }
+  __device__ static S zero() { return make_float2(0.f, 0.f); }
+  __device__ static S mul(S a, S b) { return p(df_mul(u(a), u(b))); }
+  __device__ static S nfma(S a, S b, S c) { return p(df_sub(u(c), df_mul(u(a), u(b)))); }
+  __device__ static bool ok(S a) { return a.x > 0.f && isfinite(a.x); }
+  // one Newton step from the FP32 reciprocal, its residual 1 - a y formed by
+  // FMAs (24 -> 48 bits)
+  __device__ static S rcp(S a) {
+    const float y = 1.f / a.x;
+    const float e = __fmaf_rn(-a.y, y, __fmaf_rn(-a.x, y, 1.f));
+    return p(df_make(y, __fmul_rn(y, e)));
+  }
+  __device__ static S shfl(S v, int lane) {
+    return make_float2(__shfl_sync(0xffffffffu, v.x, lane), __shfl_sync(0xffffffffu, v.y, lane));
+  }
+};
+constexpr int kLdlBw = 64;  // band widths below this
+
+// Row-major lower triangle of bw rows: entry t is (row, column) in tri[t].
+__device__ __forceinline__ void tri_table(uint16_t* tri, int bw) {
+  for (int r = threadIdx.x; r < bw; r += blockDim.x)
+    for (int c = 0; c <= r; ++c) tri[r * (r + 1) / 2 + c] = (uint16_t)((r << 8) | c);
+}
+__host__ __device__ constexpr int tri_size(int bw) { return bw * (bw + 1) / 2; }
+// band entry (i, j) of the lower band, j in [i - bw, i], in rows of bw + 1
+__device__ __forceinline__ int band_at(int i, int j, int bw) { return i * bw + j + bw; }
+
+// gband: the band in FP64 in, L (unit diagonal not stored) as Ar::S out;
+// grd: 1 / d.
+template <class Ar>
+__global__ void __launch_bounds__(1024) k_band_ldl(double* __restrict__ gband,
+                                                   double* __restrict__ grd, int n, int bw,
+                                                   int* __restrict__ err) {
+  using S = typename Ar::S;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  S* band = reinterpret_cast<S*>(smraw);
+  const int size = n * (bw + 1);
+  S* rd = band + size;
+  uint16_t* tri = reinterpret_cast<uint16_t*>(rd + n);
+  // a step's flag: the next step's goes to the other slot, so every thread
+  // reads the same value after the barrier
+  __shared__ int bad[2];
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  for (int t = tid; t < size; t += nthr) band[t] = Ar::from(gband[t]);
+  tri_table(tri, bw);
   if (tid == 0) bad[0] = bad[1] = 0;
   __syncthreads();
-  if (tid == 0) chol_pivot_df(band, rdiag, 0, ld, bw, &rpiv[0], &bad[0]);
+  if (tid == 0) {
+    const S d = band[band_at(0, 0, bw)];
+    if (!Ar::ok(d)) bad[1] = 1;
+    rd[0] = Ar::rcp(d);
+  }
   __syncthreads();
-  df lprev{0.f, 0.f};  // lane 0 of warp w: L(i, k-1) of its row in the last column
-  int64_t aprev = -1;
-  for (int k = 0; k < n; ++k) {
-    if (bad[k & 1]) break;
-    const df rp{rpiv[k & 1].x, rpiv[k & 1].y};
-    if (aprev >= 0) {
-      df_st(band + aprev, lprev);
-      aprev = -1;
-    }
-    const int m = min(k + bw, n - 1) - k;
-    if (warp < m) {
-      const int i = k + 1 + warp;
-      const int64_t ai = (int64_t)i * ld + (k - i + bw);  // A(i, k)
-      const df lik = df_mul(df_ld(band + ai), rp);
-      if (lane <= warp) {
-        const int j = k + 1 + lane;
-        const int64_t at = (int64_t)i * ld + (j - i + bw);
-        const df ljk = df_mul(df_ld(band + (int64_t)j * ld + (k - j + bw)), rp);
-        df_st(band + at, df_sub(df_ld(band + at), df_mul(lik, ljk)));
-      }
-      if (lane == 0) {
-        lprev = lik;
-        aprev = ai;
-        if (warp == 0)
-          chol_pivot_df(band, rdiag, k + 1, ld, bw, &rpiv[(k + 1) & 1], &bad[(k + 1) & 1]);
+  bool stop = bad[1] != 0;
+  for (int k = 0; k + 1 < n && !stop; ++k) {
+    const S di = rd[k];
+    const int m = min(bw, n - 1 - k), cnt = tri_size(m);
+    for (int t = tid; t < cnt; t += nthr) {
+      const int rc = tri[t], i = k + 1 + (rc >> 8), j = k + 1 + (rc & 255);
+      const S v = Ar::nfma(Ar::mul(band[band_at(i, k, bw)], di), band[band_at(j, k, bw)],
+                           band[band_at(i, j, bw)]);
+      if (CK(band_at(i, j, bw), size)) band[band_at(i, j, bw)] = v;
+      if (t == 0) {
+        if (!Ar::ok(v)) bad[k & 1] = 1;
+        rd[k + 1] = Ar::rcp(v);
       }
     }
     __syncthreads();
+    stop = bad[k & 1] != 0;
   }
-  if (aprev >= 0) df_st(band + aprev, lprev);
-  __syncthreads();
-  for (int64_t t = tid; t < size; t += blockDim.x) out[t] = band[t];
-  if (tid == 0 && (bad[0] || bad[1])) *err = MGAR_ERR_NOT_SPD;
+  S* out = reinterpret_cast<S*>(gband);
+  S* ord = reinterpret_cast<S*>(grd);
+  for (int t = tid; t < size; t += nthr) {
+    const int i = t / (bw + 1), k = t - i * (bw + 1) + i - bw;
+    out[t] = k >= 0 && k < i ? Ar::mul(band[t], rd[k]) : Ar::zero();
+  }
+  for (int t = tid; t < n; t += nthr) ord[t] = rd[t];
+  if (tid == 0 && stop) *err = MGAR_ERR_NOT_SPD;
 }
 
-// Columns of the inverse for bw < 32, one warp per column, the unknowns of
-// the substitutions in registers: lane l holds the row r = l (mod 32) of the
-// bw + 1 rows the current step touches, receives the step's solved value by
-// shuffle and takes row r + 32 (forward) or r - 32 (backward) once its own
-// row is solved, so no step waits on shared memory.  The band and the
-// reciprocal pivots are staged in shared memory; a step's coefficient and
-// pivot loads do not depend on the chain, and the solved value is stored
-// after it has been passed on.
-__global__ void k_band_inverse_df_win(const double* __restrict__ gband_d,
-                                      const double* __restrict__ grdiag_d, int n, int bw,
-                                      double* __restrict__ inv) {
+// Columns of (L D L^T)^-1, one warp per column, the unknowns of the
+// substitutions in registers: lane l holds the rows r = l (mod 32) of the next
+// 32 NW rows (NW slots, nearest first), hands the step's solved value on by
+// shuffle and takes the next row once its own is solved.  L's diagonal is one,
+// so a step's chain is a shuffle and a multiply-subtract; its coefficients and
+// the division by D are off the chain.  Few warps per block, so that the warps
+// share no FP64 pipe.
+template <class Ar, int NW>
+__global__ void k_band_ldl_inverse(const double* __restrict__ gband_d,
+                                   const double* __restrict__ grd_d, int n, int bw,
+                                   double* __restrict__ inv) {
+  using S = typename Ar::S;
   extern __shared__ __align__(16) unsigned char smraw[];
-  const float2* gband = reinterpret_cast<const float2*>(gband_d);
-  const float2* grdiag = reinterpret_cast<const float2*>(grdiag_d);
-  float2* sband = reinterpret_cast<float2*>(smraw);
-  const int ld = bw + 1;
-  const int64_t size = (int64_t)n * ld;
-  float2* srdiag = sband + size;
-  const int warps = blockDim.x >> 5;
-  const int wid = threadIdx.x >> 5;
-  for (int64_t t = threadIdx.x; t < size; t += blockDim.x) sband[t] = gband[t];
-  for (int t = threadIdx.x; t < n; t += blockDim.x) srdiag[t] = grdiag[t];
+  const S* gband = reinterpret_cast<const S*>(gband_d);
+  const S* grd = reinterpret_cast<const S*>(grd_d);
+  S* band = reinterpret_cast<S*>(smraw);
+  const int size = n * (bw + 1), warps = blockDim.x >> 5, wid = threadIdx.x >> 5;
+  S* rd = band + size;
+  for (int t = threadIdx.x; t < size; t += blockDim.x) band[t] = gband[t];
+  for (int t = threadIdx.x; t < n; t += blockDim.x) rd[t] = grd[t];
   __syncthreads();
-  float2* colbuf = srdiag + n + (int64_t)wid * n;  // the forward solution y
-  const int col = blockIdx.x * warps + wid;
-  const int lane = threadIdx.x & 31;
+  S* z = rd + n + wid * n;  // D^-1 L^-1 e_col
+  const int col = blockIdx.x * warps + wid, lane = threadIdx.x & 31;
   if (col >= n) return;
-  for (int i = lane; i < col; i += 32) colbuf[i] = make_float2(0.f, 0.f);
+  for (int i = lane; i < col; i += 32) z[i] = Ar::zero();
   // forward: L y = e_col (y_p = 0 for p < col)
-  int r = col + ((lane - col) & 31);
-  df y = r == col ? df{1.f, 0.f} : df{0.f, 0.f};
+  S y[NW];
+  int r = col + ((lane - col) & 31);  // the first slot's row
+#pragma unroll
+  for (int s = 0; s < NW; ++s) y[s] = r + 32 * s == col ? Ar::from(1.0) : Ar::zero();
   for (int p = col; p < n; ++p) {
     const int owner = p & 31;
-    const bool upd = r > p && r <= p + bw && r < n;
-    const df lrp = upd ? df_ld(sband + (int64_t)r * ld + (p - r + bw)) : df{0.f, 0.f};  // L(r, p)
-    const df rd = df_ld(srdiag + p);
-    df yp = df_mul(y, rd);  // the owner's solved value (others discard theirs)
-    yp.hi = __shfl_sync(0xffffffffu, yp.hi, owner);
-    yp.lo = __shfl_sync(0xffffffffu, yp.lo, owner);
-    if (upd) y = df_sub(y, df_mul(lrp, yp));
+    S l[NW];
+#pragma unroll
+    for (int s = 0; s < NW; ++s) {
+      const int q = r + 32 * s;
+      const bool upd = q > p && q <= p + bw && q < n;
+      l[s] = upd ? band[band_at(q, p, bw)] : Ar::zero();
+    }
+    const S yp = Ar::shfl(y[0], owner);
+#pragma unroll
+    for (int s = 0; s < NW; ++s) y[s] = Ar::nfma(l[s], yp, y[s]);
     if (lane == owner) {
-      df_st(colbuf + p, yp);
+      z[p] = Ar::mul(yp, rd[p]);
+#pragma unroll
+      for (int s = 0; s + 1 < NW; ++s) y[s] = y[s + 1];
+      y[NW - 1] = Ar::zero();
       r = p + 32;
-      y = df{0.f, 0.f};
     }
   }
   __syncwarp();
-  // backward: L^T x = y
+  // backward: L^T x = z
   r = (n - 1) - ((n - 1 - lane) & 31);
-  y = r >= 0 ? df_ld(colbuf + r) : df{0.f, 0.f};
+#pragma unroll
+  for (int s = 0; s < NW; ++s) y[s] = r - 32 * s >= 0 ? z[r - 32 * s] : Ar::zero();
   for (int i = n - 1; i >= 0; --i) {
     const int owner = i & 31;
-    const bool upd = r >= 0 && r < i && r >= i - bw;
-    const df lir = upd ? df_ld(sband + (int64_t)i * ld + (r - i + bw)) : df{0.f, 0.f};  // L(i, r)
-    const df rd = df_ld(srdiag + i);
-    df xi = df_mul(y, rd);
-    xi.hi = __shfl_sync(0xffffffffu, xi.hi, owner);
-    xi.lo = __shfl_sync(0xffffffffu, xi.lo, owner);
-    if (upd) y = df_sub(y, df_mul(lir, xi));
+    S l[NW];
+#pragma unroll
+    for (int s = 0; s < NW; ++s) {
+      const int q = r - 32 * s;
+      const bool upd = q >= 0 && q < i && q >= i - bw;
+      l[s] = upd ? band[band_at(i, q, bw)] : Ar::zero();
+    }
+    const S xi = Ar::shfl(y[0], owner);
+#pragma unroll
+    for (int s = 0; s < NW; ++s) y[s] = Ar::nfma(l[s], xi, y[s]);
     if (lane == owner) {
-      inv[(int64_t)i * n + col] = df_to_double(xi);
+      inv[(int64_t)i * n + col] = Ar::to(xi);
+#pragma unroll
+      for (int s = 0; s + 1 < NW; ++s) y[s] = y[s + 1];
       r = i - 32;
-      y = r >= 0 ? df_ld(colbuf + r) : df{0.f, 0.f};
+      const int q = r - 32 * (NW - 1);
+      y[NW - 1] = q >= 0 ? z[q] : Ar::zero();
     }
   }
 }
 
-__global__ void k_d2f(const double* a, float* b, int64_t n) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) b[i] = (float)a[i];
+// The two launches, when band, pivots and the columns of one block fit in
+// shared memory; false otherwise.
+template <class Ar>
+static size_t ldl_smem(int n, int bw) {
+  return ((size_t)n * (bw + 1) + n) * sizeof(typename Ar::S) + tri_size(bw) * sizeof(uint16_t);
+}
+template <class Ar>
+static size_t ldl_inverse_smem(int n, int bw, int warps) {
+  return ((size_t)n * (bw + 1) + n + (size_t)warps * n) * sizeof(typename Ar::S);
+}
+template <class Ar>
+static bool ldl_factor(Ctx& c, cudaStream_t s) {
+  const int n = c.nc, bw = c.bw;
+  // FP64: two columns per block share an SM's FP64 pipe
+  const int warps = std::is_same<Ar, ArD>::value ? 2 : 4;
+  const size_t sm = ldl_smem<Ar>(n, bw), smi = ldl_inverse_smem<Ar>(n, bw, warps);
+  if (bw >= kLdlBw || sm > kBandSmemMax || smi > kBandSmemMax) return false;
+  const int threads = std::min(1024, std::max(64, (tri_size(bw) + 31) / 32 * 32));
+  k_band_ldl<Ar><<<1, threads, sm, s>>>(c.band, c.rdiag, n, bw, c.derr);
+  MGAR_LAUNCH_CHECK();
+  const int blocks = (n + warps - 1) / warps;
+  if (bw < 32)
+    k_band_ldl_inverse<Ar, 1><<<blocks, 32 * warps, smi, s>>>(c.band, c.rdiag, n, bw, c.cinv);
+  else
+    k_band_ldl_inverse<Ar, 2><<<blocks, 32 * warps, smi, s>>>(c.band, c.rdiag, n, bw, c.cinv);
+  MGAR_LAUNCH_CHECK();
+  return true;
+}
+template <class Ar>
+static void ldl_attributes() {
+  MGAR_CUDA(cudaFuncSetAttribute(k_band_ldl<Ar>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kBandSmemMax));
+  MGAR_CUDA(cudaFuncSetAttribute(k_band_ldl_inverse<Ar, 1>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax));
+  MGAR_CUDA(cudaFuncSetAttribute(k_band_ldl_inverse<Ar, 2>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax));
 }
 
 // ------------------------------------------------------------------- host
@@ -789,10 +870,8 @@ void alloc_hierarchy(Ctx& c) {
                                  (int)kBandSmemMax));
   MGAR_CUDA(cudaFuncSetAttribute(k_band_inverse_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kBandSmemMax));
-  MGAR_CUDA(cudaFuncSetAttribute(k_band_cholesky_df_win, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kBandSmemMax));
-  MGAR_CUDA(cudaFuncSetAttribute(k_band_inverse_df_win, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kBandSmemMax));
+  ldl_attributes<ArD>();
+  ldl_attributes<ArDf>();
   // constant tables: k0 (nen^2) then G (3^dim * nen^2)
   const int nen = c.nen, ntypes = c.dim == 2 ? 9 : 27;
   std::vector<double> k0(nen * nen), G((size_t)ntypes * nen * nen, 0.0),
@@ -879,29 +958,26 @@ static void coarse_factor(Ctx& c, const Real* st, const Dims& dcst) {
   const size_t inv_smem = band_bytes + (size_t)8 * c.nc * sizeof(B);
   // the FP32 V-cycle's coarsest factor and inverse in df64 on the FP32 pipe
   // (same band bytes: a df64 pair is the size of a double)
-  if (sizeof(Real) == 4 && sizeof(B) == 8 && smem && inv_smem <= kBandSmemMax && c.df_coarse) {
-    // the windowed inverse also stages the n reciprocal pivots
-    const size_t win_smem = inv_smem + (size_t)c.nc * sizeof(B);
-    if (c.bw < kWinBw)
-      k_band_cholesky_df_win<<<1, 32 * std::max(c.bw, 1), band_bytes, s>>>(
-          (double*)band, (double*)rdiag, c.nc, c.bw, c.derr);
-    else
-      k_band_cholesky_df<<<1, kCholThreads, band_bytes, s>>>((double*)band, (double*)rdiag, c.nc,
-                                                             c.bw, c.derr);
-    MGAR_LAUNCH_CHECK();
-    if (c.bw < kWinBw && win_smem <= kBandSmemMax)
-      k_band_inverse_df_win<<<(c.nc + 7) / 8, 256, win_smem, s>>>(
-          (const double*)band, (const double*)rdiag, c.nc, c.bw, (double*)inv);
-    else
-      k_band_inverse_df<<<(c.nc + 7) / 8, 256, inv_smem, s>>>((const double*)band,
-                                                             (const double*)rdiag, c.nc, c.bw,
-                                                             (double*)inv);
-    MGAR_LAUNCH_CHECK();
+  const bool pairs = sizeof(Real) == 4 && c.df_coarse;
+  auto join = [&] {
     if (c.side_stream) {
       MGAR_CUDA(cudaEventRecord(c.ev_join, s));
       c.coarse_pending = true;
       c.derr_fresh = false;
     }
+  };
+  if (pairs ? ldl_factor<ArDf>(c, s) : ldl_factor<ArD>(c, s)) {
+    join();
+    return;
+  }
+  if (pairs && smem && inv_smem <= kBandSmemMax) {
+    k_band_cholesky_df<<<1, kCholThreads, band_bytes, s>>>((double*)band, (double*)rdiag, c.nc, c.bw,
+                                                           c.derr);
+    MGAR_LAUNCH_CHECK();
+    k_band_inverse_df<<<(c.nc + 7) / 8, 256, inv_smem, s>>>((const double*)band, (const double*)rdiag,
+                                                           c.nc, c.bw, (double*)inv);
+    MGAR_LAUNCH_CHECK();
+    join();
     return;
   }
   if (smem) {
@@ -916,11 +992,7 @@ static void coarse_factor(Ctx& c, const Real* st, const Dims& dcst) {
   else
     k_band_inverse<B, false><<<(c.nc + 7) / 8, 256, 0, s>>>(band, rdiag, c.nc, c.bw, inv);
   MGAR_LAUNCH_CHECK();
-  if (c.side_stream) {
-    MGAR_CUDA(cudaEventRecord(c.ev_join, s));
-    c.coarse_pending = true;
-    c.derr_fresh = false;
-  }
+  join();
 }
 
 template <typename Real, int DIM>
