@@ -359,14 +359,14 @@ __global__ void kb_check(double* bsc, int nd, cudaGraphConditionalHandle loop, i
 // unless level 1 is the coarsest)
 __global__ void __launch_bounds__(l2d::kThreads2) kb_down0(const Lev* L, const int* bdes,
                                                            const int* b0, const double* bsc) {
-  __shared__ l2d::DownSmem<float> s;
+  __shared__ l2d::DownSmem<float, l2d::kR> s;
   pdl_wait();
   const int d = bdes[blockIdx.x];
   if (!active(bsc, d)) return;
   const Lev& v = L[d];
   int tx, ty;
   tile_of(b0, d, l2d::tiles(v.f0.cNX, l2d::kCX), tx, ty);
-  l2d::fine_down<float, true>(s, v.f0, tx, ty, v.b, v.t, v.bn, v.dinv_n, v.xn);
+  l2d::fine_down<float, l2d::kR, true>(s, v.f0, tx, ty, v.b, v.t, v.bn, v.dinv_n, v.xn);
 }
 
 // levels >= 1 above the coarsest, down
@@ -410,14 +410,14 @@ __global__ void __launch_bounds__(l2d::kUpThreads) kb_up(const Lev* L, const int
 // level 0, up: x = v + w D^-1 (b - A v), v = t + P res_1
 __global__ void __launch_bounds__(l2d::kThreads2) kb_up0(const Lev* L, const int* bdes, const int* b0,
                                                          const double* bsc) {
-  __shared__ l2d::UpSmem<float> s;
+  __shared__ l2d::UpSmem<float, l2d::kR> s;
   pdl_wait();
   const int d = bdes[blockIdx.x];
   if (!active(bsc, d)) return;
   const Lev& v = L[d];
   int tx, ty;
   tile_of(b0, d, l2d::tiles(v.NX, l2d::kUX), tx, ty);
-  l2d::fine_up<float>(s, v.f0, tx, ty, v.b, v.t, v.resn, v.x, [](float, float) {});
+  l2d::fine_up<float, l2d::kR>(s, v.f0, tx, ty, v.b, v.t, v.resn, v.x, [](float, float) {});
 }
 
 // ------------------------------------------------------------------- host
@@ -498,9 +498,9 @@ static void make_level_shapes(Batch& b, int l) {
     const Ctx& c = *b.h[d];
     if (l + 1 >= c.nl) continue;
     const Dims &f = c.L[l], &n = c.L[l + 1];
-    down[d] = l == 0 ? l2d::tiles(n.NX, l2d::kCX) * l2d::tiles(n.NY, l2d::kCY)
+    down[d] = l == 0 ? l2d::tiles(n.NX, l2d::kCX) * l2d::tiles(n.NY, l2d::Geo<l2d::kR>::kCY)
                      : l2d::tiles(n.NX, l2d::kDX) * l2d::tiles(n.NY, l2d::kDY);
-    up[d] = l == 0 ? l2d::tiles(f.NX, l2d::kUX) * l2d::tiles(f.NY, l2d::kUY)
+    up[d] = l == 0 ? l2d::tiles(f.NX, l2d::kUX) * l2d::tiles(f.NY, l2d::Geo<l2d::kR>::kUY)
                    : l2d::tiles(f.NX, l2d::kPX) * l2d::tiles(f.NY, l2d::kPY);
   }
   b.s_down[l] = make_shape(down, 1, l == 0 ? l2d::kThreads2 : l2d::kDownThreads);

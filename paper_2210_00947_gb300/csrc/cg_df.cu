@@ -90,7 +90,7 @@ SumOut rz_out(Ctx& c, int slot, int old) {
 
 void df_dir2(Ctx& c, const DfOp& op, const float2* p_old, float2* p, const double* rz, bool first,
              const double* parity) {
-  const dim3 grid(l2d::tiles(op.NX, l2d::kUX), l2d::tiles(op.NY, l2d::kUY));
+  const dim3 grid(l2d::tiles(op.NX, l2d::kUX), l2d::tiles(op.NY, l2d::Geo<l2d::kR>::kUY));
   launch_pdl(c.stream, c.use_pdl, k_df_dir2, grid, dim3(l2d::kThreads2), op, (const float*)c.x32,
              p_old, p, (const double*)(c.dsc + S_BETA), first ? 1 : 0, parity, c.df_Ap);
   MGAR_LAUNCH_CHECK();
@@ -114,29 +114,6 @@ __global__ void k_df_residual(DfOp op, const float2* __restrict__ q, const float
     v = df_mul(ri, ri);
   }
   block_sum_finish_df(v, partials, counter, out);
-}
-
-// The device-side loop's test, in the last block of an update of x and r:
-// count the iteration, flip the parity, and continue while ||r|| / ||q|| >
-// eps2 (the host loop's test, same arithmetic) and fewer than cg_max
-// iterations ran; a non-finite residual stops the loop and the host reports
-// it.  The iteration's r . z (RZ1) becomes the next one's old value (RZ0).
-struct CgCheck {
-  double* dsc;  // null: no device-side loop
-  double qnorm, eps2;
-  int cg_max;
-  cudaGraphConditionalHandle loop;
-};
-
-__device__ __forceinline__ void cg_check(const CgCheck& k) {
-  double* dsc = k.dsc;
-  const double rel = sqrt(dsc[S_RR]) / k.qnorm;
-  const int it = (int)dsc[S_CGIT] + 1;
-  dsc[S_CGIT] = (double)it;
-  dsc[S_CGPAR] = (double)(((int)dsc[S_CGPAR]) ^ 1);
-  dsc[S_RZ0] = dsc[S_RZ1];
-  const bool go = isfinite(rel) && rel > k.eps2 && it < k.cg_max;
-  cudaGraphSetConditional(k.loop, go ? 1u : 0u);
 }
 
 // x += alpha p; r -= alpha Ap; ||r||^2; optionally the FP32 copy of r for the
@@ -349,8 +326,7 @@ static void cg_iteration_2d(Ctx& c, bool first, cudaGraphConditionalHandle loop)
 // iteration and whose condition the check kernel sets.  The host waits once
 // per solve instead of once per iteration.  False if the device or driver
 // refuses any part (the host loop is used then).
-static bool build_cg_graph(Ctx& c) {
-  auto iteration = c.dim == 2 ? cg_iteration_2d : cg_iteration;
+bool build_cg_graph(Ctx& c, CgIteration iteration) {
   cudaGraph_t g = nullptr;
   cudaGraphConditionalHandle loop = 0;
   cudaStream_t saved = c.stream;
@@ -432,7 +408,7 @@ static bool build_cg_graph(Ctx& c) {
 // The graph holds the iteration cap by value: one built for another cap
 // (the df64 CG finishing a reliable-update solve gets the iterations left)
 // is rebuilt.
-static void drop_stale_cg_graph(Ctx& c) {
+void drop_stale_cg_graph(Ctx& c) {
   if (c.cg_exec && c.cg_exec_cgmax != c.p.cg_max) {
     MGAR_CUDA(cudaGraphExecDestroy(c.cg_exec));
     c.cg_exec = nullptr;
@@ -455,7 +431,8 @@ static int solve_mgcg_df3(Ctx& c, double* T, int* iters, double* relres) {
   if (!(rel <= c.p.eps2) && c.cg_graph && c.prof_class == 0 && c.use_graphs) {
     require(std::isfinite(rel), MGAR_ERR_NONFINITE, "non-finite initial residual");
     drop_stale_cg_graph(c);
-    if (!c.cg_exec && !build_cg_graph(c)) c.cg_graph = false;
+    if (!c.cg_exec && !build_cg_graph(c, c.dim == 2 ? cg_iteration_2d : cg_iteration))
+      c.cg_graph = false;
   }
   if (!(rel <= c.p.eps2) && c.cg_exec && c.prof_class == 0 && c.use_graphs) {
     join_coarse(c);
@@ -883,7 +860,8 @@ int solve_mgcg_df(Ctx& c, double* T, int* iters, double* relres) {
   if (!(rel <= c.p.eps2) && graph) {
     require(std::isfinite(rel), MGAR_ERR_NONFINITE, "non-finite initial residual");
     drop_stale_cg_graph(c);
-    if (!c.cg_exec && !build_cg_graph(c)) c.cg_graph = false;
+    if (!c.cg_exec && !build_cg_graph(c, c.dim == 2 ? cg_iteration_2d : cg_iteration))
+      c.cg_graph = false;
   }
   if (!(rel <= c.p.eps2) && graph && c.cg_exec) {
     join_coarse(c);

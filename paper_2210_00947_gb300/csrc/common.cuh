@@ -820,6 +820,29 @@ __device__ __forceinline__ df block_div_df(const double* a, const double* b) {
   return df{s.x, s.y};
 }
 
+// The test of a device-side CG loop, in the last block of an update of x and
+// r: count the iteration, flip the parity, and continue while ||r|| / ||q|| >
+// eps2 (the host loop's test, same arithmetic) and fewer than cg_max
+// iterations ran; a non-finite residual stops the loop and the host reports
+// it.  The iteration's r . z (RZ1) becomes the next one's old value (RZ0).
+struct CgCheck {
+  double* dsc = nullptr;  // null: no device-side loop
+  double qnorm = 0.0, eps2 = 0.0;
+  int cg_max = 0;
+  cudaGraphConditionalHandle loop = 0;
+};
+
+__device__ __forceinline__ void cg_check(const CgCheck& k) {
+  double* dsc = k.dsc;
+  const double rel = sqrt(dsc[S_RR]) / k.qnorm;
+  const int it = (int)dsc[S_CGIT] + 1;
+  dsc[S_CGIT] = (double)it;
+  dsc[S_CGPAR] = (double)(((int)dsc[S_CGPAR]) ^ 1);
+  dsc[S_RZ0] = dsc[S_RZ1];
+  const bool go = isfinite(rel) && rel > k.eps2 && it < k.cg_max;
+  cudaGraphSetConditional(k.loop, go ? 1u : 0u);
+}
+
 // Deterministic block max (values >= 0) with the same last-block scheme.
 __device__ __forceinline__ void block_max_finish(double v, double* partials, unsigned int* counter,
                                                  double* out) {
@@ -1125,9 +1148,12 @@ void fine3d(Ctx& c, int mode, const double* ke, const double* b, const double* d
 void fine3d64_prepare(Ctx& c);
 // r = q - A x with the current k_e, ||r||^2
 void fine3d_residual64(Ctx& c, const double* q, const double* x, double* r, SumOut rr);
-// p = z + *beta p_old (p = z when p_old is null), y = A p, p . y
 void fine3d_dir64(Ctx& c, const double* z, const double* p_old, double* p, const double* beta,
-                  double* y, SumOut dot);
+                  bool first, const double* parity, double* y, SumOut dot);
+// FP64 CG direction update and product, 2D or 3D: p = z + *beta p_old (p = z
+// when first), y = A p, p . y; odd *parity (may be null) swaps p_old and p
+void cg_dir64(Ctx& c, const double* z, const double* p_old, double* p, const double* beta, bool first,
+              const double* parity, double* y, SumOut dot);
 // y = scale A x (with ksub: conductivities k_e - ksub_e, fixed rows 0), x . y
 void fine3d_apply64(Ctx& c, const double* ke, const double* ksub, const double* x, double* y,
                     double scale, SumOut dot);
@@ -1171,6 +1197,13 @@ int solve_mgcg_df(Ctx& c, double* T, int* iters, double* relres);
 void apply_df64(Ctx& c, const double* x, double* y);
 void ke_to_df(Ctx& c);
 void q_to_df(Ctx& c);
+// The graph of a whole CG after its initial residual and reset: one peeled
+// iteration, then a WHILE node repeating it (cg_df.cu).  False if the device or
+// driver refuses any part.  drop_stale_cg_graph: a graph holds the iteration
+// cap by value, so one built for another cap is dropped.
+using CgIteration = void (*)(Ctx& c, bool first, cudaGraphConditionalHandle loop);
+bool build_cg_graph(Ctx& c, CgIteration iteration);
+void drop_stale_cg_graph(Ctx& c);
 // solvers.cu
 int solve_mgcg(Ctx& c, double* T, int* iters, double* relres);
 void solve_mgar(Ctx& c, const double* T_prev, double* T, double* res, int* accepted);

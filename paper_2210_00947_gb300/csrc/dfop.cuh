@@ -152,8 +152,8 @@ __device__ __forceinline__ df unpack(float2 v) { return df{v.x, v.y}; }
 // takes 15, issue-bound, against 10 us of FP32 pipe (about 250 operations per
 // node and the rim) and 6 us of bytes.
 struct DfDirSmem {
-  float2 p[l2d::kRows + 2][l2d::kW];
-  float2 k[l2d::kRows + 1][l2d::kW];
+  float2 p[l2d::Geo<l2d::kR>::kRows + 2][l2d::kW];
+  float2 k[l2d::Geo<l2d::kR>::kRows + 1][l2d::kW];
 };
 
 __device__ __forceinline__ void df_dir_tile(DfDirSmem& s, const DfOp& op, int tx, int ty,
@@ -161,8 +161,9 @@ __device__ __forceinline__ void df_dir_tile(DfDirSmem& s, const DfOp& op, int tx
                                           const float2* __restrict__ p_old, bool first, df beta,
                                           float2* __restrict__ pn, float2* __restrict__ y) {
   using namespace l2d;
+  constexpr int kUY = Geo<kR>::kUY;
   const int fx0 = tx * kUX - 1, fy0 = ty * kUY - 1;
-  const Place p(fx0, op.ex);
+  const Place<kR> p(fx0, op.ex);
   const int64_t at = fx0 + p.lane + (int64_t)op.NX * (fy0 + p.y0);
   const int64_t eat = fx0 + p.lane + (int64_t)op.ex * (fy0 + p.y0);
   float zv[kR][2];

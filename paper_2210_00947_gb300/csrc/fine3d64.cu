@@ -34,11 +34,17 @@ struct Args {
   const double* b;     // PRE, RESID, SWEEP: right-hand side; DIR: z
   const double* dinv;  // PRE, SWEEP
   int full;            // RESID: r on fixed rows too (else 0), r . r into dout
-  const double* x;     // RESID, SWEEP, APPLY: operand; DIR: p_old (null: p = z)
+  const double* x;     // RESID, SWEEP, APPLY: operand; DIR: p_old
   double* out0;        // PRE: x; RESID: r; SWEEP: x'; DIR: p; APPLY: y
   double* out1;        // PRE: r; DIR: A p
   double omega, scale;
-  const double* beta;  // DIR
+  // DIR: *beta; p = z when first; odd *parity (may be null): p_old is x_alt
+  // and p goes to out_alt (the two buffers swap each iteration)
+  const double* beta;
+  const double* parity;
+  const double* x_alt;
+  double* out_alt;
+  int first;
   double* partials;
   unsigned int* counter;
   SumOut dout;         // SWEEP: b . x'; DIR: p . A p; APPLY: x . y
@@ -72,7 +78,11 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 3 : 2) k_fine64(Args a)
   const bool kron = kr && ki >= 0 && ki < a.ex && kj >= 0 && kj < a.ey;
   const int ocol = i + a.NX * j, rcol = ri + a.NX * rj;
   const int ecol = i + a.ex * j, kcol = ki + a.ex * kj;
-  const double om = MODE == DIRECTION ? (a.x ? *a.beta : 0.0) : a.omega;
+  const double om = MODE != DIRECTION ? a.omega : a.first ? 0.0 : *a.beta;
+  if (MODE == DIRECTION && a.parity && (((int)*a.parity) & 1)) {
+    a.x = a.x_alt;
+    a.out0 = a.out_alt;
+  }
 
   // a node's operand: the value the stencil's centre takes, and (masked) what
   // its neighbours see of it
@@ -90,7 +100,7 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 3 : 2) k_fine64(Args a)
         n.d = a.dinv[idx];
       } else if (MODE == DIRECTION) {
         n.b = a.b[idx];
-        n.d = a.x ? a.x[idx] : 0.0;
+        n.d = a.first ? 0.0 : a.x[idx];
       } else {
         n.v = a.x[idx];
         if (own && MODE != APPLY) {
@@ -103,7 +113,7 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 3 : 2) k_fine64(Args a)
   };
   auto value = [&](Node& n) {
     if (MODE == PRE_SMOOTH) n.v = om * n.d * n.b;
-    if (MODE == DIRECTION) n.v = a.x ? n.b + om * n.d : n.b;
+    if (MODE == DIRECTION) n.v = a.first ? n.b : n.b + om * n.d;
   };
   auto elem = [&](int col, bool in, int l) {
     double v = 0.0;
@@ -356,13 +366,17 @@ void fine3d_residual64(Ctx& c, const double* q, const double* x, double* r, SumO
 }
 
 void fine3d_dir64(Ctx& c, const double* z, const double* p_old, double* p, const double* beta,
-                  double* y, SumOut dot) {
+                  bool first, const double* parity, double* y, SumOut dot) {
   using namespace f64;
   Args a = base(c);
   a.ke = c.ke;
   a.b = z;
   a.x = p_old;
   a.beta = beta;
+  a.first = first ? 1 : 0;
+  a.parity = parity;
+  a.x_alt = p;
+  a.out_alt = const_cast<double*>(p_old);
   a.out0 = p;
   a.out1 = y;
   a.dout = dot;

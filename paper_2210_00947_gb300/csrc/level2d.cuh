@@ -27,19 +27,47 @@ namespace l2d {
 
 constexpr int kW = 64;        // columns of a finest-level tile with its rim
 constexpr int kThreads2 = 256;
-// Each of the eight warps owns kR consecutive rows (two columns per lane), so
+// Each of the eight warps owns R consecutive rows (two columns per lane), so
 // the rows' stencils share their neighbours' shared-memory loads, and one
-// address per array serves all six nodes of a thread.
-constexpr int kR = 3, kRows = 8 * kR;
-// down: coarse nodes per tile; fine columns 2 kCX + 3 = 63, rows 2 kCY + 3 = 23
-constexpr int kCX = 30, kCY = 10;
-// up: own nodes per tile
-constexpr int kUX = 62, kUY = kRows - 2;
+// address per array serves all nodes of a thread.  R = 3 costs the least rim;
+// R = 1 spreads a small grid over three times the blocks (best_rows).
+template <int R>
+struct Geo {
+  static constexpr int kRows = 8 * R;
+  static constexpr int kCY = (kRows - 3) / 2;  // down: coarse rows per tile (2 kCY + 3 rows)
+  static constexpr int kUY = kRows - 2;        // up, product: own rows per tile
+};
+constexpr int kR = 3;
+constexpr int kCX = 30;  // down: coarse columns per tile (2 kCX + 3 = 63)
+constexpr int kUX = 62;  // up, product: own columns per tile
 // coarse levels: down, coarse nodes per tile (31 x 7 residuals); up, own nodes
 constexpr int kDX = 15, kDY = 3, kDownThreads = 32 * (2 * kDY + 1);
 constexpr int kPX = 30, kPY = 8, kUpThreads = 32 * (kPY + 2);
 
 __host__ __device__ __forceinline__ int tiles(int n, int per) { return (n + per - 1) / per; }
+
+// Rows per warp of the finest level's tiles: a pass takes as long as the SM
+// with the most rows (FP64 passes are bound by its FP64 pipe), blocks / SMs
+// rounded up times R.  Tall tiles win from two blocks per SM on, since they
+// compute the smallest rim; a 101^2 grid takes R = 1.
+template <class Blocks>
+inline int best_rows(int sms, Blocks&& blocks) {
+  int best = 3, cost = 3 * tiles(blocks(3), sms);
+  for (int r = 2; r >= 1; --r)
+    if (const int c = r * tiles(blocks(r), sms); c < cost) {
+      best = r;
+      cost = c;
+    }
+  return best;
+}
+inline int up_rows(int NX, int NY, int sms) {
+  const int uy[4] = {0, Geo<1>::kUY, Geo<2>::kUY, Geo<3>::kUY};
+  return best_rows(sms, [&](int r) { return tiles(NX, kUX) * tiles(NY, uy[r]); });
+}
+inline int down_rows(int cNX, int cNY, int sms) {
+  const int cy[4] = {0, Geo<1>::kCY, Geo<2>::kCY, Geo<3>::kCY};
+  return best_rows(sms, [&](int r) { return tiles(cNX, kCX) * tiles(cNY, cy[r]); });
+}
 
 // A finest level (matrix-free operator).
 // dinv: 1/diag, negated on fixed nodes (one load for both)
@@ -97,17 +125,17 @@ __device__ __forceinline__ Real restrict_sum(const Real (*r)[W], int c, int y, i
   }
 }
 
-// The Q4 rows times 6 of column c at the tile rows y0 .. y0 + kR - 1, tile row
+// The Q4 rows times 6 of column c at the tile rows y0 .. y0 + R - 1, tile row
 // y at shared-memory row y + 1: x with off-grid and fixed values zero, k the
 // element to the lower right of the node; f(q, row) with row as a function of
 // the centre value.
-template <typename Real, class F>
+template <typename Real, int R, class F>
 __device__ __forceinline__ void q4_rows(const Real (*x)[kW], const Real (*k)[kW], int c, int y0, F&& f) {
   Real xl = x[y0][c - 1], xc = x[y0][c], xr = x[y0][c + 1];
   Real yl = x[y0 + 1][c - 1], yc = x[y0 + 1][c], yr = x[y0 + 1][c + 1];
   Real k00 = k[y0][c - 1], k01 = k[y0][c];
 #pragma unroll
-  for (int q = 0; q < kR; ++q) {
+  for (int q = 0; q < R; ++q) {
     const Real zl = x[y0 + q + 2][c - 1], zc = x[y0 + q + 2][c], zr = x[y0 + q + 2][c + 1];
     const Real k10 = k[y0 + q + 1][c - 1], k11 = k[y0 + q + 1][c];
     const Real s = k00 + k01, n = k10 + k11;
@@ -161,15 +189,16 @@ __device__ __forceinline__ int first_tap(int i, int nf, bool& half) {
   return (i & 1) && i == nf ? (i + 1) >> 1 : i >> 1;
 }
 
-// A thread's six nodes in a tile whose first node is (fx0, fy0): rows y0 + q,
+// A thread's 2 R nodes in a tile whose first node is (fx0, fy0): rows y0 + q,
 // columns lane + 32 h.
+template <int R>
 struct Place {
   int lane, w, y0;
   bool con[2], eon[2];  // column on the grid, its element on the grid
   __device__ __forceinline__ Place(int fx0, int ex) {
     lane = threadIdx.x & 31;
     w = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
-    y0 = kR * w;
+    y0 = R * w;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const unsigned i = (unsigned)(fx0 + lane + 32 * h);
@@ -182,8 +211,9 @@ struct Place {
 // ------------------------------------------------------------- finest, down
 // tile row y at row y + 1; the rows before the first and after the last are
 // read by the rim rows' stencils, whose results are not used
-template <typename Real>
+template <typename Real, int R>
 struct DownSmem {
+  static constexpr int kRows = Geo<R>::kRows;
   Real x[kRows + 2][kW];
   Real k[kRows + 1][kW];
   Real r[kRows][kW];
@@ -191,22 +221,23 @@ struct DownSmem {
 
 // ZERO: x = w D^-1 b, written to t; otherwise x is read from t.  bc and (not
 // null) xc of the tile's coarse nodes.
-template <typename Real, bool ZERO>
-__device__ __forceinline__ void fine_down(DownSmem<Real>& s, const Fine<Real>& f, int tx, int ty,
+template <typename Real, int R, bool ZERO>
+__device__ __forceinline__ void fine_down(DownSmem<Real, R>& s, const Fine<Real>& f, int tx, int ty,
                                           const Real* __restrict__ b, Real* __restrict__ t,
                                           Real* __restrict__ bc, const Real* __restrict__ dinvc,
                                           Real* __restrict__ xc) {
+  constexpr int kCY = Geo<R>::kCY;
   const int NX = f.ex + 1, NY = f.ey + 1;
   const int I0 = tx * kCX, J0 = ty * kCY;
   const int fx0 = 2 * I0 - 2, fy0 = 2 * J0 - 2;
-  const Place p(fx0, f.ex);
+  const Place<R> p(fx0, f.ex);
   const int64_t at = fx0 + p.lane + (int64_t)NX * (fy0 + p.y0);
   const int64_t eat = fx0 + p.lane + (int64_t)f.ex * (fy0 + p.y0);
-  Real dv[kR][2], bv[kR][2];
-  bool ron[kR];
+  Real dv[R][2], bv[R][2];
+  bool ron[R];
   // hierarchy data before the wait on the predecessor
 #pragma unroll
-  for (int q = 0; q < kR; ++q) {
+  for (int q = 0; q < R; ++q) {
     const unsigned j = (unsigned)(fy0 + p.y0 + q);
     ron[q] = j < (unsigned)NY;
     const bool reon = j < (unsigned)f.ey;
@@ -232,14 +263,14 @@ __device__ __forceinline__ void fine_down(DownSmem<Real>& s, const Fine<Real>& f
   pdl_wait();
   pdl_trigger();
 #pragma unroll
-  for (int q = 0; q < kR; ++q)
+  for (int q = 0; q < R; ++q)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       bv[q][h] = Real(0);
       if (ron[q] && p.con[h]) bv[q][h] = b[at + q * NX + 32 * h];
     }
 #pragma unroll
-  for (int q = 0; q < kR; ++q)
+  for (int q = 0; q < R; ++q)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int y = p.y0 + q, c = p.lane + 32 * h;
@@ -258,7 +289,7 @@ __device__ __forceinline__ void fine_down(DownSmem<Real>& s, const Fine<Real>& f
   for (int h = 0; h < 2; ++h) {
     const int c = p.lane + 32 * h;
     if (c >= 1 && c < 2 * kCX + 2)
-      q4_rows<Real>(s.x, s.k, c, p.y0, [&](int q, Real xi, auto&& row) {
+      q4_rows<Real, R>(s.x, s.k, c, p.y0, [&](int q, Real xi, auto&& row) {
         const Real r = bv[q][h] - sixth(row(xi));
         s.r[p.y0 + q][c] = dv[q][h] > Real(0) ? r : Real(0);
       });
@@ -276,8 +307,9 @@ __device__ __forceinline__ void fine_down(DownSmem<Real>& s, const Fine<Real>& f
 }
 
 // --------------------------------------------------------------- finest, up
-template <typename Real>
+template <typename Real, int R>
 struct UpSmem {
+  static constexpr int kRows = Geo<R>::kRows;
   Real v[kRows + 2][kW];
   Real k[kRows + 1][kW];
   Real c[kRows / 2 + 3][kW / 2 + 4];
@@ -285,22 +317,22 @@ struct UpSmem {
 
 // xout = v + w D^-1 (b - A v), v = t + P res (fixed nodes keep t); dot(b, x')
 // is called for every node of the tile.
-template <typename Real, class Dot>
-__device__ __forceinline__ void fine_up(UpSmem<Real>& s, const Fine<Real>& f, int tx, int ty,
+template <typename Real, int R, class Dot>
+__device__ __forceinline__ void fine_up(UpSmem<Real, R>& s, const Fine<Real>& f, int tx, int ty,
                                         const Real* __restrict__ b, const Real* __restrict__ t,
                                         const Real* __restrict__ res, Real* __restrict__ xout,
                                         Dot&& dot) {
-  constexpr int CR = kRows / 2 + 2, CC = kW / 2 + 2;
+  constexpr int kUY = Geo<R>::kUY, CR = Geo<R>::kRows / 2 + 2, CC = kW / 2 + 2;
   const int NX = f.ex + 1, NY = f.ey + 1;
   const int fx0 = tx * kUX - 1, fy0 = ty * kUY - 1;
   const int ci0 = max(fx0, 0) >> 1, cj0 = max(fy0, 0) >> 1;
-  const Place p(fx0, f.ex);
+  const Place<R> p(fx0, f.ex);
   const int64_t at = fx0 + p.lane + (int64_t)NX * (fy0 + p.y0);
   const int64_t eat = fx0 + p.lane + (int64_t)f.ex * (fy0 + p.y0);
-  Real dv[kR][2], bv[kR][2], tv[kR][2];
-  bool ron[kR];
+  Real dv[R][2], bv[R][2], tv[R][2];
+  bool ron[R];
 #pragma unroll
-  for (int q = 0; q < kR; ++q) {
+  for (int q = 0; q < R; ++q) {
     const unsigned j = (unsigned)(fy0 + p.y0 + q);
     ron[q] = j < (unsigned)NY;
     const bool reon = j < (unsigned)f.ey;
@@ -324,7 +356,7 @@ __device__ __forceinline__ void fine_up(UpSmem<Real>& s, const Fine<Real>& f, in
         s.c[cy][cx] = res[min(ci0 + cx, f.cNX - 1) + f.cNX * min(cj0 + cy, f.cNY - 1)];
     }
 #pragma unroll
-  for (int q = 0; q < kR; ++q)
+  for (int q = 0; q < R; ++q)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       bv[q][h] = tv[q][h] = Real(0);
@@ -339,7 +371,7 @@ __device__ __forceinline__ void fine_up(UpSmem<Real>& s, const Fine<Real>& f, in
     bool hx;
     const int cx = min(max(first_tap(fx0 + p.lane + 32 * h, f.ex, hx) - ci0, 0), CC);
 #pragma unroll
-    for (int q = 0; q < kR; ++q) {
+    for (int q = 0; q < R; ++q) {
       bool hy;
       const int cy = min(max(first_tap(fy0 + p.y0 + q, f.ey, hy) - cj0, 0), CR - 1);
       const bool in = dv[q][h] > Real(0);
@@ -352,7 +384,7 @@ __device__ __forceinline__ void fine_up(UpSmem<Real>& s, const Fine<Real>& f, in
   for (int h = 0; h < 2; ++h) {
     const int c = p.lane + 32 * h;
     if (c >= 1 && c <= kUX && p.con[h])
-      q4_rows<Real>(s.v, s.k, c, p.y0, [&](int q, Real, auto&& row) {
+      q4_rows<Real, R>(s.v, s.k, c, p.y0, [&](int q, Real, auto&& row) {
         const int y = p.y0 + q;
         if (!(y >= 1 && y <= kUY && ron[q])) return;
         const Real v = tv[q][h];
@@ -362,6 +394,68 @@ __device__ __forceinline__ void fine_up(UpSmem<Real>& s, const Fine<Real>& f, in
         dot(bv[q][h], xo);
       });
   }
+}
+
+// -------------------------------------------- finest, FP64 direction, product
+template <int R>
+struct DirSmem {
+  double p[Geo<R>::kRows + 2][kW];
+  double k[Geo<R>::kRows + 1][kW];
+};
+
+// p = z + beta p_old (p = z when first), y = A p with conductivities ke;
+// returns this thread's terms of p . y.
+template <int R>
+__device__ __forceinline__ double fine_dir(DirSmem<R>& s, const double* __restrict__ ke,
+                                           const uint8_t* __restrict__ fixed, int ex, int ey, int tx,
+                                           int ty, const double* __restrict__ z,
+                                           const double* __restrict__ p_old, bool first, double beta,
+                                           double* __restrict__ pn, double* __restrict__ y) {
+  constexpr int kUY = Geo<R>::kUY;
+  const int NX = ex + 1, NY = ey + 1;
+  const int fx0 = tx * kUX - 1, fy0 = ty * kUY - 1;
+  const Place<R> p(fx0, ex);
+  const int64_t at = fx0 + p.lane + (int64_t)NX * (fy0 + p.y0);
+  const int64_t eat = fx0 + p.lane + (int64_t)ex * (fy0 + p.y0);
+  double v[R][2];
+  bool ron[R], fx[R][2];
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    const unsigned j = (unsigned)(fy0 + p.y0 + q);
+    ron[q] = j < (unsigned)NY;
+    const bool reon = j < (unsigned)ey;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      v[q][h] = 0.0;
+      fx[q][h] = true;
+      if (ron[q] && p.con[h]) {
+        const int64_t o = at + q * NX + 32 * h;
+        v[q][h] = first ? z[o] : z[o] + beta * p_old[o];
+        fx[q][h] = fixed[o] != 0;
+      }
+      double kv = 0.0;
+      if (reon && p.eon[h]) kv = ke[eat + q * ex + 32 * h];
+      s.k[p.y0 + q + 1][p.lane + 32 * h] = kv;
+      s.p[p.y0 + q + 1][p.lane + 32 * h] = fx[q][h] ? 0.0 : v[q][h];
+    }
+  }
+  __syncthreads();
+  double dot = 0.0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int c = p.lane + 32 * h;
+    if (c >= 1 && c <= kUX && p.con[h])
+      q4_rows<double, R>(s.p, s.k, c, p.y0, [&](int q, double, auto&& row) {
+        const int t = p.y0 + q;
+        if (!(t >= 1 && t <= kUY && ron[q])) return;
+        const double xi = v[q][h], a = fx[q][h] ? xi : sixth(row(xi));
+        const int64_t o = at + q * NX + 32 * h;
+        pn[o] = xi;
+        y[o] = a;
+        dot += xi * a;
+      });
+  }
+  return dot;
 }
 
 // ------------------------------------------------------------- coarse, down

@@ -94,11 +94,14 @@ __global__ void k_residual_norm(FineOp<double> op, const double* __restrict__ q,
 // vectors are aligned; the caller's x need not be) and, as in dot, two blocks
 // per SM: with eight the FP64 shuffle trees took as long as the data.
 __global__ void __launch_bounds__(kThreads) k_cg_xr(double* __restrict__ x, double* __restrict__ r,
-                                                    const double* __restrict__ p,
+                                                    const double* p,
                                                     const double* __restrict__ Ap, int64_t n,
+                                                    const double* p_alt, const double* parity,
                                                     const double* __restrict__ alpha_p,
                                                     double* partials, unsigned int* counter,
-                                                    double* out) {
+                                                    double* out, CgCheck check) {
+  pdl_wait();
+  if (parity && (((int)*parity) & 1)) p = p_alt;
   const double alpha = *alpha_p;
   double v[1] = {0.0};
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, n2 = n >> 1;
@@ -125,7 +128,11 @@ __global__ void __launch_bounds__(kThreads) k_cg_xr(double* __restrict__ x, doub
     r[n - 1] = ri;
     v[0] += ri * ri;
   }
-  block_sum_finish<1>(v, partials, counter, out);
+  double t[1];
+  if (block_sum_last<1>(v, partials, counter, t) && threadIdx.x == 0) {
+    *out = t[0];
+    if (check.dsc) cg_check(check);
+  }
 }
 
 // p = z + beta p
@@ -343,6 +350,22 @@ int solve_mgcg(Ctx& c, double* T, int* iters, double* relres) {
   return rc;
 }
 
+// One iteration of the device-side loop: V-cycle z = M r with r . z into RZ1,
+// direction and product (beta = RZ1 / RZ0), the update of x (in R_0) and r with
+// the convergence check (which moves RZ1 to RZ0).  tm, the reanalysis's
+// solution vector, is the second direction buffer: parity 0 leaves the new p in
+// it.
+static void cg_iteration64(Ctx& c, bool first, cudaGraphConditionalHandle loop) {
+  vcycle_dot64(c, c.r, c.z, SumOut{c.dsc + S_RZ1, nullptr, c.dsc + S_RZ0, c.dsc + S_BETA, 0});
+  cg_dir64(c, c.z, c.pv, c.tm, c.dsc + S_BETA, first, c.dsc + S_CGPAR, c.Ap,
+           SumOut{c.dsc + S_PAP, c.dsc + S_RZ1, nullptr, c.dsc + S_ALPHA, 0});
+  launch_pdl(c.stream, c.use_pdl, k_cg_xr, dim3(sum_blocks(c, c.n)), dim3(kThreads), c.R, c.r,
+             (const double*)c.tm, (const double*)c.Ap, c.n, (const double*)c.pv,
+             (const double*)(c.dsc + S_CGPAR), (const double*)(c.dsc + S_ALPHA), c.partials,
+             c.counter, c.dsc + S_RR, CgCheck{c.dsc, c.qnorm, c.p.eps2, c.p.cg_max, loop});
+  MGAR_LAUNCH_CHECK();
+}
+
 static int solve_mgcg_fp(Ctx& c, double* T, int* iters, double* relres) {
   if (c.p.precision == MGAR_MIXED) return solve_mgcg_df(c, T, iters, relres);
   const int64_t n = c.n;
@@ -352,11 +375,33 @@ static int solve_mgcg_fp(Ctx& c, double* T, int* iters, double* relres) {
   fetch_scalars(c, S_RR, 1);
   double rel = std::sqrt(c.hsc[S_RR]) / c.qnorm;
   int it = 0;
+  // the device-side loop while no kernel class is being timed with events
+  const bool tiled = vcycle_dot_ok(c);
+  const bool graph = tiled && c.cg_graph && c.prof_class == 0 && c.use_graphs;
   if (!(rel <= c.p.eps2)) {
     require(std::isfinite(rel), MGAR_ERR_NONFINITE, "non-finite initial residual");
+    if (graph) {
+      drop_stale_cg_graph(c);
+      if (!c.cg_exec && c.p.cg_max > 0 && !build_cg_graph(c, cg_iteration64)) c.cg_graph = false;
+    }
+  }
+  if (!(rel <= c.p.eps2) && graph && c.cg_exec && c.p.cg_max > 0) {
+    // the solution in the handle's own vector (the graph holds no caller's
+    // pointer): R_0, which a reanalysis forms anew
+    copy_async((const double*)T, c.R, n, c.stream);
+    MGAR_LAUNCH_CHECK();
+    join_coarse(c);
+    MGAR_CUDA(cudaGraphLaunch(c.cg_exec, c.stream));
+    copy_async((const double*)c.R, T, n, c.stream);
+    MGAR_LAUNCH_CHECK();
+    fetch_scalars(c, S_RR, S_CGIT - S_RR + 1);
+    it = (int)c.hsc[S_CGIT];
+    count_launches(c.prologue_kernels + (int64_t)std::max(it - 1, 0) * c.body_kernels);
+    rel = std::sqrt(c.hsc[S_RR]) / c.qnorm;
+    require(std::isfinite(rel), MGAR_ERR_NONFINITE, "CG breakdown (non-finite residual)");
+  } else if (!(rel <= c.p.eps2)) {
     // z = M r, r . z into dsc[slot] and beta, in one with the V-cycle's tiled
-    // passes; 3D: the direction update in one with the product
-    const bool tiled = vcycle_dot_ok(c);
+    // passes; the direction update in one with the product
     auto precondition_rz = [&](int slot) {
       const SumOut out{c.dsc + slot, nullptr, c.dsc + (slot == S_RZ0 ? S_RZ1 : S_RZ0),
                        c.dsc + S_BETA, 0};
@@ -370,8 +415,7 @@ static int solve_mgcg_fp(Ctx& c, double* T, int* iters, double* relres) {
     };
     int a = S_RZ0, b = S_RZ1;
     precondition_rz(a);
-    const bool dir = c.dim == 3 && !c.untiled;
-    // tm, the reanalysis's own solution vector, is free during a solve
+    const bool dir = !c.untiled;
     double *pcur = c.pv, *pnext = c.tm;
     bool first = true;
     if (!dir)
@@ -379,15 +423,15 @@ static int solve_mgcg_fp(Ctx& c, double* T, int* iters, double* relres) {
     while (it < c.p.cg_max) {
       const SumOut pap{c.dsc + S_PAP, c.dsc + a, nullptr, c.dsc + S_ALPHA, 0};
       if (dir) {
-        ProfScope ps(c, MGAR_KC_APPLY64);
-        fine3d_dir64(c, c.z, first ? nullptr : pcur, pnext, c.dsc + S_BETA, c.Ap, pap);
+        cg_dir64(c, c.z, pcur, pnext, c.dsc + S_BETA, first, nullptr, c.Ap, pap);
         std::swap(pcur, pnext);
       } else {
         apply_fine64(c, c.ke, pcur, c.Ap, pap);
       }
       first = false;
-      k_cg_xr<<<sum_blocks(c, n), kThreads, 0, c.stream>>>(T, c.r, pcur, c.Ap, n, c.dsc + S_ALPHA,
-                                                        c.partials, c.counter, c.dsc + S_RR);
+      k_cg_xr<<<sum_blocks(c, n), kThreads, 0, c.stream>>>(T, c.r, pcur, c.Ap, n, nullptr, nullptr,
+                                                        c.dsc + S_ALPHA, c.partials, c.counter,
+                                                        c.dsc + S_RR, CgCheck{});
       MGAR_LAUNCH_CHECK();
       ++it;
       fetch_scalars(c, S_RR, 1);

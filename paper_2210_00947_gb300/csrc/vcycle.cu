@@ -12,6 +12,8 @@
 #include "level2d.cuh"
 #include "levelops.cuh"
 
+#include <type_traits>
+
 namespace mgar {
 
 const char* level_site(int kind, int level) {
@@ -93,26 +95,26 @@ __global__ void k_apply(Row row, const Real* __restrict__ x, Real* __restrict__ 
 }
 
 // The 2D levels' tiled passes (level2d.cuh).
-template <typename Real, bool ZERO>
+template <typename Real, int R, bool ZERO>
 __global__ void __launch_bounds__(l2d::kThreads2) k_down2d(l2d::Fine<Real> f, const Real* __restrict__ b,
                                                            Real* __restrict__ t, Real* __restrict__ bc,
                                                            const Real* __restrict__ dinvc,
                                                            Real* __restrict__ xc) {
-  __shared__ l2d::DownSmem<Real> s;
-  l2d::fine_down<Real, ZERO>(s, f, blockIdx.x, blockIdx.y, b, t, bc, dinvc, xc);
+  __shared__ l2d::DownSmem<Real, R> s;
+  l2d::fine_down<Real, R, ZERO>(s, f, blockIdx.x, blockIdx.y, b, t, bc, dinvc, xc);
 }
 
 // DOT (FP64): also b . xout into dout.
-template <typename Real, bool DOT>
+template <typename Real, int R, bool DOT>
 __global__ void __launch_bounds__(l2d::kThreads2) k_up2d(l2d::Fine<Real> f, const Real* __restrict__ b,
                                                          const Real* __restrict__ t,
                                                          const Real* __restrict__ res,
                                                          Real* __restrict__ xout, double* partials,
                                                          unsigned int* counter, SumOut dout) {
-  __shared__ l2d::UpSmem<Real> s;
+  __shared__ l2d::UpSmem<Real, R> s;
   double acc[1] = {0.0};
-  l2d::fine_up<Real>(s, f, blockIdx.x, blockIdx.y, b, t, res, xout,
-                     [&](Real bv, Real xo) { if (DOT) acc[0] += bv * xo; });
+  l2d::fine_up<Real, R>(s, f, blockIdx.x, blockIdx.y, b, t, res, xout,
+                        [&](Real bv, Real xo) { if (DOT) acc[0] += bv * xo; });
   if (DOT) {
     double v[1];
     if (block_sum_last_ids<1>(acc, partials, counter, v, threadIdx.x, l2d::kThreads2,
@@ -147,6 +149,34 @@ __global__ void __launch_bounds__(kThreads) k_dot_rz(const float2* __restrict__ 
           [&](int q) { return df_mulf(df{rv[q].x, rv[q].y}, xv[q]); }) &&
       threadIdx.x == 0)
     sum_out(out, t);
+}
+
+// FP64: p = z + beta p_old (p = z when first), y = A p, p . y into out; odd
+// *parity (may be null) swaps p_old and p.
+template <int R>
+__global__ void __launch_bounds__(l2d::kThreads2) k_dir2d(const double* __restrict__ ke,
+                                                          const uint8_t* __restrict__ fixed, int ex,
+                                                          int ey, const double* __restrict__ z,
+                                                          const double* p_old, double* p,
+                                                          const double* beta, int first,
+                                                          const double* parity,
+                                                          double* __restrict__ y, double* partials,
+                                                          unsigned int* counter, SumOut out) {
+  __shared__ l2d::DirSmem<R> s;
+  pdl_wait();
+  pdl_trigger();
+  if (parity && (((int)*parity) & 1)) {
+    double* t = const_cast<double*>(p_old);
+    p_old = p;
+    p = t;
+  }
+  double v[1], t[1];
+  v[0] = l2d::fine_dir<R>(s, ke, fixed, ex, ey, blockIdx.x, blockIdx.y, z, p_old, first != 0,
+                          first ? 0.0 : *beta, p, y);
+  if (block_sum_last_ids<1>(v, partials, counter, t, threadIdx.x, l2d::kThreads2,
+                            blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y) &&
+      threadIdx.x == 0)
+    sum_out(out, t[0]);
 }
 
 template <typename Real>
@@ -595,6 +625,14 @@ static void coarse_solve(Ctx& c) {
   MGAR_LAUNCH_CHECK_AT(level_site(5, l));
 }
 
+// f with the rows per warp (1, 2 or 3) as a constant
+template <class F>
+static void with_rows(int rows, F&& f) {
+  if (rows == 3) f(std::integral_constant<int, 3>{});
+  else if (rows == 2) f(std::integral_constant<int, 2>{});
+  else f(std::integral_constant<int, 1>{});
+}
+
 // The 2D V-cycle with one pre- and one post-sweep in the tiled passes: one
 // launch per level and direction and the coarsest solve, in either precision
 // (FP64 gains from the passes saved and, on small grids, from 2 instead of 5
@@ -617,9 +655,13 @@ static void vcycle_fused2(Ctx& c, const Real* b0, Real* x0, bool zero_guess,
     ProfScope ps(c, MGAR_KC_SMOOTH0);
     if (!zero_guess) sweep<Real, 2>(c, 0, b0, x0, h[0].t);
     ProfScope pr(c, MGAR_KC_RESID0);
-    const dim3 grid(l2d::tiles(c.L[1].NX, l2d::kCX), l2d::tiles(c.L[1].NY, l2d::kCY));
-    launch_pdl(c.stream, c.use_pdl, zero_guess ? k_down2d<Real, true> : k_down2d<Real, false>, grid,
-               dim3(l2d::kThreads2), f, b0, h[0].t, h[1].b, (const Real*)h[1].dinv, next_x(0));
+    auto down = [&](auto rows) {
+      constexpr int R = decltype(rows)::value;
+      const dim3 grid(l2d::tiles(c.L[1].NX, l2d::kCX), l2d::tiles(c.L[1].NY, l2d::Geo<R>::kCY));
+      launch_pdl(c.stream, c.use_pdl, zero_guess ? k_down2d<Real, R, true> : k_down2d<Real, R, false>,
+                 grid, dim3(l2d::kThreads2), f, b0, h[0].t, h[1].b, (const Real*)h[1].dinv, next_x(0));
+    };
+    with_rows(l2d::down_rows(c.L[1].NX, c.L[1].NY, c.sms), down);
     MGAR_LAUNCH_CHECK_AT(level_site(0, 0));
   }
   for (int l = 1; l + 1 < nl; ++l) {
@@ -642,10 +684,14 @@ static void vcycle_fused2(Ctx& c, const Real* b0, Real* x0, bool zero_guess,
     res = h[l].t;
   }
   ProfScope ps(c, MGAR_KC_SMOOTH0);
-  const dim3 grid(l2d::tiles(d0.NX, l2d::kUX), l2d::tiles(d0.NY, l2d::kUY));
   const bool fused = sizeof(Real) == 8 && dout.out;
-  launch_pdl(c.stream, c.use_pdl, fused ? k_up2d<Real, true> : k_up2d<Real, false>, grid,
-             dim3(l2d::kThreads2), f, b0, (const Real*)h[0].t, res, x0, c.partials, c.counter, dout);
+  auto up = [&](auto rows) {
+    constexpr int R = decltype(rows)::value;
+    const dim3 grid(l2d::tiles(d0.NX, l2d::kUX), l2d::tiles(d0.NY, l2d::Geo<R>::kUY));
+    launch_pdl(c.stream, c.use_pdl, fused ? k_up2d<Real, R, true> : k_up2d<Real, R, false>, grid,
+               dim3(l2d::kThreads2), f, b0, (const Real*)h[0].t, res, x0, c.partials, c.counter, dout);
+  };
+  with_rows(l2d::up_rows(d0.NX, d0.NY, c.sms), up);
   MGAR_LAUNCH_CHECK_AT(level_site(1, 0));
   if constexpr (sizeof(Real) == 4) {
     if (dout.out) {
@@ -829,6 +875,24 @@ void vcycle_dot(Ctx& c, const float* b, float* x, const float2* r, SumOut dout) 
 void vcycle_dot64(Ctx& c, const double* b, double* x, SumOut dout) {
   if (c.dim == 2) vcycle_fused2<double>(c, b, x, true, nullptr, dout);
   else vcycle_fused3<double>(c, b, x, true, nullptr, dout);
+}
+
+void cg_dir64(Ctx& c, const double* z, const double* p_old, double* p, const double* beta, bool first,
+              const double* parity, double* y, SumOut dot) {
+  ProfScope ps(c, MGAR_KC_APPLY64);
+  if (c.dim == 3) {
+    fine3d_dir64(c, z, p_old, p, beta, first, parity, y, dot);
+    return;
+  }
+  const Dims& d = c.L[0];
+  with_rows(l2d::up_rows(d.NX, d.NY, c.sms), [&](auto rows) {
+    constexpr int R = decltype(rows)::value;
+    const dim3 grid(l2d::tiles(d.NX, l2d::kUX), l2d::tiles(d.NY, l2d::Geo<R>::kUY));
+    launch_pdl(c.stream, c.use_pdl, k_dir2d<R>, grid, dim3(l2d::kThreads2), (const double*)c.ke,
+               (const uint8_t*)c.fixed, d.ex, d.ey, z, p_old, p, beta, first ? 1 : 0, parity, y,
+               c.partials, c.counter, dot);
+  });
+  MGAR_LAUNCH_CHECK();
 }
 
 template <typename Real, int DIM>
