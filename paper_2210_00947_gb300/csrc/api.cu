@@ -125,6 +125,7 @@ void free_ctx(Ctx& c) {
     c.prof_sites = nullptr;
   }
   cudaFree(c.f_cls);
+  cudaFree(c.kn0);
   cudaFree(c.pp_taps);
   cudaFree(c.pp_ctrl);
   cudaFree(c.run_rho);
@@ -443,7 +444,10 @@ int mgar_create(mgar_t* out, const mgar_params* p, const uint8_t* fixed_mask, co
     if (c->dim == 3) {
       fine3d_prepare(*c);
       fine3d64_prepare(*c);
-      if (P.precision == MGAR_MIXED) df3d_prepare(*c);
+      if (P.precision == MGAR_MIXED) {
+        df3d_prepare(*c);
+        fine3l_prepare(*c);
+      }
     }
   } catch (const Error& e) {
     g_create_error = e.msg;

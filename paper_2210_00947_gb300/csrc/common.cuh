@@ -243,6 +243,10 @@ struct Ctx {
   int f3d_gz[5] = {};     // z runs of the tiled finest-level kernels [mode]
   int df3d_gz[3] = {};    // z runs of the tiled df64 operator kernels [mode]
   int f64_gz[5] = {};     // z runs of the tiled FP64 kernels [mode]
+  // 3D mixed: the FP32 finest-level passes on linear segments (fine3l.cu);
+  // kn0 null: the tiled passes
+  float* kn0 = nullptr;   // K0's conductivities at node pitch
+  int f3l_L = 0, f3l_SL = 0, f3l_gz = 1;
   bool df3d_tile = false; // their tile: 32 x 8, or 43 x 11 when that leaves fewer lanes idle
   bool f3d_tile = false;  // FP32 finest-level tile: 32 x 8, or 43 x 5 when that leaves fewer lanes idle
   bool bottom_ok = false; // the V-cycle's bottom levels run as one cluster launch
@@ -1141,6 +1145,15 @@ void vcycle(Ctx& c, const Real* b, Real* x, bool zero_guess);
 void fine3d(Ctx& c, int mode, const float* ke, const float* b, const float* dinv, const float* x,
             const float* xc, float* out0, float* out1, const float2* rdot = nullptr,
             SumOut dout = {});
+// the same passes and the direction update on linear segments (no mode 1; the
+// reference conductivities, which are the current ones in a solve)
+void fine3l_prepare(Ctx& c);
+void fine3l_build(Ctx& c);
+void fine3l(Ctx& c, int mode, const float* b, const float* x, float* out0, float* out1,
+            const float2* rdot = nullptr, SumOut dout = {});
+void fine3l_dir(Ctx& c, const float* z, const float* p_old, float* p, const double* beta,
+                const double* first, const double* parity, float* y, SumOut dot,
+                const double* rz_new, double* rz_set);
 // the same passes in FP64 (fine3d64.cu; no mode 1)
 void fine3d(Ctx& c, int mode, const double* ke, const double* b, const double* dinv, const double* x,
             const double* xc, double* out0, double* out1, const float2* rdot = nullptr,
@@ -1252,12 +1265,12 @@ void oc_finish(Ctx& c, double* rho, double volfrac, double* lambda, double* chan
 namespace mgar {
 // Launch with the programmatic-dependent-launch attribute (see pdl_wait).
 template <typename... KArgs, typename... Args>
-inline void launch_pdl(cudaStream_t s, bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block,
-                       Args&&... args) {
+inline void launch_pdl_smem(cudaStream_t s, bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block,
+                            size_t smem, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1265,6 +1278,11 @@ inline void launch_pdl(cudaStream_t s, bool pdl, void (*kernel)(KArgs...), dim3 
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   MGAR_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...));
+}
+template <typename... KArgs, typename... Args>
+inline void launch_pdl(cudaStream_t s, bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block,
+                       Args&&... args) {
+  launch_pdl_smem(s, pdl, kernel, grid, block, 0, std::forward<Args>(args)...);
 }
 
 // Run `issue` (a fixed sequence of launches on c.stream) through a cached

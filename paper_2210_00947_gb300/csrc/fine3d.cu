@@ -479,6 +479,10 @@ void launch(Ctx& c, FineArgs& a) {
 // mode: 0 pre, 1 post, 2 residual, 3 sweep.
 void fine3d(Ctx& c, int mode, const float* ke, const float* b, const float* dinv, const float* x,
             const float* xc, float* out0, float* out1, const float2* rdot, SumOut dout) {
+  if (c.kn0 && mode != f3d::POST) {
+    fine3l(c, mode, b, x, out0, out1, rdot, dout);
+    return;
+  }
   using namespace f3d;
   const Dims& d = c.L[0];
   FineArgs a{};
@@ -518,6 +522,10 @@ void fine3d(Ctx& c, int mode, const float* ke, const float* b, const float* dinv
 void fine3d_dir(Ctx& c, const float* z, const float* p_old, float* p, const double* beta,
                 const double* first, const double* parity, float* y, SumOut dot,
                 const double* rz_new, double* rz_set) {
+  if (c.kn0) {
+    fine3l_dir(c, z, p_old, p, beta, first, parity, y, dot, rz_new, rz_set);
+    return;
+  }
   using namespace f3d;
   const Dims& d = c.L[0];
   FineArgs a{};

@@ -1043,6 +1043,7 @@ void build_hierarchy(Ctx& c) {
     MGAR_LAUNCH_CHECK();
     if (c.dim == 2) build_levels<float, 2>(c, c.ke0_f, c.h32);
     else build_levels<float, 3>(c, c.ke0_f, c.h32);
+    if (c.kn0) fine3l_build(c);
   }
   c.have_ref = true;
 }
