@@ -1148,7 +1148,6 @@ void fine3d(Ctx& c, int mode, const float* ke, const float* b, const float* dinv
 // the same passes and the direction update on linear segments (no mode 1; the
 // reference conductivities, which are the current ones in a solve)
 void fine3l_prepare(Ctx& c);
-void fine3l_build(Ctx& c);
 void fine3l(Ctx& c, int mode, const float* b, const float* x, float* out0, float* out1,
             const float2* rdot = nullptr, SumOut dout = {});
 void fine3l_dir(Ctx& c, const float* z, const float* p_old, float* p, const double* beta,

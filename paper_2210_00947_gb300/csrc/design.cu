@@ -122,7 +122,8 @@ __global__ void k_filter_simp_df(const float2* __restrict__ rho, const int4* __r
 template <int DIM>
 __global__ void k_sens_df(const float2* __restrict__ T, const double* __restrict__ rho,
                           const float2* __restrict__ rho_df, const float2* __restrict__ inv_hs,
-                          float2* __restrict__ out, Dims d, float2 mcoef_df, double penal) {
+                          float2* __restrict__ out, Dims d, float2 mcoef_df, double penal,
+                          int cubic) {
   constexpr int nen = 1 << DIM;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int)d.ne) return;
@@ -160,7 +161,7 @@ __global__ void k_sens_df(const float2* __restrict__ T, const double* __restrict
     }
   const df energy = df_mul(df_make(ah, al), df_from_double(DIM == 2 ? 1.0 / 6.0 : 1.0 / 12.0));
   const df r = dfk2(rho_df[e]);
-  const df rp = penal == 3.0 ? df_mul(r, r) : df_from_double(pow(rho[e], penal - 1.0));
+  const df rp = cubic ? df_mul(r, r) : df_from_double(pow(rho[e], penal - 1.0));
   const df v = df_mul(df_mul(dfk2(mcoef_df), rp), df_mul(energy, dfk2(inv_hs[e])));
   out[e] = make_float2(v.hi, v.lo);
 }
@@ -519,11 +520,22 @@ __global__ void k_oc_classify(const float2* __restrict__ s, const float2* __rest
   }
 }
 
-// Sort the ambiguous list (bitonic, shared memory), then one warp bisects
+// Sort the ambiguous list (bitonic, shared memory), then bisect
 // g(mu) = C + B mu + sum_amb dv clamp(s mu, lo, hi) = volfrac on [mu_a, mu_b].
+//
+// A step of the bisection is a chain of about 25 FP64 instructions (2 us, some
+// 35 steps).  g is piecewise linear with few breakpoints left in the bracket,
+// so the root of the chord through the bracket's ends says which way most of
+// the next steps will go: kPath steps are laid out along that guess, one warp
+// evaluates g at each of their midpoints, and the steps are taken in order as
+// long as the guess was right (a step whose guess was wrong is taken the other
+// way and ends the round).  Every step taken is the plain bisection's, on the
+// same midpoint and the same value of g, so mu is the same to the last bit.
+// 2040 x 2040 elements: 80 -> 27 us; 128^3: 58 -> 22 us.
 __global__ void k_oc_finish(const float2* __restrict__ s, const float2* __restrict__ lo,
                             const float2* __restrict__ hi, const float2* __restrict__ dv, int ne,
                             double volfrac, double* dsc, int* amb, int* namb_p) {
+  constexpr int kPath = 8, kLive = 32 * kPath;
   __shared__ int key[kOcAmbMax];
   const int namb = *namb_p;
   if (namb > kOcAmbMax) {
@@ -550,8 +562,9 @@ __global__ void k_oc_finish(const float2* __restrict__ s, const float2* __restri
       }
       __syncthreads();
     }
-  if (threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
+  if (threadIdx.x >= kLive) return;
+  auto live_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kLive) : "memory"); };
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double C = dsc[S_OC_C], B = dsc[S_OC_B];
   double a = dsc[S_OC_MUA], b = dsc[S_OC_MUB];
   // up to kCache ambiguous elements are staged in shared memory, so the
@@ -559,9 +572,12 @@ __global__ void k_oc_finish(const float2* __restrict__ s, const float2* __restri
   // same order as the loads below otherwise
   constexpr int kCache = 256;
   __shared__ double cs[kCache], cl[kCache], ch[kCache], cd[kCache];
+  __shared__ double mid[kPath], gmid[kPath], ends[4];
+  __shared__ bool guess[kPath];
+  __shared__ int steps;  // midpoints laid out this round; 0 once the bisection has ended
   const bool cached = namb <= kCache;
   if (cached) {
-    for (int i = lane; i < namb; i += 32) {
+    for (int i = threadIdx.x; i < namb; i += kLive) {
       const int e = CK(i, kOcAmbMax) ? key[i] : 0;
       const bool ok = CK(e, ne);
       cs[i] = ok ? df_to_double(ld2(s, e)) : 0.0;
@@ -569,8 +585,8 @@ __global__ void k_oc_finish(const float2* __restrict__ s, const float2* __restri
       ch[i] = ok ? df_to_double(ld2(hi, e)) : 0.0;
       cd[i] = ok ? df_to_double(ld2(dv, e)) : 0.0;
     }
-    __syncwarp();
   }
+  live_sync();
   auto g = [&](double mu) {
     double acc = 0.0;
     if (cached) {
@@ -588,19 +604,62 @@ __global__ void k_oc_finish(const float2* __restrict__ s, const float2* __restri
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     return C + B * mu + acc;
   };
-  const double ga = g(a), gb = g(b);
+  if (warp < 2) {
+    const double v = g(warp == 0 ? a : b);
+    if (lane == 0) ends[warp] = v;
+  }
+  live_sync();
+  double ga = ends[0], gb = ends[1];
   if (!(ga <= volfrac && volfrac <= gb)) {
-    if (lane == 0) dsc[S_OC_FAIL] = 1.0;
+    if (threadIdx.x == 0) dsc[S_OC_FAIL] = 1.0;
     return;
   }
-  for (int it = 0; it < 200; ++it) {
-    const double mid = 0.5 * (a + b);
-    if (!(mid > a && mid < b)) break;
-    if ((b - a) <= 1e-15 * b) break;
-    if (g(mid) >= volfrac) b = mid;
-    else a = mid;
+  // warp 0 keeps the bracket; at most 200 steps (a round takes one at least)
+  int it = 0;
+  for (int round = 0; round < 200; ++round) {
+    if (warp == 0) {
+      const double root = a + (volfrac - ga) * ((b - a) / (gb - ga));
+      double pa = a, pb = b;
+      int m = 0;
+      for (; m < kPath && it + m < 200; ++m) {
+        const double p = 0.5 * (pa + pb);
+        if (!(p > pa && p < pb)) break;
+        if ((pb - pa) <= 1e-15 * pb) break;
+        const bool below = p >= root;  // the root lies at or below p
+        if (lane == 0) {
+          mid[m] = p;
+          guess[m] = below;
+        }
+        if (below) pb = p;
+        else pa = p;
+      }
+      if (lane == 0) steps = m;
+    }
+    live_sync();
+    const int m = steps;
+    if (m == 0) break;
+    if (warp < m) {
+      const double v = g(mid[warp]);
+      if (lane == 0) gmid[warp] = v;
+    }
+    live_sync();
+    if (warp == 0) {
+      for (int q = 0; q < m; ++q) {
+        const bool below = gmid[q] >= volfrac;
+        ++it;
+        if (below) {
+          b = mid[q];
+          gb = gmid[q];
+        } else {
+          a = mid[q];
+          ga = gmid[q];
+        }
+        if (below != guess[q]) break;
+      }
+      __syncwarp();  // the round's values are read before the next ones are written
+    }
   }
-  if (lane == 0) dsc[S_OC_MU] = 0.5 * (a + b);
+  if (threadIdx.x == 0) dsc[S_OC_MU] = 0.5 * (a + b);
 }
 
 // rho <- clamp(s mu) for mu = dsc[S_OC_MU]; max |change| into dsc.  Skipped
@@ -825,7 +884,8 @@ void set_density(Ctx& c, const double* rho, bool physical) {
     k_to_df<<<blocks_for(c.ne), kThreads, 0, c.stream>>>(rho, c.df_e, (int)c.ne);
     MGAR_LAUNCH_CHECK();
     const df kmin_df = df_from_double(c.p.kmin), dk_df = df_from_double(c.p.k0 - c.p.kmin);
-    const SimpArgs a{c.inv_hs_df, c.p.k0, c.p.kmin, c.p.penal, make_float2(kmin_df.hi, kmin_df.lo),
+    const SimpArgs a{c.inv_hs_df, c.p.k0, c.p.kmin, c.p.penal, c.p.penal == 3.0,
+                     make_float2(kmin_df.hi, kmin_df.lo),
                      make_float2(dk_df.hi, dk_df.lo), c.rho_phys, c.rho_phys_df, c.ke, c.ke_f,
                      c.ke_df};
     if (filter3d_ok(c)) {
@@ -873,11 +933,11 @@ void sensitivity(Ctx& c, const double* T, double* dc, double* dv, double* compli
     if (c.dim == 2)
       k_sens_df<2><<<blocks_for(c.ne), kThreads, 0, c.stream>>>(T_df, c.rho_phys, c.rho_phys_df,
                                                                 c.inv_hs_df, c.df_e, d, mcoef_df,
-                                                                c.p.penal);
+                                                                c.p.penal, c.p.penal == 3.0);
     else
       k_sens_df<3><<<blocks_for(c.ne), kThreads, 0, c.stream>>>(T_df, c.rho_phys, c.rho_phys_df,
                                                                 c.inv_hs_df, c.df_e, d, mcoef_df,
-                                                                c.p.penal);
+                                                                c.p.penal, c.p.penal == 3.0);
     MGAR_LAUNCH_CHECK();
     if (filter3d_ok(c)) {
       filter3d_t(c, c.df_e, dc_df ? nullptr : dc, dc_df);

@@ -440,26 +440,33 @@ int runs(const Ctx& c, int sms) {
 // kd_i = 4 sum_e k_e over the (up to 8) elements around node i, df64: a
 // TwoSum chain of the high words, low words and errors added, then
 // normalised; the factor 4 is exact
-__global__ void k_node_kdiag(const float2* __restrict__ ke, float2* __restrict__ kd, int ex, int ey,
-                             int ez) {
-  const int NX = ex + 1, NY = ey + 1, NZ = ez + 1;
-  const int64_t n = (int64_t)NX * NY * NZ;
-  const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= n) return;
-  const int i = (int)(id % NX), j = (int)((id / NX) % NY), k = (int)(id / ((int64_t)NX * NY));
+__global__ void k_node_kdiag(const float2* __restrict__ ke, float2* __restrict__ kd, Dims d) {
+  const int id = blockIdx.x * blockDim.x + threadIdx.x;
+  if (id >= (int)d.n) return;
+  int i, j, k;
+  coords(id, d.fNX, d.fNXY, i, j, k);
+  // the eight loads under way together (elements off the grid: a valid
+  // address, dropped below)
+  float2 v[8];
+  bool ok[8];
+#pragma unroll
+  for (int o = 0; o < 8; ++o) {
+    const int e0 = i - 1 + (o & 1), e1 = j - 1 + ((o >> 1) & 1), e2 = k - 1 + (o >> 2);
+    ok[o] = (unsigned)e0 < (unsigned)d.ex && (unsigned)e1 < (unsigned)d.ey && (unsigned)e2 < (unsigned)d.ez;
+    v[o] = ke[ok[o] ? e0 + d.ex * (e1 + d.ey * e2) : 0];
+  }
   float s = 0.f, t = 0.f;
-  for (int dz = -1; dz <= 0; ++dz)
-    for (int dy = -1; dy <= 0; ++dy)
-      for (int dx = -1; dx <= 0; ++dx) {
-        const int e0 = i + dx, e1 = j + dy, e2 = k + dz;
-        if (e0 < 0 || e0 >= ex || e1 < 0 || e1 >= ey || e2 < 0 || e2 >= ez) continue;
-        const float2 v = ke[e0 + (int64_t)ex * (e1 + (int64_t)ey * e2)];
-        float r;
-        two_sum(s, v.x, s, r);
-        t = __fadd_rn(t, __fadd_rn(r, v.y));
-      }
-  const df d = df_make(s, t);
-  kd[id] = make_float2(4.f * d.hi, 4.f * d.lo);
+#pragma unroll
+  for (int o = 0; o < 8; ++o) {
+    float u, r;
+    two_sum(s, v[o].x, u, r);
+    if (ok[o]) {
+      s = u;
+      t = __fadd_rn(t, __fadd_rn(r, v[o].y));
+    }
+  }
+  const df q = df_make(s, t);
+  kd[id] = make_float2(4.f * q.hi, 4.f * q.lo);
 }
 
 }  // namespace d3d
@@ -467,7 +474,7 @@ __global__ void k_node_kdiag(const float2* __restrict__ ke, float2* __restrict__
 // per-node diagonal factor of the df64 operator for the current k_e
 void df3d_node_diag(Ctx& c) {
   const Dims& d = c.L[0];
-  d3d::k_node_kdiag<<<blocks_for(d.n), kThreads, 0, c.stream>>>(c.ke_df, c.kd_df, d.ex, d.ey, d.ez);
+  d3d::k_node_kdiag<<<blocks_for(d.n), kThreads, 0, c.stream>>>(c.ke_df, c.kd_df, d);
   MGAR_LAUNCH_CHECK();
 }
 

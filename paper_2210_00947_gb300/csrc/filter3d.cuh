@@ -11,6 +11,7 @@ namespace mgar {
 struct SimpArgs {
   const float2* inv_hs;
   double k0, kmin, penal;
+  int cubic;  // penal == 3, compared once on the host
   float2 kmin_df, dk_df;
   double* rho_phys;
   float2* rho_df;
@@ -26,7 +27,7 @@ __device__ __forceinline__ void simp_store(const SimpArgs& a, int e, df s) {
   a.rho_phys[e] = df_to_double(r);
   a.rho_df[e] = make_float2(r.hi, r.lo);  // the pair k_e comes from (rho_phys: its FP64 rounding)
   df kv;
-  if (a.penal == 3.0) {
+  if (a.cubic) {
     kv = df_add(df{a.kmin_df.x, a.kmin_df.y},
                 df_mul(df{a.dk_df.x, a.dk_df.y}, df_mul(df_mul(r, r), r)));
   } else {

@@ -277,20 +277,6 @@ __global__ void __launch_bounds__(NT, 2) k_fine3l(Args a) {
   }
 }
 
-// Conductivities at node pitch and the signed inverse diagonal.
-__global__ void k_node_pitch(const float* __restrict__ ke, const uint8_t* __restrict__ fixed, Dims d,
-                             float* __restrict__ kn, float* __restrict__ dinv_s,
-                             const float* __restrict__ dinv) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int)d.n) return;
-  int i, j, k;
-  coords(idx, d.fNX, d.fNXY, i, j, k);
-  float v = 0.f;
-  if (i < d.ex && j < d.ey && k < d.ez) v = ke[i + d.ex * (j + d.ey * k)];
-  kn[idx] = v;
-  dinv_s[idx] = fixed[idx] ? -1.f : dinv[idx];
-}
-
 // Segment length and cells per thread: a segment of L nodes stages L + 2 NX + 2
 // cells, NT at a time, and its cost is about 12 instructions per staged cell
 // and 45 per node.
@@ -370,14 +356,6 @@ void fine3l_prepare(Ctx& c) {
       c.f3l_gz = g;
     }
   }
-}
-
-// after every change of the reference design
-void fine3l_build(Ctx& c) {
-  const Dims& d = c.L[0];
-  f3l::k_node_pitch<<<blocks_for(d.n), kThreads, 0, c.stream>>>(c.ke0_f, c.fixed, d, c.kn0,
-                                                                 c.h32[0].dinv_s, c.h32[0].dinv);
-  MGAR_LAUNCH_CHECK();
 }
 
 void fine3l(Ctx& c, int mode, const float* b, const float* x, float* out0, float* out1,

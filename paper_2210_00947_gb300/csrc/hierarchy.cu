@@ -294,18 +294,17 @@ __global__ void k_assemble(const Real* __restrict__ elem, Dims d, Real* __restri
   dinv[idx] = Real(1) / acc[S / 2];
 }
 
-// Inverse diagonal of the matrix-free finest operator (1 on fixed nodes); 2D:
-// also negated on the fixed nodes, for the tiled passes.
+// Inverse diagonal of the matrix-free finest operator (1 on fixed nodes); also
+// negated on the fixed nodes (dinv_s: 2D, and 3D where kn is wanted) and the
+// conductivities at node pitch (kn, 3D: element (i, j, k) at node (i, j, k),
+// zero where there is none) for the passes on segments.
 template <typename Real, int DIM>
 __global__ void k_fine_dinv(const Real* __restrict__ ke, const uint8_t* __restrict__ fixed, Dims d,
-                            Real* __restrict__ dinv, Real* __restrict__ dinv_s) {
+                            Real* __restrict__ dinv, Real* __restrict__ dinv_s,
+                            Real* __restrict__ kn) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int)d.n) return;
-  if (fixed[idx]) {
-    dinv[idx] = Real(1);
-    if (DIM == 2) dinv_s[idx] = Real(-1);
-    return;
-  }
+  const bool fx = fixed[idx] != 0;
   int i, j, k;
   coords(idx, d.fNX, d.fNXY, i, j, k);
   Real ks = Real(0);
@@ -318,10 +317,11 @@ __global__ void k_fine_dinv(const Real* __restrict__ ke, const uint8_t* __restri
     const int e = ok ? exi + d.ex * (eyi + d.ey * ezi) : 0;  // valid address either way
     const Real kv = CK(e, d.ne) ? ke[e] : Real(0);
     if (ok) ks += kv;
+    if (DIM == 3 && o == 0 && kn) kn[idx] = ok ? kv : Real(0);
   }
   const Real dv = Real(1) / (ks * Real(DIM == 2 ? 4.0 / 6.0 : 4.0 / 12.0));
-  dinv[idx] = dv;
-  if (DIM == 2) dinv_s[idx] = dv;
+  dinv[idx] = fx ? Real(1) : dv;
+  if (DIM == 2 || kn) dinv_s[idx] = fx ? Real(-1) : dv;
 }
 
 // Lower band of the coarsest operator: band[i*(bw+1) + (j - i + bw)].
@@ -1001,8 +1001,9 @@ static void build_levels(Ctx& c, const Real* ke0, LevelBuf<Real>* h) {
   const int nen = 1 << DIM;
   const double* k0 = c.tables;
   const Real* G = g_tables<Real>(c);
-  k_fine_dinv<Real, DIM><<<blocks_for(c.L[0].n), kThreads, 0, s>>>(ke0, c.fixed, c.L[0], h[0].dinv,
-                                                                        h[0].dinv_s);
+  k_fine_dinv<Real, DIM><<<blocks_for(c.L[0].n), kThreads, 0, s>>>(
+      ke0, c.fixed, c.L[0], h[0].dinv, h[0].dinv_s,
+      std::is_same<Real, float>::value ? reinterpret_cast<Real*>(c.kn0) : nullptr);
   MGAR_LAUNCH_CHECK();
   for (int l = 0; l + 1 < c.nl; ++l) {
     const Dims& f = c.L[l];
@@ -1043,7 +1044,6 @@ void build_hierarchy(Ctx& c) {
     MGAR_LAUNCH_CHECK();
     if (c.dim == 2) build_levels<float, 2>(c, c.ke0_f, c.h32);
     else build_levels<float, 3>(c, c.ke0_f, c.h32);
-    if (c.kn0) fine3l_build(c);
   }
   c.have_ref = true;
 }
