@@ -317,7 +317,18 @@ struct CoarseT {
 // first thing, a hardware wait until the predecessor has completed and its
 // memory is visible, so only launch latency and block dispatch overlap.
 // pdl_trigger() lets the successor be dispatched before this grid ends.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The compiler may move a load through a const __restrict__ pointer over the
+// wait, whose memory clobber does not order loads of memory it takes to be
+// constant: in straight-line code it did, and the row read its operand before
+// the predecessor had written it.  Such loads keep their basic block, so the
+// wait ends one: the branch goes away in the assembler, after the loads have
+// been placed.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  unsigned never;
+  asm volatile("mov.u32 %0, 0;" : "=r"(never));
+  if (never != 0u) asm volatile("exit;" ::: "memory");
+}
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // handle whose API call is running on this host thread (set by the C ABI)
@@ -1102,6 +1113,46 @@ __device__ __forceinline__ Real stencil_apply(const StencilOp<Real>& op, const R
   Real acc = Real(0);
 #pragma unroll
   for (int s = 0; s < S; ++s) acc += sv[s] * xv[s];
+  return acc;
+}
+
+// The 3D row by flat offsets, for a block of nodes [i0, i1) whose neighbours'
+// flat indices all lie in the array (stencil_flat): a neighbour outside the
+// grid is the flat array's node at the other end of the row, the row before or
+// the plane before, and its coefficient is zero by itself (an upper slot holds
+// the zero; a lower one is the mirror slot of a node whose own neighbour lies
+// outside).  No coordinates, clamps or tests, the same products in the same
+// order.  65^3 nodes: residual 8.4 -> 8.2 us, sweep 7.1 -> 6.1 us; 129^3: 42.4
+// -> 39.2 and 41.2 -> 39.3 us (21 us of bytes; the 27 coefficients' loads, half
+// of them a second time through the caches, bound it).
+template <typename Real>
+__device__ __forceinline__ bool stencil_flat(const StencilOp<Real>& op, int i0, int i1) {
+  const int h = op.NX * op.NY + op.NX + 1;
+  return i0 >= h && i1 <= op.n - h;
+}
+template <typename Real>
+__device__ __forceinline__ void stencil_coefs_flat(const StencilOp<Real>& op, int idx, Real (&sv)[27]) {
+  const int NX = op.NX, NXY = op.NX * op.NY;
+#pragma unroll
+  for (int s = 0; s < 27; ++s) {
+    const int off = (s % 3 - 1) + NX * ((s / 3) % 3 - 1) + NXY * (s / 9 - 1);
+    sv[s] = s >= 13 ? op.st[(s - 13) * op.n + idx] : op.st[(13 - s) * op.n + (idx + off)];
+  }
+}
+template <typename Real>
+__device__ __forceinline__ Real stencil_apply_flat(const StencilOp<Real>& op, const Real* x, int idx,
+                                                   const Real (&sv)[27]) {
+  Real xv[27];
+#pragma unroll
+  for (int q = 0; q < 9; ++q) {
+    const Real* row = x + (idx + op.NX * (q % 3 - 1) + op.NX * op.NY * (q / 3 - 1));
+    xv[3 * q] = row[-1];
+    xv[3 * q + 1] = row[0];
+    xv[3 * q + 2] = row[1];
+  }
+  Real acc = Real(0);
+#pragma unroll
+  for (int s = 0; s < 27; ++s) acc += sv[s] * xv[s];
   return acc;
 }
 

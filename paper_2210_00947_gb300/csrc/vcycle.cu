@@ -298,18 +298,130 @@ __global__ void k_prolong3(const Real* __restrict__ xc, const Real* cur, Real* d
 // of those loads overlaps the predecessor's tail; the arithmetic and its
 // order are unchanged.
 template <typename Real, int DIM>
-__global__ void k_resid_coarse(StencilOp<Real> op, const Real* __restrict__ b,
-                               const Real* __restrict__ x, Real* __restrict__ r) {
+__global__ void k_resid_coarse(StencilOp<Real> op, const Real* b, const Real* x, Real* r) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   const bool on = idx < op.n;
   int i = 0, j = 0, k = 0;
   Real sv[stencil_size<DIM>()];
+  if constexpr (DIM == 3) {
+    const int i0 = blockIdx.x * blockDim.x;
+    if (stencil_flat(op, i0, i0 + (int)blockDim.x)) {
+      stencil_coefs_flat(op, idx, sv);
+      pdl_wait();
+      r[idx] = b[idx] - stencil_apply_flat(op, x, idx, sv);
+      pdl_trigger();
+      return;
+    }
+  }
   if (on) {
     coords(idx, op.fNX, op.fNXY, i, j, k);
     stencil_coefs<DIM>(op, i, j, k, sv);
   }
   pdl_wait();
   if (on) r[idx] = b[idx] - stencil_apply<DIM, Real, false>(op, x, i, j, k, sv);
+  pdl_trigger();
+}
+
+// Small FP32 levels, 3D: the residual and its restriction in one launch.  A
+// level of at most split_coarse_nodes nodes takes 3 to 4 us in either kernel,
+// launch and round trips; here a block forms the residuals that its 4^3 coarse
+// nodes read (9^3, one per thread, a share of 0.42 of them also formed by a
+// neighbour) in shared memory.  33^3 -> 17^3 nodes: 4.0 + 3.6 -> 6.0 us, 17^3
+// -> 9^3: 3.7 + 3.3 -> 4.6 us.
+constexpr int kRR = 4, kRRF = 2 * kRR + 1, kRRThreads = 736;  // 23 warps >= 9^3
+__global__ void __launch_bounds__(kRRThreads) k_resid_restrict3(
+    StencilOp<float> op, const float* b, const float* x, Dims f, Dims cd,
+    const float* __restrict__ dinvc, float omega, float* bc, float* xc) {
+  __shared__ float rs[kRRF][kRRF][kRRF];
+  const int t = threadIdx.x;
+  const int tx = t % kRRF, ty = (t / kRRF) % kRRF, tz = t / (kRRF * kRRF);
+  const int i = 2 * kRR * blockIdx.x - 1 + tx, j = 2 * kRR * blockIdx.y - 1 + ty,
+            k = 2 * kRR * blockIdx.z - 1 + tz;
+  const bool tile = tz < kRRF;
+  const bool on = tile && i >= 0 && i < f.NX && j >= 0 && j < f.NY && k >= 0 && k < f.NZ;
+  const int idx = i + f.NX * (j + f.NY * k);
+  float sv[27];
+  if (on) stencil_coefs<3>(op, i, j, k, sv);
+  // the coarse node of this thread
+  const int I = kRR * blockIdx.x + t % kRR, J = kRR * blockIdx.y + (t / kRR) % kRR,
+            K = kRR * blockIdx.z + t / (kRR * kRR);
+  const bool coarse = t < kRR * kRR * kRR && I < cd.NX && J < cd.NY && K < cd.NZ;
+  const int ci = I + cd.NX * (J + cd.NY * K);
+  const float dc = coarse && xc ? dinvc[ci] : 0.f;
+  pdl_wait();
+  float rv = 0.f;
+  if (on) rv = b[idx] - stencil_apply<3, float, false>(op, x, i, j, k, sv);
+  if (tile) rs[tz][ty][tx] = rv;
+  pdl_trigger();
+  __syncthreads();
+  if (!coarse) return;
+  int ix[3], iy[3], iz[3];
+  float wx[3], wy[3], wz[3];
+  restrict_taps(I, f.ex, ix, wx);
+  restrict_taps(J, f.ey, iy, wy);
+  restrict_taps(K, f.ez, iz, wz);
+  const int lx = 2 * (t % kRR), ly = 2 * ((t / kRR) % kRR), lz = 2 * (t / (kRR * kRR));
+  float acc = 0.f;
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const float wyz = wy[q] * wz[c];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) acc += (wyz * wx[a]) * rs[lz + c][ly + q][lx + a];
+    }
+  bc[ci] = acc;
+  if (xc) xc[ci] = omega * dc * acc;
+}
+
+// FP32 restriction of the finest level's residual, 3D: a thread owns a column
+// of coarse nodes and kRestrictChunk coarse planes; each fine plane's 3 x 3
+// weighted sum serves the one or two coarse planes that read it, so a coarse
+// node costs 22 loads without clamps instead of 27 with a weight and an index
+// formed for each (390 instructions).  65^3 coarse nodes: 7.6 -> 6.3 us,
+// 129^3: 41 -> 27 us; on few nodes the chain of planes costs more (38 x 27 x 21
+// coarse nodes: 3.1 -> 4.8 us), so it is taken above split_coarse_nodes.
+constexpr int kRestrictChunk = 2;
+__global__ void k_restrict3(const float* r, float* bc, Dims f, Dims cd,
+                            const float* __restrict__ dinvc, float omega, float* xc) {
+  constexpr int KC = kRestrictChunk, NP = 2 * KC + 1;
+  const int cNXY = cd.NX * cd.NY, col = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool on = col < cNXY;
+  const int J = on ? col / cd.NX : 0, I = on ? col - J * cd.NX : 0, K0 = blockIdx.y * KC;
+  int ix[3], iy[3];
+  float wx[3], wy[3];
+  restrict_taps(I, f.ex, ix, wx);
+  restrict_taps(J, f.ey, iy, wy);
+  float dc[KC];
+#pragma unroll
+  for (int u = 0; u < KC; ++u) dc[u] = on && xc && K0 + u < cd.NZ ? dinvc[col + cNXY * (K0 + u)] : 0.f;
+  pdl_wait();
+  if (on) {
+    float s[NP];  // fine planes 2 K0 - 1 .. 2 K0 + 2 KC - 1
+#pragma unroll
+    for (int t = 0; t < NP; ++t) {
+      const int k = 2 * K0 - 1 + t;
+      s[t] = 0.f;
+      if (k < 0 || k >= f.NZ) continue;
+      const float* plane = r + (int64_t)f.NX * f.NY * k;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const float* row = plane + f.NX * iy[q];
+        s[t] += wy[q] * (wx[0] * row[ix[0]] + wx[1] * row[ix[1]] + wx[2] * row[ix[2]]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < KC; ++u) {
+      const int K = K0 + u;
+      if (K >= cd.NZ) break;
+      int iz[3];
+      float wz[3];
+      restrict_taps(K, f.ez, iz, wz);
+      const float acc = wz[0] * s[2 * u] + wz[1] * s[2 * u + 1] + wz[2] * s[2 * u + 2];
+      bc[col + cNXY * K] = acc;
+      if (xc) xc[col + cNXY * K] = omega * dc[u] * acc;
+    }
+  }
   pdl_trigger();
 }
 
@@ -333,14 +445,25 @@ __global__ void k_post_coarse(StencilOp<Real> op, const Real* __restrict__ xc,
 
 // One damped-Jacobi sweep on an assembled level, x' = x + w D^-1 (b - A x).
 template <typename Real, int DIM>
-__global__ void k_jacobi_st(StencilOp<Real> op, const Real* __restrict__ b,
-                            const Real* __restrict__ xin, Real* __restrict__ xout,
+__global__ void k_jacobi_st(StencilOp<Real> op, const Real* b, const Real* xin, Real* xout,
                             const Real* __restrict__ dinv, Real omega) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   const bool on = idx < op.n;
   int i = 0, j = 0, k = 0;
   Real sv[stencil_size<DIM>()];
   Real dv = Real(0);
+  if constexpr (DIM == 3) {
+    const int i0 = blockIdx.x * blockDim.x;
+    if (stencil_flat(op, i0, i0 + (int)blockDim.x)) {
+      stencil_coefs_flat(op, idx, sv);
+      dv = dinv[idx];
+      pdl_wait();
+      const Real ax = stencil_apply_flat(op, xin, idx, sv);
+      xout[idx] = xin[idx] + omega * dv * (b[idx] - ax);
+      pdl_trigger();
+      return;
+    }
+  }
   if (on) {
     coords(idx, op.fNX, op.fNXY, i, j, k);
     stencil_coefs<DIM>(op, i, j, k, sv);
@@ -733,14 +856,38 @@ static void vcycle_fused3(Ctx& c, const Real* b0, Real* x0, bool zero_guess,
   // the tiled 3D kernels leave r = 0 on fixed nodes, which P^T = (Z P)^T ignores
   // each restriction into a level above the coarsest also leaves that
   // level's zero-guess sweep x = w D^-1 b
-  launch_pdl(c.stream, c.use_pdl, k_restrict<Real, DIM>, dim3(blocks_for(c.L[1].n)), dim3(kThreads),
-             (const Real*)h[0].r, h[1].b, d0, c.L[1], (const uint8_t*)nullptr,
-             (const Real*)h[1].dinv, om, nl > 2 ? h[1].x : (Real*)nullptr);
+  Real* const x1 = nl > 2 ? h[1].x : nullptr;
+  const Dims& d1 = c.L[1];
+  bool columns = false;
+  if constexpr (std::is_same<Real, float>::value) {
+    columns = d1.n > c.split_coarse_nodes;
+    if (columns)
+      launch_pdl(c.stream, c.use_pdl, k_restrict3,
+                 dim3(blocks_for((int64_t)d1.NX * d1.NY), (d1.NZ + kRestrictChunk - 1) / kRestrictChunk),
+                 dim3(kThreads), (const float*)h[0].r, h[1].b, d0, d1, (const float*)h[1].dinv, om, x1);
+  }
+  if (!columns) {
+    launch_pdl(c.stream, c.use_pdl, k_restrict<Real, DIM>, dim3(blocks_for(c.L[1].n)), dim3(kThreads),
+               (const Real*)h[0].r, h[1].b, d0, c.L[1], (const uint8_t*)nullptr,
+               (const Real*)h[1].dinv, om, x1);
+  }
   MGAR_LAUNCH_CHECK_AT(level_site(3, 0));
   const int lb = sizeof(Real) == 4 ? bottom_level(c) : nl;
   // coarse levels, down
   for (int l = 1; l + 1 < nl && l < lb; ++l) {
     const Dims& d = c.L[l];
+    if constexpr (std::is_same<Real, float>::value) {
+      if (d.n <= c.split_coarse_nodes) {
+        const Dims& e = c.L[l + 1];
+        const auto tiles = [](int n) { return (unsigned)((n + kRR - 1) / kRR); };
+        launch_pdl(c.stream, c.use_pdl, k_resid_restrict3, dim3(tiles(e.NX), tiles(e.NY), tiles(e.NZ)),
+                   dim3(kRRThreads), stencil_row<Real, DIM>(c, l).op, (const float*)h[l].b,
+                   (const float*)h[l].x, d, e, (const float*)h[l + 1].dinv, om, h[l + 1].b,
+                   l + 2 < nl ? h[l + 1].x : (float*)nullptr);
+        MGAR_LAUNCH_CHECK_AT(level_site(0, l));
+        continue;
+      }
+    }
     launch_pdl(c.stream, c.use_pdl, k_resid_coarse<Real, DIM>, dim3(blocks_for(d.n)), dim3(kThreads),
                stencil_row<Real, DIM>(c, l).op, (const Real*)h[l].b, (const Real*)h[l].x, h[l].r);
     MGAR_LAUNCH_CHECK_AT(level_site(0, l));
