@@ -248,6 +248,8 @@ __global__ void __launch_bounds__(kRedThreads) kb_dot_py(const Des* D, const int
   const int it = (int)s[BS_IT];
   const float2* __restrict__ p = p_new(g, it);
   const float2* __restrict__ y = g.Ap;
+  const SumOut out{s + BS_PAP, s + BS_RZ + (it & 1), nullptr, s + BS_ALPHA, 1};
+  const double other = sum_other(out, threadIdx.x == 0);
   float2 pv[kNptR * kSumVB], yv[kNptR * kSumVB];
   double t;
   if (ordered_sum<kNptR>(
@@ -258,7 +260,7 @@ __global__ void __launch_bounds__(kRedThreads) kb_dot_py(const Des* D, const int
           },
           [&](int q) { return df_mul(unpack(pv[q]), unpack(yv[q])); }) &&
       threadIdx.x == 0)
-    sum_out(SumOut{s + BS_PAP, s + BS_RZ + (it & 1), nullptr, s + BS_ALPHA, 1}, t);
+    sum_out(out, t, other);
 }
 
 // r . z and beta = r . z / (r . z)_old
@@ -272,6 +274,13 @@ __global__ void __launch_bounds__(kRedThreads) kb_dot_rz(const Des* D, const int
   const Des& g = D[d];
   double* s = bsc + d * kBS;
   const int it = (int)s[BS_IT];
+  SumOut out{s + BS_RZ + (it & 1)};
+  if (it > 0) {
+    out.den = s + BS_RZ + ((it - 1) & 1);
+    out.q = s + BS_BETA;
+    out.pair = 1;
+  }
+  const double other = sum_other(out, threadIdx.x == 0);
   float2 rv[kNptR * kSumVB];
   float zv[kNptR * kSumVB];
   double t;
@@ -282,15 +291,8 @@ __global__ void __launch_bounds__(kRedThreads) kb_dot_rz(const Des* D, const int
             zv[q] = g.x32[idx];
           },
           [&](int q) { return df_mulf(unpack(rv[q]), zv[q]); }) &&
-      threadIdx.x == 0) {
-    SumOut out{s + BS_RZ + (it & 1)};
-    if (it > 0) {
-      out.den = s + BS_RZ + ((it - 1) & 1);
-      out.q = s + BS_BETA;
-      out.pair = 1;
-    }
-    sum_out(out, t);
-  }
+      threadIdx.x == 0)
+    sum_out(out, t, other);
 }
 
 // x += alpha p; r -= alpha Ap; ||r||^2; FP32 copy of r.

@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(l2d::kThreads2) k_df_dir2(DfOp op, const float
   __shared__ DfDirSmem s;
   pdl_wait();
   pdl_trigger();
-  if (parity && (((int)*parity) & 1)) {
+  if (parity && is_set(parity)) {
     float2* t = const_cast<float2*>(p_old);
     p_old = p;
     p = t;
@@ -65,7 +65,8 @@ __global__ void __launch_bounds__(kThreads) k_dot_py(const float2* __restrict__ 
                                                      SumOut out) {
   pdl_wait();
   pdl_trigger();
-  if (parity && (((int)*parity) & 1)) p = p_alt;
+  if (parity && is_set(parity)) p = p_alt;
+  const double other = sum_other(out, threadIdx.x == 0);
   float2 pv[2 * kSumVB], yv[2 * kSumVB];
   double t;
   if (ordered_sum<2>(
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(kThreads) k_dot_py(const float2* __restrict__ 
           },
           [&](int q) { return df_mul(unpack(pv[q]), unpack(yv[q])); }) &&
       threadIdx.x == 0)
-    sum_out(out, t);
+    sum_out(out, t, other);
 }
 
 // p . A p into S_PAP and alpha = *rz / p . A p into S_ALPHA
@@ -129,7 +130,7 @@ __global__ void __launch_bounds__(kThreads) k_df_cg_xr(float2* __restrict__ x, f
   pdl_wait();
   // device-side CG loop: the two direction buffers swap with the parity
   // (every block reads it before the last one flips it)
-  if (parity && (((int)*parity) & 1)) p = p_alt;
+  if (parity && is_set(parity)) p = p_alt;
   const df alpha = load_pair(alpha_p);
   df acc{0.f, 0.f};
   const int stride = gridDim.x * blockDim.x;
@@ -525,7 +526,7 @@ __global__ void __launch_bounds__(kThreads) k_cg_xr32(float* __restrict__ xc, fl
                                                       cudaGraphConditionalHandle ru, int set) {
   pdl_wait();
   // every block reads the parity before the last one flips it
-  if (parity && (((int)*parity) & 1)) p = p_alt;
+  if (parity && is_set(parity)) p = p_alt;
   const float alpha = load_pair(alpha_p).hi;
   float acc = 0.f;
   const int stride = gridDim.x * blockDim.x;
@@ -634,17 +635,20 @@ __global__ void k_ru_loop(double* dsc, double qnorm, double eps2, int cg_max,
 // host reads the decision.
 static void ru_iteration(Ctx& c, cudaGraphConditionalHandle ru, bool set) {
   const int n = (int)c.n;
+  // the FP32 vectors read the quotients' high words
+  SumOut rz = rz_out(c, S_RZ1, S_RZ0), pap = pap_out(c, c.dsc + S_RZ1);
+  rz.pair = pap.pair = 2;
   if (set) {
-    vcycle_dot(c, c.b32, c.x32, nullptr, rz_out(c, S_RZ1, S_RZ0));
+    vcycle_dot(c, c.b32, c.x32, nullptr, rz);
   } else {
     const bool prof_inside = c.prof_class == MGAR_KC_SMOOTH0 || c.prof_class == MGAR_KC_RESID0;
     run_graph(c, 10, c.b32, c.x32, prof_inside,
-              [&] { vcycle_dot(c, c.b32, c.x32, nullptr, rz_out(c, S_RZ1, S_RZ0)); });
+              [&] { vcycle_dot(c, c.b32, c.x32, nullptr, rz); });
   }
   {
     ProfScope ps(c, MGAR_KC_APPLY32);
     fine3d_dir(c, c.x32, c.p32, c.p32b, c.dsc + S_BETA, c.dsc + S_CGFIRST, c.dsc + S_CGPAR, c.y32,
-               pap_out(c, c.dsc + S_RZ1), c.dsc + S_RZ1, c.dsc + S_RZ0);
+               pap, c.dsc + S_RZ1, c.dsc + S_RZ0);
   }
   // parity 0: the new p is in p32b
   launch_pdl(c.stream, c.use_pdl, k_cg_xr32, dim3(xr32_blocks(c)), dim3(kThreads), c.xc32,

@@ -523,9 +523,9 @@ __device__ __forceinline__ bool block_sum_last_one(bool pair, double w, df wp, d
   }
   __syncthreads();
   // 0 + v_0 + v_1 + ..., v_q in lane q
-  auto in_order = [&](double v) {
+  auto in_order = [&](double v, int count) {
     double s = 0.0;
-    for (int q = 0; q < nw; ++q) s += __shfl_sync(0xffffffffu, v, q);
+    for (int q = 0; q < count; ++q) s += __shfl_sync(0xffffffffu, v, q);
     return s;
   };
   if (warp == 0) {
@@ -538,7 +538,7 @@ __device__ __forceinline__ bool block_sum_last_one(bool pair, double w, df wp, d
         v = sh[lane];
       }
     }
-    const double s = in_order(v);
+    const double s = in_order(v, nw);
     if (lane == 0) {
       if (CK(bid, g_partials_len)) partials[bid] = s;
       __threadfence();
@@ -548,22 +548,29 @@ __device__ __forceinline__ bool block_sum_last_one(bool pair, double w, df wp, d
   __syncthreads();
   if (!last) return false;
   __threadfence();
-  // L2-coherent loads, four rows of blocks in flight together
+  // L2-coherent loads, four rows of blocks in flight together.  Additions of
+  // rows and warps without a partial are left out (they add zero): each would
+  // take about 20 clocks of the FP64 pipe per warp, 2 us for 300 partials and
+  // 16 warps.
   constexpr int U = 4;
+  const int used = min(nw, (nblk + 31) >> 5);
   double acc = 0.0;
-  for (int b = tid; b < nblk; b += U * nthr) {
+  for (int b = tid; b - lane < nblk; b += U * nthr) {
     double v[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) v[u] = b + u * nthr < nblk ? __ldcg(partials + b + u * nthr) : 0.0;
 #pragma unroll
-    for (int u = 0; u < U; ++u) acc += v[u];
+    for (int u = 0; u < U; ++u)
+      if (b - lane + u * nthr < nblk) acc += v[u];
   }
+  if (warp < used) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if (lane == 0) sh[warp] = acc;
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if (lane == 0) sh[warp] = acc;
+  }
   __syncthreads();
   if (warp == 0) {
-    total = in_order(lane < nw ? sh[lane] : 0.0);
+    total = in_order(lane < used ? sh[lane] : 0.0, used);
     if (lane == 0) *counter = 0u;
   }
   return true;
@@ -602,6 +609,16 @@ __device__ __forceinline__ bool block_sum_last_df(df v, double* partials, unsign
     v = df_add(v, df{h, l});
   }
   return block_sum_last_one(true, 0.0, v, partials, counter, total, tid, nthr, bid, nblk);
+}
+
+// The CG's scalars are read from L2: a line of them that one launch's blocks
+// bring into L1 may still be there, stale, for a launch that was started before
+// the scalar's writer had ended (the dependency wait does not drop it).
+//
+// *p != 0 for a flag kept as a double (0 or 1), by its bits: a comparison or
+// conversion on the FP64 pipe costs every warp about 20 clocks of it.
+__device__ __forceinline__ bool is_set(const double* p) {
+  return (__double_as_longlong(__ldcg(p)) << 1) != 0;
 }
 
 // Four sums at once: v[g] is thread tid's value of the virtual block vb0 + g of
@@ -652,22 +669,26 @@ __device__ __forceinline__ bool block_sums_last_df(const df (&v)[kSumVB], double
   __threadfence();
   constexpr int U = 4;
   double acc = 0.0;
-  for (int b = tid; b < nvb; b += U * kThreads) {
+  // (rows and warps without a partial add zero and are left out)
+  const int used = min(8, (nvb + 31) >> 5);
+  for (int b = tid; b - lane < nvb; b += U * kThreads) {
     double w[U];
 #pragma unroll
     for (int q = 0; q < U; ++q) w[q] = b + q * kThreads < nvb ? __ldcg(partials + b + q * kThreads) : 0.0;
 #pragma unroll
-    for (int q = 0; q < U; ++q) acc += w[q];
+    for (int q = 0; q < U; ++q)
+      if (b - lane + q * kThreads < nvb) acc += w[q];
   }
+  if (warp < used) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if (lane == 0) sh[warp] = acc;
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if (lane == 0) sh[warp] = acc;
+  }
   __syncthreads();
   if (warp == 0) {
-    const double w = sh[lane & 7];
+    const double w = lane < used ? sh[lane] : 0.0;
     double s = 0.0;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) s += __shfl_sync(0xffffffffu, w, q);
+    for (int q = 0; q < used; ++q) s += __shfl_sync(0xffffffffu, w, q);
     total = s;
     if (lane == 0) *counter = 0u;
   }
@@ -704,7 +725,10 @@ inline int sum_phys(int64_t n, int npt) {
 // Where a sum goes: *out, and with num or den also a quotient of the CG, *num
 // / sum or sum / *den, into *q as a double or as a df64 pair.  The block that
 // finishes the sum divides, so the next kernel's blocks read the quotient
-// instead of dividing each (an FP64 division is about 30 FP64 operations).
+// instead of dividing each (an FP64 division is about 30 FP64 operations, 0.6 us
+// at the end of the sum).  pair: 0 an FP64 quotient, 1 its df64 pair, 2 a df64
+// quotient (for the FP32 CG, which reads no more than its high word).  The other
+// operand is loaded before the sum (sum_other), off the chain of its last block.
 struct SumOut {
   double* out = nullptr;
   const double* num = nullptr;
@@ -712,12 +736,20 @@ struct SumOut {
   double* q = nullptr;
   int pair = 0;
 };
-__device__ __forceinline__ void sum_out(const SumOut& s, double t) {
+__device__ __forceinline__ double sum_other(const SumOut& s, bool mine) {
+  return mine && s.q ? __ldcg(s.num ? s.num : s.den) : 0.0;
+}
+__device__ __forceinline__ void sum_out(const SumOut& s, double t, double other) {
   *s.out = t;
   if (s.q) {
-    const double v = s.num ? *s.num / t : t / *s.den;
+    df p;
+    if (s.pair == 2 && df_quotient(s.num ? other : t, s.num ? t : other, p)) {
+      *reinterpret_cast<float2*>(s.q) = make_float2(p.hi, p.lo);
+      return;
+    }
+    const double v = s.num ? other / t : t / other;
     if (s.pair) {
-      const df p = df_from_double(v);
+      p = df_from_double(v);
       *reinterpret_cast<float2*>(s.q) = make_float2(p.hi, p.lo);
     } else {
       *s.q = v;
@@ -725,7 +757,7 @@ __device__ __forceinline__ void sum_out(const SumOut& s, double t) {
   }
 }
 __device__ __forceinline__ df load_pair(const double* q) {
-  const float2 v = *reinterpret_cast<const float2*>(q);
+  const float2 v = __ldcg(reinterpret_cast<const float2*>(q));
   return df{v.x, v.y};
 }
 
@@ -810,17 +842,19 @@ __device__ __forceinline__ void block_sum_finish(double (&v)[N], double* partial
 }
 __device__ __forceinline__ void block_sum_finish(double v, double* partials, unsigned int* counter,
                                                  const SumOut& out) {
+  const double other = sum_other(out, threadIdx.x == 0);
   double a[1] = {v}, t[1];
-  if (block_sum_last<1>(a, partials, counter, t) && threadIdx.x == 0) sum_out(out, t[0]);
+  if (block_sum_last<1>(a, partials, counter, t) && threadIdx.x == 0) sum_out(out, t[0], other);
 }
 
 // As block_sum_last_df over a 1D grid, storing the total to *out.
 __device__ __forceinline__ void block_sum_finish_df(df v, double* partials, unsigned int* counter,
                                                     const SumOut& out) {
+  const double other = sum_other(out, threadIdx.x == 0);
   double t;
   if (block_sum_last_df(v, partials, counter, t, threadIdx.x, blockDim.x, blockIdx.x, gridDim.x) &&
       threadIdx.x == 0)
-    sum_out(out, t);
+    sum_out(out, t, other);
 }
 
 // *a / *b for the whole block as a df64 pair, computed once by thread 0.

@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 4 : 2) k_df3d(DfArgs a)
   if (MODE == DIR) {
     if (!a.first) beta = load_pair(a.beta);
   }
-  const bool odd = MODE == DIR && a.parity && (((int)*a.parity) & 1);
+  const bool odd = MODE == DIR && a.parity && is_set(a.parity);
   const float2* const xsrc = odd ? a.x_alt : a.x;
   float2* const pdst = odd ? a.p_alt : a.p;
   const int NXY = a.NX * a.NY;
@@ -378,11 +378,12 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 4 : 2) k_df3d(DfArgs a)
 #undef D3D_FINISH_FROM
 #undef D3D_FINISH_LAYER
   if (a.out.out) {
+    const double other = sum_other(a.out, tid == 0);
     double t;
     const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     const int nb = gridDim.x * gridDim.y * gridDim.z;
     if (block_sum_last_df(dot, a.partials, a.counter, t, tid, T::NTB, bid, nb) && tid == 0)
-      sum_out(a.out, t);
+      sum_out(a.out, t, other);
   }
 }
 

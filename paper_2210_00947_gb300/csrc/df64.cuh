@@ -102,6 +102,22 @@ __device__ __forceinline__ df df_max(df a, df b) { return df_le(a, b) ? b : a; }
 __device__ __forceinline__ df df_min(df a, df b) { return df_le(a, b) ? a : b; }
 __device__ __forceinline__ df df_abs(df a) { return a.hi < 0.f ? df_neg(a) : a; }
 
+// a / b to about 2^-44: the FP32 quotient of the high words and two corrections
+// from the remainder
+__device__ __forceinline__ df df_div(df a, df b) {
+  const float q0 = __fdiv_rn(a.hi, b.hi);
+  df r = df_sub(a, df_mulf(b, q0));
+  const float q1 = __fdiv_rn(r.hi, b.hi);
+  r = df_sub(r, df_mulf(b, q1));
+  const float q2 = __fdiv_rn(r.hi, b.hi);
+  return df_add(df_make(q0, q1), df{q2, 0.f});
+}
+
+// p = a / b in df64 without an FP64 division: the quotient of the significands,
+// scaled.  False (nothing done) for zeros, denormal or non-finite operands and
+// quotients outside [2^-100, 2^100].
+__device__ __forceinline__ bool df_quotient(double a, double b, df& p);
+
 // Conversions, rounded to nearest even: hi = fl32(x), lo = fl32(x - hi), and
 // fl64(hi + lo).  Written with FP64 instructions they are four and three of
 // them, and the FP64 pipe takes about 20 clocks per instruction of a warp (a
@@ -157,6 +173,19 @@ __host__ __device__ __forceinline__ double df_to_double(df a) {
 #else
   return df_to_double_fp(a);
 #endif
+}
+
+__device__ __forceinline__ bool df_quotient(double a, double b, df& p) {
+  const int ha = __double2hiint(a), hb = __double2hiint(b);
+  const int ea = (ha >> 20) & 0x7ff, eb = (hb >> 20) & 0x7ff, e = ea - eb;
+  if (ea == 0 || ea == 0x7ff || eb == 0 || eb == 0x7ff || e < -100 || e > 100) return false;
+  const int one = 0x3ff00000, rest = (int)0x800fffff;
+  p = df_div(df_from_double(__hiloint2double((ha & rest) | one, __double2loint(a))),
+             df_from_double(__hiloint2double((hb & rest) | one, __double2loint(b))));
+  const float scale = __uint_as_float((unsigned)(127 + e) << 23);
+  p.hi *= scale;
+  p.lo *= scale;
+  return true;
 }
 
 }  // namespace mgar

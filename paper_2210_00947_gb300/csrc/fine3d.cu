@@ -255,8 +255,8 @@ __global__ void __launch_bounds__(T::NTB, f3d_minb(MODE, T::NT)) k_fine3d(FineAr
   const Real* dsrc = nullptr;
   Real* pdst = nullptr;
   if (MODE == DIR) {
-    const bool first = *a.first != 0.0;
-    const bool odd = a.parity && (((int)*a.parity) & 1);
+    const bool first = is_set(a.first);
+    const bool odd = a.parity && is_set(a.parity);
     om = first ? Real(0) : (Real)load_pair(a.beta).hi;
     dsrc = first ? nullptr : (const Real*)(odd ? a.x_alt : a.x);
     pdst = (Real*)(odd ? a.out_alt : a.out0);
@@ -409,12 +409,13 @@ __global__ void __launch_bounds__(T::NTB, f3d_minb(MODE, T::NT)) k_fine3d(FineAr
 #undef F3D_FINISH_FROM
 #undef F3D_FINISH_LAYER
   if (rdot) {
+    const double other = sum_other(a.dout, tid == 0);
     double t;
     const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     const int nb = gridDim.x * gridDim.y * gridDim.z;
     const df v = df_add(dacc, df{facc, 0.f});
     if (block_sum_last_df(v, a.partials, a.counter, t, tid, T::NTB, bid, nb) && tid == 0) {
-      sum_out(a.dout, t);
+      sum_out(a.dout, t, other);
       if (MODE == DIR) *a.rz_set = *a.rz_new;
     }
   }

@@ -78,8 +78,8 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 3 : 2) k_fine64(Args a)
   const bool kron = kr && ki >= 0 && ki < a.ex && kj >= 0 && kj < a.ey;
   const int ocol = i + a.NX * j, rcol = ri + a.NX * rj;
   const int ecol = i + a.ex * j, kcol = ki + a.ex * kj;
-  const double om = MODE != DIRECTION ? a.omega : a.first ? 0.0 : *a.beta;
-  if (MODE == DIRECTION && a.parity && (((int)*a.parity) & 1)) {
+  const double om = MODE != DIRECTION ? a.omega : a.first ? 0.0 : __ldcg(a.beta);
+  if (MODE == DIRECTION && a.parity && is_set(a.parity)) {
     a.x = a.x_alt;
     a.out0 = a.out_alt;
   }
@@ -267,11 +267,12 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 3 : 2) k_fine64(Args a)
     if (k < kb) __syncthreads();
   }
   if (sum) {
+    const double other = sum_other(a.dout, tid == 0);
     double t[1];
     const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     const int nb = gridDim.x * gridDim.y * gridDim.z;
     if (block_sum_last_ids<1>(acc, a.partials, a.counter, t, tid, T::NTB, bid, nb) && tid == 0)
-      sum_out(a.dout, t[0]);
+      sum_out(a.dout, t[0], other);
   }
 }
 

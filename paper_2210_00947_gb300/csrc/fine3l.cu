@@ -101,9 +101,9 @@ __global__ void __launch_bounds__(NT, 2) k_fine3l(Args a) {
   float* pdst = a.out0;
   bool first = false;
   if (MODE == DIR) {
-    first = *a.first != 0.0;
+    first = is_set(a.first);
     om = first ? 0.f : load_pair(a.beta).hi;
-    if (a.parity && (((int)*a.parity) & 1)) {
+    if (a.parity && is_set(a.parity)) {
       xsrc = a.x_alt;
       pdst = a.out_alt;
     }
@@ -267,11 +267,12 @@ __global__ void __launch_bounds__(NT, 2) k_fine3l(Args a) {
     }
   }
   if (rdot) {
+    const double other = sum_other(a.dout, tid == 0);
     double t;
     const int bid = blockIdx.x + gridDim.x * blockIdx.y, nblk = gridDim.x * gridDim.y;
     if (block_sum_last_df(df_add(dacc, df{facc, 0.f}), a.partials, a.counter, t, tid, NT, bid, nblk) &&
         tid == 0) {
-      sum_out(a.dout, t);
+      sum_out(a.dout, t, other);
       if (MODE == DIR) *a.rz_set = *a.rz_new;
     }
   }

@@ -116,11 +116,12 @@ __global__ void __launch_bounds__(l2d::kThreads2) k_up2d(l2d::Fine<Real> f, cons
   l2d::fine_up<Real, R>(s, f, blockIdx.x, blockIdx.y, b, t, res, xout,
                         [&](Real bv, Real xo) { if (DOT) acc[0] += bv * xo; });
   if (DOT) {
+    const double other = sum_other(dout, threadIdx.x == 0);
     double v[1];
     if (block_sum_last_ids<1>(acc, partials, counter, v, threadIdx.x, l2d::kThreads2,
                               blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y) &&
         threadIdx.x == 0)
-      sum_out(dout, v[0]);
+      sum_out(dout, v[0], other);
   }
 }
 
@@ -137,6 +138,7 @@ __global__ void __launch_bounds__(kThreads) k_dot_rz(const float2* __restrict__ 
                                                      SumOut out) {
   pdl_wait();
   pdl_trigger();
+  const double other = sum_other(out, threadIdx.x == 0);
   float2 rv[4 * kSumVB];
   float xv[4 * kSumVB];
   double t;
@@ -148,7 +150,7 @@ __global__ void __launch_bounds__(kThreads) k_dot_rz(const float2* __restrict__ 
           },
           [&](int q) { return df_mulf(df{rv[q].x, rv[q].y}, xv[q]); }) &&
       threadIdx.x == 0)
-    sum_out(out, t);
+    sum_out(out, t, other);
 }
 
 // FP64: p = z + beta p_old (p = z when first), y = A p, p . y into out; odd
@@ -165,18 +167,19 @@ __global__ void __launch_bounds__(l2d::kThreads2) k_dir2d(const double* __restri
   __shared__ l2d::DirSmem<R> s;
   pdl_wait();
   pdl_trigger();
-  if (parity && (((int)*parity) & 1)) {
+  if (parity && is_set(parity)) {
     double* t = const_cast<double*>(p_old);
     p_old = p;
     p = t;
   }
+  const double other = sum_other(out, threadIdx.x == 0);
   double v[1], t[1];
   v[0] = l2d::fine_dir<R>(s, ke, fixed, ex, ey, blockIdx.x, blockIdx.y, z, p_old, first != 0,
-                          first ? 0.0 : *beta, p, y);
+                          first ? 0.0 : __ldcg(beta), p, y);
   if (block_sum_last_ids<1>(v, partials, counter, t, threadIdx.x, l2d::kThreads2,
                             blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y) &&
       threadIdx.x == 0)
-    sum_out(out, t[0]);
+    sum_out(out, t[0], other);
 }
 
 template <typename Real>
