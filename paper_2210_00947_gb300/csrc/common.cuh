@@ -611,14 +611,10 @@ __device__ __forceinline__ bool block_sum_last_df(df v, double* partials, unsign
   return block_sum_last_one(true, 0.0, v, partials, counter, total, tid, nthr, bid, nblk);
 }
 
-// The CG's scalars are read from L2: a line of them that one launch's blocks
-// bring into L1 may still be there, stale, for a launch that was started before
-// the scalar's writer had ended (the dependency wait does not drop it).
-//
 // *p != 0 for a flag kept as a double (0 or 1), by its bits: a comparison or
 // conversion on the FP64 pipe costs every warp about 20 clocks of it.
 __device__ __forceinline__ bool is_set(const double* p) {
-  return (__double_as_longlong(__ldcg(p)) << 1) != 0;
+  return (__double_as_longlong(*p) << 1) != 0;
 }
 
 // Four sums at once: v[g] is thread tid's value of the virtual block vb0 + g of
@@ -736,6 +732,9 @@ struct SumOut {
   double* q = nullptr;
   int pair = 0;
 };
+// Read from L2: every block does, and a line of scalars that this brought into
+// its SM's L1 would still be there, stale, for the next launch, which may have
+// started before (the dependency wait does not drop it).
 __device__ __forceinline__ double sum_other(const SumOut& s, bool mine) {
   return mine && s.q ? __ldcg(s.num ? s.num : s.den) : 0.0;
 }
@@ -757,7 +756,7 @@ __device__ __forceinline__ void sum_out(const SumOut& s, double t, double other)
   }
 }
 __device__ __forceinline__ df load_pair(const double* q) {
-  const float2 v = __ldcg(reinterpret_cast<const float2*>(q));
+  const float2 v = *reinterpret_cast<const float2*>(q);
   return df{v.x, v.y};
 }
 

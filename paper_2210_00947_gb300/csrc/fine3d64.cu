@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 3 : 2) k_fine64(Args a)
   const bool kron = kr && ki >= 0 && ki < a.ex && kj >= 0 && kj < a.ey;
   const int ocol = i + a.NX * j, rcol = ri + a.NX * rj;
   const int ecol = i + a.ex * j, kcol = ki + a.ex * kj;
-  const double om = MODE != DIRECTION ? a.omega : a.first ? 0.0 : __ldcg(a.beta);
+  const double om = MODE != DIRECTION ? a.omega : a.first ? 0.0 : *a.beta;
   if (MODE == DIRECTION && a.parity && is_set(a.parity)) {
     a.x = a.x_alt;
     a.out0 = a.out_alt;

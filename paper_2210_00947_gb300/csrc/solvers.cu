@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kThreads) k_cg_xr(double* __restrict__ x, doub
                                                     double* out, CgCheck check) {
   pdl_wait();
   if (parity && is_set(parity)) p = p_alt;
-  const double alpha = __ldcg(alpha_p);
+  const double alpha = *alpha_p;
   double v[1] = {0.0};
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, n2 = n >> 1;
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

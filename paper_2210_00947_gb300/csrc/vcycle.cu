@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(l2d::kThreads2) k_dir2d(const double* __restri
   const double other = sum_other(out, threadIdx.x == 0);
   double v[1], t[1];
   v[0] = l2d::fine_dir<R>(s, ke, fixed, ex, ey, blockIdx.x, blockIdx.y, z, p_old, first != 0,
-                          first ? 0.0 : __ldcg(beta), p, y);
+                          first ? 0.0 : *beta, p, y);
   if (block_sum_last_ids<1>(v, partials, counter, t, threadIdx.x, l2d::kThreads2,
                             blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y) &&
       threadIdx.x == 0)
