@@ -57,10 +57,9 @@ __global__ void __launch_bounds__(l2d::kThreads2) k_df_dir2(DfOp op, const float
 
 // p . y over the nodes in memory order (as the sum of r . z, it does not
 // follow the tiles)
-__global__ void __launch_bounds__(kThreads) k_dot_py(const float2* __restrict__ p,
-                                                     const float2* __restrict__ p_alt,
+__global__ void __launch_bounds__(kThreads) k_dot_py(const float2* p, const float2* p_alt,
                                                      const double* parity,
-                                                     const float2* __restrict__ y, int n,
+                                                     const float2* y, int n,
                                                      double* partials, unsigned int* counter,
                                                      SumOut out) {
   pdl_wait();
@@ -122,7 +121,7 @@ __global__ void k_df_residual(DfOp op, const float2* __restrict__ q, const float
 __global__ void __launch_bounds__(kThreads) k_df_cg_xr(float2* __restrict__ x, float2* __restrict__ r,
                                                        const float2* __restrict__ p,
                                                        const float2* __restrict__ Ap, int n,
-                                                       const double* __restrict__ alpha_p,
+                                                       const double* alpha_p,
                                                        double* partials, unsigned int* counter,
                                                        double* out, float* __restrict__ r32,
                                                        const float2* __restrict__ p_alt,
@@ -519,7 +518,7 @@ __global__ void __launch_bounds__(kThreads) k_cg_xr32(float* __restrict__ xc, fl
                                                       const float* __restrict__ p_alt,
                                                       const double* parity,
                                                       const float* __restrict__ Ap, int n,
-                                                      const double* __restrict__ alpha_p,
+                                                      const double* alpha_p,
                                                       double* partials, unsigned int* counter,
                                                       double* dsc, double qnorm, double eps2,
                                                       double delta, int cg_max,

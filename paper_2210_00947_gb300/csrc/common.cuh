@@ -317,17 +317,18 @@ struct CoarseT {
 // first thing, a hardware wait until the predecessor has completed and its
 // memory is visible, so only launch latency and block dispatch overlap.
 // pdl_trigger() lets the successor be dispatched before this grid ends.
-// The compiler may move a load through a const __restrict__ pointer over the
-// wait, whose memory clobber does not order loads of memory it takes to be
-// constant: in straight-line code it did, and the row read its operand before
-// the predecessor had written it.  Such loads keep their basic block, so the
-// wait ends one: the branch goes away in the assembler, after the loads have
-// been placed.
+// A load through a const __restrict__ pointer may be moved over the wait: it
+// reads memory that the compiler takes to be constant, which neither the
+// memory clobber nor the wait itself orders.  In straight-line code it was (a
+// row read its operand, and a CG update its alpha, before the predecessor had
+// written them).  So the wait ends with a branch that no compiler stage can
+// decide and that is never taken (no SM has that number), and scalars written
+// by a predecessor come through plain pointers.
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  unsigned never;
-  asm volatile("mov.u32 %0, 0;" : "=r"(never));
-  if (never != 0u) asm volatile("exit;" ::: "memory");
+  unsigned sm;
+  asm volatile("mov.u32 %0, %%smid;" : "=r"(sm)::"memory");
+  if (sm == 0xffffffffu) asm volatile("exit;" ::: "memory");
 }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -732,9 +733,7 @@ struct SumOut {
   double* q = nullptr;
   int pair = 0;
 };
-// Read from L2: every block does, and a line of scalars that this brought into
-// its SM's L1 would still be there, stale, for the next launch, which may have
-// started before (the dependency wait does not drop it).
+// Read once per block and from L2, where the launch before this one left it.
 __device__ __forceinline__ double sum_other(const SumOut& s, bool mine) {
   return mine && s.q ? __ldcg(s.num ? s.num : s.den) : 0.0;
 }

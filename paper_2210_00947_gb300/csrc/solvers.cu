@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(kThreads) k_cg_xr(double* __restrict__ x, doub
                                                     const double* p,
                                                     const double* __restrict__ Ap, int64_t n,
                                                     const double* p_alt, const double* parity,
-                                                    const double* __restrict__ alpha_p,
+                                                    const double* alpha_p,
                                                     double* partials, unsigned int* counter,
                                                     double* out, CgCheck check) {
   pdl_wait();

@@ -131,9 +131,8 @@ __global__ void __launch_bounds__(l2d::kThreads2) k_up2d(l2d::Fine<Real> f, cons
 // iteration count of one design in sixty.  So the sum keeps the order of the
 // nodes and does not follow the tiles, where it cost 6 us on 1025^2 nodes at
 // the end of the pass.
-__global__ void __launch_bounds__(kThreads) k_dot_rz(const float2* __restrict__ r,
-                                                     const float* __restrict__ b,
-                                                     const float* __restrict__ x, int n,
+__global__ void __launch_bounds__(kThreads) k_dot_rz(const float2* r, const float* b,
+                                                     const float* x, int n,
                                                      double* partials, unsigned int* counter,
                                                      SumOut out) {
   pdl_wait();
