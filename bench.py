@@ -232,10 +232,10 @@ def kernel_model(kernel, w):
         return 45 * n, 344 * n, "alu", "fp32"
     if kernel == "apply32":
         # mixed path, 3D: FP32 product of a CG iteration with the fused
-        # direction update and p.Ap (tiled, 21-point H8 stencil): read z,
-        # p_old, k_e (4 B each) and the mask (1 B), write p and A p (4 B
-        # each): 21 B per node
-        return 21 * n, 0, "hbm", None
+        # direction update and p.Ap (21-point H8 stencil): read z, p_old, k_e
+        # and D^-1 (its sign marks fixed nodes; 4 B each), write p and A p
+        # (4 B each): 24 B per node
+        return 24 * n, 0, "hbm", None
     if kernel == "resid64":
         # mixed path, 3D: df64 residual r = q - A x in the difference form,
         # per node in FP32-pipe operations: 12 face-diagonal weight sums 96
@@ -251,11 +251,11 @@ def kernel_model(kernel, w):
         # sums, 20 FMA, 3 multiplies), + 2 for the fused p.Ap dot.
         return 25 * n, 64 * n, "alu", "fp64"
     if kernel == "smooth0":
-        # FP32 level-0 passes of the V-cycle, per node 21 B for either: the
-        # pre-smoothing pass reads b, D^-1, one k_e (4 B each) and the mask
-        # (1 B) and writes x and r (4 B each); the post-smoothing sweep reads
-        # x, b, D^-1, one k_e and the mask and writes x'
-        return 21 * n, 0, "hbm", None
+        # FP32 level-0 passes of the V-cycle, per node 20 B for either: the
+        # pre-smoothing pass reads b, D^-1 (its sign marks fixed nodes) and
+        # one k_e (4 B each) and writes x and r (4 B each); the
+        # post-smoothing sweep reads x, b, D^-1 and one k_e and writes x'
+        return 20 * n, 0, "hbm", None
     if kernel == "galerkin0":
         return 8 * e + 64 * 4 * e // 8, 0, "hbm", None
     raise ValueError(kernel)
