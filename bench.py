@@ -180,12 +180,12 @@ def shard(items, rank, world):
 # one ncu capture of the kernel as it stands; a kernel changed since its
 # capture has no entry (traffic null).
 TRAFFIC = {
-    # cold-cache ncu capture (43 x 5 tiles, layer-split stencil) of one
-    # pre-smoothing (27.73 MB) and one post-smoothing pass (36.34 MB) of the
+    # cold-cache ncu capture (passes on linear segments) of one
+    # pre-smoothing (25.78 MB) and one post-smoothing pass (34.39 MB) of the
     # 128^3 workload: their mean
-    "smooth0": 32.03e6,
+    "smooth0": 30.08e6,
     # the same capture, FP32 CG product
-    "apply32": 27.74e6,
+    "apply32": 34.39e6,
 }
 
 def load_peaks():
