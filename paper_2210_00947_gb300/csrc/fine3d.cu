@@ -1,4 +1,6 @@
-// Tiled kernels for the finest 3D (H8) level of the V-cycle.
+// Tiled kernels for the finest 3D (H8) level of the V-cycle: rows too long for
+// the segments of fine3l.cu (above 1151 nodes; on shorter ones these take up to
+// twice the time), and the interpolation fused into the sweep.
 //
 // A block of TX x TY threads owns a TX x TY column of nodes and walks along z
 // through a run of node planes.  Rotating planes of the operand
