@@ -442,11 +442,11 @@ int mgar_create(mgar_t* out, const mgar_params* p, const uint8_t* fixed_mask, co
     }
     if (const char* fc = std::getenv("MGAR_FP64_COARSE")) c->df_coarse = fc[0] != '1';
     if (c->dim == 3) {
-      fine3d_prepare(*c);
       fine3d64_prepare(*c);
       if (P.precision == MGAR_MIXED) {
         df3d_prepare(*c);
         fine3l_prepare(*c);
+        fine3d_prepare(*c);
       }
     }
   } catch (const Error& e) {

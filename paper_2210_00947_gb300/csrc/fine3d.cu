@@ -440,7 +440,8 @@ int runs_for(const Dims& d, int sms) {
 }  // namespace f3d
 
 // The tile: 32 x 8, or 43 x 5 where that leaves fewer lanes idle (129-node
-// planes: 95 % of the lanes busy instead of 76 %).
+// planes: 95 % of the lanes busy instead of 76 %).  After fine3l_prepare: no
+// occupancy query (each loads its kernel) for passes that run on segments.
 void fine3d_prepare(Ctx& c) {
   using namespace f3d;
   int dev = 0, sms = 0;
@@ -448,6 +449,11 @@ void fine3d_prepare(Ctx& c) {
   MGAR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const Dims& d = c.L[0];
   c.f3d_tile = tile_use(d.NX, d.NY, T43x5::TX, T43x5::TY) > tile_use(d.NX, d.NY, T32x8::TX, T32x8::TY);
+  if (c.kn0) {
+    if (!c.split_post)
+      c.f3d_gz[POST] = c.f3d_tile ? runs_for<float, POST, T43x5>(d, sms) : runs_for<float, POST, T32x8>(d, sms);
+    return;
+  }
   if (c.f3d_tile) {
     c.f3d_gz[PRE] = runs_for<float, PRE, T43x5>(d, sms);
     c.f3d_gz[POST] = runs_for<float, POST, T43x5>(d, sms);

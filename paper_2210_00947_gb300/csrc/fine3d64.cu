@@ -292,11 +292,12 @@ int runs_for(const Ctx& c) {
 }
 template <class T>
 void prepare(Ctx& c) {
+  c.f64_gz[APPLY] = runs_for<APPLY, T>(c);
+  if (c.p.precision != MGAR_FP64) return;  // a mixed handle takes no other FP64 pass
   c.f64_gz[PRE_SMOOTH] = runs_for<PRE_SMOOTH, T>(c);
   c.f64_gz[RESIDUAL] = runs_for<RESIDUAL, T>(c);
   c.f64_gz[SWEEP] = runs_for<SWEEP, T>(c);
   c.f64_gz[DIRECTION] = runs_for<DIRECTION, T>(c);
-  c.f64_gz[APPLY] = runs_for<APPLY, T>(c);
 }
 
 template <int MODE, class T>
