@@ -570,7 +570,7 @@ __global__ void k_oc_classify(const float2* __restrict__ s, const float2* __rest
 // long as the guess was right (a step whose guess was wrong is taken the other
 // way and ends the round).  Every step taken is the plain bisection's, on the
 // same midpoint and the same value of g, so mu is the same to the last bit.
-// 2040 x 2040 elements: 80 -> 27 us; 128^3: 58 -> 22 us.
+// 2040 x 2040 elements: 80 -> 40 us; 128^3: 58 -> 30 us.
 __global__ void k_oc_finish(const float2* __restrict__ s, const float2* __restrict__ lo,
                             const float2* __restrict__ hi, const float2* __restrict__ dv, int ne,
                             double volfrac, double* dsc, int* amb, int* namb_p) {
@@ -613,7 +613,7 @@ __global__ void k_oc_finish(const float2* __restrict__ s, const float2* __restri
   __shared__ double cs[kCache], cl[kCache], ch[kCache], cd[kCache];
   __shared__ double mid[kPath], gmid[kPath], ends[4];
   __shared__ bool guess[kPath];
-  __shared__ int steps;  // midpoints laid out this round; 0 once the bisection has ended
+  __shared__ int steps;  // midpoints laid out this time; 0 once the bisection has ended
   const bool cached = namb <= kCache;
   if (cached) {
     for (int i = threadIdx.x; i < namb; i += kLive) {
