@@ -6,6 +6,7 @@
 #include "common.cuh"
 #include "df64.cuh"
 #include "filter3d.cuh"
+#include "pplist.cuh"
 
 #include <vector>
 
@@ -1162,17 +1163,8 @@ __global__ void k_pp_nodal(const double* __restrict__ dcp, double* __restrict__ 
 // A volume per bisection step instead, 62 passes at 4.6 ms on 128^3 (FP64-bound:
 // up to 5000 FP64 operations per element), took 290 ms; this takes 1.4 ms with
 // the projection, bound by the shared-memory atomics of the first histogram.
-constexpr int kPpBins = 4096;
 constexpr unsigned kPpGuard = 64;
 constexpr int kPpShift1 = 19, kPpShift2 = 8;  // bits per bin: 2^31 in 4096 bins, then 2^19 in 2050
-
-struct PpCtrl {
-  unsigned long long hist[2][kPpBins];
-  unsigned long long above[3];  // points past the bracket of each histogram pass and of the listing
-  unsigned lo[3], hi[3];        // bracket (bit patterns, inclusive) of each pass
-  int nlist;
-  int bad;
-};
 
 // The FP32 values of an element's lattice points, clamped to its corners'
 // range: f(value, px, py, pz).
@@ -1332,7 +1324,8 @@ __global__ void __launch_bounds__(1024) k_pp_pick(PpCtrl* c, int pass, double wa
 // Points above the last bracket, counted, and the values of those inside,
 // listed: the level below which the point counts, which is its FP64 value
 // kept within its element's corners (an element whose corners all exceed the
-// level is solid, one whose corners are all below it void).
+// level is solid, one whose corners are all below it void).  Once more points
+// were met than the list holds, the elements left are skipped.
 template <int DIM>
 __global__ void __launch_bounds__(512) k_pp_list(const float* __restrict__ ns32,
                                                  const double* __restrict__ ns, Dims d, PpCtrl* c,
@@ -1352,10 +1345,13 @@ __global__ void __launch_bounds__(512) k_pp_list(const float* __restrict__ ns32,
       up += NP;
       continue;
     }
+    if (!pp_complete(__ldcg(&c->nlist), cap)) break;  // a volume per step will be taken
     pp_points32<DIM>(t, tmin, tmax, [&](float s, int px, int py, int pz) {
       const unsigned b = __float_as_uint(s);
       if (b > hi) ++up;
       else if (b >= lo) {
+        const PpCount slot = atomicAdd(&c->nlist, PpCount(1));
+        if (!pp_listed(slot, cap)) return;
         double td[nen];
         pp_corners<DIM, double>(ns, d, e, td);
         double mn = td[0], mx = td[0];
@@ -1368,8 +1364,7 @@ __global__ void __launch_bounds__(512) k_pp_list(const float* __restrict__ ns32,
         // at the level mx itself the element is not void: a value rounded
         // above mx counts there and nowhere higher
         const double eff = v > mx ? nextafter(mx, 1e300) : fmax(v, mn);
-        const int slot = atomicAdd(&c->nlist, 1);
-        if (slot < cap) list[slot] = eff;
+        list[slot] = eff;
       }
     });
   }
@@ -1388,11 +1383,12 @@ __global__ void __launch_bounds__(1024) k_pp_bisect(const PpCtrl* c, const doubl
                                                     int tie, double* out) {
   __shared__ int part[32];
   __shared__ int total;
-  const int n = c->nlist, tid = threadIdx.x;
-  if (c->bad || n > cap) {
+  const int tid = threadIdx.x;
+  if (c->bad || !pp_complete(c->nlist, cap)) {
     if (tid == 0) out[0] = 2.0;
     return;
   }
+  const int n = (int)c->nlist;
   const double base = (double)c->above[2];
   // outside [La, Lb] the answer is known (a bracket cut off at 0 knows nothing below)
   const double La = c->lo[2] ? (double)__uint_as_float(c->lo[2] + kPpGuard / 2) : -1.0;
