@@ -1,6 +1,7 @@
 // Density filter (Eq. 6-8), SIMP conductivities (Eq. 4), compliance and
 // sensitivities (Eq. 5, 9-11), and the optimality-criteria update.
 #include <algorithm>
+#include <cstddef>
 #include <vector>
 
 #include "common.cuh"
@@ -1156,7 +1157,8 @@ __global__ void k_pp_nodal(const double* __restrict__ dcp, double* __restrict__ 
 //   order non-negative floats) find the bracket that holds the level, 384
 //   ulps wide; one pass counts the points above it and lists the FP64 values
 //   of those inside (a few thousand); one block then runs the bisection on
-//   that list, step for step with the same midpoints.
+//   that list, step for step with the same midpoints.  (A count that equals
+//   the target leaves the comparison to the densities' sum: postprocess.)
 // An FP32 value is within 8 ulps of the FP64 one (positive weights, seven
 // roundings), so every bracket is widened by kPpGuard ulps and a point outside
 // the last one is on the same side of every level in it in either precision.
@@ -1374,13 +1376,10 @@ __global__ void __launch_bounds__(512) k_pp_list(const float* __restrict__ ns32,
 }
 
 // The bisection, one block: level L has the points above the last bracket
-// plus the listed values > L.  The densities' FP64 sum and this count give the
-// same answer unless the count is the target itself; then out[0] = 1 asks for
-// that answer (tie: -1 unknown, else whether the sum exceeds the target) at
-// the level in out[1].  out[0] = 2: not applicable; 0: done, level in out[1].
+// plus the listed values > L, and goes up while they are more than `want`.
+// out[0] = 2: not applicable; 0: done, level in out[1].
 __global__ void __launch_bounds__(1024) k_pp_bisect(const PpCtrl* c, const double* __restrict__ list,
-                                                    int cap, double top, double want, double slack,
-                                                    int tie, double* out) {
+                                                    int cap, double top, double want, double* out) {
   __shared__ int part[32];
   __shared__ int total;
   const int tid = threadIdx.x;
@@ -1411,20 +1410,8 @@ __global__ void __launch_bounds__(1024) k_pp_bisect(const PpCtrl* c, const doubl
         if (tid == 0) total = s;
       }
       __syncthreads();
-      const double count = base + (double)total;
+      more = base + (double)total > want;
       __syncthreads();
-      if (fabs(count - want) <= slack) {
-        if (tie < 0) {
-          if (tid == 0) {
-            out[0] = 1.0;
-            out[1] = mid;
-          }
-          return;
-        }
-        more = tie != 0;
-      } else {
-        more = count > want;
-      }
     }
     if (more) lo = mid;
     else hi = mid;
@@ -1572,7 +1559,7 @@ void postprocess(Ctx& c, const double* rho, const double* T, double volfrac, dou
   double* ns = c.tm;
   float* ns32 = reinterpret_cast<float*>(c.pv);
   PpCtrl* ctrl = reinterpret_cast<PpCtrl*>(c.pp_ctrl);
-  MGAR_CUDA(cudaMemsetAsync(ctrl, 0, sizeof(PpCtrl), c.stream));
+  MGAR_CUDA(cudaMemsetAsync(&ctrl->bad, 0, sizeof(ctrl->bad), c.stream));
   const PpTap* taps = reinterpret_cast<const PpTap*>(c.pp_taps);
   if (c.dim == 2)
     k_pp_nodal<2><<<blocks_for(c.n), kThreads, 0, c.stream>>>(c.tmp_e, ns, ns32, d, taps,
@@ -1604,44 +1591,54 @@ void postprocess(Ctx& c, const double* rho, const double* T, double volfrac, dou
     fetch_scalars(c, S_TMP, 1);
     return c.hsc[S_TMP] / (double)ne;
   };
-  // the level by counts of lattice points
+  // the level by counts of lattice points: the smallest whose points are at
+  // most `target`.  False: values outside [0, 1e37], or more equal values at
+  // the level than the list holds
   const double total = (c.dim == 3 ? 125.0 : 25.0) * (double)ne, want = volfrac * total;
   double* list = c.tmp_e;  // the element sensitivities are no longer needed
   const int hb = std::min(blocks_for(ne, 512), 4 * c.sms);
-  k_pp_first<<<1, 1, 0, c.stream>>>(ctrl);
-  MGAR_LAUNCH_CHECK();
-  for (int pass = 0; pass < 2; ++pass) {
-    if (c.dim == 2) k_pp_hist<2><<<hb, 512, 0, c.stream>>>(ns32, d, ctrl, pass);
-    else k_pp_hist<3><<<hb, 512, 0, c.stream>>>(ns32, d, ctrl, pass);
+  auto by_counts = [&](double target, double* level) {
+    MGAR_CUDA(cudaMemsetAsync(ctrl, 0, offsetof(PpCtrl, bad), c.stream));
+    k_pp_first<<<1, 1, 0, c.stream>>>(ctrl);
     MGAR_LAUNCH_CHECK();
-    k_pp_pick<<<1, 1024, 0, c.stream>>>(ctrl, pass, want);
+    for (int pass = 0; pass < 2; ++pass) {
+      if (c.dim == 2) k_pp_hist<2><<<hb, 512, 0, c.stream>>>(ns32, d, ctrl, pass);
+      else k_pp_hist<3><<<hb, 512, 0, c.stream>>>(ns32, d, ctrl, pass);
+      MGAR_LAUNCH_CHECK();
+      k_pp_pick<<<1, 1024, 0, c.stream>>>(ctrl, pass, target);
+      MGAR_LAUNCH_CHECK();
+    }
+    if (c.dim == 2) k_pp_list<2><<<hb, 512, 0, c.stream>>>(ns32, ns, d, ctrl, list, ne);
+    else k_pp_list<3><<<hb, 512, 0, c.stream>>>(ns32, ns, d, ctrl, list, ne);
     MGAR_LAUNCH_CHECK();
-  }
-  if (c.dim == 2) k_pp_list<2><<<hb, 512, 0, c.stream>>>(ns32, ns, d, ctrl, list, ne);
-  else k_pp_list<3><<<hb, 512, 0, c.stream>>>(ns32, ns, d, ctrl, list, ne);
-  MGAR_LAUNCH_CHECK();
-  // the FP64 sum of the densities is within 1e-13 of the count's share, so
-  // only a count that equals the target leaves the comparison to it
-  const double slack = 1e-12 * total;
-  double hi = top;
-  bool found = false;
-  for (int tie = -1;;) {
-    k_pp_bisect<<<1, 1024, 0, c.stream>>>(ctrl, list, ne, top, want, slack, tie, c.dsc + S_GS);
+    k_pp_bisect<<<1, 1024, 0, c.stream>>>(ctrl, list, ne, top, target, c.dsc + S_GS);
     MGAR_LAUNCH_CHECK();
     fetch_scalars(c, S_GS, 2);
-    const int state = (int)c.hsc[S_GS];
-    if (state == 1 && tie < 0) {
-      tie = volume(c.hsc[S_GS + 1], nullptr, true) > volfrac ? 1 : 0;
-      continue;
+    if (c.hsc[S_GS] != 0.0) return false;
+    *level = c.hsc[S_GS + 1];
+    return true;
+  };
+  // The comparison is the densities' FP64 sum's, within 1e-13 of the count's
+  // share: where no whole number of points lies that close to the target, the
+  // count decides it.  Otherwise the levels with that number of points are one
+  // plateau, on which the sum has one value.  The search first takes them as
+  // met (half a point more) and ends on the plateau's lower end; if its volume
+  // is above the fraction by rounding, they are not, and the level is that of
+  // half a point less, which may lie outside the first search's bracket.
+  const double whole = std::nearbyint(want);
+  const bool plateau = std::fabs(whole - want) <= 1e-12 * total;
+  double hi = top, v = 0.0;
+  bool found = by_counts(plateau ? whole + 0.5 : want, &hi);
+  if (found) {
+    v = volume(hi, rho_out, true);
+    if (plateau && v > volfrac) {
+      found = by_counts(whole - 0.5, &hi);
+      if (found) v = volume(hi, rho_out, true);
     }
-    found = state == 0;
-    if (found) hi = c.hsc[S_GS + 1];
-    break;
   }
   if (!found) {
-    // values outside [0, 1e37], or more equal values at the level than the
-    // list holds: a volume per step.  ns >= 0: below -1 every node is above
-    // the level (volume 1), at max(ns) none is (volume 0)
+    // a volume per step.  ns >= 0: below -1 every node is above the level
+    // (volume 1), at max(ns) none is (volume 0)
     double lo = -1.0;
     hi = top;
     for (int step = 0; step < 200; ++step) {
@@ -1650,8 +1647,8 @@ void postprocess(Ctx& c, const double* rho, const double* T, double volfrac, dou
       if (volume(mid, nullptr, false) > volfrac) lo = mid;
       else hi = mid;
     }
+    v = volume(hi, rho_out, false);
   }
-  const double v = volume(hi, rho_out, found);
   if (level_out) *level_out = hi;
   if (volume_out) *volume_out = v;
 }
