@@ -1432,8 +1432,9 @@ __global__ void k_pp_density32(const float* __restrict__ ns32, const double* __r
   constexpr int nen = 1 << DIM, NP = DIM == 3 ? 125 : 25;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const float l32 = (float)level;
-  // points this far (16 ulps) from the level are on the same side of it in FP64
-  const float lo = l32 * (1.f - 0x1p-19f), hi = l32 * (1.f + 0x1p-19f) + 0x1p-140f;
+  // points this far (16 ulps, denormal values 512 of theirs) from the level are
+  // on the same side of it in FP64
+  const float lo = l32 * (1.f - 0x1p-19f) - 0x1p-140f, hi = l32 * (1.f + 0x1p-19f) + 0x1p-140f;
   double v[1] = {0.0};
   if (e < (int)d.ne) {
     float t[nen], tmin, tmax;
