@@ -246,8 +246,8 @@ __global__ void __launch_bounds__(kRedThreads) kb_dot_py(const Des* D, const int
   const Des& g = D[d];
   double* s = bsc + d * kBS;
   const int it = (int)s[BS_IT];
-  const float2* __restrict__ p = p_new(g, it);
-  const float2* __restrict__ y = g.Ap;
+  const float2* p = p_new(g, it);
+  const float2* y = g.Ap;
   const SumOut out{s + BS_PAP, s + BS_RZ + (it & 1), nullptr, s + BS_ALPHA, 1};
   const double other = sum_other(out, threadIdx.x == 0);
   float2 pv[kNptR * kSumVB], yv[kNptR * kSumVB];
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kRedThreads) kb_cg_xr(const Des* D, const int*
   if (!active(bsc, d)) return;
   const Des& g = D[d];
   double* s = bsc + d * kBS;
-  const float2* __restrict__ p = p_new(g, (int)s[BS_IT]);
+  const float2* p = p_new(g, (int)s[BS_IT]);
   const df alpha = load_pair(s + BS_ALPHA);
   float2 xv[kNptR * kSumVB], pv[kNptR * kSumVB], rv[kNptR * kSumVB], qv[kNptR * kSumVB];
   int at[kNptR * kSumVB];
@@ -436,6 +436,7 @@ struct Batch {
   double* consts = nullptr;    // [nd][3] qnorm, eps2, cg_max (device)
   double* hconsts = nullptr;   // pinned
   double* hbsc = nullptr;      // pinned
+  bool pdl = true;             // dependent launches, unless a handle was made without
   double* partials = nullptr;
   unsigned int* counters = nullptr;
   Shape s_red, s_dot;          // level 0: virtual blocks of the sums, and the sums' blocks
@@ -519,7 +520,7 @@ static void make_coarse_shape(Batch& b, int warps) {
 template <typename... KArgs, typename... Args>
 static void launch_shape(Batch& b, const Shape& s, void (*kernel)(KArgs...), Args... args) {
   if (s.nblocks == 0) return;
-  launch_pdl(b.stream, true, kernel, dim3(s.nblocks), dim3(s.threads), args..., (const int*)s.bdes,
+  launch_pdl(b.stream, b.pdl, kernel, dim3(s.nblocks), dim3(s.threads), args..., (const int*)s.bdes,
              (const int*)s.b0, (const double*)b.bsc);
   MGAR_LAUNCH_CHECK();
 }
@@ -527,7 +528,7 @@ static void launch_shape(Batch& b, const Shape& s, void (*kernel)(KArgs...), Arg
 // A sum over every active design's nodes.
 static void launch_sum(Batch& b, void (*kernel)(const Des*, const int*, const int*, const int*, double*,
                                                 double*, unsigned int*)) {
-  launch_pdl(b.stream, true, kernel, dim3(b.s_dot.nblocks), dim3(kRedThreads), (const Des*)b.ddes,
+  launch_pdl(b.stream, b.pdl, kernel, dim3(b.s_dot.nblocks), dim3(kRedThreads), (const Des*)b.ddes,
              (const int*)b.s_dot.bdes, (const int*)b.s_dot.b0, (const int*)b.s_red.b0, b.bsc,
              b.partials, b.counters);
   MGAR_LAUNCH_CHECK();
@@ -555,7 +556,7 @@ static void iteration(Batch& b, cudaGraphConditionalHandle loop, int* any_out = 
   launch_shape(b, b.s_up[0], kb_dir, (const Des*)b.ddes);
   launch_sum(b, kb_dot_py);
   launch_sum(b, kb_cg_xr);
-  launch_pdl(b.stream, true, kb_check, dim3(1), dim3(256), b.bsc, b.nd, loop, any_out);
+  launch_pdl(b.stream, b.pdl, kb_check, dim3(1), dim3(256), b.bsc, b.nd, loop, any_out);
   MGAR_LAUNCH_CHECK();
   vcycle(b);
 }
@@ -971,6 +972,7 @@ int mgar_batch_create(mgar_batch_t* out, const mgar_t* handles, int count, void*
       for (Ctx* o : b->h) require(o != c, MGAR_ERR_ARG, "a handle appears twice");
       b->h.push_back(c);
       b->lmax = std::max(b->lmax, c->nl);
+      b->pdl = b->pdl && c->use_pdl;
     }
     const int nd = b->nd, lmax = b->lmax;
     b->s_down.resize(lmax);

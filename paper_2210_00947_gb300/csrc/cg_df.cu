@@ -38,11 +38,11 @@ __global__ void k_df_apply(DfOp op, const float2* __restrict__ x, float2* __rest
 
 // 2D: p = z + beta p_old (p = z when first), y = A p; odd *parity (may be
 // null) swaps p_old and p.
-__global__ void __launch_bounds__(l2d::kThreads2) k_df_dir2(DfOp op, const float* __restrict__ z,
+__global__ void __launch_bounds__(l2d::kThreads2) k_df_dir2(DfOp op, const float* z,
                                                             const float2* p_old, float2* p,
                                                             const double* beta, int first,
                                                             const double* parity,
-                                                            float2* __restrict__ y) {
+                                                            float2* y) {
   __shared__ DfDirSmem s;
   pdl_wait();
   pdl_trigger();
@@ -118,13 +118,13 @@ __global__ void k_df_residual(DfOp op, const float2* __restrict__ q, const float
 
 // x += alpha p; r -= alpha Ap; ||r||^2; optionally the FP32 copy of r for the
 // preconditioner
-__global__ void __launch_bounds__(kThreads) k_df_cg_xr(float2* __restrict__ x, float2* __restrict__ r,
-                                                       const float2* __restrict__ p,
-                                                       const float2* __restrict__ Ap, int n,
+__global__ void __launch_bounds__(kThreads) k_df_cg_xr(float2* x, float2* r,
+                                                       const float2* p,
+                                                       const float2* Ap, int n,
                                                        const double* alpha_p,
                                                        double* partials, unsigned int* counter,
-                                                       double* out, float* __restrict__ r32,
-                                                       const float2* __restrict__ p_alt,
+                                                       double* out, float* r32,
+                                                       const float2* p_alt,
                                                        const double* parity, CgCheck check) {
   pdl_wait();
   // device-side CG loop: the two direction buffers swap with the parity
@@ -513,11 +513,11 @@ __device__ void ru_decide(double* dsc, double qnorm, double eps2, double delta, 
 // xc += alpha p; r -= alpha A p; ||r||^2 into dsc[S_RR], then the update
 // decision (ru_decide) in the last block.  Two 16-byte rows of each vector in
 // flight per thread, four blocks per SM.
-__global__ void __launch_bounds__(kThreads) k_cg_xr32(float* __restrict__ xc, float* __restrict__ r,
-                                                      const float* __restrict__ p,
-                                                      const float* __restrict__ p_alt,
+__global__ void __launch_bounds__(kThreads) k_cg_xr32(float* xc, float* r,
+                                                      const float* p,
+                                                      const float* p_alt,
                                                       const double* parity,
-                                                      const float* __restrict__ Ap, int n,
+                                                      const float* Ap, int n,
                                                       const double* alpha_p,
                                                       double* partials, unsigned int* counter,
                                                       double* dsc, double qnorm, double eps2,
@@ -532,10 +532,10 @@ __global__ void __launch_bounds__(kThreads) k_cg_xr32(float* __restrict__ xc, fl
   const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
   // four nodes per access (the vectors are 256-byte aligned allocations)
   const int n4 = n >> 2;
-  float4* __restrict__ xc4 = reinterpret_cast<float4*>(xc);
-  float4* __restrict__ r4 = reinterpret_cast<float4*>(r);
-  const float4* __restrict__ p4 = reinterpret_cast<const float4*>(p);
-  const float4* __restrict__ a4 = reinterpret_cast<const float4*>(Ap);
+  float4* xc4 = reinterpret_cast<float4*>(xc);
+  float4* r4 = reinterpret_cast<float4*>(r);
+  const float4* p4 = reinterpret_cast<const float4*>(p);
+  const float4* a4 = reinterpret_cast<const float4*>(Ap);
   auto step = [&](float4& xv, float4& rv, const float4& pv, const float4& av) {
     xv.x = fmaf(alpha, pv.x, xv.x);
     xv.y = fmaf(alpha, pv.y, xv.y);

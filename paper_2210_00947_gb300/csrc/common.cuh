@@ -317,19 +317,14 @@ struct CoarseT {
 // first thing, a hardware wait until the predecessor has completed and its
 // memory is visible, so only launch latency and block dispatch overlap.
 // pdl_trigger() lets the successor be dispatched before this grid ends.
-// A load through a const __restrict__ pointer may be moved over the wait: it
-// reads memory that the compiler takes to be constant, which neither the
-// memory clobber nor the wait itself orders.  In straight-line code it was (a
-// row read its operand, and a CG update its alpha, before the predecessor had
-// written them).  So the wait ends with a branch that no compiler stage can
-// decide and that is never taken (no SM has that number), and scalars written
-// by a predecessor come through plain pointers.
-__device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  unsigned sm;
-  asm volatile("mov.u32 %0, %%smid;" : "=r"(sm)::"memory");
-  if (sm == 0xffffffffu) asm volatile("exit;" ::: "memory");
-}
+// What the predecessor writes is read through plain pointers: the wait's memory
+// clobber keeps those loads behind it.  A load through a __restrict__ pointer of
+// the kernel may be moved over the wait, since the compiler takes its memory to
+// be no one else's (in straight-line code it was: a row read its operand, and a
+// CG update its alpha, before the predecessor had written them).  __restrict__
+// is for what was complete before the predecessor started (stencils, inverse
+// diagonals, conductivities, masks).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // handle whose API call is running on this host thread (set by the C ABI)
@@ -1119,7 +1114,7 @@ __device__ __forceinline__ void stencil_coefs(const StencilOp<Real>& op, int i, 
 }
 
 template <int DIM, typename Real, bool CG = false>
-__device__ __forceinline__ Real stencil_apply(const StencilOp<Real>& op, const Real* __restrict__ x,
+__device__ __forceinline__ Real stencil_apply(const StencilOp<Real>& op, const Real* x,
                                               int i, int j, int k,
                                               const Real (&sv)[stencil_size<DIM>()]) {
   const int NX = op.NX, NXY = op.NX * op.NY;
@@ -1191,7 +1186,7 @@ __device__ __forceinline__ Real stencil_apply_flat(const StencilOp<Real>& op, co
 // The whole row: coefficients and operand values loaded before the first
 // product, so a row costs one memory round trip.
 template <typename Real, bool CG = false>
-__device__ __forceinline__ Real stencil_row2(const StencilOp<Real>& op, const Real* __restrict__ x,
+__device__ __forceinline__ Real stencil_row2(const StencilOp<Real>& op, const Real* x,
                                              int i, int j) {
   Real sv[9];
   stencil_coefs<2>(op, i, j, 0, sv);
@@ -1199,7 +1194,7 @@ __device__ __forceinline__ Real stencil_row2(const StencilOp<Real>& op, const Re
 }
 
 template <typename Real, bool CG = false>
-__device__ __forceinline__ Real stencil_row3(const StencilOp<Real>& op, const Real* __restrict__ x,
+__device__ __forceinline__ Real stencil_row3(const StencilOp<Real>& op, const Real* x,
                                              int i, int j, int k) {
   Real sv[27];
   stencil_coefs<3>(op, i, j, k, sv);

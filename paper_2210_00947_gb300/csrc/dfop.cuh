@@ -157,9 +157,9 @@ struct DfDirSmem {
 };
 
 __device__ __forceinline__ void df_dir_tile(DfDirSmem& s, const DfOp& op, int tx, int ty,
-                                          const float* __restrict__ z,
-                                          const float2* __restrict__ p_old, bool first, df beta,
-                                          float2* __restrict__ pn, float2* __restrict__ y) {
+                                          const float* z,
+                                          const float2* p_old, bool first, df beta,
+                                          float2* pn, float2* y) {
   using namespace l2d;
   constexpr int kUY = Geo<kR>::kUY;
   const int fx0 = tx * kUX - 1, fy0 = ty * kUY - 1;

@@ -223,9 +223,9 @@ struct DownSmem {
 // null) xc of the tile's coarse nodes.
 template <typename Real, int R, bool ZERO>
 __device__ __forceinline__ void fine_down(DownSmem<Real, R>& s, const Fine<Real>& f, int tx, int ty,
-                                          const Real* __restrict__ b, Real* __restrict__ t,
-                                          Real* __restrict__ bc, const Real* __restrict__ dinvc,
-                                          Real* __restrict__ xc) {
+                                          const Real* b, Real* t,
+                                          Real* bc, const Real* __restrict__ dinvc,
+                                          Real* xc) {
   constexpr int kCY = Geo<R>::kCY;
   const int NX = f.ex + 1, NY = f.ey + 1;
   const int I0 = tx * kCX, J0 = ty * kCY;
@@ -319,8 +319,8 @@ struct UpSmem {
 // is called for every node of the tile.
 template <typename Real, int R, class Dot>
 __device__ __forceinline__ void fine_up(UpSmem<Real, R>& s, const Fine<Real>& f, int tx, int ty,
-                                        const Real* __restrict__ b, const Real* __restrict__ t,
-                                        const Real* __restrict__ res, Real* __restrict__ xout,
+                                        const Real* b, const Real* t,
+                                        const Real* res, Real* xout,
                                         Dot&& dot) {
   constexpr int kUY = Geo<R>::kUY, CR = Geo<R>::kRows / 2 + 2, CC = kW / 2 + 2;
   const int NX = f.ex + 1, NY = f.ey + 1;
@@ -408,9 +408,9 @@ struct DirSmem {
 template <int R>
 __device__ __forceinline__ double fine_dir(DirSmem<R>& s, const double* __restrict__ ke,
                                            const uint8_t* __restrict__ fixed, int ex, int ey, int tx,
-                                           int ty, const double* __restrict__ z,
-                                           const double* __restrict__ p_old, bool first, double beta,
-                                           double* __restrict__ pn, double* __restrict__ y) {
+                                           int ty, const double* z,
+                                           const double* p_old, bool first, double beta,
+                                           double* pn, double* y) {
   constexpr int kUY = Geo<R>::kUY;
   const int NX = ex + 1, NY = ey + 1;
   const int fx0 = tx * kUX - 1, fy0 = ty * kUY - 1;
@@ -461,9 +461,9 @@ __device__ __forceinline__ double fine_dir(DirSmem<R>& s, const double* __restri
 // ------------------------------------------------------------- coarse, down
 template <typename Real>
 __device__ __forceinline__ void coarse_down(Real (*s)[32], const Coarse<Real>& f, int tx, int ty,
-                                            const Real* __restrict__ b, const Real* __restrict__ x,
-                                            Real* __restrict__ bc, const Real* __restrict__ dinvc,
-                                            Real* __restrict__ xc) {
+                                            const Real* b, const Real* x,
+                                            Real* bc, const Real* __restrict__ dinvc,
+                                            Real* xc) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int I0 = tx * kDX, J0 = ty * kDY;
   const int i = 2 * I0 - 1 + lane, j = 2 * J0 - 1 + w;
@@ -497,8 +497,8 @@ struct CoarseUpSmem {
 // all taps in one sum (prolong_node's).
 template <typename Real, bool AXES>
 __device__ __forceinline__ void coarse_up(CoarseUpSmem<Real>& s, const Coarse<Real>& f, int tx, int ty,
-                                          const Real* __restrict__ b, const Real* __restrict__ x,
-                                          const Real* __restrict__ res, Real* __restrict__ xout) {
+                                          const Real* b, const Real* x,
+                                          const Real* res, Real* xout) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int i = tx * kPX - 1 + lane, j = ty * kPY - 1 + w;
   const bool on = i >= 0 && i < f.op.NX && j >= 0 && j < f.op.NY;

@@ -39,7 +39,7 @@ __device__ __forceinline__ int prolong_taps(int i, int nf, int* idx, float* w) {
 
 // dst = cur + P xc at fine node idx (a fixed fine node keeps cur).
 template <typename Real, int DIM>
-__device__ __forceinline__ void prolong_node(const Real* __restrict__ xc, const Real* cur, Real* dst,
+__device__ __forceinline__ void prolong_node(const Real* xc, const Real* cur, Real* dst,
                                              const Dims& f, const Dims& cd,
                                              const uint8_t* __restrict__ fixed, int idx) {
   if (fixed && fixed[idx]) {
@@ -72,11 +72,11 @@ __device__ __forceinline__ void prolong_node(const Real* __restrict__ xc, const 
 // level, so its first sweep reduces to a residual.  The 3^d fine values are
 // loaded before the first product.
 template <typename Real, int DIM, bool CG>
-__device__ __forceinline__ void restrict_node(const Real* __restrict__ r, Real* __restrict__ bc,
+__device__ __forceinline__ void restrict_node(const Real* r, Real* bc,
                                               const Dims& f, const Dims& cd,
                                               const uint8_t* __restrict__ fixed, int idx,
                                               const Real* __restrict__ dinvc = nullptr,
-                                              Real omega = Real(0), Real* __restrict__ xc = nullptr) {
+                                              Real omega = Real(0), Real* xc = nullptr) {
   constexpr int NZ3 = DIM == 3 ? 3 : 1, NV = 9 * NZ3;
   int I, J, K;
   coords(idx, cd.fNX, cd.fNXY, I, J, K);
@@ -149,8 +149,8 @@ __device__ __forceinline__ void restrict_node(const Real* __restrict__ r, Real* 
 // that made b has already written that x, so the sweep and its residual
 // reduce to this.
 template <typename Real, int DIM, bool CG>
-__device__ __forceinline__ void resid_node(const StencilOp<Real>& op, const Real* __restrict__ b,
-                                           const Real* __restrict__ x, Real* __restrict__ r, int idx) {
+__device__ __forceinline__ void resid_node(const StencilOp<Real>& op, const Real* b,
+                                           const Real* x, Real* r, int idx) {
   int i, j, k;
   coords(idx, op.fNX, op.fNXY, i, j, k);
   const Real ax = DIM == 3 ? stencil_row3<Real, CG>(op, x, i, j, k) : stencil_row2<Real, CG>(op, x, i, j);
@@ -183,10 +183,10 @@ __device__ __forceinline__ void interp_axis(int f, int nf, int& c0, float (&w)[3
 // separably onto the 3^d fine positions.
 // PRE: the row's coefficients were gathered already (sv, slot order).
 template <typename Real, int DIM, bool CG, bool PRE = false>
-__device__ __forceinline__ void post_node(const StencilOp<Real>& op, const Real* __restrict__ xc,
-                                          const Real* __restrict__ cur, const Real* __restrict__ b,
+__device__ __forceinline__ void post_node(const StencilOp<Real>& op, const Real* xc,
+                                          const Real* cur, const Real* b,
                                           const Real* __restrict__ dinv, Real omega,
-                                          Real* __restrict__ dst, const Dims& f, const Dims& cd,
+                                          Real* dst, const Dims& f, const Dims& cd,
                                           int idx, const Real* sv = nullptr) {
   int i, j, k;
   coords(idx, op.fNX, op.fNXY, i, j, k);
@@ -259,8 +259,8 @@ __device__ __forceinline__ void post_node(const StencilOp<Real>& op, const Real*
 
 // x = C b with the explicit inverse of the coarsest operator (FP64 sums).
 template <typename Real, bool CG, typename M>
-__device__ __forceinline__ void coarse_row(const M* __restrict__ cinv, const Real* __restrict__ b,
-                                           Real* __restrict__ x, int n, int row, int lane) {
+__device__ __forceinline__ void coarse_row(const M* __restrict__ cinv, const Real* b,
+                                           Real* x, int n, int row, int lane) {
   M s = M(0);
   for (int j = lane; j < n; j += 32)
     if (CK((int64_t)row * n + j, (int64_t)n * n)) s += cinv[(int64_t)row * n + j] * (M)ldv<CG>(b + j);

@@ -93,9 +93,9 @@ __global__ void k_residual_norm(FineOp<double> op, const double* __restrict__ q,
 // x += alpha p; r -= alpha Ap; ||r||^2.  Two nodes per access (the solver's own
 // vectors are aligned; the caller's x need not be) and, as in dot, two blocks
 // per SM: with eight the FP64 shuffle trees took as long as the data.
-__global__ void __launch_bounds__(kThreads) k_cg_xr(double* __restrict__ x, double* __restrict__ r,
+__global__ void __launch_bounds__(kThreads) k_cg_xr(double* x, double* r,
                                                     const double* p,
-                                                    const double* __restrict__ Ap, int64_t n,
+                                                    const double* Ap, int64_t n,
                                                     const double* p_alt, const double* parity,
                                                     const double* alpha_p,
                                                     double* partials, unsigned int* counter,
@@ -106,21 +106,37 @@ __global__ void __launch_bounds__(kThreads) k_cg_xr(double* __restrict__ x, doub
   double v[1] = {0.0};
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, n2 = n >> 1;
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double2* __restrict__ r2 = reinterpret_cast<double2*>(r);
-  const double2* __restrict__ p2 = reinterpret_cast<const double2*>(p);
-  const double2* __restrict__ q2 = reinterpret_cast<const double2*>(Ap);
-#pragma unroll 2
-  for (int64_t i = t0; i < n2; i += stride) {
-    const double xa = x[2 * i], xb = x[2 * i + 1];
-    const double2 pv = p2[i], qv = q2[i];
-    double2 rv = r2[i];
-    x[2 * i] = xa + alpha * pv.x;
-    x[2 * i + 1] = xb + alpha * pv.y;
-    rv.x -= alpha * qv.x;
-    rv.y -= alpha * qv.y;
-    r2[i] = rv;
-    v[0] += rv.x * rv.x;
-    v[0] += rv.y * rv.y;
+  double2* r2 = reinterpret_cast<double2*>(r);
+  const double2* p2 = reinterpret_cast<const double2*>(p);
+  const double2* q2 = reinterpret_cast<const double2*>(Ap);
+  // two accesses in flight
+  for (int64_t i = t0; i < n2; i += 2 * stride) {
+    double xa[2], xb[2];
+    double2 pv[2], qv[2], rv[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int64_t j = i + u * stride;
+      if (j < n2) {
+        xa[u] = x[2 * j];
+        xb[u] = x[2 * j + 1];
+        pv[u] = p2[j];
+        qv[u] = q2[j];
+        rv[u] = r2[j];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int64_t j = i + u * stride;
+      if (j < n2) {
+        x[2 * j] = xa[u] + alpha * pv[u].x;
+        x[2 * j + 1] = xb[u] + alpha * pv[u].y;
+        rv[u].x -= alpha * qv[u].x;
+        rv[u].y -= alpha * qv[u].y;
+        r2[j] = rv[u];
+        v[0] += rv[u].x * rv[u].x;
+        v[0] += rv[u].y * rv[u].y;
+      }
+    }
   }
   if ((n & 1) && t0 == 0) {
     x[n - 1] += alpha * p[n - 1];

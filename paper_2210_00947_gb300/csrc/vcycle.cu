@@ -96,20 +96,20 @@ __global__ void k_apply(Row row, const Real* __restrict__ x, Real* __restrict__ 
 
 // The 2D levels' tiled passes (level2d.cuh).
 template <typename Real, int R, bool ZERO>
-__global__ void __launch_bounds__(l2d::kThreads2) k_down2d(l2d::Fine<Real> f, const Real* __restrict__ b,
-                                                           Real* __restrict__ t, Real* __restrict__ bc,
+__global__ void __launch_bounds__(l2d::kThreads2) k_down2d(l2d::Fine<Real> f, const Real* b,
+                                                           Real* t, Real* bc,
                                                            const Real* __restrict__ dinvc,
-                                                           Real* __restrict__ xc) {
+                                                           Real* xc) {
   __shared__ l2d::DownSmem<Real, R> s;
   l2d::fine_down<Real, R, ZERO>(s, f, blockIdx.x, blockIdx.y, b, t, bc, dinvc, xc);
 }
 
 // DOT (FP64): also b . xout into dout.
 template <typename Real, int R, bool DOT>
-__global__ void __launch_bounds__(l2d::kThreads2) k_up2d(l2d::Fine<Real> f, const Real* __restrict__ b,
-                                                         const Real* __restrict__ t,
-                                                         const Real* __restrict__ res,
-                                                         Real* __restrict__ xout, double* partials,
+__global__ void __launch_bounds__(l2d::kThreads2) k_up2d(l2d::Fine<Real> f, const Real* b,
+                                                         const Real* t,
+                                                         const Real* res,
+                                                         Real* xout, double* partials,
                                                          unsigned int* counter, SumOut dout) {
   __shared__ l2d::UpSmem<Real, R> s;
   double acc[1] = {0.0};
@@ -157,11 +157,11 @@ __global__ void __launch_bounds__(kThreads) k_dot_rz(const float2* r, const floa
 template <int R>
 __global__ void __launch_bounds__(l2d::kThreads2) k_dir2d(const double* __restrict__ ke,
                                                           const uint8_t* __restrict__ fixed, int ex,
-                                                          int ey, const double* __restrict__ z,
+                                                          int ey, const double* z,
                                                           const double* p_old, double* p,
                                                           const double* beta, int first,
                                                           const double* parity,
-                                                          double* __restrict__ y, double* partials,
+                                                          double* y, double* partials,
                                                           unsigned int* counter, SumOut out) {
   __shared__ l2d::DirSmem<R> s;
   pdl_wait();
@@ -183,29 +183,29 @@ __global__ void __launch_bounds__(l2d::kThreads2) k_dir2d(const double* __restri
 
 template <typename Real>
 __global__ void __launch_bounds__(l2d::kDownThreads) k_coarse_down2d(l2d::Coarse<Real> f,
-                                                                     const Real* __restrict__ b,
-                                                                     const Real* __restrict__ x,
-                                                                     Real* __restrict__ bc,
+                                                                     const Real* b,
+                                                                     const Real* x,
+                                                                     Real* bc,
                                                                      const Real* __restrict__ dinvc,
-                                                                     Real* __restrict__ xc) {
+                                                                     Real* xc) {
   __shared__ Real s[2 * l2d::kDY + 1][32];
   l2d::coarse_down<Real>(s, f, blockIdx.x, blockIdx.y, b, x, bc, dinvc, xc);
 }
 
 template <typename Real, bool AXES>
 __global__ void __launch_bounds__(l2d::kUpThreads) k_coarse_up2d(l2d::Coarse<Real> f,
-                                                                 const Real* __restrict__ b,
-                                                                 const Real* __restrict__ x,
-                                                                 const Real* __restrict__ res,
-                                                                 Real* __restrict__ xout) {
+                                                                 const Real* b,
+                                                                 const Real* x,
+                                                                 const Real* res,
+                                                                 Real* xout) {
   __shared__ l2d::CoarseUpSmem<Real> s;
   l2d::coarse_up<Real, AXES>(s, f, blockIdx.x, blockIdx.y, b, x, res, xout);
 }
 
 template <typename Real, int DIM>
-__global__ void k_restrict(const Real* __restrict__ r, Real* __restrict__ bc, Dims f, Dims cd,
+__global__ void k_restrict(const Real* r, Real* bc, Dims f, Dims cd,
                            const uint8_t* __restrict__ fixed, const Real* __restrict__ dinvc = nullptr,
-                           Real omega = Real(0), Real* __restrict__ xc = nullptr) {
+                           Real omega = Real(0), Real* xc = nullptr) {
   pdl_wait();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx < cd.n) restrict_node<Real, DIM, false>(r, bc, f, cd, fixed, idx, dinvc, omega, xc);
@@ -214,7 +214,7 @@ __global__ void k_restrict(const Real* __restrict__ r, Real* __restrict__ bc, Di
 
 // dst = cur + P xc (fixed fine nodes keep cur); dst may equal cur.
 template <typename Real, int DIM>
-__global__ void k_prolong(const Real* __restrict__ xc, const Real* cur, Real* dst, Dims f, Dims cd,
+__global__ void k_prolong(const Real* xc, const Real* cur, Real* dst, Dims f, Dims cd,
                           const uint8_t* __restrict__ fixed) {
   pdl_wait();
   pdl_trigger();
@@ -231,7 +231,7 @@ __global__ void k_prolong(const Real* __restrict__ xc, const Real* cur, Real* ds
 constexpr int kProlongChunk = 8;
 
 template <typename Real>
-__global__ void k_prolong3(const Real* __restrict__ xc, const Real* cur, Real* dst, Dims f, Dims cd,
+__global__ void k_prolong3(const Real* xc, const Real* cur, Real* dst, Dims f, Dims cd,
                            const uint8_t* __restrict__ fixed) {
   constexpr int KC = kProlongChunk, NP = KC / 2 + 1;
   pdl_wait();
@@ -428,9 +428,9 @@ __global__ void k_restrict3(const float* r, float* bc, Dims f, Dims cd,
 }
 
 template <typename Real, int DIM>
-__global__ void k_post_coarse(StencilOp<Real> op, const Real* __restrict__ xc,
-                              const Real* __restrict__ cur, const Real* __restrict__ b,
-                              const Real* __restrict__ dinv, Real omega, Real* __restrict__ dst,
+__global__ void k_post_coarse(StencilOp<Real> op, const Real* xc,
+                              const Real* cur, const Real* b,
+                              const Real* __restrict__ dinv, Real omega, Real* dst,
                               Dims f, Dims cd) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   const bool on = idx < op.n;
@@ -483,8 +483,8 @@ __global__ void k_jacobi_st(StencilOp<Real> op, const Real* b, const Real* xin, 
 // row, the row's entries loaded before the wait when it has at most 128
 // (four per lane), summed in the same order as coarse_row.
 template <typename Real, typename M>
-__global__ void k_coarse_solve(const M* __restrict__ cinv, const Real* __restrict__ b,
-                               Real* __restrict__ x, int n) {
+__global__ void k_coarse_solve(const M* __restrict__ cinv, const Real* b,
+                               Real* x, int n) {
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   const bool pre = n <= 128;
