@@ -425,6 +425,7 @@ int mgar_create(mgar_t* out, const mgar_params* p, const uint8_t* fixed_mask, co
     // debugging aid: MGAR_NO_GRAPHS=1 issues every V-cycle launch directly
     if (const char* ng = std::getenv("MGAR_NO_GRAPHS")) c->use_graphs = !(ng[0] == '1');
     if (const char* ut = std::getenv("MGAR_UNTILED")) c->untiled = (ut[0] == '1');
+    if (c->dim == 2 && !tiles2d_ok(*c)) c->untiled = true;
     bottom_prepare(*c);
     if (const char* np = std::getenv("MGAR_NO_PDL")) c->use_pdl = np[0] != '1';
     if (const char* ng = std::getenv("MGAR_NO_CG_GRAPH")) c->cg_graph = ng[0] != '1';

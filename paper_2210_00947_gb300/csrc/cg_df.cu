@@ -52,7 +52,8 @@ __global__ void __launch_bounds__(l2d::kThreads2) k_df_dir2(DfOp op, const float
     p = t;
   }
   const df b = first ? df{0.f, 0.f} : load_pair(beta);
-  df_dir_tile(s, op, blockIdx.x, blockIdx.y, z, p_old, first != 0, b, p, y);
+  // (the rows of tiles of a long domain go on along z, the last few past the grid)
+  df_dir_tile(s, op, blockIdx.x, blockIdx.y + gridDim.y * blockIdx.z, z, p_old, first != 0, b, p, y);
 }
 
 // p . y over the nodes in memory order (as the sum of r . z, it does not
@@ -90,7 +91,8 @@ SumOut rz_out(Ctx& c, int slot, int old) {
 
 void df_dir2(Ctx& c, const DfOp& op, const float2* p_old, float2* p, const double* rz, bool first,
              const double* parity) {
-  const dim3 grid(l2d::tiles(op.NX, l2d::kUX), l2d::tiles(op.NY, l2d::Geo<l2d::kR>::kUY));
+  const int rows = l2d::tiles(op.NY, l2d::Geo<l2d::kR>::kUY), slabs = l2d::tiles(rows, 65535);
+  const dim3 grid(l2d::tiles(op.NX, l2d::kUX), l2d::tiles(rows, slabs), slabs);
   launch_pdl(c.stream, c.use_pdl, k_df_dir2, grid, dim3(l2d::kThreads2), op, (const float*)c.x32,
              p_old, p, (const double*)(c.dsc + S_BETA), first ? 1 : 0, parity, c.df_Ap);
   MGAR_LAUNCH_CHECK();

@@ -239,7 +239,7 @@ struct Ctx {
   static constexpr int kGraphs = 16;
   GraphEntry graphs[kGraphs];
   bool use_graphs = true;
-  bool untiled = false;  // MGAR_UNTILED=1: generic finest-level kernels (debugging aid)
+  bool untiled = false;  // generic finest-level kernels: MGAR_UNTILED=1 (debugging aid), 2D domains too long for the tiles
   int f3d_gz[5] = {};     // z runs of the tiled finest-level kernels [mode]
   int df3d_gz[3] = {};    // z runs of the tiled df64 operator kernels [mode]
   int f64_gz[5] = {};     // z runs of the tiled FP64 kernels [mode]
@@ -1265,6 +1265,8 @@ void vcycle_dot(Ctx& c, const float* b, float* x, const float2* r, SumOut dout);
 void vcycle_dot64(Ctx& c, const double* b, double* x, SumOut dout);
 // launch shapes of the tiled kernels (occupancy query; call outside stream capture)
 void fine3d_prepare(Ctx& c);
+// vcycle.cu: the tiled 2D passes' launches are within the limits of a grid
+bool tiles2d_ok(const Ctx& c);
 // vcycle.cu: can the bottom levels run as one thread-block cluster launch
 void bottom_prepare(Ctx& c);
 // df3d.cu: tiled df64 finest-level operator (3D)

@@ -109,7 +109,10 @@ __global__ void __launch_bounds__(NT, R <= 4 ? 3 : 2)
     dmx[q] = cls->dmax[q];
     for (int d = 0; d <= R; ++d) wt[q][d] = cls->w[q][d];
   }
-  const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
+  // (a plane's tiles numbered along x alone: their rows may pass the second
+  // dimension's 65535)
+  const int ntx = (ex + TX - 1) / TX, by = blockIdx.x / ntx;
+  const int i0 = (blockIdx.x - by * ntx) * TX, j0 = by * TY;
   const int z0 = (int)((int64_t)blockIdx.z * ez / runs), z1 = (int)((int64_t)(blockIdx.z + 1) * ez / runs);
   const int i = i0 + tx, j = j0 + ty;
   const bool mine = i < ex && j < ey;
@@ -212,7 +215,7 @@ void launch_r(Ctx& c, const float2* in, const Out& out) {
   MGAR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter3<R, Out>, NT, 0));
   const int want = std::max(1, std::max(per_sm, 1) * c.sms / (gx * gy));
   const int runs = std::max(1, std::min(want, d.ez / (2 * R)));
-  k_filter3<R, Out><<<dim3(gx, gy, runs), NT, 0, c.stream>>>(
+  k_filter3<R, Out><<<dim3(gx * gy, 1, runs), NT, 0, c.stream>>>(
       in, reinterpret_cast<const Classes*>(c.f_cls), d.ex, d.ey, d.ez, runs, out);
   MGAR_LAUNCH_CHECK();
 }

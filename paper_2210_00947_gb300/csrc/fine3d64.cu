@@ -63,7 +63,10 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 3 : 2) k_fine64(Args a)
   pdl_trigger();
   const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
   const bool real = tid < NT;
-  const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
+  // (a plane's tiles numbered along x alone: their rows may pass the second
+  // dimension's 65535)
+  const int ntx = (a.NX + TX - 1) / TX, by = blockIdx.x / ntx;
+  const int i0 = (blockIdx.x - by * ntx) * TX, j0 = by * TY;
   const int kb = (int)(((int64_t)blockIdx.z * a.NZ) / a.gz);
   const int kend = (int)(((int64_t)(blockIdx.z + 1) * a.NZ) / a.gz);
   const int i = i0 + tx, j = j0 + ty, NXY = a.NX * a.NY;
@@ -269,8 +272,8 @@ __global__ void __launch_bounds__(T::NTB, T::NT <= 256 ? 3 : 2) k_fine64(Args a)
   if (sum) {
     const double other = sum_other(a.dout, tid == 0);
     double t[1];
-    const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    const int nb = gridDim.x * gridDim.y * gridDim.z;
+    const int bid = blockIdx.x + gridDim.x * blockIdx.z;
+    const int nb = gridDim.x * gridDim.z;
     if (block_sum_last_ids<1>(acc, a.partials, a.counter, t, tid, T::NTB, bid, nb) && tid == 0)
       sum_out(a.dout, t[0], other);
   }
@@ -304,7 +307,7 @@ template <int MODE, class T>
 void launch_t(Ctx& c, Args& a) {
   const Dims& d = c.L[0];
   a.gz = std::max(1, c.f64_gz[MODE]);
-  const dim3 grid((d.NX + T::TX - 1) / T::TX, (d.NY + T::TY - 1) / T::TY, a.gz);
+  const dim3 grid(((d.NX + T::TX - 1) / T::TX) * ((d.NY + T::TY - 1) / T::TY), 1, a.gz);
   launch_pdl(c.stream, c.use_pdl, k_fine64<MODE, T>, grid, dim3(T::NTB), a);
 }
 template <int MODE>

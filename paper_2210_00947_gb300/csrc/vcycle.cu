@@ -387,9 +387,11 @@ constexpr int kRestrictChunk = 2;
 __global__ void k_restrict3(const float* r, float* bc, Dims f, Dims cd,
                             const float* __restrict__ dinvc, float omega, float* xc) {
   constexpr int KC = kRestrictChunk, NP = 2 * KC + 1;
-  const int cNXY = cd.NX * cd.NY, col = blockIdx.x * blockDim.x + threadIdx.x;
+  // (blocks numbered along x alone: planes may pass the second dimension's 65535)
+  const int cNXY = cd.NX * cd.NY, blocks = (cNXY + (int)blockDim.x - 1) / (int)blockDim.x;
+  const int chunk = blockIdx.x / blocks, col = (blockIdx.x - chunk * blocks) * blockDim.x + threadIdx.x;
   const bool on = col < cNXY;
-  const int J = on ? col / cd.NX : 0, I = on ? col - J * cd.NX : 0, K0 = blockIdx.y * KC;
+  const int J = on ? col / cd.NX : 0, I = on ? col - J * cd.NX : 0, K0 = chunk * KC;
   int ix[3], iy[3];
   float wx[3], wy[3];
   restrict_taps(I, f.ex, ix, wx);
@@ -758,6 +760,21 @@ static void with_rows(int rows, F&& f) {
   else f(std::integral_constant<int, 1>{});
 }
 
+// Whether the tiled 2D passes can be launched: their rows of tiles are a launch's
+// second dimension, which ends at 65535 (a domain of some 390,000 rows; longer
+// ones take the general kernels).
+bool tiles2d_ok(const Ctx& c) {
+  using namespace l2d;
+  constexpr int kMax = 65535;
+  const int cy[4] = {0, Geo<1>::kCY, Geo<2>::kCY, Geo<3>::kCY}, uy[4] = {0, Geo<1>::kUY, Geo<2>::kUY, Geo<3>::kUY};
+  const Dims &d0 = c.L[0], &d1 = c.L[1];
+  if (tiles(d1.NY, cy[down_rows(d1.NX, d1.NY, c.sms)]) > kMax) return false;
+  if (tiles(d0.NY, uy[up_rows(d0.NX, d0.NY, c.sms)]) > kMax) return false;
+  for (int l = 1; l + 1 < c.nl; ++l)
+    if (tiles(c.L[l + 1].NY, kDY) > kMax || tiles(c.L[l].NY, kPY) > kMax) return false;
+  return true;
+}
+
 // The 2D V-cycle with one pre- and one post-sweep in the tiled passes: one
 // launch per level and direction and the coarsest solve, in either precision
 // (FP64 gains from the passes saved and, on small grids, from 2 instead of 5
@@ -865,7 +882,7 @@ static void vcycle_fused3(Ctx& c, const Real* b0, Real* x0, bool zero_guess,
     columns = d1.n > c.split_coarse_nodes;
     if (columns)
       launch_pdl(c.stream, c.use_pdl, k_restrict3,
-                 dim3(blocks_for((int64_t)d1.NX * d1.NY), (d1.NZ + kRestrictChunk - 1) / kRestrictChunk),
+                 dim3(blocks_for((int64_t)d1.NX * d1.NY) * ((d1.NZ + kRestrictChunk - 1) / kRestrictChunk)),
                  dim3(kThreads), (const float*)h[0].r, h[1].b, d0, d1, (const float*)h[1].dinv, om, x1);
   }
   if (!columns) {
