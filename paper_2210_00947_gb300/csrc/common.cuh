@@ -850,18 +850,6 @@ __device__ __forceinline__ void block_sum_finish_df(df v, double* partials, unsi
     sum_out(out, t, other);
 }
 
-// *a / *b for the whole block as a df64 pair, computed once by thread 0.
-// Every thread of the block must call it, once per kernel.
-__device__ __forceinline__ df block_div_df(const double* a, const double* b) {
-  __shared__ float2 s;
-  if (threadIdx.x == 0) {
-    const df d = df_from_double(*a / *b);
-    s = make_float2(d.hi, d.lo);
-  }
-  __syncthreads();
-  return df{s.x, s.y};
-}
-
 // The test of a device-side CG loop, in the last block of an update of x and
 // r: count the iteration, flip the parity, and continue while ||r|| / ||q|| >
 // eps2 (the host loop's test, same arithmetic) and fewer than cg_max
@@ -1279,7 +1267,6 @@ void df3d_dir(Ctx& c, const float* z, const float2* p_old, float2* p, const doub
               float2* y, SumOut dot, const double* parity = nullptr);
 void df3d_resid(Ctx& c, const float2* q, const float2* x, float2* r, float* r32, double* rr);
 void apply_fine64(Ctx& c, const double* ke, const double* x, double* y, SumOut dot_out = {});
-void apply_fine32(Ctx& c, const float* ke, const float* x, float* y);
 void apply_dK64(Ctx& c, const double* x, double* y);
 void apply_dK32(Ctx& c, const float* x, float* y);
 void convert_d2f(Ctx& c, const double* a, float* b, int64_t n);

@@ -1556,7 +1556,6 @@ void postprocess(Ctx& c, const double* rho, const double* T, double volfrac, dou
     k_elem_sens<3><<<blocks_for(ne), kThreads, 0, c.stream>>>(T, c.rho_phys, c.tmp_e, d, coef,
                                                               c.p.penal);
   MGAR_LAUNCH_CHECK();
-  const double r = c.p.rmin;
   double* ns = c.tm;
   float* ns32 = reinterpret_cast<float*>(c.pv);
   PpCtrl* ctrl = reinterpret_cast<PpCtrl*>(c.pp_ctrl);

@@ -70,17 +70,6 @@ __device__ __forceinline__ df df_mulf(df a, float b) {
   return df_make(p, e);
 }
 
-// (ah, al) += a * b for a float b, the pair left unnormalised: the product's
-// high part added by TwoSum, every rounding error gathered in al
-__device__ __forceinline__ void df_acc_mulf(float& ah, float& al, df a, float b) {
-  float p, pe, t, te;
-  two_prod(a.hi, b, p, pe);
-  pe = __fmaf_rn(a.lo, b, pe);
-  two_sum(ah, p, t, te);
-  ah = t;
-  al = __fadd_rn(al, __fadd_rn(te, pe));
-}
-
 // 1 / sqrt(a), a > 0: an FP32 seed and two Newton steps y <- y + y (1 - a y^2) / 2
 // with the residual 1 - a y^2 formed in df64 (each step doubles the correct bits)
 __device__ __forceinline__ df df_rsqrt(df a) {

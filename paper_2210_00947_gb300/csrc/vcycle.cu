@@ -1081,10 +1081,6 @@ void apply_fine64(Ctx& c, const double* ke, const double* x, double* y, SumOut d
   else if (!c.untiled) fine3d_apply64(c, ke, nullptr, x, y, 1.0, dot_out);
   else apply_dim<double, 3>(c, ke, nullptr, x, y, 1.0, dot_out);
 }
-void apply_fine32(Ctx& c, const float* ke, const float* x, float* y) {
-  if (c.dim == 2) apply_dim<float, 2>(c, ke, nullptr, x, y, 1.f, {});
-  else apply_dim<float, 3>(c, ke, nullptr, x, y, 1.f, {});
-}
 // y = -(A - A0) x
 void apply_dK64(Ctx& c, const double* x, double* y) {
   if (c.dim == 2) apply_dim<double, 2>(c, c.ke, c.ke0, x, y, -1.0, {});
