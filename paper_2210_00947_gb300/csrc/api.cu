@@ -426,7 +426,9 @@ int mgar_create(mgar_t* out, const mgar_params* p, const uint8_t* fixed_mask, co
     if (const char* ng = std::getenv("MGAR_NO_GRAPHS")) c->use_graphs = !(ng[0] == '1');
     if (const char* ut = std::getenv("MGAR_UNTILED")) c->untiled = (ut[0] == '1');
     if (c->dim == 2 && !tiles2d_ok(*c)) c->untiled = true;
-    bottom_prepare(*c);
+    // 3D: the bottom levels as one cluster launch, measured 2 % slower per design
+    // cycle than their separate launches, so only on request
+    if (const char* cb = std::getenv("MGAR_CLUSTER_BOTTOM"); cb && cb[0] == '1') bottom_prepare(*c);
     if (const char* np = std::getenv("MGAR_NO_PDL")) c->use_pdl = np[0] != '1';
     if (const char* ng = std::getenv("MGAR_NO_CG_GRAPH")) c->cg_graph = ng[0] != '1';
     if (const char* dc = std::getenv("MGAR_DF64_CG")) c->ru_cg = dc[0] != '1';
@@ -435,12 +437,6 @@ int mgar_create(mgar_t* out, const mgar_params* p, const uint8_t* fixed_mask, co
     if (const char* fp = std::getenv("MGAR_FUSED_POST")) c->split_post = fp[0] != '1';
     if (const char* sc = std::getenv("MGAR_SPLIT_COARSE")) c->split_coarse_nodes = std::atoll(sc);
     if (const char* bn = std::getenv("MGAR_BOTTOM_NODES")) c->bottom_nodes = std::atoll(bn);
-    // the bottom levels as one cluster launch: measured 2 % slower per design
-    // cycle than their separate launches, so only on request
-    {
-      const char* cb = std::getenv("MGAR_CLUSTER_BOTTOM");
-      c->bottom_ok = c->bottom_ok && cb && cb[0] == '1';
-    }
     if (const char* fc = std::getenv("MGAR_FP64_COARSE")) c->df_coarse = fc[0] != '1';
     if (c->dim == 3) {
       fine3d64_prepare(*c);

@@ -865,14 +865,15 @@ static bool ldl_factor(Ctx& c, cudaStream_t s) {
   MGAR_LAUNCH_CHECK();
   return true;
 }
+template <class Kernel>
+static void shared_memory(Kernel kernel) {
+  MGAR_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax));
+}
 template <class Ar>
 static void ldl_attributes() {
-  MGAR_CUDA(cudaFuncSetAttribute(k_band_ldl<Ar>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kBandSmemMax));
-  MGAR_CUDA(cudaFuncSetAttribute(k_band_ldl_inverse<Ar, 1>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax));
-  MGAR_CUDA(cudaFuncSetAttribute(k_band_ldl_inverse<Ar, 2>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax));
+  shared_memory(k_band_ldl<Ar>);
+  shared_memory(k_band_ldl_inverse<Ar, 1>);
+  shared_memory(k_band_ldl_inverse<Ar, 2>);
 }
 
 // ------------------------------------------------------------------- host
@@ -919,20 +920,20 @@ void alloc_hierarchy(Ctx& c) {
   MGAR_CUDA(cudaMalloc(&c.band, (size_t)c.nc * (c.bw + 1) * sizeof(double)));
   MGAR_CUDA(cudaMalloc(&c.rdiag, (size_t)c.nc * sizeof(double)));
   MGAR_CUDA(cudaMalloc(&c.cinv, (size_t)c.nc * c.nc * sizeof(double)));
-  MGAR_CUDA(cudaFuncSetAttribute(k_band_cholesky<double, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax));
-  MGAR_CUDA(cudaFuncSetAttribute(k_band_inverse<double, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax));
-  MGAR_CUDA(cudaFuncSetAttribute(k_band_cholesky<float, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax));
-  MGAR_CUDA(cudaFuncSetAttribute(k_band_inverse<float, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax));
-  MGAR_CUDA(cudaFuncSetAttribute(k_band_cholesky_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kBandSmemMax));
-  MGAR_CUDA(cudaFuncSetAttribute(k_band_inverse_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kBandSmemMax));
-  ldl_attributes<ArD>();
-  ldl_attributes<ArDf>();
+  // Kernels of the coarsest factor need an attribute for more than 48 KB of
+  // shared memory (1 KB of it left for their own); setting it loads them, a
+  // dozen kernels of which a handle uses two.
+  const size_t band_bytes = (size_t)c.nc * (c.bw + 1) * sizeof(double);
+  const size_t most = std::max({band_bytes + (size_t)8 * c.nc * sizeof(double), ldl_smem<ArD>(c.nc, c.bw),
+                                ldl_inverse_smem<ArD>(c.nc, c.bw, 8)});
+  if (most > 47 * 1024) {
+    shared_memory(k_band_cholesky<double, true>);
+    shared_memory(k_band_inverse<double, true>);
+    shared_memory(k_band_cholesky_df);
+    shared_memory(k_band_inverse_df);
+    ldl_attributes<ArD>();
+    ldl_attributes<ArDf>();
+  }
   // constant tables: k0 (nen^2) then G (3^dim * nen^2)
   const int nen = c.nen, ntypes = c.dim == 2 ? 9 : 27;
   std::vector<double> k0(nen * nen), G((size_t)ntypes * nen * nen, 0.0),
