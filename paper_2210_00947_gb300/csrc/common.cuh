@@ -128,7 +128,7 @@ template <typename Real>
 struct LevelBuf {
   Real* st = nullptr;    // [S][n] assembled stencil, levels >= 1
   Real* dinv = nullptr;  // [n] 1/diag, levels >= 1
-  Real* dinv_s = nullptr;  // [n] 2D, level 0: 1/diag, negated on fixed nodes
+  Real* dinv_s = nullptr;  // [n] level 0 (2D; 3D mixed): 1/diag, negated on fixed nodes
   Real* elem = nullptr;  // [ne][nen*nen] Galerkin element matrices, levels >= 1
   Real* x = nullptr;     // V-cycle iterate (levels >= 1; level 0 uses caller arrays)
   Real* b = nullptr;     // right-hand side (levels >= 1)

@@ -14,8 +14,8 @@
 // The residual never goes to memory.  1025^2 nodes in FP32: down 6.7 us (21.5
 // as three kernels), up 8.2 us (20 as two), a coarse level 2.6-5.3 us each way
 // (6-8); bound by instruction issue (100 warp instructions per node down, 130
-// up).  FP32 results are those of the separate passes bit for bit (the order
-// of a row's additions and its contractions are theirs).  Tiles are 64 columns wide with their
+// up).  FP32 results are those of the separate passes bit for bit (the mixed
+// 2D solves before and after were compared).  Tiles are 64 columns wide with their
 // rim (two nodes per lane), so a warp's rows are coalesced and no lane divides
 // to find its node; tall enough that the rim costs 8 % (residuals) to 24 %
 // (x) more, short enough that a 1024^2 grid fills the chip in one wave.
@@ -141,7 +141,8 @@ __device__ __forceinline__ void q4_rows(const Real (*x)[kW], const Real (*k)[kW]
     const Real s = k00 + k01, n = k10 + k11;
     f(q, yc, [&](Real xi) {
       if constexpr (sizeof(Real) == 4) {
-        // the order of fine_row2, as compiled
+        // fine_row2's order of additions, with the contractions that give its
+        // bits (found by comparing outputs)
         Real acc = __fmul_rn(__fmul_rn(4.f, s + n), xi);
         acc = __fmaf_rn(-(k00 + k10), yl, acc);
         acc = __fmaf_rn(-(k01 + k11), yr, acc);
