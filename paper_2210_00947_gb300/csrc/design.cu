@@ -1377,9 +1377,12 @@ __global__ void __launch_bounds__(512) k_pp_list(const float* __restrict__ ns32,
 
 // The bisection, one block: level L has the points above the last bracket
 // plus the listed values > L, and goes up while they are more than `want`.
-// out[0] = 2: not applicable; 0: done, level in out[1].
+// out[0] = 0: done, level in out[1]; 1: the level lies outside the bracket
+// (found for another target); 2: not applicable; 3: out[1] is a level with
+// `ask` points (met on the way, or the upper end of the bracket).
 __global__ void __launch_bounds__(1024) k_pp_bisect(const PpCtrl* c, const double* __restrict__ list,
-                                                    int cap, double top, double want, double* out) {
+                                                    int cap, double top, double want, double ask,
+                                                    double* out) {
   __shared__ int part[32];
   __shared__ int total;
   const int tid = threadIdx.x;
@@ -1389,37 +1392,57 @@ __global__ void __launch_bounds__(1024) k_pp_bisect(const PpCtrl* c, const doubl
   }
   const int n = (int)c->nlist;
   const double base = (double)c->above[2];
+  // points above a level within the bracket
+  auto above = [&](double level) {
+    int k = 0;
+    for (int q = tid; q < n; q += 1024) k += list[q] > level ? 1 : 0;
+    k = __reduce_add_sync(0xffffffffu, k);
+    if ((tid & 31) == 0) part[tid >> 5] = k;
+    __syncthreads();
+    if (tid < 32) {
+      const int s = __reduce_add_sync(0xffffffffu, part[tid]);
+      if (tid == 0) total = s;
+    }
+    __syncthreads();
+    const double count = base + (double)total;
+    __syncthreads();
+    return count;
+  };
   // outside [La, Lb] the answer is known (a bracket cut off at 0 knows nothing below)
   const double La = c->lo[2] ? (double)__uint_as_float(c->lo[2] + kPpGuard / 2) : -1.0;
   const double Lb = (double)__uint_as_float(c->hi[2] - kPpGuard / 2);
+  const double upper = above(Lb);
+  if ((La > 0.0 && !(above(La) > want)) || upper > want) {
+    if (tid == 0) out[0] = 1.0;
+    return;
+  }
+  auto answer = [&](double state, double level) {
+    if (tid == 0) {
+      out[0] = state;
+      out[1] = level;
+    }
+  };
+  if (upper == ask && Lb > 0.0) {
+    answer(3.0, Lb);
+    return;
+  }
   double lo = -1.0, hi = top;
   for (int step = 0; step < 200; ++step) {
     const double mid = 0.5 * (lo + hi);
     if (!(lo < mid && mid < hi)) break;
-    bool more;
-    if (mid <= La) more = true;
-    else if (mid >= Lb) more = false;
-    else {
-      int k = 0;
-      for (int q = tid; q < n; q += 1024) k += list[q] > mid ? 1 : 0;
-      k = __reduce_add_sync(0xffffffffu, k);
-      if ((tid & 31) == 0) part[tid >> 5] = k;
-      __syncthreads();
-      if (tid < 32) {
-        const int s = __reduce_add_sync(0xffffffffu, part[tid]);
-        if (tid == 0) total = s;
+    bool more = mid <= La;
+    if (!more && !(mid >= Lb)) {
+      const double count = above(mid);
+      if (count == ask) {
+        answer(3.0, mid);
+        return;
       }
-      __syncthreads();
-      more = base + (double)total > want;
-      __syncthreads();
+      more = count > want;
     }
     if (more) lo = mid;
     else hi = mid;
   }
-  if (tid == 0) {
-    out[0] = 0.0;
-    out[1] = hi;
-  }
+  answer(0.0, hi);
 }
 
 // k_pp_density for nodal values in [0, 1e37]: the same counts, the points
@@ -1592,12 +1615,12 @@ void postprocess(Ctx& c, const double* rho, const double* T, double volfrac, dou
     return c.hsc[S_TMP] / (double)ne;
   };
   // the level by counts of lattice points: the smallest whose points are at
-  // most `target`.  False: values outside [0, 1e37], or more equal values at
-  // the level than the list holds
+  // most `target`
   const double total = (c.dim == 3 ? 125.0 : 25.0) * (double)ne, want = volfrac * total;
   double* list = c.tmp_e;  // the element sensitivities are no longer needed
   const int hb = std::min(blocks_for(ne, 512), 4 * c.sms);
-  auto by_counts = [&](double target, double* level) {
+  // the bracket that holds the level, with its points listed
+  auto bracket = [&](double target) {
     MGAR_CUDA(cudaMemsetAsync(ctrl, 0, offsetof(PpCtrl, bad), c.stream));
     k_pp_first<<<1, 1, 0, c.stream>>>(ctrl);
     MGAR_LAUNCH_CHECK();
@@ -1611,33 +1634,44 @@ void postprocess(Ctx& c, const double* rho, const double* T, double volfrac, dou
     if (c.dim == 2) k_pp_list<2><<<hb, 512, 0, c.stream>>>(ns32, ns, d, ctrl, list, ne);
     else k_pp_list<3><<<hb, 512, 0, c.stream>>>(ns32, ns, d, ctrl, list, ne);
     MGAR_LAUNCH_CHECK();
-    k_pp_bisect<<<1, 1024, 0, c.stream>>>(ctrl, list, ne, top, target, c.dsc + S_GS);
+  };
+  double hi = top;
+  auto bisect = [&](double target, double ask) {
+    k_pp_bisect<<<1, 1024, 0, c.stream>>>(ctrl, list, ne, top, target, ask, c.dsc + S_GS);
     MGAR_LAUNCH_CHECK();
     fetch_scalars(c, S_GS, 2);
-    if (c.hsc[S_GS] != 0.0) return false;
-    *level = c.hsc[S_GS + 1];
-    return true;
+    hi = c.hsc[S_GS + 1];
+    return (int)c.hsc[S_GS];
   };
   // The comparison is the densities' FP64 sum's, within 1e-13 of the count's
   // share: where no whole number of points lies that close to the target, the
   // count decides it.  Otherwise the levels with that number of points are one
-  // plateau, on which the sum has one value.  The search first takes them as
-  // met (half a point more) and ends on the plateau's lower end; if its volume
-  // is above the fraction by rounding, they are not, and the level is that of
-  // half a point less, which may lie outside the first search's bracket.
+  // plateau, on which the densities and their sum are the same.  A search that
+  // meets it asks for them there: the level is the plateau's lower end (half a
+  // point more as the target) unless the volume is above the fraction by
+  // rounding, then the value above it (half a point less), mostly in the same
+  // bracket (neighbouring values further apart than that: one of their own).
   const double whole = std::nearbyint(want);
   const bool plateau = std::fabs(whole - want) <= 1e-12 * total;
-  double hi = top, v = 0.0;
-  bool found = by_counts(plateau ? whole + 0.5 : want, &hi);
-  if (found) {
+  double v = 0.0;
+  bracket(plateau ? whole + 0.5 : want);
+  int state = bisect(plateau ? whole + 0.5 : want, plateau ? whole : -1.0);
+  if (state == 3) {
     v = volume(hi, rho_out, true);
-    if (plateau && v > volfrac) {
-      found = by_counts(whole - 0.5, &hi);
-      if (found) v = volume(hi, rho_out, true);
+    const bool more = v > volfrac;
+    const double target = more ? whole - 0.5 : whole + 0.5;
+    state = bisect(target, -1.0);
+    if (state == 1) {
+      bracket(target);
+      state = bisect(target, -1.0);
     }
+    if (state == 0 && more) v = volume(hi, rho_out, true);
+  } else if (state == 0) {
+    v = volume(hi, rho_out, true);
   }
-  if (!found) {
-    // a volume per step.  ns >= 0: below -1 every node is above the level
+  if (state != 0) {
+    // values outside [0, 1e37], or more equal values at the level than the list
+    // holds: a volume per step.  ns >= 0: below -1 every node is above the level
     // (volume 1), at max(ns) none is (volume 0)
     double lo = -1.0;
     hi = top;
