@@ -1163,7 +1163,7 @@ __global__ void k_pp_nodal(const double* __restrict__ dcp, double* __restrict__ 
 // roundings), so every bracket is widened by kPpGuard ulps and a point outside
 // the last one is on the same side of every level in it in either precision.
 // A volume per bisection step instead, 62 passes at 4.6 ms on 128^3 (FP64-bound:
-// up to 5000 FP64 operations per element), took 290 ms; this takes 1.25 ms with
+// up to 5000 FP64 operations per element), took 290 ms; this takes 1.3 ms with
 // the projection, bound by the shared-memory atomics of the first histogram.
 constexpr unsigned kPpGuard = 64;
 constexpr int kPpShift1 = 19, kPpShift2 = 8;  // bits per bin: 2^31 in 4096 bins, then 2^19 in 2050
